@@ -9,6 +9,7 @@
 #include <cstring>
 #include <deque>
 #include <string>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -18,6 +19,7 @@
 #include "../../include/spm.h"
 #include "ffn_gemv.cuh"
 #include "ffn_gemv_q4.cuh"
+#include "ffn_multi.cuh"
 #include "ffn_grouped.cuh"
 #include "ffn_grouped_q4.cuh"
 #include "router_adapter.cuh"
@@ -56,6 +58,8 @@ struct spm_ctx {
     unsigned char* pools = nullptr;
     float *ws_x = nullptr, *ws_logits = nullptr, *ws_pihat = nullptr, *ws_w = nullptr;
     float *ws_scores = nullptr, *ws_partial = nullptr, *ws_h = nullptr;
+    float* mt_partial = nullptr;              // batched fp32-activation path (max_batch > 1): partial rows of ffn_multi_kernel
+    int32_t* mt_map = nullptr;                //   and where each (token, k) pair was computed
     int32_t *ws_ids = nullptr, *ws_order = nullptr;
     unsigned* ws_counters = nullptr;
     int* ws_status = nullptr;
@@ -225,6 +229,24 @@ int ffn_grid_for(const spm_ctx* c, int nb) {
     return std::max(1, kMaxCtasBatch1 / nb);
 }
 
+// CTAs of the several-sequences kernel (its workspace is sized for kMtMaxCtas)
+constexpr int kMtMaxCtas = 148;
+int mt_grid_for(const spm_ctx* c) { return std::min(c->num_sms, kMtMaxCtas); }
+// fp32-activation path of a batch. One GEMV per sequence reads an expert once per token that uses it; ffn_multi_kernel reads
+// it once per eight but has the longer chain of latencies (plan, split operands, a combine kernel instead of the fold
+// in the next routing kernel: some 17 us a layer). It pays from about 64 M weights on that are not read again; measured,
+// us a layer, GEMV per sequence -> several sequences at a time (saved reads in M weights):
+//   bf16 1280 x 896, 16 tokens 6 + 2 of 64:  120 -> 92 (213)    bf16 1280 x 200, 32 tokens 4 of 64:   48 -> 51 (49)
+//   bf16  512 x 250, 64 tokens 4 + 1 of 24:   68 -> 43 (113)    bf16  512 x 250, 16 tokens 4 + 1 of 24: 28 -> 33 (21)
+//   fp32 1024 x 250, 32 tokens 4 + 1 of 24:   66 -> 57 (104)    fp32 1024 x 250,  8 tokens 4 + 1 of 24: 27 -> 47 (12)
+//   4-bit 768 x 300, 64 tokens 4 + 1 of 60:  119 -> 63 (179)    4-bit 2048 x 500, 8 tokens 4 + 1 of 60: 50 -> 71 (0)
+constexpr size_t kMtMinSavedWeights = size_t(64) << 20;
+bool use_multi(const spm_ctx* c, int nb) {
+    const spm_model_cfg& m = c->cfg;
+    const int reads = nb * (m.top_k + m.n_shared), distinct = std::min(nb * m.top_k, m.n_experts) + m.n_shared;
+    return size_t(reads - distinct) * 3 * m.inter * m.hidden >= kMtMinSavedWeights;
+}
+
 struct Carve {
     size_t off = 0;
     size_t take(size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; }
@@ -232,6 +254,7 @@ struct Carve {
 
 struct Layout {
     size_t pools, slot_gen, x, logits, pihat, w, scores, partial, h, ids, order, clock, slot_map, codes, counters, status, total;
+    size_t mt_partial, mt_map;                                                     // max_batch > 1 only
     size_t tc_xs, tc_wrow, tc_partial, tc_desc, tc_counts, tc_act, tc_ready;       // batched tensor-core path only
     size_t desc_bytes, off_rows, off_rowmap, off_chunks, chunk_cap, off_wait;
     int rows_cap, n_jt, max_units;
@@ -250,6 +273,10 @@ Layout layout_of(const spm_model_cfg* m, int S) {
     l.w = c.take(nb * SPM_MAX_TOPK * 4);
     l.scores = c.take(n * 4);
     l.partial = c.take((kMaxCtasBatch1 + nb) * D * 4);
+    if (nb > 1) {
+        l.mt_partial = c.take(mt_partial_rows(kMtMaxCtas, m->max_batch, m->top_k, m->n_experts, m->n_shared) * D * 4);
+        l.mt_map = c.take((4 + nb * SPM_MAX_TOPK) * 4);
+    }
     l.h = c.take(nb * D * 4);
     l.ids = c.take(nb * SPM_MAX_TOPK * 4);
     l.order = c.take(n * 4);
@@ -366,6 +393,68 @@ cudaError_t launch_gemv(const spm_ctx* c, const FfnArgs<MAXNB>& a, int G, int nb
     const size_t smem = ffn_gemv_smem(c->row_bytes, warps, depth);
     if (c->cfg.dtype == SPM_DTYPE_BF16) return launch_gemv_seg<bf16_t, MAXNB>(c->nseg, a, G, nb, warps, depth, smem, c->compute, pdl);
     return launch_gemv_seg<float, MAXNB>(c->nseg, a, G, nb, warps, depth, smem, c->compute, pdl);
+}
+
+template <typename WT, int GB>
+cudaError_t launch_multi_t(const spm_ctx* c, const MtArgs& a) {
+    static bool attr_set[64] = {};          // the attribute is per device
+    auto kern = ffn_multi_kernel<WT, GB>;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFfnSmemLimit));
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    size_t smem = 0;
+    const int stages = mt_stages(c->row_bytes, std::is_same<WT, float>::value, a.n, a.nb * a.K, &smem);
+    return launch_k(kern, dim3(mt_grid_for(c)), dim3(kMtThreads), smem, c->compute, true, a, stages);
+}
+template <typename WT>
+cudaError_t launch_multi_g(const spm_ctx* c, const MtArgs& a) {
+    const int gb = (a.D / 32 + kMtWarps - 1) / kMtWarps;
+    switch (gb) {
+        case 1: return launch_multi_t<WT, 1>(c, a);
+        case 2: return launch_multi_t<WT, 2>(c, a);
+        case 3: return launch_multi_t<WT, 3>(c, a);
+        case 4: return launch_multi_t<WT, 4>(c, a);
+    }
+    if constexpr (sizeof(WT) != 4)      // (fp32: hidden <= 1024)
+        switch (gb) {
+            case 5: return launch_multi_t<WT, 5>(c, a);
+            case 6: return launch_multi_t<WT, 6>(c, a);
+            case 7: return launch_multi_t<WT, 7>(c, a);
+            case 8: return launch_multi_t<WT, 8>(c, a);
+        }
+    return cudaErrorInvalidValue;
+}
+
+// Expert FFN of several sequences with fp32 activations. In a host-free step the routing is
+// read on the device (`dev_ids`, `dev_slot`); otherwise `a.ids` / `a.slot` hold this wave's.
+int launch_multi(spm_ctx* c, int layer, MtArgs& a, const float* x, const float* w, unsigned long long* clock, bool with_shared) {
+    const spm_model_cfg& m = c->cfg;
+    a.pool = c->pools + size_t(layer) * c->S * c->blob;
+    a.shared = m.n_shared ? static_cast<const unsigned char*>(c->buf.shared_experts) + size_t(layer) * m.n_shared * c->blob : nullptr;
+    a.x = x;
+    a.w = w;
+    a.partial = c->mt_partial;
+    a.map = c->mt_map;
+    a.status = c->ws_status;
+    a.clock = clock;
+    a.blob_bytes = c->blob;
+    a.wait_limit_ns = c->wait_limit_ns;
+    a.D = m.hidden; a.I = m.inter; a.K = m.top_k; a.n = m.n_experts; a.n_slots = c->S; a.n_shared = with_shared ? m.n_shared : 0;
+    CU(c, m.dtype == SPM_DTYPE_FP32 ? launch_multi_g<float>(c, a) : m.dtype == SPM_DTYPE_BF16 ? launch_multi_g<uint16_t>(c, a) : launch_multi_g<Q4Tag>(c, a));
+    return SPM_OK;
+}
+int launch_multi_combine(spm_ctx* c, int nb, float* h, bool with_shared) {
+    const spm_model_cfg& m = c->cfg;
+    const int KS = m.top_k + (with_shared ? m.n_shared : 0);
+    unsigned long long* clock = nullptr;
+    if (int rc = take_clock(c, kClkReduce, &clock)) return rc;
+    CU(c, launch_k(mt_combine_kernel, dim3((m.hidden / 4 + 31) / 32, nb), dim3(32 * KS), 0, c->compute, true, (const float*)c->mt_partial,
+                   (const int32_t*)c->mt_map, KS, mt_grid_for(c), m.inter, m.hidden, h, clock));
+    return SPM_OK;
 }
 
 // Where a routing launch leaves its results besides the workspace: by default the context's
@@ -742,7 +831,9 @@ int launch_grouped_wave(spm_ctx* c, int layer, const float* x_norm, const int32_
 // With `launch` false only the slot table's side runs (the kernels of a host-free step were
 // enqueued earlier); a miss there would mean the step computed with a stale slot map.
 // With `leave_partial` the partial rows of the last wave stay in the workspace for the next
-// layer's routing kernel to fold into the hidden row (GEMV path only; reported through *left).
+// layer's routing kernel to fold into the hidden row (GEMV path only; reported through *left). After the grouped
+// and several-sequences kernels a combine kernel is faster than the fold in eight CTAs a token (routing kernel
+// 12.2 -> 21.6 us at 5 sequences of the Qwen3 shape, combine kernel and its launch gap 5.4 us).
 int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, const float* w, int nb,
             float* h_inout, Timing* t, int ring = -1, bool launch = true, bool leave_partial = false, bool* left = nullptr) {
     const spm_model_cfg& m = c->cfg;
@@ -771,7 +862,7 @@ int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, cons
     }
 
     const int G = ffn_grid_for(c, nb);
-    const bool use_tc = nb > 1 && c->tc_ok && c->batched_path == 0;
+    const bool use_tc = nb > 1 && c->tc_ok && c->batched_path == 0, multi = !use_tc && use_multi(c, nb);
     // kernels that can wait for a copy themselves: the batch-1 GEMV kernels and the grouped tensor-core kernels
     const bool dev_wait = c->device_wait && (nb == 1 || use_tc) && stream_write32_fn() != nullptr;
     std::vector<int16_t>& slot_of_expert = c->wave_slot;   // experts computed in the current wave
@@ -859,6 +950,14 @@ int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, cons
                 FfnArgs<1> a{};
                 fill(a);
                 CU(c, launch_gemv<1>(c, a, G, nb, true));
+            } else if (multi) {
+                MtArgs a;
+                a.dev_ids = nullptr;
+                a.dev_slot = nullptr;
+                a.nb = nb;
+                for (int i = 0; i < nb * K; ++i) a.ids[i] = short(ids[i]);
+                std::copy(slot_of_expert.begin(), slot_of_expert.end(), a.slot);
+                if (int rc = launch_multi(c, layer, a, x_norm, w, clock_slot, first)) return rc;
             } else {
                 FfnArgs<SPM_MAX_BATCH> a{};
                 fill(a);
@@ -866,7 +965,10 @@ int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, cons
             }
             if (t && last) CU(c, cudaEventRecord(t->ffn_end[layer], c->compute));
             if (ring >= 0 && last) { CU(c, cudaEventRecord(c->ring_end[ring], c->compute)); c->ring_used[ring] = 1; }
-            if (last && leave_partial) {
+            if (multi) {
+                if (int rc = launch_multi_combine(c, nb, h_inout, first)) return rc;
+                c->kernel_launches += 2;
+            } else if (last && leave_partial) {
                 if (left) *left = true;
                 c->kernel_launches += 1;
             } else {
@@ -944,7 +1046,7 @@ int step_layers(spm_ctx* c, float* h_out, int nb, Timing* t, const Mailbox* trac
         return SPM_OK;
     };
     // GEMV path: only the last layer runs the combine kernel, the others leave it to the next routing kernel
-    const bool gemv_path = !(nb > 1 && c->tc_ok && c->batched_path == 0);
+    const bool gemv_path = !(nb > 1 && c->tc_ok && c->batched_path == 0) && !use_multi(c, nb);
     if (!trace) if (int rc = enqueue_router(0)) return rc;
     for (int l = 0; l < L; ++l) {
         const bool has_adapter = l <= L - 2;
@@ -1079,7 +1181,8 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
         // On the GEMV path the routing kernel of layer l + 1 also folds layer l's partial rows into the
         // hidden row, so only the last layer needs the combine kernel.
         const bool use_tc = nb > 1 && c->tc_ok && c->batched_path == 0;
-        const bool fold = !use_tc && l > 0 && c->stub_us == 0;
+        const bool multi = !use_tc && use_multi(c, nb);
+        const bool fold = !use_tc && !multi && l > 0 && c->stub_us == 0;
         RouterRoute route{c->tr_dev + size_t(slot) * L + l, c->ws_slot_map + size_t(l) * n, codes, true,
                           fold ? c->ws_partial : nullptr, G};
         if (int rc = launch_router(c, l, h_out, nullptr, nb, c->ws_x, nullptr, true, predict && l <= L - 2, &route, false)) return rc;
@@ -1126,6 +1229,17 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             c->kernel_launches += 5;
             c->ffn_launches++;
             c->tc_launches++;
+            continue;
+        }
+        if (multi) {
+            MtArgs a;
+            a.dev_ids = c->ws_ids;
+            a.dev_slot = c->ws_slot_map + size_t(l) * n;
+            a.nb = nb;
+            if (int rc = launch_multi(c, l, a, c->ws_x, c->ws_w, clock_slot, true)) return rc;
+            if (int rc = launch_multi_combine(c, nb, h_out, true)) return rc;
+            c->kernel_launches += 3;
+            c->ffn_launches++;
             continue;
         }
         if (nb == 1) {
@@ -1300,6 +1414,10 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     c->ws_w = reinterpret_cast<float*>(base + lay.w);
     c->ws_scores = reinterpret_cast<float*>(base + lay.scores);
     c->ws_partial = reinterpret_cast<float*>(base + lay.partial);
+    if (cfg->max_batch > 1) {
+        c->mt_partial = reinterpret_cast<float*>(base + lay.mt_partial);
+        c->mt_map = reinterpret_cast<int32_t*>(base + lay.mt_map);
+    }
     c->ws_h = reinterpret_cast<float*>(base + lay.h);
     c->ws_ids = reinterpret_cast<int32_t*>(base + lay.ids);
     c->ws_order = reinterpret_cast<int32_t*>(base + lay.order);

@@ -1,0 +1,62 @@
+"""The several-sequences expert kernel with fp32 activations (fp32 weights, shared experts, sizes that do not tile by
+128) at the edges of its blocks, token runs and column groups, each against the CPU oracle."""
+import pytest
+import torch
+
+import synth
+from test_gpu_edges import build, compare_run
+
+pytestmark = pytest.mark.gpu
+
+# Tokens of an expert: runs of eight, one MMA per tile up to two tokens of a run and three above. Rows: blocks of eight.
+# Columns: groups of 32 over eight warps. The kernel takes over where 64 Mi weights and more are not read again, hence
+# few experts and many tokens.
+CASES = {
+    # every expert in every token: 64 = 8 full runs; 17 = two runs and one token; 10 = one run and two; 11 = ... and three
+    "fp32_all_experts": dict(base="tiny", hidden=256, n_experts=3, inter=463, top_k=3, slots=3, batch=64),
+    "fp32_run_of_one": dict(base="tiny", hidden=1024, n_experts=4, inter=460, top_k=4, slots=4, batch=17),
+    "fp32_idle_last_group": dict(base="tiny", hidden=384, n_experts=6, inter=511, top_k=3, slots=6, batch=48),
+    "bf16_run_of_two": dict(base="qwen3", hidden=2048, n_experts=4, inter=401, top_k=4, slots=4, batch=10),
+    "bf16_run_of_three": dict(base="qwen3", hidden=1280, n_experts=4, inter=601, top_k=4, slots=4, batch=11),
+    "bf16_shared_waves": dict(base="dsvl2", hidden=1280, n_experts=12, inter=250, top_k=3, slots=5, batch=29),
+    "bf16_narrow": dict(base="qwen3", hidden=256, n_experts=9, inter=743, top_k=2, slots=9, batch=64),
+    "q4_narrow": dict(base="qwen3_q4", hidden=256, n_experts=7, inter=777, top_k=2, slots=7, batch=64),
+    "q4_shared": dict(base="dsvl2_q4", hidden=1280, n_experts=6, inter=263, top_k=2, slots=6, batch=23),
+    "q4_widest_waves": dict(base="qwen3_q4", hidden=2048, n_experts=9, inter=129, top_k=3, slots=4, batch=32),
+}
+
+
+def config(name):
+    kw = dict(CASES[name])
+    cfg = synth.get_config(kw.pop("base"), n_layers=2, budget=1, **kw)
+    reads = cfg.batch * (cfg.top_k + cfg.n_shared)
+    distinct = min(cfg.batch * cfg.top_k, cfg.n_experts) + cfg.n_shared
+    assert (reads - distinct) * 3 * cfg.inter * cfg.hidden >= 64 << 20, "this shape would take the other kernel"
+    return cfg
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_several_sequences_match_the_oracle(name):
+    # fp32 sums of at most 2048 terms, in blocks of 16 or 32: some 1e-6 of the largest element, as on the batch-1 path
+    compare_run(config(name), steps=2, tol=4e-5 if name.startswith("fp32") else 4e-4)
+
+
+@pytest.mark.parametrize("name", ["fp32_run_of_one", "bf16_shared_waves", "q4_shared", "q4_narrow"])
+def test_several_sequences_equal_one_at_a_time(name):
+    """Same weights and rows through the batch-1 kernel: both keep activations and sums in fp32. The sums are taken in
+    another order, so they differ by the roundings of some hundred additions: 5e-6 of the largest element is ample."""
+    cfg = config(name)
+    m = build(cfg, slots=cfg.n_experts)
+    tok = synth.zipf_tokens(cfg, steps=1)
+    h = synth.embedding_rows(cfg, tok.reshape(-1)).float().cuda()
+    torch.cuda.synchronize()
+    m.set_batched_path(1)
+    x, ids, w, _ = m.router_topk(0, h)
+    both = torch.zeros(2, *h.shape, device="cuda")
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, both[0])
+    for t in range(cfg.batch):
+        m.moe_ffn(0, x[t:t + 1], ids[t:t + 1], w[t:t + 1].contiguous(), both[1, t:t + 1])
+    m.synchronize()
+    assert (both[0] - both[1]).abs().max() <= 5e-6 * both[1].abs().max()
+    m.close()
