@@ -788,7 +788,7 @@ int launch_grouped_wave(spm_ctx* c, int layer, const float* x_norm, const int32_
     c->tc_desc_ev_valid[d] = 1;
     // (all three kernels of a wave are launched so that their preambles may overlap their predecessor's tail)
     CU(c, launch_k(gg_gather_kernel, dim3(std::max(n_rows, 1)), dim3(128), 0, c->compute, true, x_norm, w,
-                   reinterpret_cast<const GgRow*>(dd + c->tc_off_rows), n_rows, (const int*)nullptr, m.hidden, K,
+                   reinterpret_cast<const GgRow*>(dd + c->tc_off_rows), n_rows, m.hidden, K,
                    c->tc_xs + size_t(off) * m.hidden, c->tc_wrow + off,
                    q4 ? 1 : 0, q4 ? (int*)nullptr : c->tc_ready, q4 ? 0 : n_units + 1));
     if (t && first) CU(c, cudaEventRecord(t->ffn_start[layer], c->compute));
@@ -1204,18 +1204,14 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             for (int tk = 0; tk < nb; ++tk) a.count[tk] = (unsigned char)(K + m.n_shared);   // launch shape only
         };
         if (use_tc) {
-            // wave plan on the device, then gather -> grouped tcgen05 FFN -> combine
+            // wave plan and gather on the device -> grouped tcgen05 FFN -> combine
             unsigned char* dd = c->tc_desc_dev;        // stream-ordered reuse of the first descriptor slot
             GgUnit* units = reinterpret_cast<GgUnit*>(dd);
-            GgRow* rows = reinterpret_cast<GgRow*>(dd + c->tc_off_rows);
             int32_t* rowmap = reinterpret_cast<int32_t*>(dd + c->tc_off_rowmap);
-            CU(c, launch_k(gg_plan_kernel, dim3(1), dim3(kGgPlanThreads), gg_plan_smem(n), c->compute, true,
-                           (const int32_t*)c->ws_ids, (const short*)(c->ws_slot_map + size_t(l) * n), l * c->S, nb, K, n, c->n_jt,
-                           units, rows, rowmap, c->tc_counts, c->ws_status));
-            CU(c, launch_k(gg_gather_kernel, dim3(nb * K), dim3(128), 0, c->compute, true, (const float*)c->ws_x, (const float*)c->ws_w,
-                           (const GgRow*)rows, 0, (const int*)(c->tc_counts + 1), m.hidden, K, c->tc_xs, c->tc_wrow,
-                           m.dtype == SPM_DTYPE_Q4 ? 1 : 0, m.dtype == SPM_DTYPE_Q4 ? (int*)nullptr : c->tc_ready,
-                           m.dtype == SPM_DTYPE_Q4 ? 0 : c->max_units + 1));
+            CU(c, launch_k(gg_plan_gather_kernel, dim3(nb * K), dim3(kGgPairThreads), 0, c->compute, true, (const float*)c->ws_x, (const float*)c->ws_w,
+                           (const int32_t*)c->ws_ids, (const short*)(c->ws_slot_map + size_t(l) * n), l * c->S, nb * K, K, n, c->n_jt, m.hidden,
+                           units, rowmap, c->tc_counts, c->tc_xs, c->tc_wrow, m.dtype == SPM_DTYPE_Q4 ? 1 : 0,
+                           m.dtype == SPM_DTYPE_Q4 ? (int*)nullptr : c->tc_ready, m.dtype == SPM_DTYPE_Q4 ? 0 : c->max_units + 1, c->ws_status));
             // (no chunk list here: the plan is built on the device, a chunk is a whole unit)
             GgArgs ga{units, 0, c->tc_counts, c->tc_wrow, c->tc_partial, c->rows_cap, m.hidden, m.inter, c->ws_status, c->wait_limit_ns,
                       nullptr, 0, c->tc_ready, c->tc_act, c->tc_ready + 1, clock_slot};
@@ -1226,7 +1222,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
                 CU(c, launch_k(ffn_grouped_kernel, dim3(c->num_sms), dim3(kGgThreads), ffn_grouped_smem(), c->compute, true, c->wmap, c->xmaps, ga));
             CU(c, launch_k(gg_combine_kernel, gg_combine_grid(m.hidden, nb), gg_combine_block(K), 0, c->compute, true,
                            (const float*)c->tc_partial, (const int32_t*)rowmap, K, c->n_jt, c->rows_cap, m.hidden, h_out));
-            c->kernel_launches += 5;
+            c->kernel_launches += 4;
             c->ffn_launches++;
             c->tc_launches++;
             continue;
@@ -1494,8 +1490,6 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
         }
         if (!cu(cudaFuncSetAttribute(ffn_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ffn_grouped_smem())), "cudaFuncSetAttribute")) return bail(SPM_ERR_CUDA);
         if (!cu(cudaFuncSetAttribute(ffn_grouped_q4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ffn_grouped_q4_smem())), "cudaFuncSetAttribute")) return bail(SPM_ERR_CUDA);
-        if (gg_plan_smem(cfg->n_experts) > 48 * 1024 &&
-            !cu(cudaFuncSetAttribute(gg_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(gg_plan_smem(cfg->n_experts))), "cudaFuncSetAttribute")) return bail(SPM_ERR_CUDA);
         c->tc_ok = true;
     }
     c->ring_start.resize(64); c->ring_end.resize(64); c->ring_used.assign(64, 0);
