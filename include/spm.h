@@ -238,8 +238,9 @@ int spm_set_ffn_ctas(spm_ctx* ctx, int ctas);             /* CTAs per token of t
 /* Expert FFN used when nb > 1. 0 (default): the grouped tensor-core kernel (tcgen05, bf16
  * activations, fp32 accumulation) whenever the shape allows it (bf16 or 4-bit weights, no shared
  * experts, inter a multiple of 128, hidden a multiple of 128 for bf16 and of 256 for 4-bit
- * weights, which are expanded to bf16 on the way to the tensor cores), else the GEMV kernel once
- * per token. 1: always the GEMV kernel per token (fp32 activations). */
+ * weights, which are expanded to bf16 on the way to the tensor cores), else fp32 activations:
+ * every expert streamed once for all its tokens where at least 64 Mi weights are shared that
+ * way, the GEMV kernel once per token below. 1: always fp32 activations. */
 int spm_set_batched_path(spm_ctx* ctx, int mode);
 /* Perfect-knowledge ranking for SPM_POLICY_HINT_TRACE: for step s (counted from the last
  * spm_cache_reset) and layer l, hint[(s*L + l)*stride .. +count[s*L+l]) are the experts that
