@@ -58,6 +58,7 @@ struct RouterArgs {
     const float* partial;    // optional [nb][G][D] partial rows of the preceding expert kernel: the hidden row is
     int G;                   //   then h + sum of them (summed here instead of by a combine kernel) ...
     float* h_out;            //   ... and written back here ([nb][D], may alias h)
+    int defer_rank;          // several tokens: leave the batch's ranking to the kernel that is given RankArgs (pihat is written)
     int publish_seq;         // fence and publish the sequence number for hosts that read untagged payload
     uint32_t seq;
     int D, n, K, r, nb, renorm, do_router, do_adapter;
@@ -189,6 +190,31 @@ __device__ __forceinline__ void half_softmax(float* v, int n, float* slots, int 
 // Mailbox words carry the launch's sequence number in their upper half, so the host can tell a
 // fresh word from a stale one without any fence between payload and flag.
 __device__ __forceinline__ int32_t tagged(uint32_t seq, int value) { return int32_t((seq << 16) | uint32_t(value)); }
+
+// The adapter's ranking of a batch: priorities summed over the tokens in token order, experts by (priority descending, id
+// ascending). By all threads of a block; sm: n floats.
+struct RankArgs {
+    const float* pihat;      // [nb][n]; null: nothing to rank
+    float* scores;
+    int32_t* order;
+    Mailbox* mailbox;
+    uint32_t tag;
+    int nb, n;
+};
+__device__ __forceinline__ void rank_batch(const RankArgs& a, float* sm) {
+    for (int e = threadIdx.x; e < a.n; e += blockDim.x) {
+        float s = 0.f;
+        for (int t = 0; t < a.nb; ++t) s += __ldcg(a.pihat + size_t(t) * a.n + e);
+        sm[e] = s;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < a.n; e += blockDim.x) {
+        const int rk = rank_of_key(reinterpret_cast<const int*>(sm), a.n, e);
+        a.order[rk] = e;
+        a.scores[e] = sm[e];
+        if (a.mailbox) { a.mailbox->order[rk] = tagged(a.tag, e); a.mailbox->scores[e] = sm[e]; }
+    }
+}
 
 // Grid (kRouterCluster, nb), cluster (kRouterCluster, 1, 1): the CTAs of a cluster split the n + r
 // weight rows of one token and deliver their dot products straight into the leader CTA's shared
@@ -466,7 +492,7 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
     }
 
     // ---- several tokens: the last leader to finish aggregates and ranks -------------------------
-    if (a.nb > 1) {
+    if (a.nb > 1 && !a.defer_rank) {
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -476,20 +502,7 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
         __syncthreads();
         if (!s_last) return;
         __threadfence();
-        if (a.do_adapter) {
-            for (int e = threadIdx.x; e < n; e += kRouterThreads) {
-                float s = 0.f;
-                for (int t = 0; t < a.nb; ++t) s += __ldcg(a.pihat + size_t(t) * n + e);
-                qs[e] = s;
-            }
-            __syncthreads();
-            for (int e = threadIdx.x; e < n; e += kRouterThreads) {
-                const int rk = rank_of_key(reinterpret_cast<const int*>(qs), n, e);
-                a.order[rk] = e;
-                a.scores[e] = qs[e];
-                if (mb) { mb->order[rk] = tagged(tag, e); mb->scores[e] = qs[e]; }
-            }
-        }
+        if (a.do_adapter) rank_batch(RankArgs{a.pihat, a.scores, a.order, mb, tag, a.nb, n}, qs);
         if (threadIdx.x == 0) a.counters[0] = 0u;
     }
     // final flag for callers that read untagged payload (scores): fence, then the sequence number

@@ -467,6 +467,7 @@ struct RouterRoute {
     bool pdl;
     const float* partial;      // partial rows of the preceding layer's expert kernel to fold into the hidden row, or null
     int G;
+    RankArgs* defer;           // several tokens: the caller's next kernel ranks the adapter's priorities and is told here with what
 };
 
 int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int nb, float* x_norm,
@@ -499,6 +500,7 @@ int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int 
     a.G = route ? route->G : 0;
     a.h_out = const_cast<float*>(h);
     a.publish_seq = publish_seq;
+    a.defer_rank = route && route->defer;
     if (int rc = take_clock(c, kClkRouter, &a.clock)) return rc;
     // Sequence numbers whose low 16 bits are zero are skipped, and the words this launch will
     // publish are zeroed first, so a word left by an older launch can never carry the current tag.
@@ -509,6 +511,7 @@ int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int 
         if (do_adapter) memset(const_cast<int32_t*>(c->mb_host->order), 0, size_t(m.n_experts) * sizeof(int32_t));
     }
     a.seq = c->seq;
+    if (a.defer_rank) *route->defer = RankArgs{do_adapter ? c->ws_pihat : nullptr, c->ws_scores, c->ws_order, a.mailbox, c->seq & 0xffffu, nb, m.n_experts};
     a.D = m.hidden; a.n = m.n_experts; a.K = m.top_k; a.r = m.adapter_rank; a.nb = nb;
     a.renorm = m.renormalize; a.do_router = do_router; a.do_adapter = do_adapter;
     a.eps = m.rms_eps;
@@ -1038,7 +1041,7 @@ int step_layers(spm_ctx* c, float* h_out, int nb, Timing* t, const Mailbox* trac
             CU(c, cudaGetLastError());
             c->kernel_launches++;
         }
-        RouterRoute fold{c->mb_dev, nullptr, nullptr, false, c->ws_partial, ffn_grid_for(c, nb)};
+        RouterRoute fold{c->mb_dev, nullptr, nullptr, false, c->ws_partial, ffn_grid_for(c, nb), nullptr};
         if (int rc = launch_router(c, l, h_out, nullptr, nb, c->ws_x, nullptr, true, predict && l <= L - 2,
                                    partial_left ? &fold : nullptr, false)) return rc;
         partial_left = false;
@@ -1183,8 +1186,9 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
         const bool use_tc = nb > 1 && c->tc_ok && c->batched_path == 0;
         const bool multi = !use_tc && use_multi(c, nb);
         const bool fold = !use_tc && !multi && l > 0 && c->stub_us == 0;
+        RankArgs rank{};               // grouped kernels: the plan and gather kernel has a block for the adapter's ranking
         RouterRoute route{c->tr_dev + size_t(slot) * L + l, c->ws_slot_map + size_t(l) * n, codes, true,
-                          fold ? c->ws_partial : nullptr, G};
+                          fold ? c->ws_partial : nullptr, G, use_tc ? &rank : nullptr};
         if (int rc = launch_router(c, l, h_out, nullptr, nb, c->ws_x, nullptr, true, predict && l <= L - 2, &route, false)) return rc;
         unsigned long long* clock_slot = nullptr;
         if (int rc = take_clock(c, kClkFfn, &clock_slot)) return rc;
@@ -1208,10 +1212,10 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             unsigned char* dd = c->tc_desc_dev;        // stream-ordered reuse of the first descriptor slot
             GgUnit* units = reinterpret_cast<GgUnit*>(dd);
             int32_t* rowmap = reinterpret_cast<int32_t*>(dd + c->tc_off_rowmap);
-            CU(c, launch_k(gg_plan_gather_kernel, dim3(nb * K), dim3(kGgPairThreads), 0, c->compute, true, (const float*)c->ws_x, (const float*)c->ws_w,
+            CU(c, launch_k(gg_plan_gather_kernel, dim3(nb * K + (rank.pihat ? 1 : 0)), dim3(kGgPairThreads), 0, c->compute, true, (const float*)c->ws_x, (const float*)c->ws_w,
                            (const int32_t*)c->ws_ids, (const short*)(c->ws_slot_map + size_t(l) * n), l * c->S, nb * K, K, n, c->n_jt, m.hidden,
                            units, rowmap, c->tc_counts, c->tc_xs, c->tc_wrow, m.dtype == SPM_DTYPE_Q4 ? 1 : 0,
-                           m.dtype == SPM_DTYPE_Q4 ? (int*)nullptr : c->tc_ready, m.dtype == SPM_DTYPE_Q4 ? 0 : c->max_units + 1, c->ws_status));
+                           m.dtype == SPM_DTYPE_Q4 ? (int*)nullptr : c->tc_ready, m.dtype == SPM_DTYPE_Q4 ? 0 : c->max_units + 1, c->ws_status, rank));
             // (no chunk list here: the plan is built on the device, a chunk is a whole unit)
             GgArgs ga{units, 0, c->tc_counts, c->tc_wrow, c->tc_partial, c->rows_cap, m.hidden, m.inter, c->ws_status, c->wait_limit_ns,
                       nullptr, 0, c->tc_ready, c->tc_act, c->tc_ready + 1, clock_slot};

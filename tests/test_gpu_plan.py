@@ -1,4 +1,4 @@
-"""Edges of the device-side plan of a batched host-free step."""
+"""Edges of the device-side plan of a batched host-free step and of the ranking made beside it."""
 import numpy as np
 import pytest
 
@@ -18,7 +18,7 @@ PLANS = {
 
 
 @pytest.mark.parametrize("name", list(PLANS))
-def test_device_plan_equals_the_host_driven_step(name):
+def test_device_plan_and_ranking_equal_the_host_driven_step(name):
     cfg = synth.get_config("qwen3", n_layers=3, hidden=256, inter=128, budget=1, **PLANS[name])
     H = rows(cfg, 3)
     results = []
