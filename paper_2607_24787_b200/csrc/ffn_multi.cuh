@@ -655,9 +655,14 @@ static __global__ void mt_combine_kernel(const float* __restrict__ partial, cons
     if (k == 0 && d < D) {
         float4 sum = part[0][c];
         for (int kk = 1; kk < KS; ++kk) { const float4 p = part[kk][c]; sum.x += p.x; sum.y += p.y; sum.z += p.z; sum.w += p.w; }
-        float4 tot = *reinterpret_cast<const float4*>(h + size_t(t) * D + d);
-        tot.x += sum.x; tot.y += sum.y; tot.z += sum.z; tot.w += sum.w;
-        *reinterpret_cast<float4*>(h + size_t(t) * D + d) = tot;
+        float* hp = h + size_t(t) * D + d;
+        if ((reinterpret_cast<uintptr_t>(hp) & 15) == 0) {
+            float4 tot = *reinterpret_cast<const float4*>(hp);
+            tot.x += sum.x; tot.y += sum.y; tot.z += sum.z; tot.w += sum.w;
+            *reinterpret_cast<float4*>(hp) = tot;
+        } else {                // the caller's rows may start at any float (spm_moe_ffn)
+            hp[0] += sum.x; hp[1] += sum.y; hp[2] += sum.z; hp[3] += sum.w;
+        }
     }
     if (clock) {
         __syncthreads();

@@ -60,3 +60,24 @@ def test_several_sequences_equal_one_at_a_time(name):
     m.synchronize()
     assert (both[0] - both[1]).abs().max() <= 5e-6 * both[1].abs().max()
     m.close()
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_hidden_rows_may_start_at_any_float(offset):
+    """spm_moe_ffn updates h_inout in place wherever it lies: an offset slice has the alignment of a float only. Same sums
+    in the same order, hence the bits of the aligned call."""
+    cfg = config("bf16_narrow")
+    m = build(cfg, slots=cfg.n_experts)
+    h = torch.randn(cfg.batch, cfg.hidden, device="cuda")
+    x, ids, w, _ = m.router_topk(0, h)
+    want = h.clone()
+    buf = torch.empty(h.numel() + 4, device="cuda")
+    at = buf[offset:offset + h.numel()].view_as(h)
+    at.copy_(h)
+    torch.cuda.synchronize()
+    assert at.data_ptr() % 16 == 4 * offset
+    m.moe_ffn(0, x, ids, w, want)
+    m.moe_ffn(0, x, ids, w, at)
+    m.synchronize()
+    assert torch.equal(at, want) and not torch.equal(want, h)
+    m.close()
