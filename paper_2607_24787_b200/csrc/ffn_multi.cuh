@@ -386,7 +386,7 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
                 f.src = a.shared + size_t(e - n) * a.blob_bytes;
             } else {
                 const int slot = a.dev_slot ? a.dev_slot[e] : a.slot[e];
-                if (slot < 0 || slot >= a.n_slots) {        // nothing more is issued; every wait of the CTA ends at once
+                if (slot < 0 || slot >= a.n_slots) {        // nothing more is issued; every wait of the CTA ends once the flag is seen
                     if (lane == 0) { atomicOr(a.status, kStatusBadSlot); *reinterpret_cast<volatile int*>(&s_abort) = 1; }
                     feeding = false;
                     return;
@@ -611,11 +611,32 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
         else segment(std::integral_constant<int, 3>{}, k, u, blk0, seg, e, ntok, mine);
         k += seg;
     }
-    if (dead) {        // leave no copy in flight into shared memory that is about to be released
-        for (int i = max(0, fgu.n - n_stages); i < fgu.n; ++i)
-            if (!mbar_wait_bounded(gu_bar + 8 * (i % n_stages), (i / n_stages) & 1, limit)) break;
-        for (int i = max(0, fdn.n - n_stages); i < fdn.n; ++i)
-            if (!mbar_wait_bounded(dn_bar + 8 * (i % n_stages), (i / n_stages) & 1, limit)) break;
+    // Wind-down after a wait ran out or a slot was bad: leave no copy in flight into shared memory that is about to be
+    // released. (The flag is raised ahead of a barrier of the loop above, so the whole CTA sees it here.) A warp that gave up
+    // stopped feeding, others went on until they saw the flag, and a stage completes only with the arrivals of all eight warps:
+    // the warps agree on the last block that any of them fed and arrive, without a copy, for the blocks up to it. Such
+    // a block's stage is free to take them: whoever fed the block had waited for the stage's block before it.
+    if (*reinterpret_cast<volatile int*>(&s_abort)) {
+        __syncthreads();
+        if (threadIdx.x == 0) { s_entries = 0; s_routed = 0; }
+        __syncthreads();
+        if (lane == 0) { atomicMax(&s_entries, fgu.n); atomicMax(&s_routed, fdn.n); }
+        __syncthreads();
+        const int n_gu = s_entries, n_dn = s_routed;
+        if (elect_one()) {
+            for (int i = fgu.n; i < n_gu; ++i) mbar_arrive(gu_bar + 8 * (i % n_stages));
+            for (int i = fdn.n; i < n_dn; ++i) mbar_arrive(dn_bar + 8 * (i % n_stages));
+        }
+        // the drain has a bound of its own: a short limit of the caller must not end it early
+        const unsigned long long t0 = global_timer_ns();
+        auto drain = [&](uint32_t bar, int n_fed) {
+            for (int i = max(0, n_fed - n_stages); i < n_fed; ++i) {
+                const unsigned long long spent = global_timer_ns() - t0;
+                mbar_wait_bounded(bar + 8 * (i % n_stages), (i / n_stages) & 1, spent < kWaitLimitNs ? kWaitLimitNs - spent : 0);
+            }
+        };
+        drain(gu_bar, n_gu);
+        drain(dn_bar, n_dn);
     }
     if (a.clock) {
         __syncthreads();

@@ -1,10 +1,15 @@
 """The several-sequences expert kernel with fp32 activations (fp32 weights, shared experts, sizes that do not tile by
 128) at the edges of its blocks, token runs and column groups, each against the CPU oracle."""
+import time
+
+import numpy as np
 import pytest
 import torch
 
 import synth
+from paper_2607_24787_b200.binding import SpmError
 from test_gpu_edges import build, compare_run
+from test_gpu_host_free import preload, rows, run
 
 pytestmark = pytest.mark.gpu
 
@@ -80,4 +85,39 @@ def test_hidden_rows_may_start_at_any_float(offset):
     m.moe_ffn(0, x, ids, w, at)
     m.synchronize()
     assert torch.equal(at, want) and not torch.equal(want, h)
+    m.close()
+
+
+@pytest.mark.parametrize("name", ["fp32_all_experts", "bf16_narrow", "q4_shared"])
+@pytest.mark.parametrize("bad", [-1, 30000])
+def test_a_slot_outside_the_pool_ends_the_launch_with_an_error(name, bad):
+    """The kernel checks the slot numbers that it reads on the device. One that names no slot (planted in the slot map of a
+    host-free step) stops the CTAs that meet it: no access, no long wait, an error status, and the context goes on."""
+    cfg = config(name).replace(slots=config(name).n_experts)
+    H = rows(cfg, 3)
+    m = build(cfg)
+    preload(cfg, m)
+    good = run(m, H)
+    assert m.stats()["host_free_steps"] == 3
+    slot_map = np.full((cfg.n_layers, cfg.n_experts), -1, np.int16)
+    for l in range(cfg.n_layers):
+        for s, e in enumerate(m.slot_table(l)):
+            slot_map[l, e] = s
+    # the map follows the pools in the arena: [layer][expert], 16-bit, 256-byte aligned
+    arena = m.arena.cpu().numpy()
+    base = (-m.arena.data_ptr()) % 256
+    first = base + -(-cfg.n_layers * cfg.slots * cfg.expert_bytes // 256) * 256
+    at = [i for i in range(first, arena.size - slot_map.nbytes, 256) if arena[i:i + slot_map.nbytes].tobytes() == slot_map.tobytes()]
+    assert len(at) == 1
+    e = 1
+    m.arena[at[0] + 2 * e:at[0] + 2 * e + 2] = torch.from_numpy(np.array([bad], np.int16).view(np.uint8)).cuda()
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    with pytest.raises(SpmError) as err:
+        run(m, H[:1])
+    assert err.value.code == -5 and time.perf_counter() - t0 < 1.5
+    m.cache_reset()
+    preload(cfg, m)
+    for a, b in zip(run(m, H), good):
+        assert np.array_equal(a, b)
     m.close()
