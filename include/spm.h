@@ -279,7 +279,7 @@ int spm_set_device_wait(spm_ctx* ctx, int on);
  * spm_cache_reset() ends the state; it is re-entered once the pools are full again. */
 int spm_set_host_free(spm_ctx* ctx, int on);
 /* Replay host-free steps from CUDA graphs (default on): the launches of such a step are the same
- * every time for a given trace slot, batch size, output buffer and launch geometry, so each
+ * every time for a given trace slot, batch size, output buffer, launch geometry and wait limit, so each
  * combination is captured once (after one step enqueued launch by launch) and replayed with a
  * single submission. Off, or with timing / an attention stand-in set, every kernel is launched
  * individually. Results are identical. */

@@ -25,6 +25,7 @@
 #include "router_adapter.cuh"
 #include "tma_maps.h"
 #include "gg_plan.h"
+#include "host_free_key.h"
 #include "slot_table.h"
 
 using namespace spm;
@@ -139,7 +140,7 @@ struct spm_ctx {
     std::deque<std::pair<int, int>> tr_pending;   // (ring slot, nb) of steps enqueued but not yet replayed
     uint64_t tr_count = 0, host_free_steps = 0;
     struct HostFreeGraph {                    // a captured host-free step and what one replay adds to the launch counters
-        int slot, nb; const float* h_out; bool predict; int G, batched_path;
+        HostFreeKey key;
         uint64_t kernels, ffns, tcs;
         cudaGraphExec_t exec;
     };
@@ -1265,7 +1266,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
 }
 
 // A host-free step is the same sequence of launches every time (for a given trace slot, batch size,
-// output buffer, prediction on/off and launch geometry), so it is captured once into a CUDA graph
+// output buffer, prediction on/off, launch geometry and wait limit), so it is captured once into a CUDA graph
 // and replayed: one submission instead of 2-5 per layer. Steps with timing or an attention
 // stand-in are enqueued launch by launch.
 int enqueue_host_free_step(spm_ctx* c, const float* h_in, int nb, float* h_out) {
@@ -1278,13 +1279,13 @@ int enqueue_host_free_step(spm_ctx* c, const float* h_in, int nb, float* h_out) 
     const bool predict = c->policy == SPM_POLICY_ADAPTER || c->policy == SPM_POLICY_PRED0;
     bool done = false;
     if (c->graph_replay && !c->timing && c->stub_us == 0) {
-        const int G = ffn_grid_for(c, nb);
+        const HostFreeKey key{slot, nb, h_out, predict, ffn_grid_for(c, nb), c->batched_path, c->wait_limit_ns};
         spm_ctx::HostFreeGraph* g = nullptr;
         for (auto& x : c->hf_graphs)
-            if (x.slot == slot && x.nb == nb && x.h_out == h_out && x.predict == predict && x.G == G && x.batched_path == c->batched_path) g = &x;
+            if (x.key == key) g = &x;
         if (!g && c->hf_warm && c->hf_graphs.size() < 64) {
             // (the first host-free step ran launch by launch, so every kernel attribute is already set)
-            spm_ctx::HostFreeGraph ng{slot, nb, h_out, predict, G, c->batched_path, 0, 0, 0, nullptr};
+            spm_ctx::HostFreeGraph ng{key, 0, 0, 0, nullptr};
             const uint64_t k0 = c->kernel_launches, f0 = c->ffn_launches, t0 = c->tc_launches;
             cudaGraph_t graph = nullptr;
             int rc = SPM_ERR_CUDA;

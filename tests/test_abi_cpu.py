@@ -82,6 +82,25 @@ def test_grouped_kernel_chunk_plan(n_units, n_dt, grid):
         assert np.all(sizes[-grid:] <= 2 * min_chunk - 1)
 
 
+def test_a_captured_step_is_replayed_only_where_everything_it_was_built_from_is_the_same(tmp_path):
+    """Launch arguments that a caller can change are frozen in a captured host-free step: two steps that differ in any of
+    them (the limit of the device-side waits among them) must not share a capture."""
+    import shutil
+    import subprocess
+    if not shutil.which("g++"):
+        pytest.skip("no host compiler")
+    base = ["3", "8", "&h", "true", "37", "0", "0ull"]
+    other = ["4", "7", "&k", "false", "36", "1", "5000ull"]
+    keys = [base] + [base[:i] + [other[i]] + base[i + 1:] for i in range(len(base))]
+    src = tmp_path / "key.cpp"
+    src.write_text('#include "host_free_key.h"\nint main() {\n  float h = 0, k = 0;\n  const spm::HostFreeKey keys[] = {'
+                   + ", ".join("{" + ", ".join(k) + "}" for k in keys)
+                   + "};\n  int same = 0;\n  for (auto& a : keys) for (auto& b : keys) same += a == b;\n"
+                   + f"  return same == {len(keys)} ? 0 : 1;\n}}\n")
+    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_2607_24787_b200", "csrc"), "-o", str(tmp_path / "key"), str(src)], check=True)
+    assert subprocess.run([str(tmp_path / "key")]).returncode == 0
+
+
 def test_noalloc_argument_checks_run_before_any_gpu_work():
     """The allocation-free entry point refuses bad shapes, indices and misaligned pointers on the
     host, before it touches the device: so this runs without a GPU (addresses below are never
