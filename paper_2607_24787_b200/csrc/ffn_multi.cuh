@@ -61,7 +61,8 @@ struct MtArgs {
     const float* x;                 // [nb][D] router input
     const float* w;                 // [nb][K] routing weights
     float* partial;                 // [(CTAs + entries) * kMtTokens][D], see mt_partial_rows
-    int32_t* map;                   // {entries, -, -, -, [nb][SPM_MAX_TOPK] entry | position << 16 of each (token, k) pair, < 0: none}
+    int32_t* map;                   // {entries, -, -, -, [nb][SPM_MAX_TOPK][2] of each (token, k) pair entry | position << 16 (< 0: none), and
+                                    //   its expert's slot (shared expert s: -1 - s)}
     int* status;
     unsigned long long* clock;      // optional {earliest CTA start, latest CTA end} in ns (globaltimer)
     const int32_t* dev_ids;         // [nb][K] expert ids left in device memory by the routing kernel, with
@@ -104,7 +105,7 @@ __device__ __forceinline__ bool mt_wait(uint32_t bar, uint32_t parity, volatile 
 
 // ---- operands ------------------------------------------------------------------
 // a (low half) and b (high half) as three bf16 pairs whose sum is exactly {a, b}: truncation leaves 16, then 8
-// significant bits. Inf and NaN stay in the first part.
+// significant bits. Of an Inf or NaN the first part is the upper half and the others are 0 (see mt_plain_y).
 struct Split3 { uint32_t part[3]; };
 __device__ __forceinline__ Split3 split3(float a, float b) {
     const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
@@ -194,6 +195,7 @@ __device__ __forceinline__ void b_parts(float a, float b, int lane, uint32_t (&o
 }
 
 // Per weight type: where a lane's operands come from. Lane (g, t) = (lane / 4, lane % 4). A group is 32 columns.
+//   weight(part, col) * scale(part, D, group): a value of one matrix's part of a blob row, for mt_plain_y
 //   phase1: acc[0..1] += gate row g, acc[2..3] += up row g, for N columns 2t, 2t + 1
 //   phase2: y[tile][0..1] += hidden column ycol(g, tile), y[tile][2..3] += ycol(g + 8, tile), for N columns 2t, 2t + 1
 // x[kb][q] is the B operand of K-block kb: the activations of columns xcol(t, kb, q, 0 / 1) of the lane's token.
@@ -204,6 +206,8 @@ template <> struct MtWeight<uint16_t> {      // bf16
     static __host__ __device__ constexpr uint32_t part_bytes(int D) { return uint32_t(D) * 2; }
     static __device__ __forceinline__ int xcol(int t, int kb, int q, int half) { return kb * 16 + 2 * t + 8 * q + half; }
     static __device__ __forceinline__ int ycol(int m, int tile) { return tile * 16 + m; }
+    static __device__ __forceinline__ float weight(const unsigned char* part, int col) { return __uint_as_float(uint32_t(reinterpret_cast<const uint16_t*>(part)[col]) << 16); }
+    static __device__ __forceinline__ float scale(const unsigned char*, int, int) { return 1.f; }
     template <int NS>
     static __device__ __forceinline__ void phase1(uint32_t rows, uint32_t stride, int D, int grp, int lane, const uint32_t (&x)[2][2][NS], float (&acc)[4]) {
         const int mat = lane >> 3;             // matrices: gate k 0-7, up k 0-7, gate k 8-15, up k 8-15
@@ -233,6 +237,8 @@ template <> struct MtWeight<float> {         // both operands in three parts: ni
     static __host__ __device__ constexpr uint32_t part_bytes(int D) { return uint32_t(D) * 4; }
     static __device__ __forceinline__ int xcol(int t, int kb, int q, int half) { return kb * 16 + 2 * t + 8 * q + half; }
     static __device__ __forceinline__ int ycol(int m, int tile) { return tile * 16 + m; }
+    static __device__ __forceinline__ float weight(const unsigned char* part, int col) { return reinterpret_cast<const float*>(part)[col]; }
+    static __device__ __forceinline__ float scale(const unsigned char*, int, int) { return 1.f; }
     template <int NS>
     static __device__ __forceinline__ void phase1(uint32_t rows, uint32_t stride, int D, int grp, int lane, const uint32_t (&x)[2][2][NS], float (&acc)[4]) {
         const uint32_t at = rows + uint32_t(lane >> 2) * stride + uint32_t(grp * 32 + 2 * (lane & 3)) * 4;
@@ -287,6 +293,8 @@ template <> struct MtWeight<Q4Tag> {         // (q - 8) through the MMA, a group
     static __device__ __forceinline__ int xcol(int t, int kb, int q, int half) { return t * 8 + 2 * kb + q + 4 * half; }
     // ... and its M positions four nibbles of half a word
     static __device__ __forceinline__ int ycol(int m, int tile) { return (m & 3) * 8 + ((m >> 2) & 1) * 4 + 2 * tile + (m >> 3); }
+    static __device__ __forceinline__ float weight(const unsigned char* part, int col) { return float(((part[col >> 1] >> (4 * (col & 1))) & 15) - 8); }
+    static __device__ __forceinline__ float scale(const unsigned char* part, int D, int grp) { return __half2float(reinterpret_cast<const __half*>(part + D / 2)[grp]); }
     template <int NS>
     static __device__ __forceinline__ void phase1(uint32_t rows, uint32_t stride, int D, int grp, int lane, const uint32_t (&x)[2][2][NS], float (&acc)[4]) {
         const uint32_t row = rows + uint32_t(lane >> 2) * stride, PART = part_bytes(D);
@@ -581,7 +589,7 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
         if (threadIdx.x == 0) a.map[0] = s_entries;
         for (int i = threadIdx.x; i < a.nb * SPM_MAX_TOPK; i += kMtThreads) {
             const int t = i / SPM_MAX_TOPK, k = i % SPM_MAX_TOPK;
-            if (k < a.K ? ids[t * a.K + k] < 0 : k >= a.K + a.n_shared) a.map[4 + i] = -1;      // not in this wave
+            if (k < a.K ? ids[t * a.K + k] < 0 : k >= a.K + a.n_shared) a.map[4 + 2 * i] = -1;      // not in this wave
         }
     }
     for (int k = 0; k < steps;) {
@@ -605,7 +613,9 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
         }
         if (blk0 == 0 && warp == 0 && lane < ntok) {        // the CTA with an entry's first block says where its pairs are
             const int tk = e >= n ? mine : mine / a.K, kk = e >= n ? a.K + (e - n) : mine - tk * a.K;
-            a.map[4 + tk * SPM_MAX_TOPK + kk] = u | (lane << 16);
+            int32_t* pair = a.map + 4 + 2 * (tk * SPM_MAX_TOPK + kk);
+            pair[0] = u | (lane << 16);
+            pair[1] = e >= n ? n - 1 - e : a.dev_slot ? a.dev_slot[e] : a.slot[e];
         }
         if (ntok <= 2) segment(std::integral_constant<int, 1>{}, k, u, blk0, seg, e, ntok, mine);
         else segment(std::integral_constant<int, 3>{}, k, u, blk0, seg, e, ntok, mine);
@@ -644,24 +654,70 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
     }
 }
 
+// Four columns of one token's y of one expert by plain fp32 multiply-adds, one warp together: the sums that the GEMV per
+// sequence takes. For operands that are not finite. The split arithmetic marks those (its result is Inf or NaN: no finite
+// sum contains one) but does not keep them apart: an infinity times an empty lower part of the other operand is NaN, and
+// a NaN whose payload is in its low 16 bits is an infinity in the first part. (Behind the segments in ffn_multi_kernel, the
+// same code cost the hot loop up to 60 registers; here it costs nothing.)
+template <typename WT>
+__device__ __noinline__ float4 mt_plain_y(const unsigned char* blob, int I, int D, const float* x, float wt, int d) {
+    using W = MtWeight<WT>;
+    const uint32_t PART = W::part_bytes(D);
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = 0; j < I; ++j) {
+        const unsigned char *gate = blob + size_t(j) * (3 * PART), *up = gate + PART, *down = up + PART;
+        float pg = 0.f, pu = 0.f;
+        for (int g = int(threadIdx.x & 31); g < D / 32; g += 32) {
+            float dg = 0.f, du = 0.f;
+            for (int i = g * 32; i < g * 32 + 32; ++i) {
+                dg = fmaf(W::weight(gate, i), x[i], dg);
+                du = fmaf(W::weight(up, i), x[i], du);
+            }
+            pg = fmaf(W::scale(gate, D, g), dg, pg);
+            pu = fmaf(W::scale(up, D, g), du, pu);
+        }
+        pg = warp_sum(pg);
+        pu = warp_sum(pu);
+        if (d < D) {
+            const float s = W::silu(pg) * pu * wt * W::scale(down, D, d / 32);
+            y.x = fmaf(s, W::weight(down, d), y.x);
+            y.y = fmaf(s, W::weight(down, d + 1), y.y);
+            y.z = fmaf(s, W::weight(down, d + 2), y.z);
+            y.w = fmaf(s, W::weight(down, d + 3), y.w);
+        }
+    }
+    return y;
+}
+
+struct MtCombineArgs {
+    const float* partial;
+    const int32_t* map;
+    float* h;                       // [nb][D]
+    const unsigned char *pool, *shared;
+    const float *x, *w;             // as in MtArgs
+    unsigned long long* clock;
+    unsigned long long blob_bytes;
+    int KS, G, I, D, K, n_slots, n_shared;      // KS: experts of a token in this wave's launch (K + shared), G: CTAs of ffn_multi_kernel
+};
+
 // h[t][d] += sum over the token's experts of this wave, in k order, of their segments' partial rows in CTA order.
 // Block = (32 groups of four columns) x (K + n_shared experts); kMtAhead loads of a thread are in flight together.
 constexpr int kMtAhead = 8;
-static __global__ void mt_combine_kernel(const float* __restrict__ partial, const int32_t* __restrict__ map, int KS, int G, int I, int D, float* h,
-                                         unsigned long long* clock) {
+template <typename WT>
+static __global__ void mt_combine_kernel(const __grid_constant__ MtCombineArgs a) {
     __shared__ float4 part[SPM_MAX_TOPK][32];
     grid_dep_launch();
     grid_dep_wait();
-    if (clock && threadIdx.x == 0) atomicMin(clock, global_timer_ns());
-    const int t = blockIdx.y, c = threadIdx.x & 31, k = threadIdx.x >> 5;
+    if (a.clock && threadIdx.x == 0) atomicMin(a.clock, global_timer_ns());
+    const int D = a.D, t = blockIdx.y, c = threadIdx.x & 31, k = threadIdx.x >> 5;
     const int d = (blockIdx.x * 32 + c) * 4;
-    const int32_t code = map[4 + t * SPM_MAX_TOPK + k];
+    const int32_t code = a.map[4 + 2 * (t * SPM_MAX_TOPK + k)];
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (code >= 0 && d < D) {
-        const int u = code & 0xffff, tl = code >> 16, NB = (I + kMtRows - 1) / kMtRows;
-        const MtSplit split(map[0] * NB, G);
+        const int u = code & 0xffff, tl = code >> 16, NB = (a.I + kMtRows - 1) / kMtRows;
+        const MtSplit split(a.map[0] * NB, a.G);
         const int c0 = split.cta_of(u * NB), total = split.cta_of(u * NB + NB - 1) - c0 + 1;
-        const float* p = partial + (size_t(c0 + u) * kMtTokens + size_t(tl)) * D + d;
+        const float* p = a.partial + (size_t(c0 + u) * kMtTokens + size_t(tl)) * D + d;
         for (int i0 = 0; i0 < total; i0 += kMtAhead) {
             float4 v[kMtAhead];
 #pragma unroll
@@ -671,12 +727,21 @@ static __global__ void mt_combine_kernel(const float* __restrict__ partial, cons
             for (int i = 0; i < kMtAhead; ++i) { acc.x += v[i].x; acc.y += v[i].y; acc.z += v[i].z; acc.w += v[i].w; }
         }
     }
+    if (code >= 0) {            // (one pair per warp)
+        const float probe = fmaf(acc.x, 0.f, fmaf(acc.y, 0.f, fmaf(acc.z, 0.f, acc.w * 0.f)));       // NaN unless all four are finite
+        if (__any_sync(0xffffffffu, probe != 0.f)) {
+            const int slot = a.map[5 + 2 * (t * SPM_MAX_TOPK + k)];
+            if (slot < a.n_slots && -1 - slot < a.n_shared)
+                acc = mt_plain_y<WT>(slot < 0 ? a.shared + size_t(-1 - slot) * a.blob_bytes : a.pool + size_t(slot) * a.blob_bytes, a.I, D, a.x + size_t(t) * D,
+                                     k < a.K ? a.w[size_t(t) * a.K + k] : 1.f, d);
+        }
+    }
     part[k][c] = acc;
     __syncthreads();
     if (k == 0 && d < D) {
         float4 sum = part[0][c];
-        for (int kk = 1; kk < KS; ++kk) { const float4 p = part[kk][c]; sum.x += p.x; sum.y += p.y; sum.z += p.z; sum.w += p.w; }
-        float* hp = h + size_t(t) * D + d;
+        for (int kk = 1; kk < a.KS; ++kk) { const float4 p = part[kk][c]; sum.x += p.x; sum.y += p.y; sum.z += p.z; sum.w += p.w; }
+        float* hp = a.h + size_t(t) * D + d;
         if ((reinterpret_cast<uintptr_t>(hp) & 15) == 0) {
             float4 tot = *reinterpret_cast<const float4*>(hp);
             tot.x += sum.x; tot.y += sum.y; tot.z += sum.z; tot.w += sum.w;
@@ -685,9 +750,9 @@ static __global__ void mt_combine_kernel(const float* __restrict__ partial, cons
             hp[0] += sum.x; hp[1] += sum.y; hp[2] += sum.z; hp[3] += sum.w;
         }
     }
-    if (clock) {
+    if (a.clock) {
         __syncthreads();
-        if (threadIdx.x == 0) atomicMax(clock + 1, global_timer_ns());
+        if (threadIdx.x == 0) atomicMax(a.clock + 1, global_timer_ns());
     }
 }
 

@@ -276,7 +276,7 @@ Layout layout_of(const spm_model_cfg* m, int S) {
     l.partial = c.take((kMaxCtasBatch1 + nb) * D * 4);
     if (nb > 1) {
         l.mt_partial = c.take(mt_partial_rows(kMtMaxCtas, m->max_batch, m->top_k, m->n_experts, m->n_shared) * D * 4);
-        l.mt_map = c.take((4 + nb * SPM_MAX_TOPK) * 4);
+        l.mt_map = c.take((4 + 2 * nb * SPM_MAX_TOPK) * 4);
     }
     l.h = c.take(nb * D * 4);
     l.ids = c.take(nb * SPM_MAX_TOPK * 4);
@@ -448,13 +448,13 @@ int launch_multi(spm_ctx* c, int layer, MtArgs& a, const float* x, const float* 
     CU(c, m.dtype == SPM_DTYPE_FP32 ? launch_multi_g<float>(c, a) : m.dtype == SPM_DTYPE_BF16 ? launch_multi_g<uint16_t>(c, a) : launch_multi_g<Q4Tag>(c, a));
     return SPM_OK;
 }
-int launch_multi_combine(spm_ctx* c, int nb, float* h, bool with_shared) {
+// ... and its combine kernel, for the launch that `a` describes.
+int launch_multi_combine(spm_ctx* c, const MtArgs& a, float* h) {
     const spm_model_cfg& m = c->cfg;
-    const int KS = m.top_k + (with_shared ? m.n_shared : 0);
-    unsigned long long* clock = nullptr;
-    if (int rc = take_clock(c, kClkReduce, &clock)) return rc;
-    CU(c, launch_k(mt_combine_kernel, dim3((m.hidden / 4 + 31) / 32, nb), dim3(32 * KS), 0, c->compute, true, (const float*)c->mt_partial,
-                   (const int32_t*)c->mt_map, KS, mt_grid_for(c), m.inter, m.hidden, h, clock));
+    MtCombineArgs b{a.partial, a.map, h, a.pool, a.shared, a.x, a.w, nullptr, a.blob_bytes, a.K + a.n_shared, mt_grid_for(c), a.I, a.D, a.K, a.n_slots, a.n_shared};
+    if (int rc = take_clock(c, kClkReduce, &b.clock)) return rc;
+    auto kern = m.dtype == SPM_DTYPE_FP32 ? mt_combine_kernel<float> : m.dtype == SPM_DTYPE_BF16 ? mt_combine_kernel<uint16_t> : mt_combine_kernel<Q4Tag>;
+    CU(c, launch_k(kern, dim3((m.hidden / 4 + 31) / 32, a.nb), dim3(32 * b.KS), 0, c->compute, true, b));
     return SPM_OK;
 }
 
@@ -950,18 +950,18 @@ int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, cons
         } else {
             if (t && first) CU(c, cudaEventRecord(t->ffn_start[layer], c->compute));
             if (ring >= 0 && first) CU(c, cudaEventRecord(c->ring_start[ring], c->compute));
+            MtArgs mt;
             if (nb == 1) {
                 FfnArgs<1> a{};
                 fill(a);
                 CU(c, launch_gemv<1>(c, a, G, nb, true));
             } else if (multi) {
-                MtArgs a;
-                a.dev_ids = nullptr;
-                a.dev_slot = nullptr;
-                a.nb = nb;
-                for (int i = 0; i < nb * K; ++i) a.ids[i] = short(ids[i]);
-                std::copy(slot_of_expert.begin(), slot_of_expert.end(), a.slot);
-                if (int rc = launch_multi(c, layer, a, x_norm, w, clock_slot, first)) return rc;
+                mt.dev_ids = nullptr;
+                mt.dev_slot = nullptr;
+                mt.nb = nb;
+                for (int i = 0; i < nb * K; ++i) mt.ids[i] = short(ids[i]);
+                std::copy(slot_of_expert.begin(), slot_of_expert.end(), mt.slot);
+                if (int rc = launch_multi(c, layer, mt, x_norm, w, clock_slot, first)) return rc;
             } else {
                 FfnArgs<SPM_MAX_BATCH> a{};
                 fill(a);
@@ -970,7 +970,7 @@ int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, cons
             if (t && last) CU(c, cudaEventRecord(t->ffn_end[layer], c->compute));
             if (ring >= 0 && last) { CU(c, cudaEventRecord(c->ring_end[ring], c->compute)); c->ring_used[ring] = 1; }
             if (multi) {
-                if (int rc = launch_multi_combine(c, nb, h_inout, first)) return rc;
+                if (int rc = launch_multi_combine(c, mt, h_inout)) return rc;
                 c->kernel_launches += 2;
             } else if (last && leave_partial) {
                 if (left) *left = true;
@@ -1238,7 +1238,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             a.dev_slot = c->ws_slot_map + size_t(l) * n;
             a.nb = nb;
             if (int rc = launch_multi(c, l, a, c->ws_x, c->ws_w, clock_slot, true)) return rc;
-            if (int rc = launch_multi_combine(c, nb, h_out, true)) return rc;
+            if (int rc = launch_multi_combine(c, a, h_out)) return rc;
             c->kernel_launches += 3;
             c->ffn_launches++;
             continue;

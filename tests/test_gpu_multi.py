@@ -121,3 +121,55 @@ def test_a_slot_outside_the_pool_ends_the_launch_with_an_error(name, bad):
     for a, b in zip(run(m, H), good):
         assert np.array_equal(a, b)
     m.close()
+
+
+def plant_infinity(cfg, m, expert, part, row, col):
+    """An infinite weight (4-bit: an infinite scale of the column's group) in one expert of layer 0 of the host store."""
+    if cfg.dtype == "q4":
+        part_bytes, at, raw = cfg.hidden // 2 + cfg.hidden // 16, cfg.hidden // 2 + col // 32 * 2, np.float16(np.inf).tobytes()
+    else:
+        part_bytes, at = cfg.hidden * cfg.elem_bytes, col * cfg.elem_bytes
+        raw = np.float32(np.inf).tobytes()[-cfg.elem_bytes:]
+    at += expert * cfg.expert_bytes + (row * 3 + part) * part_bytes
+    m.store.tensor[at:at + len(raw)] = torch.from_numpy(np.frombuffer(raw, np.uint8).copy())
+
+
+@pytest.mark.parametrize("what", ["activation_inf", "activation_nan", "gate_inf", "down_inf"])
+@pytest.mark.parametrize("name", ["fp32_run_of_one", "bf16_narrow", "q4_shared"])
+def test_infinities_and_nans_are_those_of_one_sequence_at_a_time(name, what):
+    """Activations with eight significant bits (the lower parts of their split are zero: an infinite weight times those
+    would be NaN) and a NaN that its upper half alone would turn into an infinity. Where the batch-1 kernel has a number, an
+    infinity or a NaN, so has this one; sequences that have nothing to do with it keep their bits."""
+    cfg = config(name)
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    x = torch.randn(cfg.batch, cfg.hidden, generator=gen, device="cuda").bfloat16().float()
+    x[:, 40] = 1.0
+    outs = {}
+    for planted in (False, True):
+        m = build(cfg, slots=cfg.n_experts)
+        m.set_batched_path(1)
+        _, ids, w, _ = m.router_topk(0, x)
+        if planted and what == "gate_inf":
+            plant_infinity(cfg, m, 1, 0, cfg.inter // 2, 40)
+        elif planted and what == "down_inf":
+            plant_infinity(cfg, m, 1, 2, cfg.inter - 1, 40)
+        elif planted:
+            x[3, 40] = float("inf")
+            if what == "activation_nan":
+                x[3, 40:41].copy_(torch.tensor([0x7f800001], dtype=torch.int32, device="cuda").view(torch.float32))
+        both = torch.zeros(2, cfg.batch, cfg.hidden, device="cuda")
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x, ids, w, both[0])
+        for t in range(cfg.batch):
+            m.moe_ffn(0, x[t:t + 1], ids[t:t + 1], w[t:t + 1].contiguous(), both[1, t:t + 1])
+        m.synchronize()
+        outs[planted] = both.cpu()
+        m.close()
+    got, want = outs[True]
+    hit = (ids == 1).any(1) if what.endswith("_inf") and not what.startswith("act") else np.arange(cfg.batch) == 3
+    assert hit.any() and not torch.isfinite(want[torch.from_numpy(hit)]).all()
+    assert torch.equal(got[torch.from_numpy(~hit)], outs[False][0][torch.from_numpy(~hit)])
+    assert torch.equal(got.isnan(), want.isnan())
+    assert torch.equal(got.isposinf(), want.isposinf()) and torch.equal(got.isneginf(), want.isneginf())
+    ok = want.isfinite()
+    assert not ok.any() or (got[ok] - want[ok]).abs().max() <= 5e-6 * want[ok].abs().max()
