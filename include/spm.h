@@ -155,7 +155,10 @@ typedef struct {
  * Writes the blob size to *bytes: 3*I*D*sizeof(element), or 3*I*(D/2 + D/16) for 4-bit experts. */
 int spm_expert_blob_bytes(const spm_model_cfg* cfg, size_t* bytes);
 
-/* Bytes of device arena needed for `slots_per_layer` routed slots per layer plus workspace. */
+/* Bytes of device arena needed for `slots_per_layer` routed slots per layer plus workspace. For a model whose batches may run
+ * the several-sequences FFN (spm_set_batched_path) this includes its partial rows: (148 + entries) * 8 of `hidden` floats, 9 MB
+ * for 16 sequences of a 1280 x 896 model with 6 + 2 of 64 experts, where the GEMV needs 1.6 MB. spm_init also takes an arena
+ * without that room; such a context runs the GEMV once per token. */
 int spm_query_arena(const spm_model_cfg* cfg, int slots_per_layer, size_t* bytes);
 
 /* Create a context. budget = M_max >= 0, or -1 to derive it from the profiled overlap window
@@ -240,7 +243,9 @@ int spm_set_ffn_ctas(spm_ctx* ctx, int ctas);             /* CTAs per token of t
  * experts, inter a multiple of 128, hidden a multiple of 128 for bf16 and of 256 for 4-bit
  * weights, which are expanded to bf16 on the way to the tensor cores), else fp32 activations:
  * every expert streamed once for all its tokens where at least 64 Mi weights are shared that
- * way, the GEMV kernel once per token below. 1: always fp32 activations. */
+ * way, the GEMV kernel once per token below. 1: always fp32 activations (a model that could use the
+ * tensor cores streams experts once for all tokens only where the partial rows that this takes fit into
+ * the tensor-core path's own). */
 int spm_set_batched_path(spm_ctx* ctx, int mode);
 /* Perfect-knowledge ranking for SPM_POLICY_HINT_TRACE: for step s (counted from the last
  * spm_cache_reset) and layer l, hint[(s*L + l)*stride .. +count[s*L+l]) are the experts that

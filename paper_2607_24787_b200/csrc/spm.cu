@@ -59,7 +59,7 @@ struct spm_ctx {
     unsigned char* pools = nullptr;
     float *ws_x = nullptr, *ws_logits = nullptr, *ws_pihat = nullptr, *ws_w = nullptr;
     float *ws_scores = nullptr, *ws_partial = nullptr, *ws_h = nullptr;
-    float* mt_partial = nullptr;              // batched fp32-activation path (max_batch > 1): partial rows of ffn_multi_kernel
+    float* mt_partial = nullptr;              // several-sequences kernel: its partial rows (null: the arena has no room for them)
     int32_t* mt_map = nullptr;                //   and where each (token, k) pair was computed
     int32_t *ws_ids = nullptr, *ws_order = nullptr;
     unsigned* ws_counters = nullptr;
@@ -242,11 +242,11 @@ int mt_grid_for(const spm_ctx* c) { return std::min(c->num_sms, kMtMaxCtas); }
 //   fp32 1024 x 250, 32 tokens 4 + 1 of 24:   66 -> 57 (104)    fp32 1024 x 250,  8 tokens 4 + 1 of 24: 27 -> 47 (12)
 //   4-bit 768 x 300, 64 tokens 4 + 1 of 60:  119 -> 63 (179)    4-bit 2048 x 500, 8 tokens 4 + 1 of 60: 50 -> 71 (0)
 constexpr size_t kMtMinSavedWeights = size_t(64) << 20;
-bool use_multi(const spm_ctx* c, int nb) {
-    const spm_model_cfg& m = c->cfg;
+bool multi_pays(const spm_model_cfg& m, int nb) {       // (once it pays it pays for every larger nb too)
     const int reads = nb * (m.top_k + m.n_shared), distinct = std::min(nb * m.top_k, m.n_experts) + m.n_shared;
     return size_t(reads - distinct) * 3 * m.inter * m.hidden >= kMtMinSavedWeights;
 }
+bool use_multi(const spm_ctx* c, int nb) { return c->mt_partial && multi_pays(c->cfg, nb); }
 
 struct Carve {
     size_t off = 0;
@@ -255,14 +255,18 @@ struct Carve {
 
 struct Layout {
     size_t pools, slot_gen, x, logits, pihat, w, scores, partial, h, ids, order, clock, slot_map, codes, counters, status, total;
-    size_t mt_partial, mt_map;                                                     // max_batch > 1 only
-    size_t tc_xs, tc_wrow, tc_partial, tc_desc, tc_counts, tc_act, tc_ready;       // batched tensor-core path only
+    size_t mt_map;                                                                 // several-sequences kernel only
+    size_t tc_xs, tc_wrow, tc_desc, tc_counts, tc_act, tc_ready;       // batched tensor-core path only
     size_t desc_bytes, off_rows, off_rowmap, off_chunks, chunk_cap, off_wait;
     int rows_cap, n_jt, max_units;
-    bool tc;
+    bool tc, multi;
 };
 
-Layout layout_of(const spm_model_cfg* m, int S) {
+// Partial rows of the GEMV, grouped and several-sequences kernels share one region: a layer's expert kernels are all of one kind,
+// and what they leave there is consumed before another kind is launched. With `with_multi` the region also holds what the
+// several-sequences kernel needs, where this model can reach it (22 MB at 64 sequences of the Qwen3 shape). Models that batch
+// on the tensor cores reach it only by spm_set_batched_path(1) and give it no more than the grouped kernels' share.
+Layout layout_of(const spm_model_cfg* m, int S, bool with_multi = true) {
     Layout l{};
     Carve c;
     const size_t nb = m->max_batch, D = m->hidden, n = m->n_experts;
@@ -273,21 +277,29 @@ Layout layout_of(const spm_model_cfg* m, int S) {
     l.pihat = c.take(nb * n * 4);
     l.w = c.take(nb * SPM_MAX_TOPK * 4);
     l.scores = c.take(n * 4);
-    l.partial = c.take((kMaxCtasBatch1 + nb) * D * 4);
-    if (nb > 1) {
-        l.mt_partial = c.take(mt_partial_rows(kMtMaxCtas, m->max_batch, m->top_k, m->n_experts, m->n_shared) * D * 4);
-        l.mt_map = c.take((4 + 2 * nb * SPM_MAX_TOPK) * 4);
+    l.tc = tc_supported(m);
+    size_t partial = (kMaxCtasBatch1 + nb) * D * 4;
+    if (l.tc) {
+        l.rows_cap = m->max_batch * m->top_k;
+        l.n_jt = m->inter / kGgTileRows;
+        partial = std::max(partial, size_t(l.n_jt) * l.rows_cap * D * 4);
     }
+    if (with_multi && nb > 1 && multi_pays(*m, m->max_batch)) {
+        const size_t need = mt_partial_rows(kMtMaxCtas, m->max_batch, m->top_k, m->n_experts, m->n_shared) * D * 4;
+        l.multi = !l.tc || need <= partial;
+        if (l.multi) {
+            partial = std::max(partial, need);
+            l.mt_map = c.take((4 + 2 * nb * SPM_MAX_TOPK) * 4);
+        }
+    }
+    l.partial = c.take(partial);
     l.h = c.take(nb * D * 4);
     l.ids = c.take(nb * SPM_MAX_TOPK * 4);
     l.order = c.take(n * 4);
     l.clock = c.take(size_t(kClockSlots) * 16);
     l.slot_map = c.take(size_t(m->n_layers) * n * sizeof(short));
     l.codes = c.take(size_t(m->n_layers) * nb * SPM_MAX_TOPK * sizeof(short));
-    l.tc = tc_supported(m);
     if (l.tc) {
-        l.rows_cap = m->max_batch * m->top_k;
-        l.n_jt = m->inter / kGgTileRows;
         l.max_units = std::min(S, m->n_experts) * l.n_jt;
         l.off_rows = align_up(size_t(l.max_units) * sizeof(GgUnit), 256);
         l.off_rowmap = l.off_rows + align_up(size_t(l.rows_cap) * sizeof(GgRow), 256);
@@ -298,7 +310,6 @@ Layout layout_of(const spm_model_cfg* m, int S) {
         l.desc_bytes = l.off_wait + align_up(size_t(l.max_units) * sizeof(GgWait), 256);
         l.tc_xs = c.take(size_t(l.rows_cap + kGgTokens) * D * 2);
         l.tc_wrow = c.take(size_t(l.rows_cap) * 4);
-        l.tc_partial = c.take(size_t(l.n_jt) * l.rows_cap * D * 4);
         l.tc_desc = c.take(size_t(kDescRing) * l.desc_bytes);
         l.tc_counts = c.take(2 * sizeof(int));
         l.tc_act = c.take(size_t(l.max_units) * kGgActBytes);
@@ -1379,7 +1390,8 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     if (b->compute_stream == b->copy_stream) return fail(nullptr, SPM_ERR_INVALID_ARG, "compute and copy stream must differ");
     if (b->host_store_layers < 0 || b->host_store_layers > cfg->n_layers) return fail(nullptr, SPM_ERR_INVALID_ARG, "host_store_layers out of range");
     if (reinterpret_cast<uintptr_t>(b->arena) % 256) return fail(nullptr, SPM_ERR_INVALID_ARG, "arena must be 256-byte aligned");
-    const Layout lay = layout_of(cfg, slots_per_layer);
+    Layout lay = layout_of(cfg, slots_per_layer);
+    if (b->arena_bytes < lay.total) lay = layout_of(cfg, slots_per_layer, false);      // one GEMV per sequence then takes every such batch
     if (b->arena_bytes < lay.total) return fail(nullptr, SPM_ERR_INVALID_ARG, "arena too small: %zu < %zu", b->arena_bytes, lay.total);
 
     int dev_count = 0;
@@ -1415,8 +1427,8 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     c->ws_w = reinterpret_cast<float*>(base + lay.w);
     c->ws_scores = reinterpret_cast<float*>(base + lay.scores);
     c->ws_partial = reinterpret_cast<float*>(base + lay.partial);
-    if (cfg->max_batch > 1) {
-        c->mt_partial = reinterpret_cast<float*>(base + lay.mt_partial);
+    if (lay.multi) {
+        c->mt_partial = c->ws_partial;
         c->mt_map = reinterpret_cast<int32_t*>(base + lay.mt_map);
     }
     c->ws_h = reinterpret_cast<float*>(base + lay.h);
@@ -1471,7 +1483,7 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
         c->rows_cap = lay.rows_cap; c->n_jt = lay.n_jt; c->max_units = lay.max_units;
         c->tc_xs = reinterpret_cast<__nv_bfloat16*>(base + lay.tc_xs);
         c->tc_wrow = reinterpret_cast<float*>(base + lay.tc_wrow);
-        c->tc_partial = reinterpret_cast<float*>(base + lay.tc_partial);
+        c->tc_partial = c->ws_partial;
         c->tc_desc_dev = base + lay.tc_desc;
         c->tc_counts = reinterpret_cast<int*>(base + lay.tc_counts);
         c->tc_desc_bytes = lay.desc_bytes; c->tc_off_rows = lay.off_rows; c->tc_off_rowmap = lay.off_rowmap;

@@ -41,6 +41,38 @@ def test_query_and_config_errors():
         B.spm_query_arena(B.make_cfg(2, 256, 16, 128, 2, 15, 8, B.DTYPE_FP32), 4)   # top_k + shared too large
 
 
+# Arena sizes from before the several-sequences kernel existed: device memory that callers have set aside.
+# (layers, hidden, experts, inter, top_k, shared, rank, dtype, max_batch, slots): bytes, and whether the kernel is the default path
+ARENAS = {
+    (48, 2048, 128, 768, 8, 0, 16, B.DTYPE_BF16, 1, 16): (7250423296, False),
+    (48, 2048, 128, 768, 8, 0, 16, B.DTYPE_BF16, 64, 32): (14530726656, False),
+    (48, 2048, 128, 768, 8, 0, 16, B.DTYPE_Q4, 64, 32): (4112075520, False),
+    (3, 2048, 1024, 128, 16, 0, 8, B.DTYPE_BF16, 64, 64): (320763904, False),
+    (2, 256, 16, 128, 2, 0, 8, B.DTYPE_FP32, 64, 16): (13301248, False),
+    (3, 512, 24, 250, 4, 1, 8, B.DTYPE_BF16, 4, 24): (56127232, False),
+    (12, 1280, 64, 896, 6, 2, 16, B.DTYPE_BF16, 16, 64): (5286802944, True),
+    (12, 1280, 64, 896, 6, 2, 16, B.DTYPE_Q4, 64, 8): (188558336, True),
+    (2, 1024, 96, 640, 4, 1, 8, B.DTYPE_FP32, 64, 96): (1512209152, True),
+}
+
+
+@pytest.mark.parametrize("shape", list(ARENAS))
+def test_arena_needs_no_more_than_it_did(shape):
+    """Models that batch on the tensor cores or too little for the several-sequences kernel pay nothing for it; the others
+    are told what it wants but are not refused without (checked on the host, ahead of the device)."""
+    import torch
+    L, d, n, i, k, s, r, dtype, nb, S = shape
+    cfg = B.make_cfg(L, d, n, i, k, s, r, dtype, max_batch=nb)
+    before, wants_more = ARENAS[shape]
+    assert (B.spm_query_arena(cfg, S) > before) == wants_more
+    if torch.cuda.is_available():
+        return                                     # made-up addresses below: they must not reach a device
+    for size, code in ((before, -3), (L * S * B.spm_expert_blob_bytes(cfg), -1)):
+        with pytest.raises(B.SpmError) as e:
+            B.spm_init(cfg, S, 2, B.Buffers(256, 256, 256, 256, 256, 256, 256, size, 1, 2, 0))
+        assert e.value.code == code, str(e.value)
+
+
 def test_init_fails_loudly_without_gpu():
     import torch
     if torch.cuda.is_available():

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 import synth
+from paper_2607_24787_b200 import binding as B
 from paper_2607_24787_b200.binding import SpmError
 from test_gpu_edges import build, compare_run
 from test_gpu_host_free import preload, rows, run
@@ -173,3 +174,21 @@ def test_infinities_and_nans_are_those_of_one_sequence_at_a_time(name, what):
     assert torch.equal(got.isposinf(), want.isposinf()) and torch.equal(got.isneginf(), want.isneginf())
     ok = want.isfinite()
     assert not ok.any() or (got[ok] - want[ok]).abs().max() <= 5e-6 * want[ok].abs().max()
+
+
+def test_an_arena_without_room_for_the_kernel_is_accepted(monkeypatch):
+    """An arena of the size that the model needed without this kernel: one GEMV per sequence serves the batch."""
+    cfg = config("bf16_shared_waves").replace(slots=12)
+    H = rows(cfg, 2)
+    outs = []
+    ask = B.spm_query_arena
+    rows_of = lambda n: n * cfg.hidden * 4
+    entries = min(cfg.batch * cfg.top_k, cfg.n_experts) + cfg.batch * cfg.top_k // 8 + cfg.n_shared * -(-cfg.batch // 8)
+    extra = rows_of((148 + entries) * 8) - rows_of(296 + cfg.batch)          # partial rows beyond the GEMV's
+    for less in (0, extra):
+        monkeypatch.setattr(B, "spm_query_arena", lambda c, s: ask(c, s) - less // 256 * 256)
+        m = build(cfg)
+        outs.append(run(m, H))
+        m.close()
+    for a, b in zip(*outs):
+        assert not np.array_equal(a, b) and np.abs(a - b).max() <= 1e-5 * np.abs(b).max()
