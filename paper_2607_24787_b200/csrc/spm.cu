@@ -1238,7 +1238,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
                 CU(c, launch_k(ffn_grouped_kernel, dim3(c->num_sms), dim3(kGgThreads), ffn_grouped_smem(), c->compute, true, c->wmap, c->xmaps, ga));
             CU(c, launch_k(gg_combine_kernel, gg_combine_grid(m.hidden, nb), gg_combine_block(K), 0, c->compute, true,
                            (const float*)c->tc_partial, (const int32_t*)rowmap, K, c->n_jt, c->rows_cap, m.hidden, h_out));
-            c->kernel_launches += 4;
+            c->kernel_launches += 3;       // (launch_router has counted itself)
             c->ffn_launches++;
             c->tc_launches++;
             continue;
@@ -1250,7 +1250,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             a.nb = nb;
             if (int rc = launch_multi(c, l, a, c->ws_x, c->ws_w, clock_slot, true)) return rc;
             if (int rc = launch_multi_combine(c, a, h_out)) return rc;
-            c->kernel_launches += 3;
+            c->kernel_launches += 2;
             c->ffn_launches++;
             continue;
         }
@@ -1270,7 +1270,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
                            c->compute, true, (const float*)c->ws_partial, (const float*)h_out, h_out, G, m.hidden, reduce_clock));
             c->kernel_launches++;
         }
-        c->kernel_launches += 2;
+        c->kernel_launches++;
         c->ffn_launches++;
     }
     return SPM_OK;

@@ -192,3 +192,32 @@ def test_an_arena_without_room_for_the_kernel_is_accepted(monkeypatch):
         m.close()
     for a, b in zip(*outs):
         assert not np.array_equal(a, b) and np.abs(a - b).max() <= 1e-5 * np.abs(b).max()
+
+
+# kernels of a layer and of the end of a step: routing + GEMV (folded by the next routing kernel) and one combine kernel; routing,
+# gather, grouped FFN, combine; routing, several-sequences FFN, combine
+COUNTS = {
+    "one_sequence": (synth.get_config("tiny", slots=16), 2, 1),
+    "gemv_per_sequence": (synth.get_config("tiny", slots=16, batch=3), 2, 1),
+    "tensor_cores": (synth.get_config("qwen3", n_layers=3, hidden=256, n_experts=8, inter=128, top_k=2, slots=8, budget=1, batch=5), 4, 0),
+    "several_sequences": (config("bf16_run_of_three"), 3, 0),
+    "several_sequences_shared": (config("q4_shared"), 3, 0),
+}
+
+
+@pytest.mark.parametrize("host_free", [0, 1])
+@pytest.mark.parametrize("name", list(COUNTS))
+def test_kernels_of_a_step_are_counted_once(name, host_free):
+    """spm_stats.kernel_launches says what was launched, whichever way a step is enqueued (12 steps: replayed captures among
+    them); it also tells which expert kernel a batch ran."""
+    cfg, a_layer, at_the_end = COUNTS[name]
+    m = build(cfg)
+    m.set_host_free(host_free)
+    preload(cfg, m)
+    m.reset_stats()
+    run(m, rows(cfg, 12))
+    st = m.stats()
+    assert st["host_free_steps"] == (12 if host_free else 0)
+    assert st["ffn_launches"] == 12 * cfg.n_layers
+    assert st["kernel_launches"] == 12 * (a_layer * cfg.n_layers + at_the_end)
+    m.close()
