@@ -128,7 +128,8 @@ typedef struct {
     uint64_t ffn_launches;       /* expert-FFN kernel launches timed below                               */
     uint64_t kernel_launches;    /* all kernels this context launched                                    */
     double   ffn_us;             /* summed CUDA-event time around those launches (needs spm_set_timing(ctx, 1)) */
-    double   ffn_window_us;      /* same launches, first CTA start to last CTA end read from %globaltimer
+    double   ffn_window_us;      /* same launches, first CTA start (of a kernel launched ahead of its predecessor's
+                                    end: first CTA past the wait for it) to last CTA end read from %globaltimer
                                     inside the kernel: excludes launch latency (profiling aid)            */
     double   stall_us;           /* summed gap "routing kernel done -> expert FFN may start" per layer    */
     double   ready_sum;          /* sum over (step, layer >= 1, token) of |T ∩ has-slot| / K at demand   */
@@ -137,7 +138,9 @@ typedef struct {
     uint64_t recall_count;       /*   ExpertRecall@M = recall_sum / recall_count  (Section 4.1)          */
     uint64_t host_free_steps;    /* decode steps enqueued without a host turn (spm_set_host_free)        */
     double router_window_us;     /* in-kernel windows of the routing kernels (first leader past its launch      */
-    double reduce_window_us;     /*   dependency -> last leader done) and of the combine kernels, timing on     */
+    double reduce_window_us;     /*   dependency -> last leader done; the adapter's ranking of a batch is not in
+                                    it where the tensor-core path's gather kernel makes it) and of the combine
+                                    kernels (not the tensor-core path's), timing on                             */
     double gap_us;               /* device idle time between consecutive clocked kernels of the compute stream  */
     double recall_at[3];         /* sums like recall_sum for M = max(1, K/2), K, K+2 (the coverage levels of
                                     the paper's model-level table); divide by recall_count                    */

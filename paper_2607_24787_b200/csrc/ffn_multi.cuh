@@ -64,7 +64,7 @@ struct MtArgs {
     int32_t* map;                   // {entries, -, -, -, [nb][SPM_MAX_TOPK][2] of each (token, k) pair entry | position << 16 (< 0: none), and
                                     //   its expert's slot (shared expert s: -1 - s)}
     int* status;
-    unsigned long long* clock;      // optional {earliest CTA start, latest CTA end} in ns (globaltimer)
+    unsigned long long* clock;      // optional {first CTA past its dependency wait, latest CTA end} in ns (globaltimer)
     const int32_t* dev_ids;         // [nb][K] expert ids left in device memory by the routing kernel, with
     const short* dev_slot;          //   [n] slot of each expert; null: `ids` and `slot` below
     unsigned long long blob_bytes, wait_limit_ns;
@@ -350,7 +350,6 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
     const uint32_t ring = smem_u32(smem), gu_bar = smem_u32(bars), dn_bar = gu_bar + 8 * kMtMaxStages;
 
     grid_dep_launch();
-    const unsigned long long t_entry = (a.clock && threadIdx.x == 0) ? global_timer_ns() : 0ull;
     if (threadIdx.x == 0) {
         for (int s = 0; s < n_stages; ++s) { mbar_init(gu_bar + 8 * s, kMtRows); mbar_init(dn_bar + 8 * s, kMtRows); }
         s_abort = 0;
@@ -546,8 +545,11 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
     };
 
     // With the routing among the launch arguments the plan and the first weight copies need not wait for the preceding kernel.
-    if (!early) grid_dep_wait();
-    if (a.clock && threadIdx.x == 0) atomicMin(a.clock, early ? t_entry : global_timer_ns());
+    auto depend = [&]() {
+        grid_dep_wait();
+        if (a.clock && threadIdx.x == 0) atomicMin(a.clock, global_timer_ns());
+    };
+    if (!early) depend();
     __syncthreads();
     for (int i = threadIdx.x; i < n_pairs; i += kMtThreads) {
         int e = a.dev_ids ? __ldcg(a.dev_ids + i) : int(a.ids[i]);
@@ -583,7 +585,7 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
     fdn = fgu;
     feeding = true;
     for (int i = 0; i < n_stages; ++i) { feed_gu(); feed_dn(); }
-    if (early) grid_dep_wait();          // activations and routing weights come from the preceding kernel
+    if (early) depend();                 // activations and routing weights come from the preceding kernel
 
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0) a.map[0] = s_entries;

@@ -511,6 +511,7 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
         __syncthreads();
         if (threadIdx.x == 0 && mb) mb->seq = a.seq;
     }
+    if (a.clock && a.defer_rank) __syncthreads();      // both halves of this leader (the path above has been through a barrier)
     if (threadIdx.x == 0 && a.clock) atomicMax(a.clock + 1, global_timer_ns());
 }
 
