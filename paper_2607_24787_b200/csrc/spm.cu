@@ -248,6 +248,13 @@ bool multi_pays(const spm_model_cfg& m, int nb) {       // (once it pays it pays
 }
 bool use_multi(const spm_ctx* c, int nb) { return c->mt_partial && multi_pays(c->cfg, nb); }
 
+// The expert kernel that a call with nb sequences runs.
+enum class FfnPath { kGemv, kGrouped, kMulti };
+FfnPath ffn_path(const spm_ctx* c, int nb) {
+    if (nb > 1 && c->tc_ok && c->batched_path == 0) return FfnPath::kGrouped;
+    return use_multi(c, nb) ? FfnPath::kMulti : FfnPath::kGemv;
+}
+
 struct Carve {
     size_t off = 0;
     size_t take(size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; }
@@ -877,7 +884,7 @@ int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, cons
     }
 
     const int G = ffn_grid_for(c, nb);
-    const bool use_tc = nb > 1 && c->tc_ok && c->batched_path == 0, multi = !use_tc && use_multi(c, nb);
+    const bool use_tc = ffn_path(c, nb) == FfnPath::kGrouped, multi = ffn_path(c, nb) == FfnPath::kMulti;
     // kernels that can wait for a copy themselves: the batch-1 GEMV kernels and the grouped tensor-core kernels
     const bool dev_wait = c->device_wait && (nb == 1 || use_tc) && stream_write32_fn() != nullptr;
     std::vector<int16_t>& slot_of_expert = c->wave_slot;   // experts computed in the current wave
@@ -1061,7 +1068,7 @@ int step_layers(spm_ctx* c, float* h_out, int nb, Timing* t, const Mailbox* trac
         return SPM_OK;
     };
     // GEMV path: only the last layer runs the combine kernel, the others leave it to the next routing kernel
-    const bool gemv_path = !(nb > 1 && c->tc_ok && c->batched_path == 0) && !use_multi(c, nb);
+    const bool gemv_path = ffn_path(c, nb) == FfnPath::kGemv;
     if (!trace) if (int rc = enqueue_router(0)) return rc;
     for (int l = 0; l < L; ++l) {
         const bool has_adapter = l <= L - 2;
@@ -1195,8 +1202,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
         short* codes = c->ws_codes + size_t(l) * m.max_batch * SPM_MAX_TOPK;
         // On the GEMV path the routing kernel of layer l + 1 also folds layer l's partial rows into the
         // hidden row, so only the last layer needs the combine kernel.
-        const bool use_tc = nb > 1 && c->tc_ok && c->batched_path == 0;
-        const bool multi = !use_tc && use_multi(c, nb);
+        const bool use_tc = ffn_path(c, nb) == FfnPath::kGrouped, multi = ffn_path(c, nb) == FfnPath::kMulti;
         const bool fold = !use_tc && !multi && l > 0 && c->stub_us == 0;
         RankArgs rank{};               // grouped kernels: the plan and gather kernel has a block for the adapter's ranking
         RouterRoute route{c->tr_dev + size_t(slot) * L + l, c->ws_slot_map + size_t(l) * n, codes, true,
@@ -1342,6 +1348,8 @@ int check_layer(spm_ctx* c, int layer, int nb) {
     return SPM_OK;
 }
 
+bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+
 int check_status(spm_ctx* c) {
     int st = 0;
     CU(c, cudaMemcpy(&st, c->ws_status, sizeof st, cudaMemcpyDeviceToHost));
@@ -1390,6 +1398,8 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     if (b->compute_stream == b->copy_stream) return fail(nullptr, SPM_ERR_INVALID_ARG, "compute and copy stream must differ");
     if (b->host_store_layers < 0 || b->host_store_layers > cfg->n_layers) return fail(nullptr, SPM_ERR_INVALID_ARG, "host_store_layers out of range");
     if (reinterpret_cast<uintptr_t>(b->arena) % 256) return fail(nullptr, SPM_ERR_INVALID_ARG, "arena must be 256-byte aligned");
+    if (!aligned16(b->rms_gamma) || !aligned16(b->router_w) || !aligned16(b->adapter_a) || !aligned16(b->shared_experts))
+        return fail(nullptr, SPM_ERR_INVALID_ARG, "rms_gamma, router_w, adapter_a and shared_experts must be 16-byte aligned");
     Layout lay = layout_of(cfg, slots_per_layer);
     if (b->arena_bytes < lay.total) lay = layout_of(cfg, slots_per_layer, false);      // one GEMV per sequence then takes every such batch
     if (b->arena_bytes < lay.total) return fail(nullptr, SPM_ERR_INVALID_ARG, "arena too small: %zu < %zu", b->arena_bytes, lay.total);
@@ -1558,6 +1568,7 @@ int spm_router_topk(spm_ctx* c, int layer, const float* h, int nb, float* x_norm
     if (int rc = check_layer(c, layer, nb)) return rc;
     if (int rc = flush_trace(c)) return rc;
     if (!h || !x_norm || !ids || !w) return fail(c, SPM_ERR_INVALID_ARG, "null argument");
+    if (!aligned16(h) || !aligned16(x_norm)) return fail(c, SPM_ERR_INVALID_ARG, "h and x_norm must be 16-byte aligned");
     if (int rc = launch_router(c, layer, h, nullptr, nb, x_norm, logits, true, false)) return rc;
     CU(c, cudaMemcpyAsync(w, c->ws_w, size_t(nb) * c->cfg.top_k * 4, cudaMemcpyDeviceToDevice, c->compute));
     if (int rc = wait_mailbox(c)) return rc;
@@ -1610,6 +1621,10 @@ int spm_moe_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, 
     if (int rc = check_layer(c, layer, nb)) return rc;
     if (int rc = flush_trace(c)) return rc;
     if (!x_norm || !ids || !w || !h_inout) return fail(c, SPM_ERR_INVALID_ARG, "null argument");
+    const FfnPath path = ffn_path(c, nb);
+    if (!aligned16(x_norm) && path != FfnPath::kMulti && !(path == FfnPath::kGemv && c->cfg.dtype == SPM_DTYPE_Q4))
+        return fail(c, SPM_ERR_INVALID_ARG, "x_norm must be 16-byte aligned here");
+    if (!aligned16(h_inout) && path == FfnPath::kGrouped) return fail(c, SPM_ERR_INVALID_ARG, "h_inout must be 16-byte aligned on the tensor-core path");
     int ring = -1;
     if (c->timing) {
         ring = int(c->ring_pos++ % c->ring_start.size());
@@ -1621,6 +1636,7 @@ int spm_moe_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, 
 int spm_decode_step(spm_ctx* c, const float* h_in, int nb, float* h_out) {
     if (int rc = check_layer(c, 0, nb)) return rc;
     if (!h_in || !h_out) return fail(c, SPM_ERR_INVALID_ARG, "null argument");
+    if (!aligned16(h_out)) return fail(c, SPM_ERR_INVALID_ARG, "h_out must be 16-byte aligned");
     const spm_model_cfg& m = c->cfg;
     if (c->policy == SPM_POLICY_HINT_TRACE && c->table->step() + int(c->tr_pending.size()) >= c->hint_steps)
         return fail(c, SPM_ERR_STATE, "no hint trace for step %d", c->table->step() + int(c->tr_pending.size()));
@@ -1986,6 +2002,7 @@ int spm_time_ffn_kernel(spm_ctx* c, int first_layer, const float* x_norm, const 
                         int chained, double* us_per_launch, double* window_us) {
     if (int rc = check_layer(c, first_layer, 1)) return rc;
     if (!x_norm || !ids || !w || !us_per_launch || launches < 1) return fail(c, SPM_ERR_INVALID_ARG, "bad argument");
+    if (!aligned16(x_norm) && c->cfg.dtype != SPM_DTYPE_Q4) return fail(c, SPM_ERR_INVALID_ARG, "x_norm must be 16-byte aligned");
     if (int rc = flush_trace(c)) return rc;
     const spm_model_cfg& m = c->cfg;
     const int K = m.top_k, L = m.n_layers;

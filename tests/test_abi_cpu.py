@@ -27,6 +27,19 @@ def test_header_symbols_exported(lib):
         assert hasattr(lib, name), name
 
 
+def test_misaligned_buffers_are_refused_ahead_of_the_device():
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("made-up addresses")
+    cfg = B.make_cfg(2, 256, 16, 128, 2, 1, 8, B.DTYPE_FP32)
+    for i, what in enumerate(("rms_gamma", "router_w", "adapter_a", None, "shared_experts")):
+        at = [256] * 5
+        at[i] += 8
+        with pytest.raises(B.SpmError) as e:
+            B.spm_init(cfg, 4, 2, B.Buffers(*at, 256, 256, 1 << 40, 1, 2, 0))
+        assert e.value.code == (-1 if what else -3)          # (adapter_b is read one element at a time)
+
+
 def test_query_and_config_errors():
     cfg = B.make_cfg(48, 2048, 128, 768, 8, 0, 16, B.DTYPE_BF16)
     assert B.spm_expert_blob_bytes(cfg) == 9437184

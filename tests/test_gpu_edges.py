@@ -388,3 +388,43 @@ def test_ffn_kernel_probe_in_all_launch_modes_leaves_the_context_usable():
             assert M.rel_linf(out.cpu().numpy().astype(np.float64)[0], want[0]) < 4e-5
     finally:
         m.close()
+
+
+def test_rows_off_a_16_byte_boundary_are_refused_or_served():
+    """The kernels read most rows 16 bytes at a time. A call whose rows do not start on such a boundary is refused on the host,
+    nothing is enqueued; rows that are read one float at a time may start anywhere."""
+    from paper_2607_24787_b200 import binding as B
+
+    def shifted(t):
+        buf = torch.empty(t.numel() + 4, dtype=t.dtype, device="cuda")
+        out = buf[1:1 + t.numel()].view_as(t)
+        out.copy_(t)
+        torch.cuda.synchronize()
+        return out
+
+    for base, batch, x_any, h_any in (("tiny", 1, False, True), ("tiny", 3, False, True), ("qwen3_q4", 1, True, True), ("qwen3", 4, False, False)):
+        cfg = synth.get_config(base, n_layers=2, hidden=256, n_experts=8, inter=128, top_k=2, slots=8, budget=1, batch=batch)
+        m = build(cfg)
+        h = torch.randn(batch, cfg.hidden, device="cuda")
+        x, ids, w, _ = m.router_topk(0, h)
+        want = h.clone()
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x, ids, w, want)
+        m.synchronize()
+        m.reset_stats()
+        refused = [lambda: m.router_topk(0, shifted(h)), lambda: m.decode_step(h, shifted(h))]
+        for any_float, xs, hs in ((x_any, shifted(x), h.clone()), (h_any, x, shifted(h))):
+            call = lambda xs=xs, hs=hs: m.moe_ffn(0, xs, ids, w, hs)
+            if not any_float:
+                refused.append(call)
+                continue
+            call()
+            m.synchronize()
+            assert torch.equal(hs, want)
+            m.reset_stats()
+        for call in refused:
+            with pytest.raises(B.SpmError) as e:
+                call()
+            assert e.value.code == -1
+        assert m.stats()["kernel_launches"] == 0
+        m.close()
