@@ -249,8 +249,8 @@ int spm_set_ffn_ctas(spm_ctx* ctx, int ctas);             /* CTAs per token of t
  * activations, fp32 accumulation) whenever the shape allows it (bf16 or 4-bit weights, no shared
  * experts, inter a multiple of 128, hidden a multiple of 128 for bf16 and of 256 for 4-bit
  * weights, which are expanded to bf16 on the way to the tensor cores), else fp32 activations:
- * every expert streamed once for all its tokens where at least 64 Mi weights are shared that
- * way, the GEMV kernel once per token below. 1: always fp32 activations (a model that could use the
+ * every expert streamed once per eight of its tokens where at least 64 Mi weights (for some shapes more)
+ * need not be read again that way, the GEMV kernel once per token below. 1: always fp32 activations (a model that could use the
  * tensor cores streams experts once for all tokens only where the partial rows that this takes fit into
  * the tensor-core path's own). */
 int spm_set_batched_path(spm_ctx* ctx, int mode);

@@ -235,16 +235,34 @@ constexpr int kMtMaxCtas = 148;
 int mt_grid_for(const spm_ctx* c) { return std::min(c->num_sms, kMtMaxCtas); }
 // fp32-activation path of a batch. One GEMV per sequence reads an expert once per token that uses it; ffn_multi_kernel reads
 // it once per eight but has the longer chain of latencies (plan, split operands, a combine kernel instead of the fold
-// in the next routing kernel: some 17 us a layer). It pays from about 64 M weights on that are not read again; measured,
-// us a layer, GEMV per sequence -> several sequences at a time (saved reads in M weights):
-//   bf16 1280 x 896, 16 tokens 6 + 2 of 64:  120 -> 92 (213)    bf16 1280 x 200, 32 tokens 4 of 64:   48 -> 51 (49)
-//   bf16  512 x 250, 64 tokens 4 + 1 of 24:   68 -> 43 (113)    bf16  512 x 250, 16 tokens 4 + 1 of 24: 28 -> 33 (21)
-//   fp32 1024 x 250, 32 tokens 4 + 1 of 24:   66 -> 57 (104)    fp32 1024 x 250,  8 tokens 4 + 1 of 24: 27 -> 47 (12)
-//   4-bit 768 x 300, 64 tokens 4 + 1 of 60:  119 -> 63 (179)    4-bit 2048 x 500, 8 tokens 4 + 1 of 60: 50 -> 71 (0)
-constexpr size_t kMtMinSavedWeights = size_t(64) << 20;
-bool multi_pays(const spm_model_cfg& m, int nb) {       // (once it pays it pays for every larger nb too)
-    const int reads = nb * (m.top_k + m.n_shared), distinct = std::min(nb * m.top_k, m.n_experts) + m.n_shared;
-    return size_t(reads - distinct) * 3 * m.inter * m.hidden >= kMtMinSavedWeights;
+// in the next routing kernel: some 17 us a layer, more for wide rows). It pays from about 64 Mi weights on that are not read
+// again, and by weight type
+//   bf16   a little later for wide rows (59 Mi + hidden / 128 Mi);
+//   4-bit  where the saved reads also outweigh the unpacking of the experts it computes, which grows with the row;
+//   fp32   where the reads exceed the experts it computes by a quarter: a block's arithmetic, nine MMAs a tile over columns
+//          padded to 256 and a latency worth another 256, outweighs its bytes.
+// Measured on 253 shapes (hidden 256 - 2048, 12 - 128 experts, 3 - 64 sequences), us a layer of a whole host-free step, GEMV
+// per sequence -> several sequences at a time (saved reads in Mi weights); first its own side of the line, then the GEMV's:
+//   bf16  1280 x 896, 16 tokens 6 + 2 of 64: 121 -> 94 (203)     1280 x 653,  6 tokens 7 + 2 of 24:   51 -> 55 (67)
+//         1280 x 200, 40 tokens 4 of 64:      57 -> 54 (70)      the same, 32 tokens:                 49 -> 51 (47)
+//          512 x 250, 40 tokens 4 + 1 of 24:  45 -> 34 (64)      the same, 16 tokens:                 28 -> 33 (20)
+//   4-bit  768 x 300, 64 tokens 4 + 1 of 60: 119 -> 63 (171)     2048 x 906, 15 tokens 2 + 1 of 96:   74 -> 98 (74)
+//         2048 x 500, 24 tokens 4 + 1 of 60: 104 -> 99 (173)     the same, 16 tokens:                 76 -> 90 (56)
+//   fp32  1024 x 250, 32 tokens 4 + 1 of 24:  67 -> 58 (99)      the same, 24 tokens:                 53 -> 56 (70)
+//          768 x 640, 24 tokens 6 + 2 of 60: 119 -> 112 (183)    the same, 16 tokens:                 91 -> 102 (93)
+//          512 x 384, 64 tokens 3 + 1 of 96: 104 -> 91 (89)       640 x 735, 31 tokens 7 + 1 of 128: 173 -> 191 (160)
+// Of 124 shapes that it chooses four are slower than with the GEMV, by 2 - 3 %; of those above 64 Mi that it leaves to the GEMV
+// two would gain 7 - 8 %.
+constexpr size_t kMi = size_t(1) << 20;
+bool multi_pays(const spm_model_cfg& m, int nb) {
+    const size_t D = m.hidden, expert = size_t(3) * m.inter * D;
+    const size_t distinct = std::min(nb * m.top_k, m.n_experts) + m.n_shared;
+    const size_t reads = nb * (m.top_k + m.n_shared) * expert, computed = distinct * expert, saved = reads - computed;
+    if (saved < 64 * kMi) return false;
+    if (m.dtype == SPM_DTYPE_BF16) return saved >= 59 * kMi + D * kMi / 128;
+    if (m.dtype == SPM_DTYPE_Q4) return saved >= computed / 4096 * D;
+    const size_t cols = align_up(D, 256);
+    return 4 * reads >= 5 * computed / D * (cols + 256) + 4 * (12 * kMi + 3 * cols * kMi / 64);
 }
 bool use_multi(const spm_ctx* c, int nb) { return c->mt_partial && multi_pays(c->cfg, nb); }
 
@@ -291,7 +309,9 @@ Layout layout_of(const spm_model_cfg* m, int S, bool with_multi = true) {
         l.n_jt = m->inter / kGgTileRows;
         partial = std::max(partial, size_t(l.n_jt) * l.rows_cap * D * 4);
     }
-    if (with_multi && nb > 1 && multi_pays(*m, m->max_batch)) {
+    bool reached = false;
+    for (int b = 2; b <= m->max_batch; ++b) reached = reached || multi_pays(*m, b);
+    if (with_multi && reached) {
         const size_t need = mt_partial_rows(kMtMaxCtas, m->max_batch, m->top_k, m->n_experts, m->n_shared) * D * 4;
         l.multi = !l.tc || need <= partial;
         if (l.multi) {

@@ -15,8 +15,8 @@ from test_gpu_host_free import preload, rows, run
 pytestmark = pytest.mark.gpu
 
 # Tokens of an expert: runs of eight, one MMA per tile up to two tokens of a run and three above. Rows: blocks of eight.
-# Columns: groups of 32 over eight warps. The kernel takes over where 64 Mi weights and more are not read again, hence
-# few experts and many tokens.
+# Columns: groups of 32 over eight warps. The kernel takes over where enough weights are not read again (takes_kernel),
+# hence few experts and many tokens.
 CASES = {
     # every expert in every token: 64 = 8 full runs; 17 = two runs and one token; 10 = one run and two; 11 = ... and three
     "fp32_all_experts": dict(base="tiny", hidden=256, n_experts=3, inter=463, top_k=3, slots=3, batch=64),
@@ -32,12 +32,25 @@ CASES = {
 }
 
 
+def takes_kernel(cfg, nb):
+    """The rule by which a batch that keeps fp32 activations is given to this kernel."""
+    expert = 3 * cfg.inter * cfg.hidden
+    distinct = min(nb * cfg.top_k, cfg.n_experts) + cfg.n_shared
+    reads, computed = nb * (cfg.top_k + cfg.n_shared) * expert, distinct * expert
+    if reads - computed < 64 << 20:
+        return False
+    if cfg.dtype == "bf16":
+        return reads - computed >= (59 << 20) + cfg.hidden * 8192
+    if cfg.dtype == "q4":
+        return reads - computed >= computed // 4096 * cfg.hidden
+    cols = -(-cfg.hidden // 256) * 256
+    return 4 * reads >= 5 * computed // cfg.hidden * (cols + 256) + 4 * ((12 << 20) + 3 * cols * 16384)
+
+
 def config(name):
     kw = dict(CASES[name])
     cfg = synth.get_config(kw.pop("base"), n_layers=2, budget=1, **kw)
-    reads = cfg.batch * (cfg.top_k + cfg.n_shared)
-    distinct = min(cfg.batch * cfg.top_k, cfg.n_experts) + cfg.n_shared
-    assert (reads - distinct) * 3 * cfg.inter * cfg.hidden >= 64 << 20, "this shape would take the other kernel"
+    assert takes_kernel(cfg, cfg.batch), "this shape would take the other kernel"
     return cfg
 
 
@@ -220,4 +233,33 @@ def test_kernels_of_a_step_are_counted_once(name, host_free):
     assert st["host_free_steps"] == (12 if host_free else 0)
     assert st["ffn_launches"] == 12 * cfg.n_layers
     assert st["kernel_launches"] == 12 * (a_layer * cfg.n_layers + at_the_end)
+    m.close()
+
+
+# around the line of each weight type: (shape, sequences below it, sequences above it)
+LINES = {
+    "bf16_wide": (dict(base="dsvl2", hidden=1280, n_experts=24, inter=653, top_k=7, slots=24, adapter_rank=8), 6, 8),
+    "q4_one_token_each": (dict(base="dsvl2_q4", hidden=2048, n_experts=30, inter=906, top_k=2, n_shared=1, slots=30, adapter_rank=8), 15, 18),
+    "fp32": (dict(base="tiny", hidden=1024, n_experts=24, inter=250, top_k=4, n_shared=1, slots=24), 24, 32),
+}
+
+
+@pytest.mark.parametrize("name", list(LINES))
+def test_the_line_between_the_kernels(name):
+    """Where this kernel was measured slower than one GEMV per sequence, the batch runs the GEMV: seen in the launches of a
+    step (routing and GEMV a layer and one combine kernel; routing, FFN and combine kernel a layer)."""
+    kw, below, above = LINES[name]
+    kw = dict(kw)
+    cfg = synth.get_config(kw.pop("base"), n_layers=2, budget=1, batch=above, **kw)
+    assert not takes_kernel(cfg, below) and takes_kernel(cfg, above)
+    m = build(cfg, store_layers=1)
+    preload(cfg, m)
+    H = torch.as_tensor(rows(cfg, 1)[0], dtype=torch.float32).cuda()
+    for nb, launches in ((below, 2 * cfg.n_layers + 1), (above, 3 * cfg.n_layers)):
+        h = H[:nb].contiguous()
+        torch.cuda.synchronize()
+        m.reset_stats()
+        m.decode_step(h)
+        m.synchronize()
+        assert m.stats()["kernel_launches"] == launches, nb
     m.close()
