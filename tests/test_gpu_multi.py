@@ -22,6 +22,7 @@ CASES = {
     "fp32_all_experts": dict(base="tiny", hidden=256, n_experts=3, inter=463, top_k=3, slots=3, batch=64),
     "fp32_run_of_one": dict(base="tiny", hidden=1024, n_experts=4, inter=460, top_k=4, slots=4, batch=17),
     "fp32_idle_last_group": dict(base="tiny", hidden=384, n_experts=6, inter=511, top_k=3, slots=6, batch=48),
+    "fp32_half_the_warps": dict(base="tiny", hidden=128, n_experts=12, inter=461, top_k=8, slots=12, batch=64),       # four groups of columns
     "bf16_run_of_two": dict(base="qwen3", hidden=2048, n_experts=4, inter=401, top_k=4, slots=4, batch=10),
     "bf16_run_of_three": dict(base="qwen3", hidden=1280, n_experts=4, inter=601, top_k=4, slots=4, batch=11),
     "bf16_shared_waves": dict(base="dsvl2", hidden=1280, n_experts=12, inter=250, top_k=3, slots=5, batch=29),
@@ -263,3 +264,90 @@ def test_the_line_between_the_kernels(name):
         m.synchronize()
         assert m.stats()["kernel_launches"] == launches, nb
     m.close()
+
+
+HOST_FREE = ["fp32_all_experts", "fp32_idle_last_group", "bf16_run_of_three", "bf16_shared_waves", "q4_shared", "q4_widest_waves"]
+
+
+@pytest.mark.parametrize("name", HOST_FREE)
+def test_host_free_steps_equal_host_driven_ones(name):
+    """The routing read on the device (launch by launch, then replayed from captures) against the routing in the launch
+    arguments: same bits, events and statistics. The launch counts say that both ran this kernel."""
+    cfg = config(name).replace(slots=config(name).n_experts)
+    steps = 20                      # every slot of the trace ring is captured and replayed
+    H = rows(cfg, steps)
+    results = []
+    for host_free in (1, 0):
+        m = build(cfg)
+        m.set_host_free(host_free)
+        m.set_policy("adapter")
+        preload(cfg, m)
+        m.reset_stats()
+        outs = run(m, H, sync_every=0 if host_free else 1)
+        st = m.stats()
+        assert st["host_free_steps"] == (steps if host_free else 0) and st["misses"] == 0
+        assert st["kernel_launches"] == 3 * cfg.n_layers * steps
+        results.append((outs, m.events(), {k: st[k] for k in ("hits", "touches", "steps", "tokens", "recall_sum", "ready_sum")}))
+        m.close()
+    (a, ev_a, st_a), (b, ev_b, st_b) = results
+    for s in range(steps):
+        assert np.array_equal(a[s], b[s]), s
+    assert ev_a == ev_b and st_a == st_b
+
+
+@pytest.mark.parametrize("name", ["fp32_all_experts", "bf16_shared_waves", "q4_narrow"])
+def test_fewer_sequences_than_the_context_was_made_for(name):
+    """One context over both sides of the rule: which kernel a call takes follows its own number of sequences, and the
+    results are those of one sequence at a time either way (5e-6: the roundings of some hundred additions)."""
+    cfg = config(name).replace(slots=config(name).n_experts)
+    first = next(nb for nb in range(1, cfg.batch + 1) if takes_kernel(cfg, nb))
+    m = build(cfg)
+    preload(cfg, m)
+    H = torch.as_tensor(rows(cfg, 1)[0], dtype=torch.float32).cuda()
+    for nb in sorted({2, first - 1, first, cfg.batch - 1}):
+        h = H[:nb].contiguous()
+        torch.cuda.synchronize()
+        x, ids, w, _ = m.router_topk(0, h)
+        both = torch.zeros(2, *h.shape, device="cuda")
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x, ids, w, both[0])
+        for t in range(nb):
+            m.moe_ffn(0, x[t:t + 1], ids[t:t + 1], w[t:t + 1].contiguous(), both[1, t:t + 1])
+        m.synchronize()
+        assert (both[0] - both[1]).abs().max() <= 5e-6 * both[1].abs().max()
+        m.reset_stats()
+        m.decode_step(h)
+        m.synchronize()
+        assert m.stats()["kernel_launches"] == (3 * cfg.n_layers if nb >= first else 2 * cfg.n_layers + 1), nb
+    m.close()
+
+
+def test_error_against_64_bits_is_that_of_fp32_sums():
+    """Distance of one layer's output from 64-bit arithmetic, this kernel against one GEMV (fp32 multiply-adds) per sequence.
+    Products are exact in both and both round some hundred partial sums: neither is better in general, so a shape may
+    favour one by a quarter, and all shapes together by a tenth at most."""
+    ratios = {}
+    for name in ("fp32_all_experts", "fp32_run_of_one", "fp32_idle_last_group", "bf16_run_of_two", "bf16_shared_waves", "bf16_narrow", "q4_narrow", "q4_shared"):
+        cfg = config(name)
+        m = build(cfg, slots=cfg.n_experts)
+        h = torch.randn(cfg.batch, cfg.hidden, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+        torch.cuda.synchronize()
+        x, ids, w, _ = m.router_topk(0, h)
+        both = torch.zeros(2, *h.shape, device="cuda")
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x, ids, w, both[0])
+        for t in range(cfg.batch):
+            m.moe_ffn(0, x[t:t + 1], ids[t:t + 1], w[t:t + 1].contiguous(), both[1, t:t + 1])
+        m.synchronize()
+        m.close()
+        want = torch.zeros_like(h, dtype=torch.float64)
+        for e in range(cfg.n_experts + cfg.n_shared):
+            gate, up, down = (a[0].double() for a in synth.expert_matrices(cfg, 0, [e], device="cuda"))
+            part = torch.from_numpy(ids).cuda() == e if e < cfg.n_experts else torch.zeros(cfg.batch, cfg.top_k, device="cuda")
+            weight = (w.double() * part).sum(1) if e < cfg.n_experts else torch.ones(cfg.batch, dtype=torch.float64, device="cuda")
+            xd = x.double()
+            want += weight[:, None] * ((torch.nn.functional.silu(xd @ gate.T) * (xd @ up.T)) @ down.T)
+        err = [((b.double() - want).norm() / want.norm()).item() for b in both]
+        assert err[0] <= 4e-7, (name, err)
+        ratios[name] = err[0] / err[1]
+    assert max(ratios.values()) <= 1.25 and np.exp(np.mean(np.log(list(ratios.values())))) <= 1.1, ratios
