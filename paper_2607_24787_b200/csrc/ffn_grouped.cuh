@@ -666,7 +666,7 @@ static_assert(SPM_MAX_BATCH * SPM_MAX_TOPK < (1 << 21), "three counts of pairs s
 static __global__ void __launch_bounds__(kGgPairThreads)
 gg_plan_gather_kernel(const float* __restrict__ x, const float* __restrict__ w, const int32_t* __restrict__ ids, const short* __restrict__ slot_map,
                       int slot_base, int n_pairs, int K, int n, int n_jt, int D, GgUnit* __restrict__ units, int32_t* __restrict__ rowmap,
-                      int* __restrict__ counts /* {n_units, n_rows} */, __nv_bfloat16* __restrict__ xs, float* __restrict__ wrow, int perm8,
+                      int* __restrict__ n_units, __nv_bfloat16* __restrict__ xs, float* __restrict__ wrow, int perm8,
                       int* act_ready, int n_ready, int* status, const RankArgs rank) {
     __shared__ __align__(16) float rank_sm[SPM_MAX_EXPERTS];
     __shared__ unsigned used[SPM_MAX_EXPERTS / 32];          // experts that some pair names
@@ -709,7 +709,7 @@ gg_plan_gather_kernel(const float* __restrict__ x, const float* __restrict__ w, 
             routed += __popc(m);
             rank += v < (e >> 5) ? __popc(m) : v == (e >> 5) ? __popc(m & ((1u << (e & 31)) - 1u)) : 0;
         }
-        if (i == 0 && tid == 0) { counts[0] = routed * n_jt; counts[1] = n_pairs; }
+        if (i == 0 && tid == 0) *n_units = routed * n_jt;
         if (before == 0) {
             const int slot = slot_map[e];
             if (slot < 0 && tid == 0) atomicOr(status, kStatusBadSlot);

@@ -79,7 +79,7 @@ struct spm_ctx {
     float *tc_wrow = nullptr, *tc_partial = nullptr;
     unsigned char* tc_desc_dev = nullptr;     // kDescRing wave descriptors
     unsigned char* tc_desc_host = nullptr;    // pinned staging, same layout
-    int* tc_counts = nullptr;                 // {units, rows} of a wave planned on the device
+    int* tc_n_units = nullptr;                // units of a wave planned on the device
     size_t tc_desc_bytes = 0, tc_off_rows = 0, tc_off_rowmap = 0, tc_off_chunks = 0, tc_chunk_cap = 0, tc_off_wait = 0;
     int wave_row_off = 0;                     // rows of the sorted token arrays taken by the earlier waves of this layer
     std::vector<int32_t> wave_rowmap;         // [nb][SPM_MAX_TOPK] row of each (token, k) pair over all waves so far
@@ -281,7 +281,7 @@ struct Carve {
 struct Layout {
     size_t pools, slot_gen, x, logits, pihat, w, scores, partial, h, ids, order, clock, slot_map, codes, counters, status, total;
     size_t mt_map;                                                                 // several-sequences kernel only
-    size_t tc_xs, tc_wrow, tc_desc, tc_counts, tc_act, tc_ready;       // batched tensor-core path only
+    size_t tc_xs, tc_wrow, tc_desc, tc_n_units, tc_act, tc_ready;       // batched tensor-core path only
     size_t desc_bytes, off_rows, off_rowmap, off_chunks, chunk_cap, off_wait;
     int rows_cap, n_jt, max_units;
     bool tc, multi;
@@ -338,7 +338,7 @@ Layout layout_of(const spm_model_cfg* m, int S, bool with_multi = true) {
         l.tc_xs = c.take(size_t(l.rows_cap + kGgTokens) * D * 2);
         l.tc_wrow = c.take(size_t(l.rows_cap) * 4);
         l.tc_desc = c.take(size_t(kDescRing) * l.desc_bytes);
-        l.tc_counts = c.take(2 * sizeof(int));
+        l.tc_n_units = c.take(sizeof(int));
         l.tc_act = c.take(size_t(l.max_units) * kGgActBytes);
         l.tc_ready = c.take(size_t(l.max_units + 1) * sizeof(int));
     }
@@ -1252,10 +1252,10 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             int32_t* rowmap = reinterpret_cast<int32_t*>(dd + c->tc_off_rowmap);
             CU(c, launch_k(gg_plan_gather_kernel, dim3(nb * K + (rank.pihat ? 1 : 0)), dim3(kGgPairThreads), 0, c->compute, true, (const float*)c->ws_x, (const float*)c->ws_w,
                            (const int32_t*)c->ws_ids, (const short*)(c->ws_slot_map + size_t(l) * n), l * c->S, nb * K, K, n, c->n_jt, m.hidden,
-                           units, rowmap, c->tc_counts, c->tc_xs, c->tc_wrow, m.dtype == SPM_DTYPE_Q4 ? 1 : 0,
+                           units, rowmap, c->tc_n_units, c->tc_xs, c->tc_wrow, m.dtype == SPM_DTYPE_Q4 ? 1 : 0,
                            m.dtype == SPM_DTYPE_Q4 ? (int*)nullptr : c->tc_ready, m.dtype == SPM_DTYPE_Q4 ? 0 : c->max_units + 1, c->ws_status, rank));
             // (no chunk list here: the plan is built on the device, a chunk is a whole unit)
-            GgArgs ga{units, 0, c->tc_counts, c->tc_wrow, c->tc_partial, c->rows_cap, m.hidden, m.inter, c->ws_status, c->wait_limit_ns,
+            GgArgs ga{units, 0, c->tc_n_units, c->tc_wrow, c->tc_partial, c->rows_cap, m.hidden, m.inter, c->ws_status, c->wait_limit_ns,
                       nullptr, 0, c->tc_ready, c->tc_act, c->tc_ready + 1, clock_slot};
             if (m.dtype == SPM_DTYPE_Q4)
                 CU(c, launch_k(ffn_grouped_q4_kernel, dim3(c->num_sms), dim3(kQgThreads), ffn_grouped_q4_smem(), c->compute, true,
@@ -1515,7 +1515,7 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
         c->tc_wrow = reinterpret_cast<float*>(base + lay.tc_wrow);
         c->tc_partial = c->ws_partial;
         c->tc_desc_dev = base + lay.tc_desc;
-        c->tc_counts = reinterpret_cast<int*>(base + lay.tc_counts);
+        c->tc_n_units = reinterpret_cast<int*>(base + lay.tc_n_units);
         c->tc_desc_bytes = lay.desc_bytes; c->tc_off_rows = lay.off_rows; c->tc_off_rowmap = lay.off_rowmap;
         c->tc_off_chunks = lay.off_chunks; c->tc_chunk_cap = lay.chunk_cap; c->tc_off_wait = lay.off_wait;
         c->tc_act = base + lay.tc_act;
