@@ -368,17 +368,23 @@ cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
     return cudaLaunchKernelEx(&lc, kern, std::forward<Args>(args)...);
 }
 
-template <typename WT, int NSEG, int MAXNB>
-cudaError_t launch_gemv_t(const FfnArgs<MAXNB>& a, int G, int nb, int warps, int depth, size_t smem, cudaStream_t st, bool pdl) {
-    static bool attr_set[64] = {};          // the attribute is per device
-    auto kern = ffn_gemv_kernel<WT, NSEG, MAXNB>;
+// The attribute is per kernel and device; set once (by several threads at worst).
+template <auto kern>
+cudaError_t allow_full_smem() {
+    static std::atomic<bool> done[64];
     int dev = 0;
     cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFfnSmemLimit));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
+    const bool known = dev >= 0 && dev < 64;
+    if (known && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFfnSmemLimit));
+    if (e == cudaSuccess && known) done[dev].store(true, std::memory_order_relaxed);
+    return e;
+}
+
+template <typename WT, int NSEG, int MAXNB>
+cudaError_t launch_gemv_t(const FfnArgs<MAXNB>& a, int G, int nb, int warps, int depth, size_t smem, cudaStream_t st, bool pdl) {
+    constexpr auto kern = ffn_gemv_kernel<WT, NSEG, MAXNB>;
+    if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
     return launch_k(kern, dim3(G, nb), dim3(warps * 32), smem, st, pdl, a, depth);
 }
 
@@ -399,15 +405,8 @@ cudaError_t launch_gemv_seg(int nseg, const FfnArgs<MAXNB>& a, int G, int nb, in
 
 template <int NCH, int MAXNB>
 cudaError_t launch_gemv_q4_t(int D, const FfnArgs<MAXNB>& a, int G, int nb, int warps, int depth, size_t smem, cudaStream_t st, bool pdl) {
-    static bool attr_set[64] = {};
-    auto kern = ffn_gemv_q4_kernel<NCH, MAXNB>;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFfnSmemLimit));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
+    constexpr auto kern = ffn_gemv_q4_kernel<NCH, MAXNB>;
+    if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
     return launch_k(kern, dim3(G, nb), dim3(warps * 32), smem, st, pdl, a, depth, D);
 }
 
@@ -436,15 +435,8 @@ cudaError_t launch_gemv(const spm_ctx* c, const FfnArgs<MAXNB>& a, int G, int nb
 
 template <typename WT, int GB>
 cudaError_t launch_multi_t(const spm_ctx* c, const MtArgs& a) {
-    static bool attr_set[64] = {};          // the attribute is per device
-    auto kern = ffn_multi_kernel<WT, GB>;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFfnSmemLimit));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
+    constexpr auto kern = ffn_multi_kernel<WT, GB>;
+    if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
     size_t smem = 0;
     const int stages = mt_stages(c->row_bytes, std::is_same<WT, float>::value, a.n, a.nb * a.K, &smem);
     return launch_k(kern, dim3(mt_grid_for(c)), dim3(kMtThreads), smem, c->compute, true, a, stages);
