@@ -142,9 +142,8 @@ typedef struct {
     uint64_t recall_count;       /*   ExpertRecall@M = recall_sum / recall_count  (Section 4.1)          */
     uint64_t host_free_steps;    /* decode steps enqueued without a host turn (spm_set_host_free)        */
     double router_window_us;     /* in-kernel windows of the routing kernels (first leader past its launch      */
-    double reduce_window_us;     /*   dependency -> last leader done; the adapter's ranking of a batch is not in
-                                    it where the tensor-core path's gather kernel makes it) and of the combine
-                                    kernels (not the tensor-core path's), timing on                             */
+    double reduce_window_us;     /*   dependency -> last leader done, or the batch's ranking made, wherever that is)
+                                    and of the combine kernels (not the tensor-core path's), timing on          */
     double gap_us;               /* device idle time between consecutive clocked kernels of the compute stream  */
     double recall_at[3];         /* sums like recall_sum for M = max(1, K/2), K, K+2 (the coverage levels of
                                     the paper's model-level table); divide by recall_count                    */

@@ -678,6 +678,10 @@ gg_plan_gather_kernel(const float* __restrict__ x, const float* __restrict__ w, 
     if (i == n_pairs) {                  // one block more: the adapter's ranking,
         // beside the gather instead of behind the routing: 511 -> 488 us a step of six layers at 5 sequences of the Qwen3 shape
         rank_batch(rank, rank_sm);
+        if (rank.clock) {
+            __syncthreads();
+            if (tid == 0) atomicMax(rank.clock + 1, global_timer_ns());
+        }
         return;
     }
     // the grouped kernel that follows counts arrivals per unit from zero

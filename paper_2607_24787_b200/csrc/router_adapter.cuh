@@ -200,6 +200,7 @@ struct RankArgs {
     Mailbox* mailbox;
     uint32_t tag;
     int nb, n;
+    unsigned long long* clock;   // a kernel that ranks for a routing launch ends that launch's window
 };
 __device__ __forceinline__ void rank_batch(const RankArgs& a, float* sm) {
     for (int e = threadIdx.x; e < a.n; e += blockDim.x) {
@@ -502,7 +503,7 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
         __syncthreads();
         if (!s_last) return;
         __threadfence();
-        if (a.do_adapter) rank_batch(RankArgs{a.pihat, a.scores, a.order, mb, tag, a.nb, n}, qs);
+        if (a.do_adapter) rank_batch(RankArgs{a.pihat, a.scores, a.order, mb, tag, a.nb, n, nullptr}, qs);
         if (threadIdx.x == 0) a.counters[0] = 0u;
     }
     // final flag for callers that read untagged payload (scores): fence, then the sequence number
@@ -511,7 +512,6 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
         __syncthreads();
         if (threadIdx.x == 0 && mb) mb->seq = a.seq;
     }
-    if (a.clock && a.defer_rank) __syncthreads();      // both halves of this leader (the path above has been through a barrier)
     if (threadIdx.x == 0 && a.clock) atomicMax(a.clock + 1, global_timer_ns());
 }
 

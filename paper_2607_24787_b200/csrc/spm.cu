@@ -542,7 +542,7 @@ int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int 
         if (do_adapter) memset(const_cast<int32_t*>(c->mb_host->order), 0, size_t(m.n_experts) * sizeof(int32_t));
     }
     a.seq = c->seq;
-    if (a.defer_rank) *route->defer = RankArgs{do_adapter ? c->ws_pihat : nullptr, c->ws_scores, c->ws_order, a.mailbox, c->seq & 0xffffu, nb, m.n_experts};
+    if (a.defer_rank) *route->defer = RankArgs{do_adapter ? c->ws_pihat : nullptr, c->ws_scores, c->ws_order, a.mailbox, c->seq & 0xffffu, nb, m.n_experts, a.clock};
     a.D = m.hidden; a.n = m.n_experts; a.K = m.top_k; a.r = m.adapter_rank; a.nb = nb;
     a.renorm = m.renormalize; a.do_router = do_router; a.do_adapter = do_adapter;
     a.eps = m.rms_eps;
