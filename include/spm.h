@@ -30,8 +30,8 @@
  *     returns as soon as the host has what it needs (calls that hand expert ids to the host
  *     wait, with a deadline, for the routing kernel only).
  *   - layers, experts, slots are 0-based. Adapter `l` scores layer l+1 and exists for l <= L-2.
- *   - rows that a kernel reads 16 bytes at a time must start on a 16-byte boundary (rms_gamma, router_w, adapter_a,
- *     shared_experts; h and x_norm of spm_router_topk, h_out of spm_decode_step, x_norm of spm_moe_ffn and
+ *   - rows that a kernel reads 16 bytes at a time must start on a 16-byte boundary (rms_gamma, router_w,
+ *     shared_experts, adapter_a where the adapter runs; h and x_norm of spm_router_topk, h_out of spm_decode_step, x_norm of spm_moe_ffn and
  *     spm_time_ffn_kernel, h_inout of spm_moe_ffn on the batched tensor-core path). Where a call would read one that does not,
  *     it returns SPM_ERR_INVALID_ARG and enqueues nothing; all other rows may start at any element.
  *   - all matrices are row-major. dtype applies to every weight matrix (router, adapter,

@@ -37,6 +37,7 @@ thread_local std::string g_init_error;
 struct bf16_t { uint16_t v; };
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
 enum ClockKind : uint8_t { kClkFfn = 0, kClkRouter = 1, kClkReduce = 2 };   // owners of in-kernel clock slots
 
@@ -504,6 +505,7 @@ struct RouterRoute {
 int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int nb, float* x_norm,
                   float* logits_out, bool do_router, bool do_adapter, const RouterRoute* route = nullptr, bool publish_seq = true) {
     const spm_model_cfg& m = c->cfg;
+    if (do_adapter && !aligned16(c->buf.adapter_a)) return fail(c, SPM_ERR_INVALID_ARG, "adapter_a must be 16-byte aligned");
     RouterArgs a{};
     const size_t D = m.hidden, n = m.n_experts, r = m.adapter_rank;
     a.h = h;
@@ -1360,8 +1362,6 @@ int check_layer(spm_ctx* c, int layer, int nb) {
     return SPM_OK;
 }
 
-bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
-
 int check_status(spm_ctx* c) {
     int st = 0;
     CU(c, cudaMemcpy(&st, c->ws_status, sizeof st, cudaMemcpyDeviceToHost));
@@ -1410,8 +1410,8 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     if (b->compute_stream == b->copy_stream) return fail(nullptr, SPM_ERR_INVALID_ARG, "compute and copy stream must differ");
     if (b->host_store_layers < 0 || b->host_store_layers > cfg->n_layers) return fail(nullptr, SPM_ERR_INVALID_ARG, "host_store_layers out of range");
     if (reinterpret_cast<uintptr_t>(b->arena) % 256) return fail(nullptr, SPM_ERR_INVALID_ARG, "arena must be 256-byte aligned");
-    if (!aligned16(b->rms_gamma) || !aligned16(b->router_w) || !aligned16(b->adapter_a) || !aligned16(b->shared_experts))
-        return fail(nullptr, SPM_ERR_INVALID_ARG, "rms_gamma, router_w, adapter_a and shared_experts must be 16-byte aligned");
+    if (!aligned16(b->rms_gamma) || !aligned16(b->router_w) || (cfg->n_shared > 0 && !aligned16(b->shared_experts)))
+        return fail(nullptr, SPM_ERR_INVALID_ARG, "rms_gamma, router_w and shared_experts must be 16-byte aligned");
     Layout lay = layout_of(cfg, slots_per_layer);
     if (b->arena_bytes < lay.total) lay = layout_of(cfg, slots_per_layer, false);      // one GEMV per sequence then takes every such batch
     if (b->arena_bytes < lay.total) return fail(nullptr, SPM_ERR_INVALID_ARG, "arena too small: %zu < %zu", b->arena_bytes, lay.total);

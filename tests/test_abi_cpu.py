@@ -31,13 +31,15 @@ def test_misaligned_buffers_are_refused_ahead_of_the_device():
     import torch
     if torch.cuda.is_available():
         pytest.skip("made-up addresses")
-    cfg = B.make_cfg(2, 256, 16, 128, 2, 1, 8, B.DTYPE_FP32)
-    for i, what in enumerate(("rms_gamma", "router_w", "adapter_a", None, "shared_experts")):
-        at = [256] * 5
-        at[i] += 8
-        with pytest.raises(B.SpmError) as e:
-            B.spm_init(cfg, 4, 2, B.Buffers(*at, 256, 256, 1 << 40, 1, 2, 0))
-        assert e.value.code == (-1 if what else -3)          # (adapter_b is read one element at a time)
+    for shared in (0, 1):
+        cfg = B.make_cfg(2, 256, 16, 128, 2, shared, 8, B.DTYPE_FP32)
+        # rms_gamma, router_w, adapter_a (checked where the adapter runs), adapter_b (read one element at a time), shared_experts
+        for i, refused in enumerate((True, True, False, False, shared > 0)):
+            at = [256] * 5
+            at[i] += 8
+            with pytest.raises(B.SpmError) as e:
+                B.spm_init(cfg, 4, 2, B.Buffers(*at, 256, 256, 1 << 40, 1, 2, 0))
+            assert e.value.code == (-1 if refused else -3)
 
 
 def test_query_and_config_errors():

@@ -428,3 +428,25 @@ def test_rows_off_a_16_byte_boundary_are_refused_or_served():
             assert e.value.code == -1
         assert m.stats()["kernel_launches"] == 0
         m.close()
+
+
+def test_a_misaligned_adapter_is_refused_where_it_would_run():
+    from paper_2607_24787_b200 import binding as B
+    cfg = synth.get_config("tiny", slots=16)
+    a, b = synth.adapter_a(cfg, 0, "cuda")[None], synth.adapter_b(cfg, 0, "cuda")[None]
+    buf = torch.empty(a.numel() + 1, dtype=a.dtype, device="cuda")
+    off = buf[1:].view_as(a)
+    off.copy_(a)
+    h = torch.randn(1, cfg.hidden, device="cuda")
+    good, m = build(cfg, adapter=(a, b)), build(cfg, adapter=(off, b))
+    x, _, _, _ = m.router_topk(0, h)
+    for call in (lambda: m.adapter_predict(0, x), lambda: m.decode_step(h)):
+        with pytest.raises(B.SpmError) as e:
+            call()
+        assert e.value.code == -1
+    m.set_policy("on_demand"); good.set_policy("on_demand")
+    torch.cuda.synchronize()
+    outs = [c.decode_step(h) for c in (m, good)]
+    m.synchronize(); good.synchronize()
+    assert torch.equal(*outs)
+    m.close(); good.close()
