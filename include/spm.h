@@ -30,10 +30,10 @@
  *     returns as soon as the host has what it needs (calls that hand expert ids to the host
  *     wait, with a deadline, for the routing kernel only).
  *   - layers, experts, slots are 0-based. Adapter `l` scores layer l+1 and exists for l <= L-2.
- *   - rows that a kernel reads 16 bytes at a time must start on a 16-byte boundary (rms_gamma, router_w,
- *     shared_experts, adapter_a where the adapter runs; h and x_norm of spm_router_topk, h_out of spm_decode_step, x_norm of spm_moe_ffn and
- *     spm_time_ffn_kernel, h_inout of spm_moe_ffn on the batched tensor-core path). Where a call would read one that does not,
- *     it returns SPM_ERR_INVALID_ARG and enqueues nothing; all other rows may start at any element.
+ *   - rows that a kernel reads 16 bytes at a time must start on a 16-byte boundary: rms_gamma, router_w, shared_experts, and
+ *     adapter_a where the adapter runs; h and x_norm of spm_router_topk; h_out of spm_decode_step; x_norm of spm_moe_ffn and
+ *     spm_time_ffn_kernel; h_inout of spm_moe_ffn on the batched tensor-core path. A call that would read one that does not
+ *     returns SPM_ERR_INVALID_ARG and launches no kernel. All other rows may start at any element.
  *   - all matrices are row-major. dtype applies to every weight matrix (router, adapter,
  *     experts); activations, logits, scores and routing weights are fp32.
  */
@@ -221,7 +221,9 @@ int spm_prefetch_async(spm_ctx* ctx, int target_layer, const int32_t* ids, int c
  * When more distinct experts are needed than there are slots the work is split in waves. On the
  * batched tensor-core path the sum of a token's experts is taken in rank order whatever the waves
  * were, and at batch 1 a layer is one launch whenever slots >= top_k, so in both cases the result
- * does not depend on the cache state, bit for bit. */
+ * does not depend on the cache state, bit for bit. A batch with fp32 activations (spm_set_batched_path) is summed wave by
+ * wave; where experts are streamed once for several tokens, the order of a token's sums also follows how the call's other tokens
+ * are routed. The same call on the same cache state gives the same bits. */
 int spm_moe_ffn(spm_ctx* ctx, int layer, const float* x_norm, const int32_t* ids,
                 const float* w, int nb, float* h_inout);
 
@@ -248,10 +250,10 @@ int spm_set_ffn_ctas(spm_ctx* ctx, int ctas);             /* CTAs per token of t
  * activations, fp32 accumulation) whenever the shape allows it (bf16 or 4-bit weights, no shared
  * experts, inter a multiple of 128, hidden a multiple of 128 for bf16 and of 256 for 4-bit
  * weights, which are expanded to bf16 on the way to the tensor cores), else fp32 activations:
- * every expert streamed once per eight of its tokens where at least 64 Mi weights (for some shapes more)
- * need not be read again that way, the GEMV kernel once per token below. 1: always fp32 activations (a model that could use the
- * tensor cores streams experts once for all tokens only where the partial rows that this takes fit into
- * the tensor-core path's own). */
+ * every expert streamed once per eight of its tokens where at least 64 Mi weights (for some shapes
+ * more) need not be read again that way, else the GEMV kernel once per token. 1: always fp32
+ * activations (a model that could use the tensor cores streams experts once per eight tokens only
+ * where the partial rows that this takes fit into the tensor-core path's own). */
 int spm_set_batched_path(spm_ctx* ctx, int mode);
 /* Perfect-knowledge ranking for SPM_POLICY_HINT_TRACE: for step s (counted from the last
  * spm_cache_reset) and layer l, hint[(s*L + l)*stride .. +count[s*L+l]) are the experts that

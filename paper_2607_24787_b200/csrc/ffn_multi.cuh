@@ -1,11 +1,11 @@
 // Slot-indexed SwiGLU expert FFN for several sequences with fp32 activations: every expert's weights
-// are streamed once for all the tokens that were routed to it (up to kMtTokens at a time).
+// are streamed once per kMtTokens of the tokens that were routed to it.
 //
 // The batched path where the grouped tcgen05 kernels do not apply (fp32 weights, shared experts, intermediate or hidden
-// sizes that do not tile by 128, spm_set_batched_path(1)) and enough expert reads are shared (use_multi). One GEMV
+// sizes that do not tile by 128, spm_set_batched_path(1)) and enough expert reads are shared (multi_pays). One GEMV
 // per sequence, the other kernel of that path, reads an expert once per token: 16 sequences of the DeepSeek shape
-// (1280 x 896, 6 of 64 and 2 shared experts) ask for 880 MB a layer where the distinct experts hold 310 MB.
-// Measured there: 104 us a layer with it, 77 us here (310 MB at the card's copy rate: 47 us).
+// (1280 x 896, 6 of 64 and 2 shared experts) ask for 880 MB a layer where the distinct experts hold 350 MB.
+// Measured there, the kernel's window in a host-free step: 104 us a layer with it, 76 us here (350 MB at the card's copy rate: 54 us).
 //
 // Work. An entry is an expert with at most kMtTokens of its tokens. Its rows (row j = gate[j][:], up[j][:] and
 // column j of W_down, contiguous in the blob) are taken in blocks of kMtRows; the blocks of all entries, in
@@ -18,19 +18,22 @@
 // number already and an fp32 weight is split likewise. All products are exact in the tensor core's fp32
 // accumulator, which is only trusted with 16 or 32 terms (8 in phase 2) of each part, small parts first, before the
 // sum is added to an fp32 register with an ordinary rounded addition. Error against 64 bits over eight shapes of
-// all three weight types: 1.9e-7 to 2.3e-7 of the result, with fp32 FMAs (the GEMV per sequence) 1.7e-7 to 2.4e-7, geometric
-// mean of the ratio 0.99. With plain fp32 FMAs, columns split over the lanes, this kernel needed 944 warp instructions
-// per row of 1280 columns (its rows arrive every 1280 issue slots) and 108 us for the layer above; with MMAs about 400.
+// all three weight types: 1.9e-7 to 2.2e-7 of the result, with fp32 FMAs (one sequence at a time, sums cut over all 148 CTAs)
+// 1.8e-7 to 2.1e-7, geometric mean of the ratio 1.04 (tests/test_gpu_multi.py). With plain fp32 FMAs, columns split over
+// the lanes, this kernel needed 944 warp instructions per row of 1280 columns (its rows arrive every 1280 issue slots) and 108 us
+// for the layer above; with MMAs about 400.
 // mma.sync and not tcgen05: the accumulator has to come back to registers every 16 terms.
 //   Phase 1 (M = 8 gate rows over 8 up rows, N = tokens, K = hidden): the warps split the columns in groups
 // of 32; a lane ends up with gate and up of the same (row, token); the warps' sums meet in shared memory.
 //   Phase 2 (M = hidden, N = tokens, K = the block's 8 rows): the same groups of columns; y stays in registers
 // for the whole segment and is written once, to slot (segment, token) of `partial`.
 //   The phases are one block apart: while the warps' sums of block i become activations, phase 2 of block i - 1
-// runs, and one CTA barrier a block is enough. What bounds it now: copies alone take 56 us of the 77, arithmetic and
-// barriers alone 55; with two to three blocks in the ring they overlap only in part.
+// runs, and one CTA barrier a block is enough. What bounds it now is the chain of latencies of a block: HBM is busy half of
+// the time and a quarter of the issue slots are used; with two to three blocks in the ring, copies and arithmetic overlap only in part.
 // mt_combine_kernel adds a token's experts in k order, each over its segments in CTA order. Every sum has
-// a fixed order given the routing, so results are bitwise reproducible.
+// a fixed order given the routing of the whole call, so results are bitwise reproducible. They depend on the call in the last
+// bits: how many tokens share an expert picks one of two summation orders (NS), and the even split of all entries' blocks says
+// where an expert's sum is cut. (With one GEMV per sequence they depend on the sequence's own routing and nb.)
 //
 // The routing is turned into entries inside the kernel, by every CTA for itself (counts by shared-memory
 // atomics, a prefix sum over the experts, token lists by ballot): 1 - 2 us in place of a planning kernel and
