@@ -129,7 +129,7 @@ typedef struct {
     uint64_t prefetch_issued, touches, waves, planned, dropped;
     uint64_t late_arrivals;      /* needed expert whose prefetch copy was still in flight (timing only) */
     uint64_t h2d_bytes;          /* expert bytes copied host -> HBM                                      */
-    uint64_t ffn_launches;       /* expert-FFN kernel launches timed below                               */
+    uint64_t ffn_launches;       /* expert-FFN kernel launches timed below (a step that is one kernel: its layers) */
     uint64_t kernel_launches;    /* all kernels this context launched                                    */
     double   ffn_us;             /* summed CUDA-event time around those launches (needs spm_set_timing(ctx, 1)) */
     double   ffn_window_us;      /* same launches, first CTA start (of a kernel launched ahead of its predecessor's

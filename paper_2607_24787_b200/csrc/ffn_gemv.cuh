@@ -33,7 +33,7 @@
 
 namespace spm {
 
-constexpr int kFfnMaxWarps = 9;                    // 9 * 32 threads * 216 registers fit one SM
+constexpr int kFfnMaxWarps = 9;                    // (three warps to a quarter of the SM: 168 registers a thread)
 constexpr int kFfnMaxThreads = kFfnMaxWarps * 32;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default limit of every device-side wait (2 s): give up, set status, return
 
@@ -128,13 +128,83 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
     return v;
 }
 
+// One row of a blob against this warp's token: ya += silu(gate . x) * (up . x) * wk * down. `b32`: shared-memory address of the row,
+// this lane's first 16 bytes.
+template <typename WT, int NSEG>
+__device__ __forceinline__ void gemv_row(uint32_t b32, const float (&xr)[NSEG][16 / sizeof(WT)], float wk, uint64_t (&ya)[NSEG][8 / sizeof(WT)]) {
+    constexpr int VEC = 16 / int(sizeof(WT));
+    constexpr uint32_t PART = uint32_t(NSEG) * 32 * 16;      // bytes of one matrix's part of a blob row
+    // gate / up rows first (16 reads), then the down row's reads go out ahead of the reductions
+    uint4 vg[NSEG], vu[NSEG];
+#pragma unroll
+    for (int s = 0; s < NSEG; ++s) { vg[s] = lds128(b32 + s * 512); vu[s] = lds128(b32 + PART + s * 512); }
+    uint64_t ag[2] = {0ull, 0ull}, au[2] = {0ull, 0ull};
+#pragma unroll
+    for (int s = 0; s < NSEG; ++s) {
+        uint64_t fg[VEC / 2], fu[VEC / 2];
+        unpack16p(vg[s], fg);
+        unpack16p(vu[s], fu);
+#pragma unroll
+        for (int v = 0; v < VEC / 2; ++v) {
+            const uint64_t xp = pack2(xr[s][2 * v], xr[s][2 * v + 1]);
+            ag[v & 1] = fma2(fg[v], xp, ag[v & 1]);
+            au[v & 1] = fma2(fu[v], xp, au[v & 1]);
+        }
+    }
+    uint4 vd[NSEG];
+#pragma unroll
+    for (int s = 0; s < NSEG; ++s) vd[s] = lds128(b32 + 2 * PART + s * 512);
+    float a0, a1, a2, a3;
+    unpack2(ag[0], a0, a1); unpack2(ag[1], a2, a3);
+    float pg = (a0 + a1) + (a2 + a3);
+    unpack2(au[0], a0, a1); unpack2(au[1], a2, a3);
+    float pu = (a0 + a1) + (a2 + a3);
+    pg = warp_sum(pg);
+    pu = warp_sum(pu);
+    const float act = __fdividef(pg, 1.f + __expf(-pg)) * pu * wk;
+    const uint64_t ap = pack2(act, act);
+#pragma unroll
+    for (int s = 0; s < NSEG; ++s) {
+        uint64_t fd[VEC / 2];
+        unpack16p(vd[s], fd);
+#pragma unroll
+        for (int v = 0; v < VEC / 2; ++v) ya[s][v] = fma2(ap, fd[v], ya[s][v]);
+    }
+}
+
+// A warp's partial y as float4s, one per (segment, quad, lane), so that stores and loads of a warp are contiguous.
+template <int NSEG, int PAIRS>
+__device__ __forceinline__ void gemv_stage_y(unsigned char* ring, int lane, const uint64_t (&ya)[NSEG][PAIRS]) {
+    float4* mine = reinterpret_cast<float4*>(ring);
+#pragma unroll
+    for (int s = 0; s < NSEG; ++s)
+#pragma unroll
+        for (int h = 0; h < PAIRS / 2; ++h) {
+            float4 t;
+            unpack2(ya[s][2 * h], t.x, t.y);
+            unpack2(ya[s][2 * h + 1], t.z, t.w);
+            mine[s * (16 * PAIRS) + h * 32 + lane] = t;
+        }
+}
+// The values of all warps at one position, in flight at once and added in warp order.
+__device__ __forceinline__ float4 gemv_sum_warps(const unsigned char* first, size_t ring_stride, int nw) {
+    float4 v[kFfnMaxWarps];
+#pragma unroll
+    for (int w2 = 0; w2 < kFfnMaxWarps; ++w2)
+        if (w2 < nw) v[w2] = *reinterpret_cast<const float4*>(first + w2 * ring_stride);
+    float4 acc = v[0];
+#pragma unroll
+    for (int w2 = 1; w2 < kFfnMaxWarps; ++w2)
+        if (w2 < nw) { acc.x += v[w2].x; acc.y += v[w2].y; acc.z += v[w2].z; acc.w += v[w2].w; }
+    return acc;
+}
+
 template <typename WT, int NSEG, int MAXNB>
 __global__ void __launch_bounds__(kFfnMaxThreads, 1)
 ffn_gemv_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int depth) {
     constexpr int VEC = 16 / int(sizeof(WT));
     constexpr int D = NSEG * 32 * VEC;
     constexpr uint32_t ROWB = 3u * D * sizeof(WT);
-    constexpr uint32_t PART = D * sizeof(WT);      // bytes of one matrix's part of a blob row
 
     extern __shared__ __align__(128) unsigned char smem[];
     grid_dep_launch();
@@ -259,43 +329,7 @@ ffn_gemv_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int depth) {
                 const int kk = a.kidx_of(tok, ent);
                 wk = kk == 255 ? 1.f : a.w[size_t(tok) * a.K + kk];
             }
-            // gate / up rows first (16 reads), then the down row's reads go out ahead of the reductions
-            const uint32_t b32 = ring0 + uint32_t(st) * ROWB + lane * 16;
-            uint4 vg[NSEG], vu[NSEG];
-#pragma unroll
-            for (int s = 0; s < NSEG; ++s) { vg[s] = lds128(b32 + s * 512); vu[s] = lds128(b32 + PART + s * 512); }
-            uint64_t ag[2] = {0ull, 0ull}, au[2] = {0ull, 0ull};
-#pragma unroll
-            for (int s = 0; s < NSEG; ++s) {
-                uint64_t fg[VEC / 2], fu[VEC / 2];
-                unpack16p(vg[s], fg);
-                unpack16p(vu[s], fu);
-#pragma unroll
-                for (int v = 0; v < VEC / 2; ++v) {
-                    const uint64_t xp = pack2(xr[s][2 * v], xr[s][2 * v + 1]);
-                    ag[v & 1] = fma2(fg[v], xp, ag[v & 1]);
-                    au[v & 1] = fma2(fu[v], xp, au[v & 1]);
-                }
-            }
-            uint4 vd[NSEG];
-#pragma unroll
-            for (int s = 0; s < NSEG; ++s) vd[s] = lds128(b32 + 2 * PART + s * 512);
-            float a0, a1, a2, a3;
-            unpack2(ag[0], a0, a1); unpack2(ag[1], a2, a3);
-            float pg = (a0 + a1) + (a2 + a3);
-            unpack2(au[0], a0, a1); unpack2(au[1], a2, a3);
-            float pu = (a0 + a1) + (a2 + a3);
-            pg = warp_sum(pg);
-            pu = warp_sum(pu);
-            const float act = __fdividef(pg, 1.f + __expf(-pg)) * pu * wk;
-            const uint64_t ap = pack2(act, act);
-#pragma unroll
-            for (int s = 0; s < NSEG; ++s) {
-                uint64_t fd[VEC / 2];
-                unpack16p(vd[s], fd);
-#pragma unroll
-                for (int v = 0; v < VEC / 2; ++v) ya[s][v] = fma2(ap, fd[v], ya[s][v]);
-            }
+            gemv_row<WT, NSEG>(ring0 + uint32_t(st) * ROWB + lane * 16, xr, wk, ya);
             __syncwarp();   // every lane is done with this buffer before it is refilled
             if (lane == 0 && n_issued < my_n && !halt) {
                 if (issue(n_issued)) ++n_issued;
@@ -317,30 +351,12 @@ ffn_gemv_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int depth) {
     constexpr int Q = VEC / 4;                  // float4s per lane and segment
     constexpr int NP = D / 4;                   // float4 positions of a row
     static_assert(ROWB >= NP * sizeof(float4), "a ring row holds a warp's partial y");
-    {
-        float4* mine = reinterpret_cast<float4*>(ring);
-#pragma unroll
-        for (int s = 0; s < NSEG; ++s)
-#pragma unroll
-            for (int h = 0; h < Q; ++h) {
-                float4 t;
-                unpack2(ya[s][2 * h], t.x, t.y);
-                unpack2(ya[s][2 * h + 1], t.z, t.w);
-                mine[s * (32 * Q) + h * 32 + lane] = t;
-            }
-    }
+    gemv_stage_y<NSEG>(ring, lane, ya);
     __syncthreads();
     const size_t ring_stride = size_t(depth) * ROWB;
     float* out = a.partial + (size_t(tok) * G + c) * D;
     for (int p = threadIdx.x; p < NP; p += blockDim.x) {
-        float4 v[kFfnMaxWarps];
-#pragma unroll
-        for (int w2 = 0; w2 < kFfnMaxWarps; ++w2)
-            if (w2 < nw) v[w2] = reinterpret_cast<const float4*>(smem + w2 * ring_stride)[p];
-        float4 acc = v[0];
-#pragma unroll
-        for (int w2 = 1; w2 < kFfnMaxWarps; ++w2)
-            if (w2 < nw) { acc.x += v[w2].x; acc.y += v[w2].y; acc.z += v[w2].z; acc.w += v[w2].w; }
+        const float4 acc = gemv_sum_warps(smem + size_t(p) * sizeof(float4), ring_stride, nw);
         const int s = p / (32 * Q), h = (p / 32) % Q, ln = p % 32;
         *reinterpret_cast<float4*>(out + s * 32 * VEC + ln * VEC + 4 * h) = acc;
     }

@@ -1,0 +1,489 @@
+// One decode step of one sequence whose experts are all in HBM, as one kernel: routing, adapter and expert FFN of every layer.
+//
+// A host-free batch-1 step used to be two launches a layer (routing kernel, expert GEMV). What a layer of the Qwen3 shape spent
+// its 26 us on: 14.5 in the GEMV, 9.1 in a routing kernel on the 8 SMs of one cluster (3.4 of them to pull 148 partial rows, 1.2 MB,
+// through one GPC's port), 3.4 between the kernels. Here every CTA keeps its SM for the whole step and the routing is split over
+// all of them; three exchanges a layer take the place of the launches:
+//
+//   partial rows   each CTA's sum over its share of the (expert, row) pairs -> the CTAs that own 16 columns of the hidden row each
+//   hidden row     16 updated columns of each owner                         -> every CTA, which normalises the row for itself
+//   logits         router and adapter rows, one warp each, over all CTAs    -> every CTA, which does the Top-K for itself
+//
+// A value travels as an 8-byte word {fp32, tag of the exchange}, so that it needs no flag and no fence: whoever reads a word with
+// the tag of this layer has the value (8-byte accesses are single). A hop costs one store and one load through L2, about a
+// microsecond; the logits, which have a writer each, have a 128-byte line each (sixteen writers to a line that all SMs poll took 4 us).
+// One buffer per exchange is enough: a CTA overwrites a word one layer later, when it holds data that every reader of
+// the old word contributed to after reading it.
+//
+// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 17.2 (21): the FFN 11.5 - 13 and 9 - 11 with the slowest SM 2 us
+// behind the mean, and a chain of latencies of 6 (partial rows 1.4, hidden row 1, norm and dot products 1.5, logits 1.1, Top-K to the
+// first copies 1.3).
+//
+// The arithmetic, the orders of all sums and the split of the rows are those of router_adapter_kernel and ffn_gemv_kernel, so the
+// outputs have the same bits as host-driven steps. The adapter's ranking, which only the host reads, is done by the last
+// CTA (which owns no columns where there are fewer than 16 a CTA) while the others exchange the hidden row.
+//
+// The CTAs wait for one another, so the launch is cooperative (one CTA per SM, all resident or none). Every wait is
+// bounded: a CTA that gives up raises a flag that the others' waits look at, and all of them return with nothing in flight.
+#pragma once
+
+#include "ffn_gemv.cuh"
+#include "router_adapter.cuh"
+
+namespace spm {
+
+// Warps of a CTA: as many as the GEMV may take (those it does not use only route). Rows of 9216 bytes and more leave it eight at most,
+// whose threads then have 255 registers.
+constexpr int step_warps(int nseg) { return nseg >= 6 ? 8 : kFfnMaxWarps; }
+constexpr int kStepCols = 16;                     // columns of the hidden row that an owner adds up
+constexpr int kStepMaxCtas = kReduceGroupsR * kReduceChunkR;
+constexpr unsigned long long kStepStartNs = 30000000000ull;     // limit of the first exchange: kernels of other streams may hold SMs until then
+
+struct StepArgs {
+    const float* h_in;              // [D]
+    float* h_out;                   // [D], may be h_in
+    const float* gamma;             // [L][D]
+    const void* router_w;           // [L][n][D]
+    const void* adapter_a;          // [L - 1][r][D]
+    const void* adapter_b;          // [L - 1][n][r]
+    const unsigned char* pools;     // [L] pools of pool_bytes
+    const unsigned char* shared;    // [L][n_shared] blobs (may be null)
+    const short* slot_map;          // [L][n]
+    unsigned long long* part;       // exchange: [CTAs][D] ...
+    unsigned long long* hx;         // [D] ...
+    unsigned long long* zx;         // [n + r][z_stride], words {fp32 bits, tag << 32}
+    int z_stride;                   // 16, a line of its own for each writer, where there is room
+    unsigned* abort_word;           // tag0 of a launch that gave up
+    Mailbox* mailbox;               // [L]
+    int* status;
+    unsigned long long pool_bytes, blob_bytes, wait_limit_ns;
+    uint32_t tag0;                  // layer l's exchanges carry tag0 + l, different from what any word holds before
+    int I, K, n, r, L, n_slots, n_shared;
+    int nw, depth;                  // GEMV warps and rows of a warp's ring
+    uint32_t ring_bytes;            // shared memory ahead of the routing arrays
+    int renorm, predict, xs_in_ring;
+    float eps;
+};
+
+__device__ __forceinline__ unsigned long long ll_word(float v, uint32_t tag) { return (static_cast<unsigned long long>(tag) << 32) | __float_as_uint(v); }
+__device__ __forceinline__ float ll_value(unsigned long long w) { return __uint_as_float(uint32_t(w)); }
+__device__ __forceinline__ void ll_store(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ void ll_store2(unsigned long long* p, unsigned long long v0, unsigned long long v1) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(v0), "l"(v1) : "memory");
+}
+__device__ __forceinline__ unsigned long long ll_load(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void ll_load2(const unsigned long long* p, unsigned long long& v0, unsigned long long& v1) {
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v0), "=l"(v1) : "l"(p) : "memory");
+}
+
+// Bound of a thread's polling: true when the limit has run out or another CTA has given up.
+struct StepSpin {
+    const StepArgs& a;
+    unsigned long long limit, t0 = 0;
+    int polls = 0;
+    __device__ StepSpin(const StepArgs& args, unsigned long long limit_ns) : a(args), limit(limit_ns) {}
+    __device__ __forceinline__ bool give_up() {
+        if ((++polls & 63) != 0) return false;
+        unsigned flag;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(flag) : "l"(a.abort_word) : "memory");
+        if (flag == a.tag0) return true;
+        const unsigned long long now = global_timer_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 <= limit) return false;
+        raise(a);
+        return true;
+    }
+    static __device__ __forceinline__ void raise(const StepArgs& a) {
+        atomicOr(a.status, kStatusCopyTimeout);
+        asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(a.abort_word), "r"(a.tag0) : "memory");
+    }
+};
+
+// Elements of k[j0..j1) that come before e in (key descending, index ascending); j0 a multiple of 4, k 16-byte aligned.
+__device__ __forceinline__ int count_before(const int* k, int j0, int j1, int e) {
+    const int ke = k[e];
+    int c0 = 0, c1 = 0, c2 = 0, c3 = 0, j = j0;
+#pragma unroll 4
+    for (; j + 4 <= j1; j += 4) {
+        const int4 t = *reinterpret_cast<const int4*>(k + j);
+        const int d = e - j;
+        c0 += t.x > ke - int(0 < d);
+        c1 += t.y > ke - int(1 < d);
+        c2 += t.z > ke - int(2 < d);
+        c3 += t.w > ke - int(3 < d);
+    }
+    for (; j < j1; ++j) c0 += k[j] > ke - int(j < e);
+    return c0 + c1 + c2 + c3;
+}
+
+// Shared memory behind the GEMV's ring and barriers, in floats: [normalised row][n logits][n probabilities, or sums of the owned columns]
+// [r adapter hidden][scratch 32][16 residuals][experts, weights and slots of the chosen, 3 x 16][slot map, shorts]
+__host__ __device__ constexpr size_t step_route_bytes(int D, int n, int r, bool xs_in_ring) {
+    const size_t n4 = (size_t(n) + 3) & ~size_t(3), sums = size_t(kReduceGroupsR) * kStepCols;
+    return sizeof(float) * ((xs_in_ring ? 0 : size_t(D)) + n4 + (n4 > sums ? n4 : sums) + ((size_t(r) + 3) & ~size_t(3)) + 32 + kStepCols + 3 * SPM_MAX_TOPK) +
+           n4 * sizeof(short);
+}
+
+template <typename WT, int NSEG>
+__global__ void __launch_bounds__(step_warps(NSEG) * 32, 1)
+resident_step_kernel(const __grid_constant__ StepArgs a) {
+    constexpr int kStepWarps = step_warps(NSEG), kStepThreads = kStepWarps * 32;
+    static_assert(kStepThreads >= kRouterThreads, "the hidden row is normalised by the routing kernel's number of threads");
+    constexpr int VEC = 16 / int(sizeof(WT));
+    constexpr int D = NSEG * 32 * VEC;
+    constexpr uint32_t ROWB = 3u * D * uint32_t(sizeof(WT));
+    constexpr int NV4 = (D / 4 + kRouterThreads - 1) / kRouterThreads;     // float4s of the hidden row per routing thread
+
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, wi = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // (wi: uniform)
+    const int G = gridDim.x, c = blockIdx.x, n = a.n, I = a.I, nw = a.nw, depth = a.depth;
+    const int n4 = (n + 3) & ~3;
+    unsigned char* ring = smem + size_t(wi < nw ? wi : 0) * depth * ROWB;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + size_t(nw) * depth * ROWB);
+    float* route = reinterpret_cast<float*>(smem + a.ring_bytes);
+    float* xs = a.xs_in_ring ? reinterpret_cast<float*>(smem) : route;
+    float* zs = route + (a.xs_in_ring ? 0 : D);
+    float* ps = zs + n4;
+    float* us = ps + max(n4, kReduceGroupsR * kStepCols);
+    float* scratch = us + ((a.r + 3) & ~3);
+    float* hres = scratch + 32;             // residual of the owned columns
+    int* isel = reinterpret_cast<int*>(hres + kStepCols);
+    float* s_w = reinterpret_cast<float*>(isel + SPM_MAX_TOPK);
+    int* s_code = reinterpret_cast<int*>(s_w + SPM_MAX_TOPK);
+    short* smap = reinterpret_cast<short*>(s_code + SPM_MAX_TOPK);
+
+    // even split of the (expert, j) rows over the CTAs, then over the warps, as in ffn_gemv_kernel
+    const int entries = a.K + a.n_shared, R = entries * I;
+    const int q_rows = R / G, rem_rows = R - q_rows * G;
+    const int r_begin = q_rows * c + min(c, rem_rows);
+    const int span = q_rows + (c < rem_rows ? 1 : 0);
+    const int my_n = wi < nw && span > wi ? (span - wi + nw - 1) / nw : 0;
+    const uint32_t bar0 = smem_u32(bars + (wi < nw ? wi : 0) * depth), ring0 = smem_u32(ring);
+    // the warp's first rows of a layer are looked up by a lane each, which knows where they are but for the slot
+    const int n_first = min(depth, my_n), first_r = r_begin + wi + min(lane, max(n_first - 1, 0)) * nw;
+    const int first_ent = first_r / I, first_j = first_r - first_ent * I;
+    const unsigned long long limit = a.wait_limit_ns ? a.wait_limit_ns : kWaitLimitNs;
+    if (wi < nw && lane == 0) {
+        for (int d = 0; d < depth; ++d) mbar_init(bar0 + 8u * d, 1);
+        fence_barrier_init();
+    }
+    if (tid < a.n_shared) s_code[a.K + tid] = -1 - tid;
+
+    const bool owner = c * kStepCols < D, ranks = c == G - 1;
+    if (owner && tid < kStepCols) hres[tid] = a.h_in[c * kStepCols + tid];
+
+    // what routing reads of a layer: this warp's first weight row, the gain, the slot map
+    const int my_row = c + G * wi;
+    uint4 v[NSEG];
+    float4 gv[NV4];
+    short slot0 = 0;
+    auto row_ptr = [&](int l, int row) {
+        return row < n ? static_cast<const WT*>(a.router_w) + (size_t(l) * n + row) * D
+                       : static_cast<const WT*>(a.adapter_a) + (size_t(l) * a.r + (row - n)) * D;
+    };
+    auto load_row = [&](int l, int row, int rows) {
+        const uint4* p = reinterpret_cast<const uint4*>(row_ptr(l, row < rows ? row : 0));
+#pragma unroll
+        for (int it = 0; it < NSEG; ++it) v[it] = row < rows ? __ldg(p + it * 32 + lane) : make_uint4(0, 0, 0, 0);
+    };
+    auto rows_of = [&](int l) { return n + (a.predict && l <= a.L - 2 ? a.r : 0); };
+    auto preload = [&](int l) {
+        load_row(l, my_row, rows_of(l));
+#pragma unroll
+        for (int i = 0; i < NV4; ++i) {
+            const int at = (i * kRouterThreads + tid) * 4;
+            if (tid < kRouterThreads && at < D) gv[i] = __ldg(reinterpret_cast<const float4*>(a.gamma + size_t(l) * D + at));
+        }
+        if (tid < n) slot0 = __ldg(a.slot_map + size_t(l) * n + tid);
+    };
+    preload(0);
+
+    int st_in = 0, st_out = 0;          // ring stages of the next copy and the next row, and the phase of the latter
+    uint32_t ph = 0;
+    for (int l = 0; l < a.L; ++l) {
+        const uint32_t tag = a.tag0 + uint32_t(l);
+        const int rows = rows_of(l);
+        int dead = 0;
+
+        // ---- hidden row -> normalised row, in every CTA (the sums of router_adapter_kernel) ----
+        float4 hv[NV4];
+        if (tid < kRouterThreads) {
+            if (l == 0) {
+#pragma unroll
+                for (int i = 0; i < NV4; ++i) {
+                    const int at = (i * kRouterThreads + tid) * 4;
+                    if (at < D) hv[i] = *reinterpret_cast<const float4*>(a.h_in + at);
+                }
+            } else {
+                StepSpin spin(a, limit);
+                unsigned long long w[NV4][4];
+#pragma unroll
+                for (int i = 0; i < NV4; ++i)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) w[i][q] = 0ull;
+                for (;;) {
+                    bool missing = false;
+#pragma unroll
+                    for (int i = 0; i < NV4; ++i) {
+                        const int at = (i * kRouterThreads + tid) * 4;
+                        if (at >= D) continue;
+#pragma unroll
+                        for (int q = 0; q < 4; q += 2)
+                            if (uint32_t(w[i][q] >> 32) != tag || uint32_t(w[i][q + 1] >> 32) != tag) {
+                                ll_load2(a.hx + at + q, w[i][q], w[i][q + 1]);
+                                missing = true;
+                            }
+                    }
+                    if (!missing) break;
+                    if (spin.give_up()) { dead = 1; break; }
+                }
+#pragma unroll
+                for (int i = 0; i < NV4; ++i) hv[i] = make_float4(ll_value(w[i][0]), ll_value(w[i][1]), ll_value(w[i][2]), ll_value(w[i][3]));
+            }
+        }
+        float ss = 0.f;
+        if (tid < kRouterThreads) {
+#pragma unroll
+            for (int i = 0; i < NV4; ++i)
+                if ((i * kRouterThreads + tid) * 4 < D) {
+                    ss = fmaf(hv[i].x, hv[i].x, ss); ss = fmaf(hv[i].y, hv[i].y, ss);
+                    ss = fmaf(hv[i].z, hv[i].z, ss); ss = fmaf(hv[i].w, hv[i].w, ss);
+                }
+        }
+        ss = block_reduce(ss, scratch, false);
+        const float inv = 1.0f / sqrtf(ss / float(D) + a.eps);
+        if (tid < kRouterThreads) {
+#pragma unroll
+            for (int i = 0; i < NV4; ++i) {
+                const int at = (i * kRouterThreads + tid) * 4;
+                if (at < D)
+                    *reinterpret_cast<float4*>(xs + at) = make_float4(hv[i].x * gv[i].x * inv, hv[i].y * gv[i].y * inv, hv[i].z * gv[i].z * inv, hv[i].w * gv[i].w * inv);
+            }
+        }
+        if (tid < n) smap[tid] = slot0;
+        for (int e = tid + kStepThreads; e < n; e += kStepThreads) smap[e] = a.slot_map[size_t(l) * n + e];
+        if (__syncthreads_or(dead)) return;
+
+        // ---- logits: one warp per router or adapter row ----
+        for (int row = my_row; row < rows; row += G * kStepWarps) {
+            if (row != my_row) load_row(l, row, rows);
+            float acc = 0.f;
+#pragma unroll
+            for (int it = 0; it < NSEG; ++it) {
+                float f[VEC];
+                unpack16(v[it], f);
+#pragma unroll
+                for (int q = 0; q < VEC; q += 4) {
+                    const float4 t = *reinterpret_cast<const float4*>(xs + (it * 32 + lane) * VEC + q);
+                    acc = fmaf(f[q], t.x, acc); acc = fmaf(f[q + 1], t.y, acc);
+                    acc = fmaf(f[q + 2], t.z, acc); acc = fmaf(f[q + 3], t.w, acc);
+                }
+            }
+            acc = warp_sum(acc);
+            if (lane == 0) ll_store(a.zx + row * a.z_stride, ll_word(acc, tag));
+        }
+        // the GEMV's copy of the row: like one 16-byte weight vector per lane and segment
+        float xr[NSEG][VEC];
+#pragma unroll
+        for (int s = 0; s < NSEG; ++s)
+#pragma unroll
+            for (int q = 0; q < VEC; q += 4) {
+                const float4 t = *reinterpret_cast<const float4*>(xs + (s * 32 + lane) * VEC + q);
+                xr[s][q] = t.x; xr[s][q + 1] = t.y; xr[s][q + 2] = t.z; xr[s][q + 3] = t.w;
+            }
+        for (int i = tid; i < rows; i += kStepThreads) {
+            StepSpin spin(a, l == 0 ? max(limit, kStepStartNs) : limit);
+            unsigned long long w;
+            while (uint32_t((w = ll_load(a.zx + i * a.z_stride)) >> 32) != tag)
+                if (spin.give_up()) { dead = 1; break; }
+            float z = ll_value(w);
+            if (i >= n) { us[i - n] = z; continue; }
+            if (!isfinite(z)) {          // ids are meaningless then; keep the ordering total so that every rank is filled
+                if (c == 0) atomicOr(a.status, kStatusNonFinite);
+                z = -3.0e38f;
+            }
+            ps[i] = z;
+            reinterpret_cast<int*>(zs)[i] = order_key(z);
+        }
+        if (a.xs_in_ring) fence_proxy_async();      // the row was written and read where copies are about to land
+        if (__syncthreads_or(dead)) return;
+
+        // ---- Top-K, two threads an expert; then the first weight copies go out, and the routing weights are computed behind them ----
+        const int half_n = (n / 2) & ~3;
+        for (int u0 = 0; u0 < 2 * n; u0 += kStepThreads) {
+            const int u = u0 + tid, e = u >> 1;
+            int rk = u < 2 * n ? count_before(reinterpret_cast<const int*>(zs), (u & 1) ? half_n : 0, (u & 1) ? n : half_n, e) : 0;
+            rk += __shfl_xor_sync(0xffffffffu, rk, 1);
+            if (u < 2 * n && (u & 1) == 0 && rk < a.K) {
+                isel[rk] = e;
+                s_code[rk] = smap[e];
+                if (c == 0) a.mailbox[l].ids[rk] = tagged(tag & 0xffffu, e);
+            }
+        }
+        __syncthreads();
+        auto blob = [&](int ent) -> const unsigned char* {          // null after a bad slot number
+            const int code = s_code[ent];
+            if (code >= a.n_slots) { atomicOr(a.status, kStatusBadSlot); return nullptr; }
+            return code < 0 ? a.shared + (size_t(l) * a.n_shared + size_t(-1 - code)) * a.blob_bytes
+                            : a.pools + size_t(l) * a.pool_bytes + size_t(code) * a.blob_bytes;
+        };
+        // The row at `src` into the next stage of the warp's ring, by one elected lane with operands that are the same in the warp (lanes that
+        // ask side by side are taken one by one; this took the DeepSeek shape from 19.3 to 17.8 us a layer). A bad slot's row is whatever
+        // was there: the status word says so.
+        auto ask = [&](const unsigned char* src) {
+            if (elect_one()) {
+                if (src) {
+                    mbar_arrive_expect_tx(bar0 + 8u * st_in, ROWB);
+                    bulk_g2s(ring0 + uint32_t(st_in) * ROWB, src, ROWB, bar0 + 8u * st_in, policy_evict_first());
+                } else {
+                    mbar_arrive(bar0 + 8u * st_in);
+                }
+            }
+            __syncwarp();
+            st_in = st_in + 1 == depth ? 0 : st_in + 1;
+        };
+        int n_in = n_first;                 // rows that the warp has asked for
+        {       // (the lanes look the rows up side by side)
+            const unsigned char* base = lane < n_first ? blob(first_ent) : nullptr;
+            const unsigned long long at = base ? reinterpret_cast<unsigned long long>(base + size_t(first_j) * ROWB) : 0ull;
+            for (int i = 0; i < n_first; ++i) ask(reinterpret_cast<const unsigned char*>(__shfl_sync(0xffffffffu, at, i)));
+        }
+        // Routing weights: the router tail's softmax over all experts, by every warp for itself. The four butterflies are the sums
+        // of that tail's four warps, added in their order.
+        float wk = 1.f;                     // lane k: weight of entry k
+        {
+            float top = -INFINITY, part[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int e = lane; e < n; e += 32) top = fmaxf(top, ps[e]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+            for (int e0 = 0; e0 < n; e0 += 128)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (e0 + q * 32 + lane < n) part[q] += expf(ps[e0 + q * 32 + lane] - top);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) part[q] += __shfl_xor_sync(0xffffffffu, part[q], o);
+            const float sum = ((part[0] + part[1]) + part[2]) + part[3];
+            const float p = lane < a.K ? expf(ps[isel[lane]] - top) / sum : 0.f;
+            float tot = 0.f;
+            for (int k = 0; k < a.K; ++k) tot += __shfl_sync(0xffffffffu, p, k);
+            if (lane < a.K) wk = a.renorm ? p / tot : p;
+        }
+
+        // ---- expert FFN: this CTA's rows, as in ffn_gemv_kernel ----
+        unsigned long long* out = a.part + size_t(c) * D;
+        auto send = [&](int col, float4 y) {        // four consecutive columns of the CTA's partial row
+            ll_store2(out + col, ll_word(y.x, tag), ll_word(y.y, tag));
+            ll_store2(out + col + 2, ll_word(y.z, tag), ll_word(y.w, tag));
+        };
+        uint64_t ya[NSEG][VEC / 2];
+#pragma unroll
+        for (int s = 0; s < NSEG; ++s)
+#pragma unroll
+            for (int q = 0; q < VEC / 2; ++q) ya[s][q] = 0ull;
+        int done = 0;
+        for (; done < n_in; ++done) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8u * st_out, ph, limit))) {
+                if (lane == 0) StepSpin::raise(a);
+                dead = 1;
+                break;
+            }
+            gemv_row<WT, NSEG>(ring0 + uint32_t(st_out) * ROWB + lane * 16, xr, __shfl_sync(0xffffffffu, wk, (r_begin + wi + done * nw) / I), ya);
+            __syncwarp();
+            st_out = st_out + 1 == depth ? 0 : st_out + 1;
+            if (st_out == 0) ph ^= 1;
+            if (n_in < my_n) {
+                const int r = r_begin + wi + n_in * nw, e = r / I;
+                const unsigned char* base = blob(e);
+                ask(base ? base + size_t(r - e * I) * ROWB : nullptr);
+                ++n_in;
+            }
+        }
+        if (dead)           // leave no copy in flight
+            for (; done < n_in; ++done) {
+                if (!mbar_wait_bounded(bar0 + 8u * st_out, ph, kWaitLimitNs)) break;
+                st_out = st_out + 1 == depth ? 0 : st_out + 1;
+                if (st_out == 0) ph ^= 1;
+            }
+        if (wi < nw && !dead) gemv_stage_y<NSEG>(ring, lane, ya);
+        if (__syncthreads_or(dead)) return;
+
+        // ---- partial rows -> owned columns -> hidden row of the next layer ----
+        {
+            constexpr int Q = VEC / 4;
+            const size_t ring_stride = size_t(depth) * ROWB;
+            for (int p = tid; p < D / 4; p += kStepThreads) {
+                const float4 y = gemv_sum_warps(smem + size_t(p) * sizeof(float4), ring_stride, nw);
+                const int s = p / (32 * Q), h = (p / 32) % Q, ln = p % 32;
+                send(s * 32 * VEC + ln * VEC + 4 * h, y);
+            }
+            fence_proxy_async();            // the ring held partial sums: ordered before the next layer's copies
+        }
+        if (l + 1 < a.L) preload(l + 1);
+        if (owner && tid < kReduceGroupsR * kStepCols) {
+            // the combine kernel's order: kReduceGroupsR runs of consecutive rows, each front to back, the runs in order, the residual last
+            const int g = tid / kStepCols, col = tid % kStepCols;
+            const int per = (G + kReduceGroupsR - 1) / kReduceGroupsR;
+            const int c0 = g * per, cnt = min(G, c0 + per) - c0;
+            const unsigned long long* p = a.part + size_t(c0) * D + c * kStepCols + col;
+            unsigned long long w[kReduceChunkR];
+#pragma unroll
+            for (int i = 0; i < kReduceChunkR; ++i) w[i] = i < cnt ? ll_load(p + size_t(i) * D) : 0ull;
+            StepSpin spin(a, limit);
+            for (;;) {
+                bool missing = false;
+#pragma unroll
+                for (int i = 0; i < kReduceChunkR; ++i)
+                    if (i < cnt && uint32_t(w[i] >> 32) != tag) {
+                        w[i] = ll_load(p + size_t(i) * D);
+                        missing = true;
+                    }
+                if (!missing) break;
+                if (spin.give_up()) break;          // (raised: the next exchange ends the launch)
+            }
+            float acc = 0.f;
+#pragma unroll
+            for (int i = 0; i < kReduceChunkR; ++i) acc += ll_value(w[i]);
+            ps[g * kStepCols + col] = acc;
+            asm volatile("bar.sync 3, %0;" ::"n"(kReduceGroupsR * kStepCols) : "memory");
+            if (tid < kStepCols) {
+                float tot = ps[tid];
+#pragma unroll
+                for (int i = 1; i < kReduceGroupsR; ++i) tot += ps[i * kStepCols + tid];
+                tot += hres[tid];
+                hres[tid] = tot;
+                if (l + 1 < a.L) ll_store(a.hx + c * kStepCols + tid, ll_word(tot, tag + 1));
+                else a.h_out[c * kStepCols + tid] = tot;
+            }
+        }
+        if (ranks && rows > n && tid >= 128 && tid < 256) {      // the adapter's tail, as in router_adapter_kernel
+            const WT* B = static_cast<const WT*>(a.adapter_b) + size_t(l) * n * a.r;
+            for (int e = tid - 128; e < n; e += 128) {
+                float acc = 0.f;
+                for (int q = 0; q < a.r; ++q) acc = fmaf(load_weight(B, size_t(e) * a.r + q), us[q], acc);
+                if (!isfinite(acc)) {
+                    atomicOr(a.status, kStatusNonFinite);
+                    acc = -3.0e38f;
+                }
+                zs[e] = acc;
+            }
+            asm volatile("bar.sync 2, 128;" ::: "memory");
+            half_softmax(zs, n, scratch + 16, 2);
+            Mailbox* mb = a.mailbox + l;
+            for (int e = tid - 128; e < n; e += 128) {
+                const int rk = rank_of_key(reinterpret_cast<const int*>(zs), n, e);
+                mb->order[rk] = tagged(tag & 0xffffu, e);
+                mb->scores[e] = zs[e];
+            }
+        }
+    }
+}
+
+}  // namespace spm

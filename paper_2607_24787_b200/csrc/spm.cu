@@ -22,6 +22,7 @@
 #include "ffn_multi.cuh"
 #include "ffn_grouped.cuh"
 #include "ffn_grouped_q4.cuh"
+#include "resident_step.cuh"
 #include "router_adapter.cuh"
 #include "tma_maps.h"
 #include "gg_plan.h"
@@ -147,6 +148,11 @@ struct spm_ctx {
     };
     std::vector<HostFreeGraph> hf_graphs;
     bool graph_replay = true, hf_warm = false;
+    // one sequence: the whole host-free step as one cooperative kernel
+    unsigned long long* step_hx = nullptr;
+    uint32_t step_tag = 1;                    // tag of the next launch's first layer
+    bool step_clean = false;                  // no other kernel has written the partial rows since the last such step
+    bool coop = false;                        // the device takes cooperative launches
     std::vector<std::vector<int32_t>> prev_rank;   // Naive Prefetch: experts the preceding step used, per layer
     std::vector<std::vector<int32_t>> pending_protect;
     std::vector<uint8_t> has_plan;
@@ -210,7 +216,8 @@ size_t blob_bytes_of(const spm_model_cfg* m) {
 }
 
 constexpr int kMaxCtasBatch1 = 296;
-constexpr int kClockSlots = 12288;    // in-kernel {start, end} pairs between two harvests
+constexpr int kClockSlots = 8192;     // in-kernel {start, end} pairs between two harvests
+constexpr size_t kStepExchangeBytes = 65536;     // resident_step_kernel: hidden row, logits and adapter rows as 8-byte words, abort word
 constexpr int kDescRing = 8;          // wave descriptors in flight for the batched tensor-core path
 constexpr int kTraceRing = 8;         // host-free steps whose bookkeeping may be outstanding
 static_assert(sizeof(GgTask) == sizeof(GgTaskHost), "host plan and device task share one layout");
@@ -281,6 +288,7 @@ struct Carve {
 
 struct Layout {
     size_t pools, slot_gen, x, logits, pihat, w, scores, partial, h, ids, order, clock, slot_map, codes, counters, status, total;
+    size_t step;                                                                   // exchange buffers of resident_step_kernel
     size_t mt_map;                                                                 // several-sequences kernel only
     size_t tc_xs, tc_wrow, tc_desc, tc_n_units, tc_act, tc_ready;       // batched tensor-core path only
     size_t desc_bytes, off_rows, off_rowmap, off_chunks, chunk_cap, off_wait;
@@ -325,6 +333,7 @@ Layout layout_of(const spm_model_cfg* m, int S, bool with_multi = true) {
     l.ids = c.take(nb * SPM_MAX_TOPK * 4);
     l.order = c.take(n * 4);
     l.clock = c.take(size_t(kClockSlots) * 16);
+    l.step = c.take(kStepExchangeBytes);
     l.slot_map = c.take(size_t(m->n_layers) * n * sizeof(short));
     l.codes = c.take(size_t(m->n_layers) * nb * SPM_MAX_TOPK * sizeof(short));
     if (l.tc) {
@@ -897,6 +906,7 @@ int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, cons
         return SPM_OK;
     }
 
+    c->step_clean = false;
     const int G = ffn_grid_for(c, nb);
     const bool use_tc = ffn_path(c, nb) == FfnPath::kGrouped, multi = ffn_path(c, nb) == FfnPath::kMulti;
     // kernels that can wait for a copy themselves: the batch-1 GEMV kernels and the grouped tensor-core kernels
@@ -1296,6 +1306,117 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
     return SPM_OK;
 }
 
+template <typename WT, int NSEG>
+cudaError_t launch_resident_t(const StepArgs& a, int G, size_t smem, cudaStream_t st) {
+    constexpr auto kern = resident_step_kernel<WT, NSEG>;
+    if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(G);
+    lc.blockDim = dim3(step_warps(NSEG) * 32);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;      // the CTAs wait for one another
+    at[0].val.cooperative = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kern, a);
+}
+template <typename WT>
+cudaError_t launch_resident_seg(int nseg, const StepArgs& a, int G, size_t smem, cudaStream_t st) {
+    switch (nseg) {
+        case 1: return launch_resident_t<WT, 1>(a, G, smem, st);
+        case 2: return launch_resident_t<WT, 2>(a, G, smem, st);
+        case 3: return launch_resident_t<WT, 3>(a, G, smem, st);
+        case 4: return launch_resident_t<WT, 4>(a, G, smem, st);
+        case 5: return launch_resident_t<WT, 5>(a, G, smem, st);
+        case 6: return launch_resident_t<WT, 6>(a, G, smem, st);
+        case 7: return launch_resident_t<WT, 7>(a, G, smem, st);
+        case 8: return launch_resident_t<WT, 8>(a, G, smem, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// Shared memory of resident_step_kernel: the GEMV's ring first, as deep as the routing arrays leave room for. False where they
+// do not fit beside two rows a warp (more than some 900 experts with the widest rows).
+bool resident_shape(const spm_ctx* c, int G, StepArgs* a, size_t* smem) {
+    const spm_model_cfg& m = c->cfg;
+    const int rows_per_cta = ((m.top_k + m.n_shared) * m.inter + G - 1) / G;
+    ffn_gemv_shape(c->row_bytes, rows_per_cta, &a->nw, &a->depth);
+    for (; a->depth >= 2; --a->depth)
+        for (const int in_ring : {0, 1}) {
+            const size_t ring = align_up(ffn_gemv_smem(c->row_bytes, a->nw, a->depth), 16);
+            *smem = ring + step_route_bytes(m.hidden, m.n_experts, m.adapter_rank, in_ring);
+            a->ring_bytes = uint32_t(ring);
+            a->xs_in_ring = in_ring;
+            if (*smem <= kFfnSmemLimit - 1024) return true;
+        }
+    return false;
+}
+
+// One sequence, everything resident, the default geometry: the step as one kernel. Not with in-kernel clocks or an attention
+// stand-in, which belong to separate launches, and not for fp32 models (parity checks) of one or two layers, where it gains too little
+// to keep other streams' kernels off the SMs for a step (us a step: 27 -> 25 - 27 with two layers, 76 -> 45 with eight).
+int enqueue_resident_step(spm_ctx* c, const float* h_in, float* h_out, int slot, bool predict, bool* done) {
+    const spm_model_cfg& m = c->cfg;
+    *done = false;
+    const int G = c->num_sms;
+    StepArgs a{};
+    size_t smem = 0;
+    if (!c->coop || m.dtype == SPM_DTYPE_Q4 || (m.dtype == SPM_DTYPE_FP32 && m.n_layers < 3) || c->timing || c->stub_us > 0 || ffn_grid_for(c, 1) != G ||
+        G > kStepMaxCtas || 2 * G > kMaxCtasBatch1 || m.hidden > G * kStepCols || !resident_shape(c, G, &a, &smem)) return SPM_OK;
+    predict = predict && m.n_layers > 1;
+    if (predict && !aligned16(c->buf.adapter_a)) return fail(c, SPM_ERR_INVALID_ARG, "adapter_a must be 16-byte aligned");
+    // the kernel reads the rows where they are if they are this device's memory; anything else that a copy takes is copied
+    cudaPointerAttributes pa{};
+    int dev = -1;
+    if (h_in != h_out && !(aligned16(h_in) && cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&pa, h_in) == cudaSuccess &&
+                           pa.type == cudaMemoryTypeDevice && pa.device == dev)) {
+        cudaGetLastError();
+        CU(c, cudaMemcpyAsync(h_out, h_in, size_t(m.hidden) * 4, cudaMemcpyDeviceToDevice, c->compute));
+        h_in = h_out;
+    }
+    a.h_in = h_in;
+    a.h_out = h_out;
+    a.gamma = static_cast<const float*>(c->buf.rms_gamma);
+    a.router_w = c->buf.router_w;
+    a.adapter_a = c->buf.adapter_a;
+    a.adapter_b = c->buf.adapter_b;
+    a.pools = c->pools;
+    a.shared = static_cast<const unsigned char*>(c->buf.shared_experts);
+    a.slot_map = c->ws_slot_map;
+    a.part = reinterpret_cast<unsigned long long*>(c->ws_partial);
+    a.hx = c->step_hx;
+    a.zx = a.hx + m.hidden;
+    const size_t words = size_t(m.n_experts) + m.adapter_rank;
+    for (a.z_stride = 16; a.z_stride > 1 && (m.hidden + words * a.z_stride + 1) * 8 > kStepExchangeBytes;) a.z_stride /= 2;
+    a.abort_word = reinterpret_cast<unsigned*>(a.zx + words * a.z_stride);
+    a.mailbox = c->tr_dev + size_t(slot) * m.n_layers;
+    a.status = c->ws_status;
+    a.pool_bytes = size_t(c->S) * c->blob;
+    a.blob_bytes = c->blob;
+    a.wait_limit_ns = c->wait_limit_ns;
+    a.I = m.inter; a.K = m.top_k; a.n = m.n_experts; a.r = m.adapter_rank; a.L = m.n_layers; a.n_slots = c->S; a.n_shared = m.n_shared;
+    a.renorm = m.renormalize; a.predict = predict;
+    a.eps = m.rms_eps;
+    if (!c->step_clean) {           // words of other kernels (or of the memory's last owner) could carry a tag
+        CU(c, cudaMemsetAsync(a.part, 0, size_t(G) * m.hidden * 8, c->compute));
+        CU(c, cudaMemsetAsync(a.hx, 0, kStepExchangeBytes, c->compute));
+        c->step_tag = 1;
+        c->step_clean = true;
+    }
+    if (c->step_tag > 0xffffffffu - 2u * m.n_layers) c->step_tag = 1;        // (the words hold tags of the last two layers)
+    a.tag0 = c->step_tag;
+    c->step_tag += m.n_layers;
+    const cudaError_t launched = m.dtype == SPM_DTYPE_FP32 ? launch_resident_seg<float>(c->nseg, a, G, smem, c->compute)
+                                                           : launch_resident_seg<bf16_t>(c->nseg, a, G, smem, c->compute);
+    CU(c, launched);
+    c->kernel_launches++;
+    c->ffn_launches += m.n_layers;
+    *done = true;
+    return SPM_OK;
+}
+
 // A host-free step is the same sequence of launches every time (for a given trace slot, batch size,
 // output buffer, prediction on/off, launch geometry and wait limit), so it is captured once into a CUDA graph
 // and replayed: one submission instead of 2-5 per layer. Steps with timing or an attention
@@ -1305,11 +1426,16 @@ int enqueue_host_free_step(spm_ctx* c, const float* h_in, int nb, float* h_out) 
     if (int(c->tr_pending.size()) == kTraceRing)
         if (int rc = replay_oldest(c)) return rc;
     const int slot = int(c->tr_count++ % kTraceRing);
-    if (h_out != h_in)
-        CU(c, cudaMemcpyAsync(h_out, h_in, size_t(nb) * m.hidden * 4, cudaMemcpyDeviceToDevice, c->compute));
     const bool predict = c->policy == SPM_POLICY_ADAPTER || c->policy == SPM_POLICY_PRED0;
     bool done = false;
-    if (c->graph_replay && !c->timing && c->stub_us == 0) {
+    if (nb == 1)
+        if (int rc = enqueue_resident_step(c, h_in, h_out, slot, predict, &done)) return rc;
+    if (!done) {
+        c->step_clean = false;
+        if (h_out != h_in)
+            CU(c, cudaMemcpyAsync(h_out, h_in, size_t(nb) * m.hidden * 4, cudaMemcpyDeviceToDevice, c->compute));
+    }
+    if (!done && c->graph_replay && !c->timing && c->stub_us == 0) {
         const HostFreeKey key{slot, nb, h_out, predict, ffn_grid_for(c, nb), c->batched_path, c->wait_limit_ns};
         spm_ctx::HostFreeGraph* g = nullptr;
         for (auto& x : c->hf_graphs)
@@ -1438,6 +1564,8 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     cudaGetDevice(&dev);
     cudaDeviceProp prop{};
     if (cudaGetDeviceProperties(&prop, dev) == cudaSuccess) c->num_sms = prop.multiProcessorCount;
+    int coop = 0;
+    c->coop = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop;
     if (prop.major != 10) { c->err = "this library is built for sm_100a (B200) only"; return bail(SPM_ERR_CONFIG); }
 
     unsigned char* base = static_cast<unsigned char*>(b->arena);
@@ -1457,6 +1585,7 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     c->ws_ids = reinterpret_cast<int32_t*>(base + lay.ids);
     c->ws_order = reinterpret_cast<int32_t*>(base + lay.order);
     c->ws_clock = reinterpret_cast<unsigned long long*>(base + lay.clock);
+    c->step_hx = reinterpret_cast<unsigned long long*>(base + lay.step);
     c->ws_slot_map = reinterpret_cast<short*>(base + lay.slot_map);
     c->ws_codes = reinterpret_cast<short*>(base + lay.codes);
     c->ws_counters = reinterpret_cast<unsigned*>(base + lay.counters);
@@ -2016,6 +2145,7 @@ int spm_time_ffn_kernel(spm_ctx* c, int first_layer, const float* x_norm, const 
     if (!x_norm || !ids || !w || !us_per_launch || launches < 1) return fail(c, SPM_ERR_INVALID_ARG, "bad argument");
     if (!aligned16(x_norm) && c->cfg.dtype != SPM_DTYPE_Q4) return fail(c, SPM_ERR_INVALID_ARG, "x_norm must be 16-byte aligned");
     if (int rc = flush_trace(c)) return rc;
+    c->step_clean = false;
     const spm_model_cfg& m = c->cfg;
     const int K = m.top_k, L = m.n_layers;
     SlotTable& tb = *c->table;

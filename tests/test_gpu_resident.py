@@ -1,0 +1,138 @@
+"""Batch-1 host-free steps as one cooperative kernel: the bits, events and statistics of host-driven steps at the edges of its
+exchanges (owned columns, rows over all CTAs, more experts than threads) and of its shared-memory layouts."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+from paper_2607_24787_b200.binding import SpmError
+from test_gpu_host_free import build, preload, rows, run
+
+pytestmark = pytest.mark.gpu
+
+# hidden: one 16-column owner a 16 columns, 8 to 128 of them; inter * top_k: CTAs without a row, with one, with ragged shares; n_experts:
+# ranked by two threads each, from 3 to more than the threads, and more rows than warps of all CTAs; odd adapter ranks.
+CASES = {
+    "fp32_smallest": dict(base="tiny", hidden=128, n_experts=3, inter=7, top_k=1, adapter_rank=1),
+    "fp32_widest": dict(base="tiny", hidden=1024, n_experts=20, inter=331, top_k=4, adapter_rank=7),
+    "fp32_shared": dict(base="tiny", hidden=640, n_experts=37, inter=50, top_k=3, n_shared=2, adapter_rank=5),
+    "bf16_widest": dict(base="qwen3", hidden=2048, n_experts=24, inter=129, top_k=8, adapter_rank=16),
+    "bf16_many_experts": dict(base="qwen3", hidden=256, n_experts=600, inter=24, top_k=16, adapter_rank=3),
+    "bf16_row_in_ring": dict(base="qwen3", hidden=2048, n_experts=513, inter=10, top_k=2, adapter_rank=63),
+    "bf16_nine_warps": dict(base="dsvl2", hidden=1280, n_experts=16, inter=224, top_k=6, n_shared=2, adapter_rank=16),
+    "bf16_raw_weights": dict(base="qwen3", hidden=1792, n_experts=9, inter=100, top_k=3, renormalize=0, adapter_rank=4),
+}
+
+
+def config(name, **over):
+    kw = dict(CASES[name], **over)
+    n = kw["n_experts"]
+    return synth.get_config(kw.pop("base"), n_layers=3, slots=n, budget=2, batch=1, **kw)
+
+
+@pytest.mark.parametrize("policy", ["adapter", "on_demand"])
+@pytest.mark.parametrize("name", list(CASES))
+def test_one_kernel_gives_the_bits_of_host_driven_steps(name, policy):
+    cfg = config(name)
+    steps = 10                      # more than the trace ring holds
+    H = rows(cfg, steps)
+    results = []
+    for host_free in (1, 0):
+        m = build(cfg, store_layers=1)
+        m.set_host_free(host_free)
+        m.set_policy(policy)
+        preload(cfg, m)
+        m.reset_stats()
+        outs = run(m, H, sync_every=0 if host_free else 1)
+        st = m.stats()
+        assert st["host_free_steps"] == (steps if host_free else 0) and st["ffn_launches"] == steps * cfg.n_layers
+        assert st["kernel_launches"] == (steps if host_free else steps * (2 * cfg.n_layers + 1))
+        results.append((outs, m.events(), {k: st[k] for k in ("hits", "touches", "steps", "tokens", "recall_sum", "ready_sum")}))
+        m.close()
+    (a, ev_a, st_a), (b, ev_b, st_b) = results
+    for s in range(steps):
+        assert np.array_equal(a[s], b[s]), s
+    assert ev_a == ev_b and st_a == st_b
+
+
+def test_other_launches_in_between_and_rows_from_anywhere():
+    """The exchange words share memory with other kernels' partial rows: steps before and after such kernels, in place, from rows
+    at any float and from pinned host rows."""
+    cfg = config("bf16_nine_warps")
+    H = torch.as_tensor(rows(cfg, 4), dtype=torch.float32).cuda()
+    m = build(cfg, store_layers=1)
+    preload(cfg, m)
+    torch.cuda.synchronize()
+    want = [m.decode_step(H[s]) for s in range(4)]
+    m.synchronize()
+    want = [w.clone() for w in want]
+    x, ids, w, _ = m.router_topk(0, H[0])
+    scratch = H[0].clone()
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, scratch)            # writes partial rows
+    in_place = H[1].clone()
+    odd = torch.empty(cfg.hidden + 1, device="cuda")
+    odd[1:].copy_(H[2][0])
+    torch.cuda.synchronize()
+    third = torch.empty_like(H[2])
+    got = [m.decode_step(H[0]), m.decode_step(in_place, in_place), m.decode_step(odd[1:].view(1, -1), third)]
+    m.set_timing(1)                             # the separate launches
+    timed = m.decode_step(H[3])
+    m.set_timing(0)
+    got.append(m.decode_step(H[3]))
+    host = torch.empty(1, cfg.hidden).pin_memory()
+    m.decode_step_host(H[3].cpu().pin_memory(), host)
+    m.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    assert torch.equal(timed, want[3]) and torch.equal(host.cuda(), want[3])
+    m.close()
+
+
+def test_non_finite_logits_are_reported_once():
+    cfg = config("fp32_shared")
+    m = build(cfg, store_layers=1)
+    preload(cfg, m)
+    h = torch.as_tensor(rows(cfg, 1)[0], dtype=torch.float32).cuda()
+    torch.cuda.synchronize()
+    want = m.decode_step(h)
+    m.synchronize()
+    want = want.clone()
+    bad = h.clone()
+    bad[0, 3] = float("nan")
+    torch.cuda.synchronize()
+    m.decode_step(bad)
+    with pytest.raises(SpmError) as e:
+        m.synchronize()
+    assert e.value.code == -7
+    got = m.decode_step(h)
+    m.synchronize()
+    assert torch.equal(got, want)
+    m.close()
+
+
+def test_two_contexts_at_once():
+    """Two threads, each with a context and streams of its own: both kernels want every SM, one waits for the other."""
+    cfg = config("bf16_nine_warps")
+    H = rows(cfg, 24)
+    ms = [build(cfg, store_layers=1) for _ in range(2)]
+    for m in ms:
+        preload(cfg, m)
+    want = run(ms[0], H)
+    outs = [None, None]
+
+    def work(i):
+        outs[i] = run(ms[i], H)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for o in outs:
+        for a, b in zip(o, want):
+            assert np.array_equal(a, b)
+    for m in ms:
+        m.close()
