@@ -28,6 +28,7 @@
 // router input and the routing weights do, and those are read after the wait.
 #pragma once
 
+#include "mma_ops.cuh"
 #include "ptx.cuh"
 #include "../../include/spm.h"
 
@@ -121,11 +122,6 @@ __device__ __forceinline__ void unpack16p(const uint4& v, uint64_t (&f)[4]) {   
 }
 __device__ __forceinline__ void unpack16p(const uint4& v, uint64_t (&f)[2]) {   // fp32: 4 values
     f[0] = pack2u(v.x, v.y); f[1] = pack2u(v.z, v.w);
-}
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
 }
 
 // One row of a blob against this warp's token: ya += silu(gate . x) * (up . x) * wk * down. `b32`: shared-memory address of the row,

@@ -1,84 +1,300 @@
 // Slot-indexed SwiGLU expert FFN for decode with 4-bit experts (the paper's on-device setting:
-// 4-bit weights, 1.94 MB per DeepSeek-VL2-Tiny expert).
+// 4-bit weights, 1.94 MB per DeepSeek-VL2-Tiny expert), one activation row per token.
 //
-// Quantisation: groups of 32 weights along a row share one fp16 scale, value = scale * (q - 8),
-// q in 0..15. A packed row of D weights is D/2 bytes of nibbles (element 2b in the low half of
-// byte b, 2b+1 in the high half) followed by D/32 fp16 scales; a blob row j holds the packed
-// gate[j][:], up[j][:] and column j of W_down back to back, so the kernel keeps the structure of
-// ffn_gemv_kernel: per-warp rings of row triples filled by 1-D bulk async copies, the two dot
-// products and the rank-1 update of y from one row, deterministic partial rows per CTA.
-// A lane owns whole groups: 16 bytes of nibbles = 32 weights = one scale, so de-quantisation needs
-// no cross-lane traffic: nibbles become exact (q - 8) halves with one lop3 + one half2 subtract
-// per pair, are widened to fp32 and multiplied with fp32 activations; the scale is applied once
-// per group. Transfers and HBM traffic shrink 3.56x against bf16.
+// A blob row j holds the packed gate[j][:], up[j][:] and column j of W_down back to back (q4_mma.cuh has the format). The
+// (expert, j) rows of a token are split evenly over the CTAs, as in ffn_gemv_kernel; a CTA takes its rows in tiles of 16, whatever
+// experts they belong to, one bulk copy a row.
+//
+// All arithmetic on weights is mma.sync, with the fp32 operand as the sum of three bf16 numbers (split3) in three columns of N, so
+// that nothing is rounded to 16 bits. The warps split the columns in groups of 32 (one scale):
+//   Phase 1 (M = 16 gate rows, then 16 up rows; K = the group): the group's scale goes onto the fp32 sum of its 32 products; the warps' sums
+// meet in shared memory, a warp takes a row's activation from them.
+//   Phase 2 (M = hidden columns, K = the tile's 16 rows): act * scale is the split operand; two groups, whose scales differ, use columns of
+// N of their own. y stays in the accumulators for all tiles of the CTA, each column in one warp: no sum over warps.
+//
+// Why MMAs: with fp32 FMAs the kernel was bound by instruction issue, 27 warp instructions per eight weights and lane, eight of which
+// widened halves to floats and eight multiplied; an MMA operand needs five. A layer of the Qwen3 shape (a step as one kernel; with
+// separate launches before) 26.5 -> 18.6 us, of the DeepSeek shape 25.6 -> 16.1; its part of that, 14.6 -> 9. What bounds it now: the
+// chain of latencies of a tile, of which a CTA has three or four, and still instruction issue (some 400 a warp and tile).
+// Error against 64 bits, 18 shapes of hidden 256 to 2048: 0.93 of the FMAs' on normally distributed rows (2.4e-7 of the result at
+// worst, as before), 1.4 on log-normal ones (5e-7 at worst: the -8 is a sum of its own).
 #pragma once
 
+#include <type_traits>
+
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "ffn_gemv.cuh"
+#include "q4_mma.cuh"
 
 namespace spm {
 
-// 8 nibbles of one 32-bit word -> fp32 (q - 8), in element order 0..7
-__device__ __forceinline__ void unpack_q4_word(uint32_t w, float (&f)[8]) {
-    const __half2 bias = __floats2half2_rn(1032.f, 1032.f);      // 1024 + 8
+// One of the three parts of split3 by a lane that wants only that: what is left of a number after the parts before it. An infinity
+// leaves NaNs (`guarded`: zeros).
+struct Q4Part {
+    uint32_t m1, m2;               // masks of the parts that go first
+    __device__ __forceinline__ explicit Q4Part(int p) : m1(p >= 1 ? 0xffff0000u : 0u), m2(p >= 2 ? 0xffff0000u : 0u) {}
+    __device__ __forceinline__ float left(float v, bool guarded) const {
+        float r = v - __uint_as_float(__float_as_uint(v) & m1);
+        if (guarded && m1 != 0 && !(fabsf(v) < INFINITY)) r = 0.f;
+        return r - __uint_as_float(__float_as_uint(r) & m2);
+    }
+    __device__ __forceinline__ uint32_t pair(float a, float b, bool guarded = false) const {
+        return __byte_perm(__float_as_uint(left(a, guarded)), __float_as_uint(left(b, guarded)), 0x7632);
+    }
+};
+
+// Where the tiles of a CTA are: a ring of stages of kQ4Rows rows, one barrier a stage that completes when all rows of it have been asked for
+// and have landed, the phase-1 sums [warps][kQ4Red], gate and up of each row, and the activations [2][rows].
+constexpr int kQ4Red = 33;             // (a lane reads one row's sum of one warp)
+template <int NW>
+struct Q4Ring {
+    uint32_t rows, bars, pitch;
+    float *red, *act;
+    int stages;
+    int st = 0, st_in = 0;         // stage of the next tile to use, of the next to fill
+    uint32_t ph = 0;
+    __device__ __forceinline__ Q4Ring(unsigned char* smem, int D, int n_stages, int thread) : stages(n_stages) {
+        pitch = mt_pitch(3 * q4_part_bytes(D), false);
+        uint64_t* b = reinterpret_cast<uint64_t*>(smem + size_t(n_stages) * kQ4Rows * pitch);
+        rows = smem_u32(smem);
+        bars = smem_u32(b);
+        red = reinterpret_cast<float*>(b + kQ4MaxStages);
+        act = red + (NW * kQ4Red + 3) / 4 * 4;
+        if (thread == 0) {
+            for (int s = 0; s < stages; ++s) mbar_init(bars + 8u * s, kQ4Rows);
+            fence_barrier_init();
+        }
+    }
+    // The warp's rows (warp, warp + NW) of `count` tiles from `tile` on; row_at(row) is null for rows that are not there. The lanes look the rows up side
+    // by side, one elected lane asks for them (lanes that ask side by side are taken one by one).
+    template <typename F>
+    __device__ __forceinline__ void fill(int tile, int count, int warp, int lane, uint32_t bytes, F row_at) {
+        constexpr int kPer = q4_rows_per_warp(NW);
+        const int mine = warp + lane % kPer * NW;
+        const bool in = lane < count * kPer && mine < kQ4Rows;
+        const unsigned long long at = in ? reinterpret_cast<unsigned long long>(row_at((tile + lane / kPer) * kQ4Rows + mine)) : 0ull;
+        for (int k = 0; k < count; ++k) {
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        // nibbles p and p + 4 sit at the same position of the two 16-bit halves
-        uint32_t h = ((w >> (4 * p)) & 0x000f000fu) | 0x64006400u;          // half2 {1024 + q_p, 1024 + q_{p+4}}
-        const __half2 v = __hsub2(*reinterpret_cast<__half2*>(&h), bias);   // exact q - 8
-        const float2 t = __half22float2(v);
-        f[p] = t.x;
-        f[p + 4] = t.y;
+            for (int r = 0; r < kPer; ++r) {
+                const int i = warp + r * NW;
+                const unsigned long long src = __shfl_sync(0xffffffffu, at, k * kPer + r);
+                if (kQ4Rows % NW != 0 && i >= kQ4Rows) continue;
+                if (elect_one()) {
+                    if (src) {
+                        mbar_arrive_expect_tx(bars + 8u * st_in, bytes);
+                        bulk_g2s(rows + uint32_t(st_in * kQ4Rows + i) * pitch, reinterpret_cast<const void*>(src), bytes, bars + 8u * st_in, policy_evict_first());
+                    } else {
+                        mbar_arrive(bars + 8u * st_in);
+                    }
+                }
+                __syncwarp();
+            }
+            st_in = st_in + 1 == stages ? 0 : st_in + 1;
+        }
+    }
+};
+
+// B operand of phase 1: the lane's part (N column = part) of the activations of its eight columns in each of the warp's groups, scaled up
+// by the warp's power of two; returns its exponent. get(col, v): eight consecutive fp32 from column col on.
+template <int GB, typename F>
+__device__ __forceinline__ int q4_operand(uint32_t (&x)[GB][4], float (&off)[GB][2], int warp, int lane, F get) {
+    const int g = lane >> 2, t = lane & 3;
+    float v[GB][8];
+    uint32_t top = 0;
+#pragma unroll
+    for (int i = 0; i < GB; ++i) {
+        get((warp * GB + i) * 32 + t * 8, v[i]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) top = max(top, __float_as_uint(v[i][q]) & 0x7fffffffu);
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    const int e = q4_exponent(top);
+    const bool guarded = top >= 0x7f800000u;
+    const float even = g < 3 ? q4_up(e) : 0.f, odd = even * 0.0625f;
+    const Q4Part part(g);
+#pragma unroll
+    for (int i = 0; i < GB; ++i) {
+        // (a NaN comes out as the one whose upper half is one too)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float f = (q & 1) ? odd : even;
+            x[i][q] = guarded ? (g < 3 ? part.pair(v[i][q] * f, v[i][q + 4] * f, true) : 0u) : part.pair(v[i][q] * f, v[i][q + 4] * f);
+        }
+        q4_offset(x[i], off[i]);
+    }
+    return e;
+}
+
+// The CTA's rows 0 .. span - 1, tile by tile. fill(tile): ask for the warp's rows of a tile; the first `stages` tiles have been
+// asked for. weight(row): routing weight. Every thread of the CTA takes part. Returns false, in every
+// thread, when a wait ran out (the caller drains and leaves).
+template <int GB, int NW, typename Fill, typename Weight>
+__device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[GB][4], const float (&off)[GB][2], int x_exp, float (&y)[GB][2][4], Q4ActScale& scale,
+                                         int D, int span, int warp, int lane, unsigned long long limit, Fill fill, Weight weight) {
+    const int g = lane >> 2, t = lane & 3, grp0 = warp * GB;
+    const int tiles = (span + kQ4Rows - 1) / kQ4Rows;
+    const uint32_t P = ring.pitch, PART = q4_part_bytes(D);
+    const float x_down = q4_down(x_exp);
+    for (int k = 0; k < tiles; ++k) {
+        const int nr = span - k * kQ4Rows;
+        const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(ring.bars + 8u * ring.st, ring.ph, limit));
+        const uint32_t rows = ring.rows + uint32_t(ring.st * kQ4Rows) * P;
+        if (++ring.st == ring.stages) { ring.st = 0; ring.ph ^= 1; }
+        float* acts = ring.act + (k & 1) * kQ4Rows;
+        // `whole`: for the case below, exact operands, and a group's three parts added up before the scale goes onto them
+        auto phase1 = [&](auto whole) {
+            constexpr bool kWhole = decltype(whole)::value;
+            float ag[4], au[4];
+            q4_phase1<GB, kWhole>(rows, P, D, grp0, lane, x, off, ag, au, [](float (&acc)[4], const float (&c)[4], float s0, float s1) {
+                if constexpr (kWhole) {
+                    float lo = c[0] + c[1], hi = c[2] + c[3];
+                    lo += __shfl_xor_sync(0xffffffffu, lo, 1);
+                    hi += __shfl_xor_sync(0xffffffffu, hi, 1);
+                    acc[0] = fmaf(s0, lo, acc[0]); acc[2] = fmaf(s1, hi, acc[2]);
+                } else {
+                    acc[0] = fmaf(s0, c[0], acc[0]); acc[1] = fmaf(s0, c[1], acc[1]);
+                    acc[2] = fmaf(s1, c[2], acc[2]); acc[3] = fmaf(s1, c[3], acc[3]);
+                }
+            });
+            // columns 0 and 1 are in lane t = 0, column 2 in lane t = 1 (the others hold zeros)
+            float v[4] = {ag[0] + ag[1], ag[2] + ag[3], au[0] + au[1], au[2] + au[3]};
+            if constexpr (!kWhole)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], 1);
+            if (t == 0) {
+                float* r = ring.red + warp * kQ4Red + g;
+                r[0] = v[0] * x_down; r[8] = v[1] * x_down; r[16] = v[2] * x_down; r[24] = v[3] * x_down;
+            }
+        };
+        auto activations = [&]() {       // warp w: rows w, w + NW; even lanes take a row's gate, odd ones its up
+#pragma unroll
+            for (int r0 = 0; r0 < kQ4Rows; r0 += NW) {
+                const int r = r0 + warp;
+                if (kQ4Rows % NW != 0 && r >= kQ4Rows) continue;
+                const float* p = ring.red + (lane & 1) * 16 + r;
+                float sum = 0.f;         // (front to back: the loads overlap, so it takes no longer than shuffles between lanes)
+#pragma unroll
+                for (int w = 0; w < NW; ++w) sum += p[w * kQ4Red];
+                const float up = __shfl_xor_sync(0xffffffffu, sum, 1);
+                if (lane == 0) acts[r] = r < nr ? __fdividef(sum, 1.f + __expf(-sum)) * up * weight(k * kQ4Rows + r) : 0.f;
+            }
+        };
+        float a0, a1, a2, a3;            // activations of rows 2t, 2t + 1, 2t + 8, 2t + 9
+        auto take = [&]() {
+            const float2 lo = *reinterpret_cast<const float2*>(acts + 2 * t), hi = *reinterpret_cast<const float2*>(acts + 2 * t + 8);
+            a0 = lo.x; a1 = lo.y; a2 = hi.x; a3 = hi.y;
+            return fmaxf(fmaxf(fabsf(a0), fabsf(a1)), fmaxf(fabsf(a2), fabsf(a3)));
+        };
+        phase1(std::false_type{});
+        if (!__syncthreads_and(ok)) return false;
+        // every warp is done with the tile before this one
+        if (k > 0 && k - 1 + ring.stages < tiles) fill(k - 1 + ring.stages);
+        activations();
+        __syncthreads();
+        float largest = take();
+        if (__any_sync(0xffffffffu, !isfinite(a0 * 0.f + a1 * 0.f + a2 * 0.f + a3 * 0.f))) {       // (so in all warps or in none)
+            // An infinite scale times a part that is zero is a NaN where the scale times the sum is an infinity, and so are q and -8
+            // times an infinity where q - 8 times it is one.
+            phase1(std::true_type{});
+            __syncthreads();
+            activations();
+            __syncthreads();
+            largest = take();
+        }
+        scale.fit<GB>(largest, y);
+        // N columns 0-2: the parts for one group, 4-6: for the next (where there is one)
+        const bool second = g >= 4;
+        const float up = (g & 3) < 3 ? scale.up : 0.f;
+        a0 *= up; a1 *= up; a2 *= up; a3 *= up;
+        const uint32_t at = rows + 2 * PART + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * P + uint32_t(grp0) * 16;
+        const uint32_t sc = rows + 2 * PART + uint32_t(2 * t) * P + uint32_t(D / 2 + grp0 * 2);
+        float s0[GB], s1[GB], s2[GB], s3[GB];
+        q4_scales<GB>(sc, s0);
+        q4_scales<GB>(sc + P, s1);
+        q4_scales<GB>(sc + 8 * P, s2);
+        q4_scales<GB>(sc + 9 * P, s3);
+        if (nr < kQ4Rows) {          // rows past the last one hold whatever was there: their activations are 0, so their scales must be finite
+#pragma unroll
+            for (int i = 0; i < GB; ++i) {
+                s0[i] = 2 * t < nr ? s0[i] : 0.f; s1[i] = 2 * t + 1 < nr ? s1[i] : 0.f;
+                s2[i] = 2 * t + 8 < nr ? s2[i] : 0.f; s3[i] = 2 * t + 9 < nr ? s3[i] : 0.f;
+            }
+        }
+        uint32_t b[(GB + 1) / 2][2];
+        const Q4Part part(g & 3);
+        auto operand = [&](bool guarded) {
+#pragma unroll
+            for (int i = 0; i < GB; i += 2) {
+                const int j = i + 1 < GB ? i + 1 : GB - 1;
+                const float v0 = a0 * (second ? s0[j] : s0[i]), v1 = a1 * (second ? s1[j] : s1[i]), v2 = a2 * (second ? s2[j] : s2[i]), v3 = a3 * (second ? s3[j] : s3[i]);
+                b[i / 2][0] = part.pair(v0, v1, guarded);
+                b[i / 2][1] = part.pair(v2, v3, guarded);
+                if ((i + 1 >= GB && second) || (guarded && (g & 3) == 3)) b[i / 2][0] = b[i / 2][1] = 0u;
+            }
+        };
+        operand(false);
+        auto phase2 = [&](auto exact) {
+#pragma unroll
+            for (int i = 0; i < GB; i += 2) {
+                // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word
+                const uint4 w = ldsm4t(at + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
+                q4_phase2<decltype(exact)::value>(y[i], w.x, w.y, b[i / 2][0], b[i / 2][1]);
+                if (i + 1 < GB) q4_phase2<decltype(exact)::value>(y[i + 1 < GB ? i + 1 : i], w.z, w.w, b[i / 2][0], b[i / 2][1]);
+            }
+        };
+        if (q4_any_nonfinite(b)) {
+            operand(true);
+            phase2(std::true_type{});
+        } else {
+            phase2(std::false_type{});
+        }
+    }
+    return true;
+}
+
+// After the last tile: put(column, four consecutive y) for the columns of the warp's groups
+template <int GB, typename F>
+__device__ __forceinline__ void q4_result(const float (&y)[GB][2][4], const Q4ActScale& scale, int warp, int lane, F put) {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int i = 0; i < GB; ++i) {
+        float4 o = make_float4(y[i][0][0] + y[i][0][1], y[i][0][2] + y[i][0][3], y[i][1][0] + y[i][1][1], y[i][1][2] + y[i][1][3]);
+        o.x += __shfl_xor_sync(0xffffffffu, o.x, 1); o.y += __shfl_xor_sync(0xffffffffu, o.y, 1);
+        o.z += __shfl_xor_sync(0xffffffffu, o.z, 1); o.w += __shfl_xor_sync(0xffffffffu, o.w, 1);
+        if (t == (i & 1) * 2) put((warp * GB + i) * 32 + g * 4, scale.out(o.x, o.y, o.z, o.w));
     }
 }
 
-constexpr int kQ4MaxWarps = 16;    // activations live in shared memory here, so registers allow 16 warps
-constexpr int kQ4Pad = 36;         // floats per 32-wide group in shared memory: lanes then start 4 banks apart
-
-template <int NCH, int MAXNB>     // NCH = 16-byte nibble chunks (groups of 32 weights) per lane
-__global__ void __launch_bounds__(kQ4MaxWarps * 32, 1)
-ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int depth, const int D) {
+template <int NSEG, int MAXNB>
+__global__ void __launch_bounds__(q4_warps(NSEG) * 32, 1)
+ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages) {
+    constexpr int D = NSEG * 256, GB = q4_groups(NSEG), NW = q4_warps(NSEG);
+    constexpr uint32_t ROWB = 3 * q4_part_bytes(D);
     extern __shared__ __align__(128) unsigned char smem[];
     grid_dep_launch();
     const unsigned long long t_entry = (a.clock && threadIdx.x == 0) ? global_timer_ns() : 0ull;
-    const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nw = blockDim.x >> 5;
-    const int tok = blockIdx.y;
-    const int G = gridDim.x, c = blockIdx.x;
-    const int I = a.I;
-    const int n_grp = D / 32;                         // groups per row
-    const uint32_t RB = uint32_t(D / 2 + D / 16);     // bytes of one packed row
-    const uint32_t ROWB = 3u * RB;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0), lane = threadIdx.x & 31;      // (warp: uniform)
+    const int tok = blockIdx.y, G = gridDim.x, c = blockIdx.x, I = a.I;
     const int R = a.entries(tok) * I;
-    // even split: CTA c takes q rows, the first R % G CTAs one more (one 32-bit division)
     const int q_rows = R / G, rem_rows = R - q_rows * G;
-    const int r_begin = q_rows * c + min(c, rem_rows);
-    const int r_end = r_begin + q_rows + (c < rem_rows ? 1 : 0);
-    const int span = r_end - r_begin - wi;
-    const int my_n = span > 0 ? (span + nw - 1) / nw : 0;
+    const int r_begin = q_rows * c + min(c, rem_rows), span = q_rows + (c < rem_rows ? 1 : 0);
+    const unsigned long long limit = a.limit();
+    Q4Ring<NW> ring(smem, D, n_stages, threadIdx.x);
+    __syncthreads();
+    // Everything above is independent of the preceding kernel; with `early` so are the first weight copies (see ffn_gemv_kernel).
+    const bool early = a.early && !a.dev_code;
+    auto depend = [&]() {
+        grid_dep_wait();
+        // window start: kernel entry, or the end of the dependency wait when launched ahead of its predecessor's end
+        if (a.clock && threadIdx.x == 0) atomicMin(a.clock, a.dev_code || early ? global_timer_ns() : t_entry);
+    };
+    if (!early) depend();
 
-    unsigned char* ring = smem + size_t(wi) * depth * ROWB;
-    // layout: [ring, reused for the cross-warp reduction][barriers][activations, padded per group]
-    const size_t ring_bytes = size_t(nw) * depth * ROWB, red_bytes = size_t(nw) * n_grp * kQ4Pad * sizeof(float);
-    const size_t area = ((ring_bytes > red_bytes ? ring_bytes : red_bytes) + 15) & ~size_t(15);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + area);
-    float* xs = reinterpret_cast<float*>(smem + area + ((size_t(nw) * depth * 8 + 15) & ~size_t(15)));
-    const uint32_t bar0 = smem_u32(bars + wi * depth);
-    const uint32_t ring0 = smem_u32(ring);
-    if (lane == 0) {
-        for (int d = 0; d < depth; ++d) mbar_init(bar0 + 8u * d, 1);
-        fence_barrier_init();
-    }
-    __syncwarp();
-    grid_dep_wait();          // routing results (slot codes, activations, weights) are read from here on
-    // window start: kernel entry, or the end of the dependency wait when launched ahead of its predecessor's end
-    if (a.clock && threadIdx.x == 0) atomicMin(a.clock, a.dev_code ? global_timer_ns() : t_entry);
-
-    const uint64_t pol = policy_evict_first();
-    bool ok = true;
-    int src_ent = -1;                          // lane 0: entry being streamed and where its blob starts
-    const unsigned char* src_base = nullptr;   //         (null: the entry cannot be served)
+    int src_ent = -1;                          // (per lane) entry whose blob was looked up last
+    const unsigned char* src_base = nullptr;   // (null: it cannot be served; its rows are skipped)
+    bool gave_up = false;
     auto resolve = [&](int ent) -> const unsigned char* {
         const int code = a.code_of(tok, ent);
         if (code < 0) {
@@ -86,168 +302,68 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int depth, co
             return a.shared + size_t(-1 - code) * a.blob_bytes;
         }
         if (code >= a.n_slots) { atomicOr(a.status, kStatusBadSlot); return nullptr; }
-        // device-side wait for the batch of copies that fills this slot (see ffn_gemv_kernel)
-        if (a.ready && !ffn_wait_arrival(a.ready + a.watch[ent], a.want[ent], a.limit())) {
+        // device-side wait for the batch of copies that fills this slot; after one has run out no other is begun
+        if (a.ready && (gave_up || !ffn_wait_arrival(a.ready + a.watch[ent], a.want[ent], limit))) {
+            gave_up = true;
             atomicOr(a.status, kStatusCopyTimeout);
             return nullptr;
         }
         return a.pool + size_t(code) * a.blob_bytes;
     };
-    auto issue = [&](int i) {
-        const int r = r_begin + wi + i * nw;
-        const int ent = r / I;
-        const int j = r - ent * I;
+    auto row_at = [&](int row) -> const unsigned char* {
+        if (row >= span) return nullptr;
+        const int ent = (r_begin + row) / I;
         if (ent != src_ent) { src_ent = ent; src_base = resolve(ent); }
-        const unsigned char* base = src_base;
-        if (!base) return false;
-        const int st = i % depth;
-        mbar_arrive_expect_tx(bar0 + 8u * st, ROWB);
-        bulk_g2s(ring0 + uint32_t(st) * ROWB, base + size_t(j) * ROWB, ROWB, bar0 + 8u * st, pol);
-        return true;
+        return src_base ? src_base + size_t(r_begin + row - ent * I) * ROWB : nullptr;
     };
-    int n_issued = 0;
-    if (lane == 0) {
-        for (; n_issued < depth && n_issued < my_n; ++n_issued)
-            if (!issue(n_issued)) { ok = false; break; }
-    }
+    int filled = min(n_stages, (span + kQ4Rows - 1) / kQ4Rows);
+    ring.fill(0, filled, warp, lane, ROWB, row_at);
+    if (early) depend();
 
-    // activations go to shared memory once (group g at xs[g * kQ4Pad ..]); the partial y of this
-    // lane's groups (g = ch * 32 + lane) stays in registers
-    for (int i = threadIdx.x; i < D; i += blockDim.x) xs[(i >> 5) * kQ4Pad + (i & 31)] = a.x[size_t(tok) * D + i];
-    float ya[NCH][32];
+    uint32_t x[GB][4];
+    float off[GB][2];
+    const float* xt = a.x + size_t(tok) * D;
+    const bool vec = (reinterpret_cast<uintptr_t>(xt) & 15) == 0;       // the caller's rows may start at any float
+    const int x_exp = q4_operand<GB>(x, off, warp, lane, [&](int col, float (&v)[8]) {
+        if (vec) {
+            const float4 lo = *reinterpret_cast<const float4*>(xt + col), hi = *reinterpret_cast<const float4*>(xt + col + 4);
+            v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w; v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
+        } else {
 #pragma unroll
-    for (int ch = 0; ch < NCH; ++ch)
-#pragma unroll
-        for (int v = 0; v < 32; ++v) ya[ch][v] = 0.f;
-    __syncthreads();
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-
-    int cur_ent = -1;
-    float wk = 0.f;
-    int done = 0;
-    bool halt = false;
-    if (ok) {
-        for (int i = 0; i < my_n; ++i) {
-            if (i >= __shfl_sync(0xffffffffu, n_issued, 0)) break;
-            const int st = i % depth;
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8u * st, (i / depth) & 1, a.limit()))) {
-                if (lane == 0) atomicOr(a.status, kStatusCopyTimeout);
-                ok = false;
-                break;
-            }
-            done = i + 1;
-            const int r = r_begin + wi + i * nw;
-            const int ent = r / I;
-            if (ent != cur_ent) {
-                cur_ent = ent;
-                const int kk = a.kidx_of(tok, ent);
-                wk = kk == 255 ? 1.f : a.w[size_t(tok) * a.K + kk];
-            }
-            const unsigned char* buf = ring + size_t(st) * ROWB;
-            float pg = 0.f, pu = 0.f;
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
-                const int g = ch * 32 + lane;
-                if (g < n_grp) {
-                    const uint4 vg = *reinterpret_cast<const uint4*>(buf + g * 16);
-                    const uint4 vu = *reinterpret_cast<const uint4*>(buf + RB + g * 16);
-                    const float sg = __half2float(*reinterpret_cast<const __half*>(buf + D / 2 + g * 2));
-                    const float su = __half2float(*reinterpret_cast<const __half*>(buf + RB + D / 2 + g * 2));
-                    const uint32_t wg[4] = {vg.x, vg.y, vg.z, vg.w}, wu[4] = {vu.x, vu.y, vu.z, vu.w};
-                    const float* xg = xs + g * kQ4Pad;
-                    float dg = 0.f, du = 0.f;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float fg[8], fu[8];
-                        unpack_q4_word(wg[q], fg);
-                        unpack_q4_word(wu[q], fu);
-                        const float4 x0 = *reinterpret_cast<const float4*>(xg + q * 8);
-                        const float4 x1 = *reinterpret_cast<const float4*>(xg + q * 8 + 4);
-                        const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-#pragma unroll
-                        for (int v = 0; v < 8; ++v) {
-                            dg = fmaf(fg[v], xv[v], dg);
-                            du = fmaf(fu[v], xv[v], du);
-                        }
-                    }
-                    pg = fmaf(sg, dg, pg);
-                    pu = fmaf(su, du, pu);
-                }
-            }
-            pg = warp_sum(pg);
-            pu = warp_sum(pu);
-            const float act = pg / (1.f + expf(-pg)) * pu * wk;
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
-                const int g = ch * 32 + lane;
-                if (g < n_grp) {
-                    const uint4 vd = *reinterpret_cast<const uint4*>(buf + 2 * RB + g * 16);
-                    const float sd = act * __half2float(*reinterpret_cast<const __half*>(buf + 2 * RB + D / 2 + g * 2));
-                    const uint32_t wd[4] = {vd.x, vd.y, vd.z, vd.w};
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float fd[8];
-                        unpack_q4_word(wd[q], fd);
-#pragma unroll
-                        for (int v = 0; v < 8; ++v) ya[ch][q * 8 + v] = fmaf(sd, fd[v], ya[ch][q * 8 + v]);
-                    }
-                }
-            }
-            __syncwarp();
-            if (lane == 0 && n_issued < my_n && !halt) {
-                if (issue(n_issued)) ++n_issued;
-                else halt = true;
-            }
+            for (int q = 0; q < 8; ++q) v[q] = xt[col + q];
         }
-    }
+    });
+    float y[GB][2][4] = {};
+    Q4ActScale scale;
+    const bool ok = q4_tiles<GB, NW>(ring, x, off, x_exp, y, scale, D, span, warp, lane, limit,
+        [&](int tile) { ring.fill(tile, 1, warp, lane, ROWB, row_at); ++filled; },
+        [&](int row) {
+            const int kk = a.kidx_of(tok, (r_begin + row) / I);
+            return kk == 255 ? 1.f : a.w[size_t(tok) * a.K + kk];
+        });
     if (!ok) {
-        n_issued = __shfl_sync(0xffffffffu, n_issued, 0);
-        for (int i = done; i < n_issued; ++i)
-            if (!mbar_wait_bounded(bar0 + 8u * (i % depth), (i / depth) & 1, a.limit())) break;
+        if (lane == 0) atomicOr(a.status, kStatusCopyTimeout);
+        // leave no copy in flight into shared memory that is about to be released
+        for (int k = max(0, filled - n_stages); k < filled; ++k)
+            if (!mbar_wait_bounded(ring.bars + 8u * (k % n_stages), (k / n_stages) & 1, kWaitLimitNs)) break;
     }
-
-    // sum the warps' partial y in warp order, one partial row per CTA
-    __syncthreads();
-    float* red = reinterpret_cast<float*>(smem);
-#pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-        const int g = ch * 32 + lane;
-        if (g < n_grp) {
-#pragma unroll
-            for (int v = 0; v < 32; v += 4)
-                *reinterpret_cast<float4*>(red + (size_t(wi) * n_grp + g) * kQ4Pad + v) = make_float4(ya[ch][v], ya[ch][v + 1], ya[ch][v + 2], ya[ch][v + 3]);
-        }
-    }
-    __syncthreads();
     float* out = a.partial + (size_t(tok) * G + c) * D;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) {
-        const int o = (d >> 5) * kQ4Pad + (d & 31);
-        float acc = red[o];
-        for (int w2 = 1; w2 < nw; ++w2) acc += red[size_t(w2) * n_grp * kQ4Pad + o];
-        out[d] = acc;
-    }
+    q4_result<GB>(y, scale, warp, lane, [&](int col, float4 v) { *reinterpret_cast<float4*>(out + col) = v; });
     if (a.clock) {
         __syncthreads();
         if (threadIdx.x == 0) atomicMax(a.clock + 1, global_timer_ns());
     }
 }
 
-// Launch shape for 4-bit rows: the warp count that leaves the fewest rows on the busiest warp, a
-// ring deep enough to hold a warp's whole share when it fits, and room for the cross-warp reduction.
-inline void ffn_gemv_q4_shape(size_t row_bytes, int D, int rows_per_cta, int* warps, int* depth, size_t* smem) {
-    int best_w = 8, best_cost = 1 << 30;
-    for (int w = 4; w <= kQ4MaxWarps; ++w) {
-        const int cost = (rows_per_cta + w - 1) / w;
-        if (cost < best_cost || (cost == best_cost && w < best_w)) { best_w = w; best_cost = cost; }
-    }
-    int d = best_cost < 2 ? 2 : (best_cost > 6 ? 6 : best_cost);
-    while (d > 2 && size_t(best_w) * d * row_bytes > 150 * 1024) --d;
-    size_t area = size_t(best_w) * d * row_bytes;
-    const size_t red = size_t(best_w) * (D / 32) * kQ4Pad * sizeof(float);
-    if (area < red) area = red;
-    *warps = best_w;
-    *depth = d;
-    *smem = ((area + 15) & ~size_t(15)) + ((size_t(best_w) * d * 8 + 15) & ~size_t(15)) + size_t(D / 32) * kQ4Pad * sizeof(float) + 16;
+// Ring of a CTA with rows_per_cta rows: all its tiles where they fit beside `reserve` bytes. Returns the bytes of ring, barriers and sums.
+inline size_t ffn_gemv_q4_shape(int D, int rows_per_cta, size_t reserve, int* stages) {
+    const size_t stage = size_t(kQ4Rows) * mt_pitch(3 * q4_part_bytes(D), false);
+    const size_t rest = kQ4MaxStages * 8 + size_t(kQ4MaxWarps) * kQ4Red * 4 + 16 + 2 * kQ4Rows * 4;
+    const size_t fit = (kFfnSmemLimit - 1024 - rest - reserve) / stage;
+    const int want = rows_per_cta < kQ4Rows ? 1 : (rows_per_cta + kQ4Rows - 1) / kQ4Rows;
+    *stages = int(fit < size_t(want) ? fit : size_t(want));
+    if (*stages > kQ4MaxStages) *stages = kQ4MaxStages;
+    return size_t(*stages) * stage + rest;
 }
 
 }  // namespace spm

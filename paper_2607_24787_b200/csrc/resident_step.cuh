@@ -28,13 +28,14 @@
 #pragma once
 
 #include "ffn_gemv.cuh"
+#include "ffn_gemv_q4.cuh"
 #include "router_adapter.cuh"
 
 namespace spm {
 
 // Warps of a CTA: as many as the GEMV may take (those it does not use only route). Rows of 9216 bytes and more leave it eight at most,
 // whose threads then have 255 registers.
-constexpr int step_warps(int nseg) { return nseg >= 6 ? 8 : kFfnMaxWarps; }
+constexpr int step_warps(int nseg, bool q4) { return q4 ? q4_warps(nseg) : nseg >= 6 ? 8 : kFfnMaxWarps; }
 constexpr int kStepCols = 16;                     // columns of the hidden row that an owner adds up
 constexpr int kStepMaxCtas = kReduceGroupsR * kReduceChunkR;
 constexpr unsigned long long kStepStartNs = 30000000000ull;     // limit of the first exchange: kernels of other streams may hold SMs until then
@@ -59,7 +60,7 @@ struct StepArgs {
     unsigned long long pool_bytes, blob_bytes, wait_limit_ns;
     uint32_t tag0;                  // layer l's exchanges carry tag0 + l, different from what any word holds before
     int I, K, n, r, L, n_slots, n_shared;
-    int nw, depth;                  // GEMV warps and rows of a warp's ring
+    int nw, depth;                  // GEMV warps and rows of a warp's ring (4-bit experts: -, tiles of the CTA's ring)
     uint32_t ring_bytes;            // shared memory ahead of the routing arrays
     int renorm, predict, xs_in_ring;
     float eps;
@@ -130,14 +131,15 @@ __host__ __device__ constexpr size_t step_route_bytes(int D, int n, int r, bool 
            n4 * sizeof(short);
 }
 
-template <typename WT, int NSEG>
-__global__ void __launch_bounds__(step_warps(NSEG) * 32, 1)
+template <typename WT, int NSEG, bool Q4>
+__global__ void __launch_bounds__(step_warps(NSEG, Q4) * 32, 1)
 resident_step_kernel(const __grid_constant__ StepArgs a) {
-    constexpr int kStepWarps = step_warps(NSEG), kStepThreads = kStepWarps * 32;
+    constexpr int kStepWarps = step_warps(NSEG, Q4), kStepThreads = kStepWarps * 32;
     static_assert(kStepThreads >= kRouterThreads, "the hidden row is normalised by the routing kernel's number of threads");
     constexpr int VEC = 16 / int(sizeof(WT));
     constexpr int D = NSEG * 32 * VEC;
-    constexpr uint32_t ROWB = 3u * D * uint32_t(sizeof(WT));
+    constexpr uint32_t ROWB = Q4 ? 3 * q4_part_bytes(D) : 3u * D * uint32_t(sizeof(WT));
+    constexpr int GB = Q4 ? q4_groups(NSEG) : 1;
     constexpr int NV4 = (D / 4 + kRouterThreads - 1) / kRouterThreads;     // float4s of the hidden row per routing thread
 
     extern __shared__ __align__(128) unsigned char smem[];
@@ -169,7 +171,8 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
     const int n_first = min(depth, my_n), first_r = r_begin + wi + min(lane, max(n_first - 1, 0)) * nw;
     const int first_ent = first_r / I, first_j = first_r - first_ent * I;
     const unsigned long long limit = a.wait_limit_ns ? a.wait_limit_ns : kWaitLimitNs;
-    if (wi < nw && lane == 0) {
+    Q4Ring<kStepWarps> tiles(smem, D, Q4 ? depth : 0, tid);         // (4-bit experts)
+    if (!Q4 && wi < nw && lane == 0) {
         for (int d = 0; d < depth; ++d) mbar_init(bar0 + 8u * d, 1);
         fence_barrier_init();
     }
@@ -288,15 +291,25 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
             acc = warp_sum(acc);
             if (lane == 0) ll_store(a.zx + row * a.z_stride, ll_word(acc, tag));
         }
-        // the GEMV's copy of the row: like one 16-byte weight vector per lane and segment
-        float xr[NSEG][VEC];
+        // the GEMV's copy of the row: like one 16-byte weight vector per lane and segment, or as an MMA operand
+        float xr[Q4 ? 1 : NSEG][VEC];
+        uint32_t xq[GB][4];
+        float xoff[GB][2];
+        int x_exp = 0;
+        if constexpr (Q4) {
+            x_exp = q4_operand<GB>(xq, xoff, wi, lane, [&](int col, float (&f)[8]) {
+                const float4 lo = *reinterpret_cast<const float4*>(xs + col), hi = *reinterpret_cast<const float4*>(xs + col + 4);
+                f[0] = lo.x; f[1] = lo.y; f[2] = lo.z; f[3] = lo.w; f[4] = hi.x; f[5] = hi.y; f[6] = hi.z; f[7] = hi.w;
+            });
+        } else {
 #pragma unroll
-        for (int s = 0; s < NSEG; ++s)
+            for (int s = 0; s < NSEG; ++s)
 #pragma unroll
-            for (int q = 0; q < VEC; q += 4) {
-                const float4 t = *reinterpret_cast<const float4*>(xs + (s * 32 + lane) * VEC + q);
-                xr[s][q] = t.x; xr[s][q + 1] = t.y; xr[s][q + 2] = t.z; xr[s][q + 3] = t.w;
-            }
+                for (int q = 0; q < VEC; q += 4) {
+                    const float4 t = *reinterpret_cast<const float4*>(xs + (s * 32 + lane) * VEC + q);
+                    xr[s][q] = t.x; xr[s][q + 1] = t.y; xr[s][q + 2] = t.z; xr[s][q + 3] = t.w;
+                }
+        }
         for (int i = tid; i < rows; i += kStepThreads) {
             StepSpin spin(a, l == 0 ? max(limit, kStepStartNs) : limit);
             unsigned long long w;
@@ -333,6 +346,12 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
             return code < 0 ? a.shared + (size_t(l) * a.n_shared + size_t(-1 - code)) * a.blob_bytes
                             : a.pools + size_t(l) * a.pool_bytes + size_t(code) * a.blob_bytes;
         };
+        auto row_at = [&](int row) -> const unsigned char* {        // (4-bit experts)
+            if (row >= span) return nullptr;
+            const int ent = (r_begin + row) / I;
+            const unsigned char* base = blob(ent);
+            return base ? base + size_t(r_begin + row - ent * I) * ROWB : nullptr;
+        };
         // The row at `src` into the next stage of the warp's ring, by one elected lane with operands that are the same in the warp (lanes that
         // ask side by side are taken one by one; this took the DeepSeek shape from 19.3 to 17.8 us a layer). A bad slot's row is whatever
         // was there: the status word says so.
@@ -349,7 +368,9 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
             st_in = st_in + 1 == depth ? 0 : st_in + 1;
         };
         int n_in = n_first;                 // rows that the warp has asked for
-        {       // (the lanes look the rows up side by side)
+        if constexpr (Q4) {
+            tiles.fill(0, min(depth, (span + kQ4Rows - 1) / kQ4Rows), wi, lane, ROWB, row_at);
+        } else {       // (the lanes look the rows up side by side)
             const unsigned char* base = lane < n_first ? blob(first_ent) : nullptr;
             const unsigned long long at = base ? reinterpret_cast<unsigned long long>(base + size_t(first_j) * ROWB) : 0ull;
             for (int i = 0; i < n_first; ++i) ask(reinterpret_cast<const unsigned char*>(__shfl_sync(0xffffffffu, at, i)));
@@ -357,7 +378,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
         // Routing weights: the router tail's softmax over all experts, by every warp for itself. The four butterflies are the sums
         // of that tail's four warps, added in their order.
         float wk = 1.f;                     // lane k: weight of entry k
-        {
+        if (!Q4 || wi == 0) {
             float top = -INFINITY, part[4] = {0.f, 0.f, 0.f, 0.f};
             for (int e = lane; e < n; e += 32) top = fmaxf(top, ps[e]);
 #pragma unroll
@@ -375,6 +396,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
             float tot = 0.f;
             for (int k = 0; k < a.K; ++k) tot += __shfl_sync(0xffffffffu, p, k);
             if (lane < a.K) wk = a.renorm ? p / tot : p;
+            if (Q4 && lane < SPM_MAX_TOPK) s_w[lane] = wk;
         }
 
         // ---- expert FFN: this CTA's rows, as in ffn_gemv_kernel ----
@@ -383,48 +405,66 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
             ll_store2(out + col, ll_word(y.x, tag), ll_word(y.y, tag));
             ll_store2(out + col + 2, ll_word(y.z, tag), ll_word(y.w, tag));
         };
-        uint64_t ya[NSEG][VEC / 2];
-#pragma unroll
-        for (int s = 0; s < NSEG; ++s)
-#pragma unroll
-            for (int q = 0; q < VEC / 2; ++q) ya[s][q] = 0ull;
-        int done = 0;
-        for (; done < n_in; ++done) {
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8u * st_out, ph, limit))) {
-                if (lane == 0) StepSpin::raise(a);
-                dead = 1;
-                break;
+        if constexpr (Q4) {
+            float y[GB][2][4] = {};
+            Q4ActScale scale;
+            if (!q4_tiles<GB, kStepWarps>(tiles, xq, xoff, x_exp, y, scale, D, span, wi, lane, limit, [&](int tile) { tiles.fill(tile, 1, wi, lane, ROWB, row_at); },
+                                          [&](int row) { return s_w[(r_begin + row) / I]; })) {
+                if (tid == 0) StepSpin::raise(a);
+                // leave no copy in flight: the tile that was waited for and those asked for since
+                int st = tiles.st == 0 ? depth - 1 : tiles.st - 1;
+                uint32_t phase = tiles.st == 0 ? tiles.ph ^ 1 : tiles.ph;
+                do {
+                    mbar_wait_bounded(tiles.bars + 8u * st, phase, kWaitLimitNs);
+                    if (++st == depth) { st = 0; phase ^= 1; }
+                } while (st != tiles.st_in);
+                return;
             }
-            gemv_row<WT, NSEG>(ring0 + uint32_t(st_out) * ROWB + lane * 16, xr, __shfl_sync(0xffffffffu, wk, (r_begin + wi + done * nw) / I), ya);
-            __syncwarp();
-            st_out = st_out + 1 == depth ? 0 : st_out + 1;
-            if (st_out == 0) ph ^= 1;
-            if (n_in < my_n) {
-                const int r = r_begin + wi + n_in * nw, e = r / I;
-                const unsigned char* base = blob(e);
-                ask(base ? base + size_t(r - e * I) * ROWB : nullptr);
-                ++n_in;
-            }
-        }
-        if (dead)           // leave no copy in flight
+            q4_result<GB>(y, scale, wi, lane, send);
+        } else {
+            uint64_t ya[NSEG][VEC / 2];
+#pragma unroll
+            for (int s = 0; s < NSEG; ++s)
+#pragma unroll
+                for (int q = 0; q < VEC / 2; ++q) ya[s][q] = 0ull;
+            int done = 0;
             for (; done < n_in; ++done) {
-                if (!mbar_wait_bounded(bar0 + 8u * st_out, ph, kWaitLimitNs)) break;
+                if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8u * st_out, ph, limit))) {
+                    if (lane == 0) StepSpin::raise(a);
+                    dead = 1;
+                    break;
+                }
+                gemv_row<WT, NSEG>(ring0 + uint32_t(st_out) * ROWB + lane * 16, xr, __shfl_sync(0xffffffffu, wk, (r_begin + wi + done * nw) / I), ya);
+                __syncwarp();
                 st_out = st_out + 1 == depth ? 0 : st_out + 1;
                 if (st_out == 0) ph ^= 1;
+                if (n_in < my_n) {
+                    const int r = r_begin + wi + n_in * nw, e = r / I;
+                    const unsigned char* base = blob(e);
+                    ask(base ? base + size_t(r - e * I) * ROWB : nullptr);
+                    ++n_in;
+                }
             }
-        if (wi < nw && !dead) gemv_stage_y<NSEG>(ring, lane, ya);
-        if (__syncthreads_or(dead)) return;
+            if (dead)           // leave no copy in flight
+                for (; done < n_in; ++done) {
+                    if (!mbar_wait_bounded(bar0 + 8u * st_out, ph, kWaitLimitNs)) break;
+                    st_out = st_out + 1 == depth ? 0 : st_out + 1;
+                    if (st_out == 0) ph ^= 1;
+                }
+            if (wi < nw && !dead) gemv_stage_y<NSEG>(ring, lane, ya);
+            if (__syncthreads_or(dead)) return;
 
-        // ---- partial rows -> owned columns -> hidden row of the next layer ----
-        {
-            constexpr int Q = VEC / 4;
-            const size_t ring_stride = size_t(depth) * ROWB;
-            for (int p = tid; p < D / 4; p += kStepThreads) {
-                const float4 y = gemv_sum_warps(smem + size_t(p) * sizeof(float4), ring_stride, nw);
-                const int s = p / (32 * Q), h = (p / 32) % Q, ln = p % 32;
-                send(s * 32 * VEC + ln * VEC + 4 * h, y);
+            // ---- partial rows -> owned columns -> hidden row of the next layer ----
+            {
+                constexpr int Q = VEC / 4;
+                const size_t ring_stride = size_t(depth) * ROWB;
+                for (int p = tid; p < D / 4; p += kStepThreads) {
+                    const float4 y = gemv_sum_warps(smem + size_t(p) * sizeof(float4), ring_stride, nw);
+                    const int s = p / (32 * Q), h = (p / 32) % Q, ln = p % 32;
+                    send(s * 32 * VEC + ln * VEC + 4 * h, y);
+                }
+                fence_proxy_async();            // the ring held partial sums: ordered before the next layer's copies
             }
-            fence_proxy_async();            // the ring held partial sums: ordered before the next layer's copies
         }
         if (l + 1 < a.L) preload(l + 1);
         if (owner && tid < kReduceGroupsR * kStepCols) {

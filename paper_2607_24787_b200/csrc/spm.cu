@@ -413,17 +413,28 @@ cudaError_t launch_gemv_seg(int nseg, const FfnArgs<MAXNB>& a, int G, int nb, in
     return cudaErrorInvalidValue;
 }
 
-template <int NCH, int MAXNB>
-cudaError_t launch_gemv_q4_t(int D, const FfnArgs<MAXNB>& a, int G, int nb, int warps, int depth, size_t smem, cudaStream_t st, bool pdl) {
-    constexpr auto kern = ffn_gemv_q4_kernel<NCH, MAXNB>;
+template <int NSEG, int MAXNB>
+cudaError_t launch_gemv_q4_t(const FfnArgs<MAXNB>& a, int G, int nb, int stages, size_t smem, cudaStream_t st, bool pdl) {
+    constexpr auto kern = ffn_gemv_q4_kernel<NSEG, MAXNB>;
     if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
-    return launch_k(kern, dim3(G, nb), dim3(warps * 32), smem, st, pdl, a, depth, D);
+    return launch_k(kern, dim3(G, nb), dim3(q4_warps(NSEG) * 32), smem, st, pdl, a, stages);
 }
 
 template <int MAXNB>
-cudaError_t launch_gemv_q4(int D, const FfnArgs<MAXNB>& a, int G, int nb, int warps, int depth, size_t smem, cudaStream_t st, bool pdl) {
-    if (D <= 1024) return launch_gemv_q4_t<1, MAXNB>(D, a, G, nb, warps, depth, smem, st, pdl);
-    return launch_gemv_q4_t<2, MAXNB>(D, a, G, nb, warps, depth, smem, st, pdl);
+cudaError_t launch_gemv_q4(int D, const FfnArgs<MAXNB>& a, int G, int nb, int rows_per_cta, cudaStream_t st, bool pdl) {
+    int stages = 1;
+    const size_t smem = ffn_gemv_q4_shape(D, rows_per_cta, 0, &stages);
+    switch (D / 256) {
+        case 1: return launch_gemv_q4_t<1, MAXNB>(a, G, nb, stages, smem, st, pdl);
+        case 2: return launch_gemv_q4_t<2, MAXNB>(a, G, nb, stages, smem, st, pdl);
+        case 3: return launch_gemv_q4_t<3, MAXNB>(a, G, nb, stages, smem, st, pdl);
+        case 4: return launch_gemv_q4_t<4, MAXNB>(a, G, nb, stages, smem, st, pdl);
+        case 5: return launch_gemv_q4_t<5, MAXNB>(a, G, nb, stages, smem, st, pdl);
+        case 6: return launch_gemv_q4_t<6, MAXNB>(a, G, nb, stages, smem, st, pdl);
+        case 7: return launch_gemv_q4_t<7, MAXNB>(a, G, nb, stages, smem, st, pdl);
+        case 8: return launch_gemv_q4_t<8, MAXNB>(a, G, nb, stages, smem, st, pdl);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <int MAXNB>
@@ -432,11 +443,7 @@ cudaError_t launch_gemv(const spm_ctx* c, const FfnArgs<MAXNB>& a, int G, int nb
     for (int t = 0; t < nb; ++t) max_cnt = std::max(max_cnt, int(a.count[t]));
     const int rows_per_cta = (max_cnt * c->cfg.inter + G - 1) / G;
     int warps = 8, depth = 2;
-    if (c->cfg.dtype == SPM_DTYPE_Q4) {
-        size_t smem = 0;
-        ffn_gemv_q4_shape(c->row_bytes, c->cfg.hidden, rows_per_cta, &warps, &depth, &smem);
-        return launch_gemv_q4<MAXNB>(c->cfg.hidden, a, G, nb, warps, depth, smem, c->compute, pdl);
-    }
+    if (c->cfg.dtype == SPM_DTYPE_Q4) return launch_gemv_q4<MAXNB>(c->cfg.hidden, a, G, nb, rows_per_cta, c->compute, pdl);
     ffn_gemv_shape(c->row_bytes, rows_per_cta, &warps, &depth);
     const size_t smem = ffn_gemv_smem(c->row_bytes, warps, depth);
     if (c->cfg.dtype == SPM_DTYPE_BF16) return launch_gemv_seg<bf16_t, MAXNB>(c->nseg, a, G, nb, warps, depth, smem, c->compute, pdl);
@@ -1306,13 +1313,13 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
     return SPM_OK;
 }
 
-template <typename WT, int NSEG>
+template <typename WT, int NSEG, bool Q4>
 cudaError_t launch_resident_t(const StepArgs& a, int G, size_t smem, cudaStream_t st) {
-    constexpr auto kern = resident_step_kernel<WT, NSEG>;
+    constexpr auto kern = resident_step_kernel<WT, NSEG, Q4>;
     if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(G);
-    lc.blockDim = dim3(step_warps(NSEG) * 32);
+    lc.blockDim = dim3(step_warps(NSEG, Q4) * 32);
     lc.dynamicSmemBytes = smem;
     lc.stream = st;
     cudaLaunchAttribute at[1];
@@ -1322,17 +1329,17 @@ cudaError_t launch_resident_t(const StepArgs& a, int G, size_t smem, cudaStream_
     lc.numAttrs = 1;
     return cudaLaunchKernelEx(&lc, kern, a);
 }
-template <typename WT>
+template <typename WT, bool Q4>
 cudaError_t launch_resident_seg(int nseg, const StepArgs& a, int G, size_t smem, cudaStream_t st) {
     switch (nseg) {
-        case 1: return launch_resident_t<WT, 1>(a, G, smem, st);
-        case 2: return launch_resident_t<WT, 2>(a, G, smem, st);
-        case 3: return launch_resident_t<WT, 3>(a, G, smem, st);
-        case 4: return launch_resident_t<WT, 4>(a, G, smem, st);
-        case 5: return launch_resident_t<WT, 5>(a, G, smem, st);
-        case 6: return launch_resident_t<WT, 6>(a, G, smem, st);
-        case 7: return launch_resident_t<WT, 7>(a, G, smem, st);
-        case 8: return launch_resident_t<WT, 8>(a, G, smem, st);
+        case 1: return launch_resident_t<WT, 1, Q4>(a, G, smem, st);
+        case 2: return launch_resident_t<WT, 2, Q4>(a, G, smem, st);
+        case 3: return launch_resident_t<WT, 3, Q4>(a, G, smem, st);
+        case 4: return launch_resident_t<WT, 4, Q4>(a, G, smem, st);
+        case 5: return launch_resident_t<WT, 5, Q4>(a, G, smem, st);
+        case 6: return launch_resident_t<WT, 6, Q4>(a, G, smem, st);
+        case 7: return launch_resident_t<WT, 7, Q4>(a, G, smem, st);
+        case 8: return launch_resident_t<WT, 8, Q4>(a, G, smem, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -1342,6 +1349,13 @@ cudaError_t launch_resident_seg(int nseg, const StepArgs& a, int G, size_t smem,
 bool resident_shape(const spm_ctx* c, int G, StepArgs* a, size_t* smem) {
     const spm_model_cfg& m = c->cfg;
     const int rows_per_cta = ((m.top_k + m.n_shared) * m.inter + G - 1) / G;
+    if (m.dtype == SPM_DTYPE_Q4) {
+        const size_t route = step_route_bytes(m.hidden, m.n_experts, m.adapter_rank, false);
+        const size_t ring = align_up(ffn_gemv_q4_shape(m.hidden, rows_per_cta, route + 16, &a->depth), 16);
+        *smem = ring + route;
+        a->ring_bytes = uint32_t(ring);
+        return a->depth >= 1 && *smem <= kFfnSmemLimit - 1024;
+    }
     ffn_gemv_shape(c->row_bytes, rows_per_cta, &a->nw, &a->depth);
     for (; a->depth >= 2; --a->depth)
         for (const int in_ring : {0, 1}) {
@@ -1363,7 +1377,7 @@ int enqueue_resident_step(spm_ctx* c, const float* h_in, float* h_out, int slot,
     const int G = c->num_sms;
     StepArgs a{};
     size_t smem = 0;
-    if (!c->coop || m.dtype == SPM_DTYPE_Q4 || (m.dtype == SPM_DTYPE_FP32 && m.n_layers < 3) || c->timing || c->stub_us > 0 || ffn_grid_for(c, 1) != G ||
+    if (!c->coop || (m.dtype == SPM_DTYPE_FP32 && m.n_layers < 3) || c->timing || c->stub_us > 0 || ffn_grid_for(c, 1) != G ||
         G > kStepMaxCtas || 2 * G > kMaxCtasBatch1 || m.hidden > G * kStepCols || !resident_shape(c, G, &a, &smem)) return SPM_OK;
     predict = predict && m.n_layers > 1;
     if (predict && !aligned16(c->buf.adapter_a)) return fail(c, SPM_ERR_INVALID_ARG, "adapter_a must be 16-byte aligned");
@@ -1408,8 +1422,9 @@ int enqueue_resident_step(spm_ctx* c, const float* h_in, float* h_out, int slot,
     if (c->step_tag > 0xffffffffu - 2u * m.n_layers) c->step_tag = 1;        // (the words hold tags of the last two layers)
     a.tag0 = c->step_tag;
     c->step_tag += m.n_layers;
-    const cudaError_t launched = m.dtype == SPM_DTYPE_FP32 ? launch_resident_seg<float>(c->nseg, a, G, smem, c->compute)
-                                                           : launch_resident_seg<bf16_t>(c->nseg, a, G, smem, c->compute);
+    const cudaError_t launched = m.dtype == SPM_DTYPE_FP32 ? launch_resident_seg<float, false>(c->nseg, a, G, smem, c->compute)
+                               : m.dtype == SPM_DTYPE_BF16 ? launch_resident_seg<bf16_t, false>(c->nseg, a, G, smem, c->compute)
+                                                           : launch_resident_seg<bf16_t, true>(c->nseg, a, G, smem, c->compute);
     CU(c, launched);
     c->kernel_launches++;
     c->ffn_launches += m.n_layers;

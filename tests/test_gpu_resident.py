@@ -22,6 +22,10 @@ CASES = {
     "bf16_many_experts": dict(base="qwen3", hidden=256, n_experts=600, inter=24, top_k=16, adapter_rank=3),
     "bf16_row_in_ring": dict(base="qwen3", hidden=2048, n_experts=513, inter=10, top_k=2, adapter_rank=63),
     "bf16_nine_warps": dict(base="dsvl2", hidden=1280, n_experts=16, inter=224, top_k=6, n_shared=2, adapter_rank=16),
+    "q4_narrow": dict(base="qwen3_q4", hidden=256, n_experts=12, inter=96, top_k=3, adapter_rank=4),
+    "q4_shared": dict(base="dsvl2_q4", hidden=1280, n_experts=16, inter=224, top_k=6, n_shared=2, adapter_rank=16),
+    "q4_widest": dict(base="qwen3_q4", hidden=2048, n_experts=20, inter=450, top_k=8, adapter_rank=16),
+    "q4_many_experts": dict(base="qwen3_q4", hidden=768, n_experts=300, inter=33, top_k=10, adapter_rank=2),
     "bf16_raw_weights": dict(base="qwen3", hidden=1792, n_experts=9, inter=100, top_k=3, renormalize=0, adapter_rank=4),
 }
 
