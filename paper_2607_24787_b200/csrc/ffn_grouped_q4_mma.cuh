@@ -1,0 +1,344 @@
+// Batched decode with 4-bit experts, few tokens an expert: the grouped SwiGLU expert FFN with the unpacked weights going from
+// registers straight into mma.sync.
+//
+// Takes the place of ffn_grouped_q4_kernel (tcgen05) where an expert has few tokens, which is the rule in decode: 64 sequences of
+// the Qwen3 shape give an expert about four. There the tensor cores idle either way, and what the tcgen05 kernel spends its time on
+// is the way of an operand: unpack, store to tensor or shared memory, fence, hand-shake, 1050 cycles for an item that HBM
+// delivers in 340. An mma.sync operand is where the unpacking leaves it, in the registers of the lane that needs it. A layer of a whole
+// host-free step of that shape: 198 -> 142 us (HBM time of its experts: 49). What bounds it now: instruction issue and dependent-issue
+// latency, 107,000 instructions a scheduler at 0.5 a cycle, 330 of a warp's 620 a tile for what is done once a tile.
+//
+// Work. A task is 128 intermediate rows of an expert (GgUnit) for up to kMqTokens of its tokens; CTA b runs the tasks b, b + grid, ...
+// of all experts in order (a hot expert's runs of tokens go to different CTAs). A task goes through its rows in tiles of 16; the
+// warps split the columns in groups of 32 (one scale), GB consecutive groups a warp.
+//   Phase 1 (M = 16 gate rows, then 16 up rows; N = tokens; K = 32 columns, two MMAs): the group's scale goes onto the fp32 sum. The
+// warps' sums meet in shared memory.
+//   Phase 2 (M = 16 hidden columns, N = tokens, K = 16 rows): the warp's own columns; the scale goes onto the activation, rounded
+// to bf16 once. y stays in the accumulators for the whole task.
+// Phase 2 is one tile behind phase 1, so that one CTA barrier a tile is enough. The rows of a tile come as two bulk copies each, gate /
+// up and W_down, into rings of their own.
+//
+// A token's result depends on its own row and the expert only (a column of the MMAs), so outputs do not depend on waves, batch
+// mates or the CTA. Rounding: activations to bf16, act * scale to bf16, all else exact or fp32 (the tcgen05 kernel also rounds
+// the scales and the products of scale and weight).
+#pragma once
+
+#include <type_traits>
+
+#include "ffn_grouped.cuh"
+#include "ffn_multi.cuh"
+#include "q4_mma.cuh"
+
+namespace spm {
+
+constexpr int kMqTokens = 8;                  // tokens of a task: N of the MMAs
+constexpr int kMqTiles = kGgTileRows / kQ4Rows;
+constexpr int kMqRed = 264;                   // pitch of a warp's phase-1 sums: 256 floats, the next warp's eight banks on
+constexpr int kMqMaxTasks = 512;              // tasks of a CTA
+
+struct MqArgs {
+    const unsigned char* pools;     // all layers' slots
+    const __nv_bfloat16* xs;        // sorted token rows, columns 8g .. 8g + 7 in the order 0 4 1 5 2 6 3 7
+    unsigned long long blob_bytes;
+    GgArgs g;
+};
+struct MqTask { int slot, jt_n, row, unit; };         // global slot, 128-row tile * 16 + tokens, first token row, unit
+
+// Tasks of a CTA at worst: every expert's last run partly filled
+inline int mq_max_tasks(int nb, int K, int n, int n_jt, int grid) {
+    const int pairs = nb * K, runs = (pairs < n ? pairs : n) + pairs / kMqTokens;
+    return (runs * n_jt + grid - 1) / grid;
+}
+inline size_t mq_rest_bytes(int n) {
+    return 2 * kQ4MaxStages * 8 + 2 * size_t(kQ4MaxWarps) * kMqRed * 4 + 2 * kMqTokens * kQ4Rows * 4 + 2 * kMqTokens * 4 + 16 +
+           size_t(kMqMaxTasks) * sizeof(MqTask) + size_t(n + 1) * 4;
+}
+inline int mq_stages(int D, int n, size_t* smem) {
+    const size_t stage = size_t(kQ4Rows) * (mt_pitch(2 * q4_part_bytes(D), false) + mt_pitch(q4_part_bytes(D), false));
+    size_t s = (kFfnSmemLimit - mq_rest_bytes(n)) / stage;
+    if (s > size_t(kQ4MaxStages)) s = kQ4MaxStages;
+    *smem = s * stage + mq_rest_bytes(n);
+    return int(s);
+}
+
+template <int NSEG>
+__global__ void __launch_bounds__(q4_warps(NSEG) * 32, 1)
+ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) {
+    constexpr int D = NSEG * 256, GB = q4_groups(NSEG), NW = q4_warps(NSEG);
+    constexpr uint32_t PART = q4_part_bytes(D), GU = mt_pitch(2 * PART, false), DN = mt_pitch(PART, false);      // row pitches
+    extern __shared__ __align__(128) unsigned char smem[];
+    const GgArgs& a = m.g;
+    const uint32_t dn_ring = uint32_t(n_stages) * kQ4Rows * GU;               // the gate / up ring, then the W_down ring
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + dn_ring + uint32_t(n_stages) * kQ4Rows * DN);
+    MqTask* tasks = reinterpret_cast<MqTask*>(bars + 2 * kQ4MaxStages);
+    float* red = reinterpret_cast<float*>(tasks + kMqMaxTasks);               // [2][warps] phase-1 sums
+    float* actv = red + 2 * NW * kMqRed;                                      // [2][token][row]
+    float* s_w = actv + 2 * kMqTokens * kQ4Rows;                              // [2 tasks][token]
+    int& s_abort = *reinterpret_cast<int*>(s_w + 2 * kMqTokens);
+    int& s_gu = (&s_abort)[1];
+    int& s_dn = (&s_abort)[2];
+    int* runs = &s_abort + 4;                                                 // [experts + 1] runs of tokens before each expert
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;      // (warp: uniform)
+    const uint32_t ring = smem_u32(smem), gu_bar = smem_u32(bars), dn_bar = gu_bar + 8 * kQ4MaxStages;
+    const unsigned long long limit = a.wait_limit_ns ? a.wait_limit_ns : kWaitLimitNs;
+
+    grid_dep_launch();
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < n_stages; ++s) { mbar_init(gu_bar + 8 * s, kQ4Rows); mbar_init(dn_bar + 8 * s, kQ4Rows); }
+        s_abort = 0;
+        fence_barrier_init();
+    }
+    grid_dep_wait();
+    if (a.clock && threadIdx.x == 0) atomicMin(a.clock, global_timer_ns());
+
+    // ---- the CTA's tasks ----
+    const int n_jt = a.I / kGgTileRows, n_exp = (a.n_units_dev ? __ldcg(a.n_units_dev) : a.n_units) / n_jt;
+    for (int e = threadIdx.x; e < n_exp; e += NW * 32) runs[e + 1] = (__ldcg(&a.units[e * n_jt].ntok) + kMqTokens - 1) / kMqTokens;
+    __syncthreads();
+    if (warp == 0) {
+        int run = 0;
+        for (int e0 = 0; e0 < n_exp; e0 += 32) {
+            int v = e0 + lane < n_exp ? runs[e0 + lane + 1] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            if (e0 + lane < n_exp) runs[e0 + lane + 1] = run + v;
+            run += __shfl_sync(0xffffffffu, v, 31);
+        }
+        if (lane == 0) runs[0] = 0;
+    }
+    __syncthreads();
+    const int n_all = n_exp > 0 ? runs[n_exp] * n_jt : 0, G = int(gridDim.x);
+    const int n_tasks = min(kMqMaxTasks, int(blockIdx.x) < n_all ? (n_all - 1 - int(blockIdx.x)) / G + 1 : 0);
+    for (int i = threadIdx.x; i < n_tasks; i += NW * 32) {
+        const int task = int(blockIdx.x) + i * G, run = task / n_jt, jt = task - run * n_jt;
+        int lo = 0, hi = n_exp;              // the expert whose runs hold this one
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (runs[mid] <= run) lo = mid; else hi = mid;
+        }
+        const int4 v = __ldcg(reinterpret_cast<const int4*>(a.units + lo * n_jt + jt));      // GgUnit{slot, jt, row0, ntok}
+        const int tok = (run - runs[lo]) * kMqTokens;
+        tasks[i] = MqTask{v.x, v.y * 16 + min(kMqTokens, v.w - tok), v.z + tok, lo * n_jt + jt};
+    }
+    __syncthreads();
+
+    // ---- The warps fill the rings, warp i the rows i, i + NW of every tile. One elected lane asks, with operands that are the same in
+    // the warp: with a row a lane, which the compiler takes one by one, the two rings cost a warp 110 instructions a tile more. ----
+    struct Feed { int task, tile, n, st; const unsigned char* src; };       // next tile; tiles asked for; stage of the next; the tile's first row
+    const uint64_t pol = policy_evict_first();
+    bool feeding = true;
+    auto open = [&](Feed& f, uint32_t off, bool wait) {
+        if (f.task >= n_tasks) return;
+        const MqTask k = tasks[f.task];
+        f.src = m.pools + size_t(k.slot) * m.blob_bytes + size_t(k.jt_n >> 4) * kGgTileRows * (3 * PART) + off;
+        if (wait && a.unit_wait) {       // the expert's copy may still be on its way
+            const GgWait uw = a.unit_wait[k.unit];
+            const GgAbort ab{&s_abort, a.status, limit};
+            if (uw.watch >= 0 && !__all_sync(0xffffffffu, gg_wait_arrival(a.ready + uw.watch, uw.want, ab))) feeding = false;
+        }
+    };
+    auto feed = [&](Feed& f, uint32_t ring_at, uint32_t bar, uint32_t pitch, uint32_t off, uint32_t bytes, bool wait) {
+        if (!feeding || f.task >= n_tasks) return;
+        if (elect_one())
+#pragma unroll
+            for (int r = 0; r < kQ4Rows; r += NW)
+                if (kQ4Rows % NW == 0 || r + warp < kQ4Rows) {
+                    mbar_arrive_expect_tx(bar + 8 * f.st, bytes);
+                    bulk_g2s(ring_at + uint32_t(f.st * kQ4Rows + r + warp) * pitch, f.src + size_t(r + warp) * (3 * PART), bytes, bar + 8 * f.st, pol);
+                }
+        __syncwarp();
+        ++f.n;
+        f.st = f.st + 1 == n_stages ? 0 : f.st + 1;
+        f.src += size_t(kQ4Rows) * (3 * PART);
+        if (++f.tile < kMqTiles) return;
+        f.tile = 0;
+        ++f.task;
+        open(f, off, wait);
+    };
+    Feed fgu{0, 0, 0, 0, nullptr}, fdn = fgu;
+    auto feed_gu = [&]() { feed(fgu, ring, gu_bar, GU, 0, 2 * PART, true); };
+    auto feed_dn = [&]() { feed(fdn, ring + dn_ring, dn_bar, DN, 2 * PART, PART, false); };     // (never ahead of the other)
+    open(fgu, 0, true);
+    open(fdn, 2 * PART, false);
+    for (int i = 0; i < n_stages; ++i) { feed_gu(); feed_dn(); }
+
+    // ---- tiles: phase 1 of tile k, phase 2 of tile k - 1 ----
+    const int grp0 = warp * GB;
+    uint32_t x[GB][4];
+    float off[GB][2], down[2] = {0.f, 0.f};      // down: 2^133 over the scale of the tokens 2t and 2t + 1
+    float y[GB][2][4];
+    Q4ActScale scale;
+    auto load_x = [&](int task) {           // token rows, and the routing weights, of the task that phase 1 comes to
+        const MqTask k = task < n_tasks ? tasks[task] : MqTask{0, 0, 0, 0};
+        const bool on = g < (k.jt_n & 15);
+        const __nv_bfloat16* p = m.xs + size_t(k.row + g) * D + grp0 * 32 + t * 8;
+#pragma unroll
+        for (int i = 0; i < GB; ++i) {
+            const uint4 v = on ? __ldcg(reinterpret_cast<const uint4*>(p + i * 32)) : make_uint4(0, 0, 0, 0);
+            x[i][0] = v.x; x[i][1] = v.y; x[i][2] = v.z; x[i][3] = v.w;
+        }
+        if (threadIdx.x < kMqTokens) s_w[(task & 1) * kMqTokens + threadIdx.x] = int(threadIdx.x) < (k.jt_n & 15) ? __ldcg(a.wrow + k.row + threadIdx.x) : 0.f;
+    };
+    auto scale_x = [&]() {                  // a token's columns of this warp by one power of two
+        uint32_t top = 0;
+#pragma unroll
+        for (int i = 0; i < GB; ++i)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) top = __vmaxu2(top, x[i][q] & 0x7fff7fffu);
+        top = max(top & 0xffffu, top >> 16);
+        top = max(top, __shfl_xor_sync(0xffffffffu, top, 1));
+        top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
+        const int e = q4_exponent(top << 16);
+        const float up = q4_up(e), dn = q4_down(e);
+        const __nv_bfloat162 even = __float2bfloat162_rn(up), odd = __float2bfloat162_rn(up * 0.0625f);
+#pragma unroll
+        for (int i = 0; i < GB; ++i) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const __nv_bfloat162 v = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&x[i][q]), (q & 1) ? odd : even);
+                x[i][q] = *reinterpret_cast<const uint32_t*>(&v);
+            }
+            q4_offset(x[i], off[i]);
+        }
+        down[0] = __shfl_sync(0xffffffffu, dn, 8 * t);
+        down[1] = __shfl_sync(0xffffffffu, dn, 8 * t + 4);
+    };
+    auto clear_y = [&]() {
+#pragma unroll
+        for (int i = 0; i < GB; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) y[i][j][v] = 0.f;
+    };
+    load_x(0);
+    clear_y();
+    bool dead = false;
+    int st1 = 0, st2 = 0;
+    uint32_t ph1 = 0, ph2 = 0;
+    const int n_tiles = n_tasks * kMqTiles;
+    for (int k = 0; k <= n_tiles && n_tiles > 0; ++k) {
+        const bool p1 = k < n_tiles, p2 = k > 0;
+        const int task1 = k / kMqTiles;
+        if (p1) {
+            if (k % kMqTiles == 0) scale_x();
+            if (!dead) dead = !__all_sync(0xffffffffu, mt_wait(gu_bar + 8 * st1, ph1, &s_abort, a.status, limit));
+            const uint32_t rows = ring + uint32_t(st1) * kQ4Rows * GU;
+            if (++st1 == n_stages) { st1 = 0; ph1 ^= 1; }
+            float ag[4], au[4];
+            q4_phase1<GB, false>(rows, GU, D, grp0, lane, x, off, ag, au, [](float (&acc)[4], const float (&c)[4], float s0, float s1) {
+                acc[0] = fmaf(s0, c[0], acc[0]); acc[1] = fmaf(s0, c[1], acc[1]);
+                acc[2] = fmaf(s1, c[2], acc[2]); acc[3] = fmaf(s1, c[3], acc[3]);
+            });
+            float* r = red + ((k & 1) * NW + warp) * kMqRed + lane * 4;
+            *reinterpret_cast<float4*>(r) = make_float4(ag[0] * down[0], ag[1] * down[1], ag[2] * down[0], ag[3] * down[1]);
+            *reinterpret_cast<float4*>(r + 128) = make_float4(au[0] * down[0], au[1] * down[1], au[2] * down[0], au[3] * down[1]);
+            if (k % kMqTiles == kMqTiles - 1) load_x(task1 + 1);        // the next task's rows are on their way while this tile is finished
+        }
+        if (p2 && !dead) dead = !__all_sync(0xffffffffu, mt_wait(dn_bar + 8 * st2, ph2, &s_abort, a.status, limit));
+        __syncthreads();
+        // every warp is done with the gate / up rows of tile k and with the W_down rows of tile k - 2
+        if (!dead) {
+            if (p1) feed_gu();
+            if (k >= 2 && fdn.n < k - 1 + n_stages) feed_dn();
+        }
+        if (p1) {       // 128 (row, token) pairs, eight at a time; four lanes share the warps' sums of one
+            for (int q = warp; q < 16; q += NW) {
+                const int pair = q * 8 + (lane & 7);
+                const float* r = red + ((k & 1) * NW + (lane >> 3)) * kMqRed + pair;
+                float vg = 0.f, vu = 0.f;
+#pragma unroll
+                for (int w = 0; w < (NW + 3) / 4; ++w)
+                    if (NW % 4 == 0 || w * 4 + (lane >> 3) < NW) { vg += r[w * 4 * kMqRed]; vu += r[w * 4 * kMqRed + 128]; }
+                vg += __shfl_xor_sync(0xffffffffu, vg, 8);
+                vu += __shfl_xor_sync(0xffffffffu, vu, 8);
+                vg += __shfl_xor_sync(0xffffffffu, vg, 16);
+                vu += __shfl_xor_sync(0xffffffffu, vu, 16);
+                const int row = (pair >> 4) + 8 * ((pair >> 1) & 1), tok = 2 * ((pair >> 2) & 3) + (pair & 1);
+                if (lane < 8) actv[((k & 1) * kMqTokens + tok) * kQ4Rows + row] = __fdividef(vg, 1.f + __expf(-vg)) * vu * s_w[(task1 & 1) * kMqTokens + tok];
+            }
+        }
+        if (!p2) continue;
+        {
+            const float* av = actv + (((k - 1) & 1) * kMqTokens + g) * kQ4Rows + 2 * t;
+            float2 a0 = *reinterpret_cast<const float2*>(av), a1 = *reinterpret_cast<const float2*>(av + 8);
+            scale.fit<GB>(fmaxf(fmaxf(fabsf(a0.x), fabsf(a0.y)), fmaxf(fabsf(a1.x), fabsf(a1.y))), y);
+            a0.x *= scale.up; a0.y *= scale.up; a1.x *= scale.up; a1.y *= scale.up;
+            const uint32_t rows = ring + dn_ring + uint32_t(st2) * kQ4Rows * DN;
+            if (++st2 == n_stages) { st2 = 0; ph2 ^= 1; }
+            const uint32_t at = rows + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * DN + uint32_t(grp0) * 16;
+            const uint32_t sc = rows + uint32_t(2 * t) * DN + uint32_t(D / 2 + grp0 * 2);
+            uint32_t b[GB][2];
+            {
+                float s0[GB], s1[GB], s2[GB], s3[GB];
+                q4_scales<GB>(sc, s0);
+                q4_scales<GB>(sc + DN, s1);
+                q4_scales<GB>(sc + 8 * DN, s2);
+                q4_scales<GB>(sc + 9 * DN, s3);
+#pragma unroll
+                for (int i = 0; i < GB; ++i) {
+                    const __nv_bfloat162 b0 = __floats2bfloat162_rn(a0.x * s0[i], a0.y * s1[i]), b1 = __floats2bfloat162_rn(a1.x * s2[i], a1.y * s3[i]);
+                    b[i][0] = *reinterpret_cast<const uint32_t*>(&b0);
+                    b[i][1] = *reinterpret_cast<const uint32_t*>(&b1);
+                }
+            }
+            auto phase2 = [&](auto exact) {
+#pragma unroll
+                for (int i = 0; i < GB; i += 2) {
+                    // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word
+                    const int j = i + 1 < GB ? i + 1 : i;
+                    const uint4 w = ldsm4t(at + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
+                    q4_phase2<decltype(exact)::value>(y[i], w.x, w.y, b[i][0], b[i][1]);
+                    if (i + 1 < GB) q4_phase2<decltype(exact)::value>(y[j], w.z, w.w, b[j][0], b[j][1]);
+                }
+            };
+            if (q4_any_nonfinite(b)) phase2(std::true_type{});
+            else phase2(std::false_type{});
+        }
+        if ((k - 1) % kMqTiles == kMqTiles - 1) {            // end of a task: a lane has four consecutive columns of two tokens
+            const MqTask kk = tasks[(k - 1) / kMqTiles];
+            const int n_tok = kk.jt_n & 15;
+            float* out = a.partial + (size_t(kk.jt_n >> 4) * a.rows_cap + kk.row) * D + grp0 * 32 + g * 4;
+#pragma unroll
+            for (int i = 0; i < GB; ++i) {
+                if (2 * t < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t) * D + i * 32) = scale.out(y[i][0][0], y[i][0][2], y[i][1][0], y[i][1][2]);
+                if (2 * t + 1 < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t + 1) * D + i * 32) = scale.out(y[i][0][1], y[i][0][3], y[i][1][1], y[i][1][3]);
+            }
+            clear_y();
+            scale = Q4ActScale{};
+        }
+    }
+    // Wind-down after a wait ran out, as in ffn_multi_kernel: the warps agree on the last tile that any of them fed, arrive without a
+    // copy for the tiles up to it, and wait for what is in flight.
+    __syncthreads();
+    if (*reinterpret_cast<volatile int*>(&s_abort)) {
+        if (threadIdx.x == 0) { s_gu = 0; s_dn = 0; }
+        __syncthreads();
+        if (lane == 0) { atomicMax(&s_gu, fgu.n); atomicMax(&s_dn, fdn.n); }
+        __syncthreads();
+        const int n_gu = s_gu, n_dn = s_dn;
+        if (elect_one())
+            for (int r = warp; r < kQ4Rows; r += NW) {
+                for (int i = fgu.n; i < n_gu; ++i) mbar_arrive(gu_bar + 8 * (i % n_stages));
+                for (int i = fdn.n; i < n_dn; ++i) mbar_arrive(dn_bar + 8 * (i % n_stages));
+            }
+        const unsigned long long t0 = global_timer_ns();
+        auto drain = [&](uint32_t bar, int n_fed) {
+            for (int i = max(0, n_fed - n_stages); i < n_fed; ++i) {
+                const unsigned long long spent = global_timer_ns() - t0;
+                mbar_wait_bounded(bar + 8 * (i % n_stages), (i / n_stages) & 1, spent < kWaitLimitNs ? kWaitLimitNs - spent : 0);
+            }
+        };
+        drain(gu_bar, n_gu);
+        drain(dn_bar, n_dn);
+    }
+    if (a.clock) {
+        __syncthreads();
+        if (threadIdx.x == 0) atomicMax(a.clock + 1, global_timer_ns());
+    }
+}
+
+}  // namespace spm

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -22,6 +23,7 @@
 #include "ffn_multi.cuh"
 #include "ffn_grouped.cuh"
 #include "ffn_grouped_q4.cuh"
+#include "ffn_grouped_q4_mma.cuh"
 #include "resident_step.cuh"
 #include "router_adapter.cuh"
 #include "tma_maps.h"
@@ -505,6 +507,50 @@ int launch_multi_combine(spm_ctx* c, const MtArgs& a, float* h) {
     return SPM_OK;
 }
 
+template <int NSEG>
+cudaError_t launch_grouped_q4_mma_t(const spm_ctx* c, const MqArgs& a) {
+    constexpr auto kern = ffn_grouped_q4_mma_kernel<NSEG>;
+    if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
+    size_t smem = 0;
+    const int stages = mq_stages(a.g.D, c->cfg.n_experts, &smem);
+    return launch_k(kern, dim3(c->num_sms), dim3(q4_warps(NSEG) * 32), smem, c->compute, true, a, stages);
+}
+// 4-bit grouped FFN of nb sequences. Which kernel follows from the call alone, not from a wave: the two round differently.
+// ffn_grouped_q4_mma_kernel costs a CTA's tasks (an expert's 128 rows for up to eight tokens) and depends little on hidden, the
+// tcgen05 kernel costs a CTA's units (an expert's 128 rows), in proportion to hidden and up to twice as much with many tokens. The
+// costs below are in us per 16 rows, from whole host-free steps (us a layer, tcgen05 -> mma.sync; sequences, top-k of experts, hidden;
+// 768 rows an expert):
+//   64, 8 of 128, 2048: 198 -> 142     8, 8 of 128, 2048: 103 -> 68     64, 8 of 60, 2048: 140 -> 108     64, 8 of 24, 2048:  85 -> 98
+//   64, 8 of 128, 1280: 134 -> 120     2, 8 of 128, 2048:  52 -> 38     32, 4 of 12, 2048:  61 -> 42      64, 8 of 12, 2048:  95 -> 91
+//   64, 8 of 128,  768:  98 -> 97     64, 8 of 128,  256:  57 -> 93
+bool grouped_q4_mma_pays(const spm_ctx* c, int nb) {
+    const spm_model_cfg& m = c->cfg;
+    if (mq_max_tasks(nb, m.top_k, m.n_experts, c->n_jt, c->num_sms) > kMqMaxTasks) return false;
+    const double n = m.n_experts, used = n * (1.0 - std::pow(1.0 - m.top_k / n, nb)), tokens = double(nb) * m.top_k / used, seg = m.hidden / 256;
+    auto rounds = [&](double work) { return std::ceil(work * c->n_jt / c->num_sms); };
+    const double mma = rounds(used * std::max(1.0, (tokens + 3) / 8)) * (1.35 + 0.14 * seg);
+    const double tc = rounds(used) * (0.2 + 0.49 * seg) * (1 + 0.5 * std::max(0.0, (std::min(tokens, 48.0) - 8) / 16));
+    return mma < tc;
+}
+cudaError_t launch_grouped_q4(const spm_ctx* c, int nb, int grid, const GgArgs& a) {
+    const spm_model_cfg& m = c->cfg;
+    if (grouped_q4_mma_pays(c, nb)) {
+        MqArgs q{c->pools, c->tc_xs, c->blob, a};
+        switch (m.hidden / 256) {
+            case 1: return launch_grouped_q4_mma_t<1>(c, q);
+            case 2: return launch_grouped_q4_mma_t<2>(c, q);
+            case 3: return launch_grouped_q4_mma_t<3>(c, q);
+            case 4: return launch_grouped_q4_mma_t<4>(c, q);
+            case 5: return launch_grouped_q4_mma_t<5>(c, q);
+            case 6: return launch_grouped_q4_mma_t<6>(c, q);
+            case 7: return launch_grouped_q4_mma_t<7>(c, q);
+            case 8: return launch_grouped_q4_mma_t<8>(c, q);
+        }
+        return cudaErrorInvalidValue;
+    }
+    return launch_k(ffn_grouped_q4_kernel, dim3(grid), dim3(kQgThreads), ffn_grouped_q4_smem(), c->compute, true, c->qmapn, c->qmapsc, c->xmaps, a);
+}
+
 // Where a routing launch leaves its results besides the workspace: by default the context's
 // mailbox, which the host polls; a host-free step names a trace mailbox, the device-side slot
 // map and the slot-code row of its layer, and lets the kernel start ahead of its predecessor's end.
@@ -855,8 +901,7 @@ int launch_grouped_wave(spm_ctx* c, int layer, const float* x_norm, const int32_
     if (n_units == 0) {
         // (nothing to compute in this wave; the combine below still closes the layer)
     } else if (q4) {
-        CU(c, launch_k(ffn_grouped_q4_kernel, dim3(std::min(c->num_sms, n_units)), dim3(kQgThreads), ffn_grouped_q4_smem(), c->compute, true,
-                       c->qmapn, c->qmapsc, c->xmaps, a));
+        CU(c, launch_grouped_q4(c, nb, std::min(c->num_sms, n_units), a));
     } else {
         a.chunks = reinterpret_cast<const GgTask*>(dd + c->tc_off_chunks);
         a.n_chunks = int(c->plan_chunks.size());
@@ -1269,8 +1314,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             GgArgs ga{units, 0, c->tc_n_units, c->tc_wrow, c->tc_partial, c->rows_cap, m.hidden, m.inter, c->ws_status, c->wait_limit_ns,
                       nullptr, 0, c->tc_ready, c->tc_act, c->tc_ready + 1, clock_slot};
             if (m.dtype == SPM_DTYPE_Q4)
-                CU(c, launch_k(ffn_grouped_q4_kernel, dim3(c->num_sms), dim3(kQgThreads), ffn_grouped_q4_smem(), c->compute, true,
-                               c->qmapn, c->qmapsc, c->xmaps, ga));
+                CU(c, launch_grouped_q4(c, nb, c->num_sms, ga));
             else
                 CU(c, launch_k(ffn_grouped_kernel, dim3(c->num_sms), dim3(kGgThreads), ffn_grouped_smem(), c->compute, true, c->wmap, c->xmaps, ga));
             CU(c, launch_k(gg_combine_kernel, gg_combine_grid(m.hidden, nb), gg_combine_block(K), 0, c->compute, true,

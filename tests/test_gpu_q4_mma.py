@@ -1,4 +1,5 @@
-"""4-bit experts through mma.sync operands: the one-token kernel at the edges of its tiles against 64-bit sums."""
+"""4-bit experts through mma.sync operands: the one-token kernel at the edges of its tiles against 64-bit sums, the batched kernel at
+the edges of its runs of tokens against the one-token kernel."""
 import numpy as np
 import pytest
 import torch
@@ -63,4 +64,37 @@ def test_infinite_operands_reach_the_result():
     want = exact(cfg, x, ids, w)                # finite in 64 bits, beyond fp32
     big = want.abs() > 1e39
     assert big.any() and not got[big].isfinite().any()
+    m.close()
+
+
+# tokens of an expert: runs of eight (every expert in every token), one short and one over; few and many tasks a CTA; every split of the columns
+BATCHED = {
+    "one_run": (2048, 128, 3, 3, 8), "run_and_one": (2048, 256, 3, 3, 9), "run_short": (1792, 384, 2, 2, 15), "eight_runs": (1536, 128, 2, 2, 64),
+    "narrow": (512, 2048, 12, 2, 3), "wide_spread": (1280, 768, 60, 6, 24), "many_tasks": (1024, 1152, 128, 8, 5), "three_segments": (768, 768, 9, 3, 4),
+    "one_segment": (256, 256, 2, 1, 2),
+}
+
+
+@pytest.mark.parametrize("name", list(BATCHED))
+def test_batched(name):
+    """bf16 activations against the one-token kernel's fp32 ones, on either side of the line between the two batched kernels: both operands
+    that are rounded carry 2^-9, over all terms some 3e-3 of a row. A row keeps its bits in another place of the batch."""
+    hidden, inter, n, k, nb = BATCHED[name]
+    cfg = make(hidden, inter, n, k, batch=nb)
+    m = build(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    for scale in (1.0, 2e4):
+        x = torch.randn(nb, hidden, generator=gen, device="cuda") * scale
+        torch.cuda.synchronize()
+        _, ids, w, _ = m.router_topk(0, torch.randn(nb, hidden, generator=gen, device="cuda"))
+        got, turned, rows = torch.zeros_like(x), torch.zeros_like(x), torch.zeros_like(x)
+        x2, w2 = x.roll(1, 0), w.roll(1, 0)
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x, ids, w, got)
+        m.moe_ffn(0, x2, np.roll(ids, 1, 0), w2, turned)
+        for t in range(nb):
+            m.moe_ffn(0, x[t:t + 1], ids[t:t + 1], w[t:t + 1].contiguous(), rows[t:t + 1])
+        m.synchronize()
+        assert torch.equal(turned.roll(-1, 0), got)
+        assert ((got - rows).norm(dim=1) <= 1e-2 * rows.norm(dim=1)).all()
     m.close()
