@@ -551,6 +551,15 @@ cudaError_t launch_grouped_q4(const spm_ctx* c, int nb, int grid, const GgArgs& 
     return launch_k(ffn_grouped_q4_kernel, dim3(grid), dim3(kQgThreads), ffn_grouped_q4_smem(), c->compute, true, c->qmapn, c->qmapsc, c->xmaps, a);
 }
 
+// Whether a pointer names this device's own memory
+bool device_memory(const void* p) {
+    cudaPointerAttributes pa{};
+    int dev = -1;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&pa, p) == cudaSuccess) return pa.type == cudaMemoryTypeDevice && pa.device == dev;
+    cudaGetLastError();
+    return false;
+}
+
 // Where a routing launch leaves its results besides the workspace: by default the context's
 // mailbox, which the host polls; a host-free step names a trace mailbox, the device-side slot
 // map and the slot-code row of its layer, and lets the kernel start ahead of its predecessor's end.
@@ -565,7 +574,7 @@ struct RouterRoute {
 };
 
 int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int nb, float* x_norm,
-                  float* logits_out, bool do_router, bool do_adapter, const RouterRoute* route = nullptr, bool publish_seq = true) {
+                  float* logits_out, bool do_router, bool do_adapter, const RouterRoute* route = nullptr, bool publish_seq = true, float* w_out = nullptr) {
     const spm_model_cfg& m = c->cfg;
     if (do_adapter && !aligned16(c->buf.adapter_a)) return fail(c, SPM_ERR_INVALID_ARG, "adapter_a must be 16-byte aligned");
     RouterArgs a{};
@@ -583,7 +592,7 @@ int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int 
     a.logits_out = logits_out;
     a.pihat = c->ws_pihat;
     a.ids = c->ws_ids;
-    a.w = c->ws_w;
+    a.w = w_out ? w_out : c->ws_w;
     a.scores = c->ws_scores;
     a.order = c->ws_order;
     a.counters = c->ws_counters;
@@ -1426,11 +1435,7 @@ int enqueue_resident_step(spm_ctx* c, const float* h_in, float* h_out, int slot,
     predict = predict && m.n_layers > 1;
     if (predict && !aligned16(c->buf.adapter_a)) return fail(c, SPM_ERR_INVALID_ARG, "adapter_a must be 16-byte aligned");
     // the kernel reads the rows where they are if they are this device's memory; anything else that a copy takes is copied
-    cudaPointerAttributes pa{};
-    int dev = -1;
-    if (h_in != h_out && !(aligned16(h_in) && cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&pa, h_in) == cudaSuccess &&
-                           pa.type == cudaMemoryTypeDevice && pa.device == dev)) {
-        cudaGetLastError();
+    if (h_in != h_out && !(aligned16(h_in) && device_memory(h_in))) {
         CU(c, cudaMemcpyAsync(h_out, h_in, size_t(m.hidden) * 4, cudaMemcpyDeviceToDevice, c->compute));
         h_in = h_out;
     }
@@ -1769,8 +1774,12 @@ int spm_router_topk(spm_ctx* c, int layer, const float* h, int nb, float* x_norm
     if (int rc = flush_trace(c)) return rc;
     if (!h || !x_norm || !ids || !w) return fail(c, SPM_ERR_INVALID_ARG, "null argument");
     if (!aligned16(h) || !aligned16(x_norm)) return fail(c, SPM_ERR_INVALID_ARG, "h and x_norm must be 16-byte aligned");
-    if (int rc = launch_router(c, layer, h, nullptr, nb, x_norm, logits, true, false)) return rc;
-    CU(c, cudaMemcpyAsync(w, c->ws_w, size_t(nb) * c->cfg.top_k * 4, cudaMemcpyDeviceToDevice, c->compute));
+    // The kernel leaves the weights where they are wanted (a copy behind it cost its launch, and the expert kernel its early start); anything
+    // but this device's memory is copied to.
+    const bool direct = device_memory(w);
+    const RouterRoute route{c->mb_dev, nullptr, nullptr, true, nullptr, 0, nullptr};
+    if (int rc = launch_router(c, layer, h, nullptr, nb, x_norm, logits, true, false, &route, true, direct ? w : nullptr)) return rc;
+    if (!direct) CU(c, cudaMemcpyAsync(w, c->ws_w, size_t(nb) * c->cfg.top_k * 4, cudaMemcpyDeviceToDevice, c->compute));
     if (int rc = wait_mailbox(c)) return rc;
     for (int i = 0; i < nb * c->cfg.top_k; ++i) ids[i] = c->mb_host->ids[i] & 0xffff;
     return SPM_OK;
@@ -1781,7 +1790,8 @@ int spm_adapter_predict(spm_ctx* c, int layer, const float* x_norm, int nb, floa
     if (int rc = flush_trace(c)) return rc;
     if (layer > c->cfg.n_layers - 2) return fail(c, SPM_ERR_INVALID_ARG, "layer %d has no adapter (L-1 adapters)", layer);
     if (!x_norm || !scores || !order) return fail(c, SPM_ERR_INVALID_ARG, "null argument");
-    if (int rc = launch_router(c, layer, nullptr, x_norm, nb, nullptr, nullptr, false, true)) return rc;
+    const RouterRoute route{c->mb_dev, nullptr, nullptr, true, nullptr, 0, nullptr};
+    if (int rc = launch_router(c, layer, nullptr, x_norm, nb, nullptr, nullptr, false, true, &route)) return rc;
     if (int rc = wait_mailbox(c)) return rc;
     memcpy(scores, c->mb_host->scores, size_t(c->cfg.n_experts) * 4);
     for (int i = 0; i < c->cfg.n_experts; ++i) order[i] = c->mb_host->order[i] & 0xffff;
