@@ -149,6 +149,9 @@ def load() -> C.CDLL:
     return _lib
 
 
+_NO_BYTES = C.c_char * 0
+
+
 def _ptr(x):
     """Raw address of a torch tensor, numpy array, int or None."""
     if x is None:
@@ -157,7 +160,8 @@ def _ptr(x):
         return x
     if isinstance(x, np.ndarray):
         assert x.flags["C_CONTIGUOUS"]
-        return x.ctypes.data
+        # (x.ctypes builds an object: 1.0 us against 0.3, seven times a layer in the stand-alone calls)
+        return C.addressof(_NO_BYTES.from_buffer(x)) if x.flags.writeable else x.ctypes.data
     assert x.is_contiguous()
     return x.data_ptr()
 
