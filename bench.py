@@ -174,7 +174,7 @@ def config_block(cfg, args):
 
 def ffn_kernel_name(cfg):
     if cfg.batch > 1 and cfg.n_shared == 0 and cfg.dtype in ("bf16", "q4"):
-        return "ffn_grouped_q4_kernel" if cfg.dtype == "q4" else "ffn_grouped_kernel"
+        return "ffn_grouped_q4_mma_kernel" if cfg.dtype == "q4" else "ffn_grouped_kernel"
     if cfg.dtype == "q4":
         return "ffn_gemv_q4_kernel"
     return "ffn_gemv_kernel"

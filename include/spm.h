@@ -287,14 +287,15 @@ int spm_set_device_wait(spm_ctx* ctx, int on);
  * slot table's bookkeeping (hits, LRU ticks, recall statistics, event log) is replayed in order,
  * at the latest when a call reads or changes that state. Outputs, events and statistics are the
  * same as with the option off; per-layer event timings are not taken in such steps (the in-kernel
- * window still is). On the batched tensor-core path the wave plan (token rows sorted by expert,
+ * window still is). A step of one sequence in the default geometry is one cooperative kernel over all SMs (not with timing or an
+ * attention stand-in set, nor for fp32 models of one or two layers). On the batched tensor-core path the wave plan (token rows sorted by expert,
  * work units, combine map) is then built by a kernel instead of the host.
  * spm_cache_reset() ends the state; it is re-entered once the pools are full again. */
 int spm_set_host_free(spm_ctx* ctx, int on);
 /* Replay host-free steps from CUDA graphs (default on): the launches of such a step are the same
  * every time for a given trace slot, batch size, output buffer, launch geometry and wait limit, so each
  * combination is captured once (after one step enqueued launch by launch) and replayed with a
- * single submission. Off, or with timing / an attention stand-in set, every kernel is launched
+ * single submission. (A step that is one kernel needs none.) Off, or with timing / an attention stand-in set, every kernel is launched
  * individually. Results are identical. */
 int spm_set_graph_replay(spm_ctx* ctx, int on);
 /* Stand-in for the attention block the synthetic configurations omit: before each layer's router a
