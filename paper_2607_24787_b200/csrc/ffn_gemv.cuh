@@ -8,7 +8,7 @@
 // back to back, so one contiguous 3*D-element read yields everything intermediate unit j
 // contributes: its two dot products and its rank-1 update of y.
 //
-// Work decomposition: the (expert, j) rows of a token are split evenly over gridDim.x CTAs; in
+// Work decomposition: the (expert, j) rows of a token are split evenly over gridDim.x CTAs (GemvShare); in
 // a CTA each warp owns a private ring of row buffers in shared memory that lane 0 keeps full
 // with 1-D bulk async copies (cp.async.bulk + mbarrier byte counting, no multicast), so about
 // 170-220 KB per SM are in flight without costing registers. The host picks the number of warps
@@ -59,6 +59,7 @@ struct FfnArgs {
     short watch[SPM_MAX_TOPK];      //   (the counter of the slot that leads the batch of copies entry k's slot was filled by)
     unsigned long long blob_bytes;
     int I, K, n_slots, n_shared;
+    int n_tail;                     // how many of a token's last entries are shared experts (fp32 and bf16 weights: see GemvShare)
     unsigned long long wait_limit_ns;   // every wait in the kernel gives up after this long (0: the 2 s default)
     int early;                      // 1: start the first weight copies before the launch dependency resolves (needs slot numbers in `code`)
     unsigned char count[MAXNB];                     // expert entries of token t in this launch
@@ -123,6 +124,26 @@ __device__ __forceinline__ void unpack16p(const uint4& v, uint64_t (&f)[4]) {   
 __device__ __forceinline__ void unpack16p(const uint4& v, uint64_t (&f)[2]) {   // fp32: 4 values
     f[0] = pack2u(v.x, v.y); f[1] = pack2u(v.z, v.w);
 }
+
+// A CTA's rows: its even share of the shared experts' (expert, j) rows, then its even share of the routed ones'. Every CTA then begins with rows
+// that are known ahead of the routing. Row i of the share is row j of entry ent.
+struct GemvShare {
+    int I, entries, tail, r_begin, s_begin, n_shared_rows, span;
+    __device__ __forceinline__ GemvShare(int inter, int n_entries, int n_tail, int c, int G) : I(inter), entries(n_entries), tail(n_tail) {
+        const int R = (entries - tail) * I, S = tail * I, q = R / G, rem = R - q * G, qs = S / G, rems = S - qs * G;
+        r_begin = q * c + min(c, rem);
+        const int first = G - rems;                     // (the remainders go to opposite ends)
+        s_begin = qs * c + max(c - first, 0);
+        n_shared_rows = qs + (c >= first ? 1 : 0);
+        span = n_shared_rows + q + (c < rem ? 1 : 0);
+    }
+    __device__ __forceinline__ void row(int i, int& ent, int& j) const {
+        const bool sh = i < n_shared_rows;
+        const int r = sh ? s_begin + i : r_begin + i - n_shared_rows, e = r / I;
+        j = r - e * I;
+        ent = sh ? entries - tail + e : e;
+    }
+};
 
 // One row of a blob against this warp's token: ya += silu(gate . x) * (up . x) * wk * down. `b32`: shared-memory address of the row,
 // this lane's first 16 bytes.
@@ -211,12 +232,8 @@ ffn_gemv_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int depth) {
     const int tok = blockIdx.y;
     const int G = gridDim.x, c = blockIdx.x;
     const int I = a.I;
-    const int R = a.entries(tok) * I;
-    // even split: CTA c takes q rows, the first R % G CTAs one more (one 32-bit division)
-    const int q_rows = R / G, rem_rows = R - q_rows * G;
-    const int r_begin = q_rows * c + min(c, rem_rows);
-    const int r_end = r_begin + q_rows + (c < rem_rows ? 1 : 0);
-    const int span = r_end - r_begin - wi;
+    const GemvShare share(I, a.entries(tok), a.n_tail, c, G);
+    const int span = share.span - wi;
     const int my_n = span > 0 ? (span + nw - 1) / nw : 0;
 
     unsigned char* ring = smem + size_t(wi) * depth * ROWB;
@@ -258,9 +275,8 @@ ffn_gemv_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int depth) {
     };
 
     auto issue = [&](int i) {
-        const int r = r_begin + wi + i * nw;
-        const int ent = r / I;
-        const int j = r - ent * I;
+        int ent, j;
+        share.row(wi + i * nw, ent, j);
         if (ent != src_ent) { src_ent = ent; src_base = resolve(ent); }
         const unsigned char* base = src_base;
         if (!base) return false;
@@ -318,8 +334,8 @@ ffn_gemv_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int depth) {
                 break;
             }
             done = i + 1;
-            const int r = r_begin + wi + i * nw;
-            const int ent = r / I;
+            int ent, j;
+            share.row(wi + i * nw, ent, j);
             if (ent != cur_ent) {
                 cur_ent = ent;
                 const int kk = a.kidx_of(tok, ent);

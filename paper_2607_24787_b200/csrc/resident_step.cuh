@@ -15,7 +15,7 @@
 // One buffer per exchange is enough: a CTA overwrites a word one layer later, when it holds data that every reader of
 // the old word contributed to after reading it.
 //
-// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 17.2 (21): the FFN 11.5 - 13 and 9 - 11 with the slowest SM 2 us
+// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 16.2 (21): the FFN 11.5 - 13 and 8 - 10 with the slowest SM 2 us
 // behind the mean, and a chain of latencies of 6 (partial rows 1.4, hidden row 1, norm and dot products 1.5, logits 1.1, Top-K to the
 // first copies 1.3).
 //
@@ -161,15 +161,17 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
     short* smap = reinterpret_cast<short*>(s_code + SPM_MAX_TOPK);
 
     // even split of the (expert, j) rows over the CTAs, then over the warps, as in ffn_gemv_kernel
-    const int entries = a.K + a.n_shared, R = entries * I;
-    const int q_rows = R / G, rem_rows = R - q_rows * G;
-    const int r_begin = q_rows * c + min(c, rem_rows);
-    const int span = q_rows + (c < rem_rows ? 1 : 0);
+    const GemvShare share(I, a.K + a.n_shared, Q4 ? 0 : a.n_shared, c, G);
+    const int r_begin = share.r_begin, span = share.span;
     const int my_n = wi < nw && span > wi ? (span - wi + nw - 1) / nw : 0;
     const uint32_t bar0 = smem_u32(bars + (wi < nw ? wi : 0) * depth), ring0 = smem_u32(ring);
-    // the warp's first rows of a layer are looked up by a lane each, which knows where they are but for the slot
-    const int n_first = min(depth, my_n), first_r = r_begin + wi + min(lane, max(n_first - 1, 0)) * nw;
-    const int first_ent = first_r / I, first_j = first_r - first_ent * I;
+    // The warp's first rows of a layer are looked up by a lane each, which knows where they are but for the slot. The first n_early, of shared
+    // experts, are asked for ahead of the routing, while the ring has nothing else to do (DeepSeek shape, two shared experts of eight:
+    // 17.9 -> 16.2 us a layer).
+    const int n_first = min(depth, my_n);
+    const int n_early = Q4 || a.xs_in_ring ? 0 : min(n_first, share.n_shared_rows > wi ? (share.n_shared_rows - wi + nw - 1) / nw : 0);
+    int first_ent, first_j;
+    share.row(wi + min(lane, max(n_first - 1, 0)) * nw, first_ent, first_j);
     const unsigned long long limit = a.wait_limit_ns ? a.wait_limit_ns : kWaitLimitNs;
     Q4Ring<kStepWarps> tiles(smem, D, Q4 ? depth : 0, tid);         // (4-bit experts)
     if (!Q4 && wi < nw && lane == 0) {
@@ -209,6 +211,37 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
 
     int st_in = 0, st_out = 0;          // ring stages of the next copy and the next row, and the phase of the latter
     uint32_t ph = 0;
+    // The row at `src` into the next stage of the warp's ring, by one elected lane with operands that are the same in the warp (lanes that
+    // ask side by side are taken one by one; this took the DeepSeek shape from 19.3 to 17.8 us a layer). A bad slot's row is whatever
+    // was there: the status word says so.
+    auto ask = [&](const unsigned char* src) {
+        if (elect_one()) {
+            if (src) {
+                mbar_arrive_expect_tx(bar0 + 8u * st_in, ROWB);
+                bulk_g2s(ring0 + uint32_t(st_in) * ROWB, src, ROWB, bar0 + 8u * st_in, policy_evict_first());
+            } else {
+                mbar_arrive(bar0 + 8u * st_in);
+            }
+        }
+        __syncwarp();
+        st_in = st_in + 1 == depth ? 0 : st_in + 1;
+    };
+    auto ask_early = [&](int l) {
+        for (int i = 0; i < n_early; ++i) {
+            const int e = __shfl_sync(0xffffffffu, first_ent, i) - a.K, j = __shfl_sync(0xffffffffu, first_j, i);
+            ask(a.shared + (size_t(l) * a.n_shared + e) * a.blob_bytes + size_t(j) * ROWB);
+        }
+    };
+    __syncwarp();
+    ask_early(0);
+    // Leaves no copy of the `asked` last ones in flight
+    auto drain = [&](int asked) {
+        for (; asked > 0; --asked) {
+            if (!mbar_wait_bounded(bar0 + 8u * st_out, ph, kWaitLimitNs)) break;
+            st_out = st_out + 1 == depth ? 0 : st_out + 1;
+            if (st_out == 0) ph ^= 1;
+        }
+    };
     for (int l = 0; l < a.L; ++l) {
         const uint32_t tag = a.tag0 + uint32_t(l);
         const int rows = rows_of(l);
@@ -271,7 +304,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
         }
         if (tid < n) smap[tid] = slot0;
         for (int e = tid + kStepThreads; e < n; e += kStepThreads) smap[e] = a.slot_map[size_t(l) * n + e];
-        if (__syncthreads_or(dead)) return;
+        if (__syncthreads_or(dead)) { drain(n_early); return; }
 
         // ---- logits: one warp per router or adapter row ----
         for (int row = my_row; row < rows; row += G * kStepWarps) {
@@ -325,7 +358,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
             reinterpret_cast<int*>(zs)[i] = order_key(z);
         }
         if (a.xs_in_ring) fence_proxy_async();      // the row was written and read where copies are about to land
-        if (__syncthreads_or(dead)) return;
+        if (__syncthreads_or(dead)) { drain(n_early); return; }
 
         // ---- Top-K, two threads an expert; then the first weight copies go out, and the routing weights are computed behind them ----
         const int half_n = (n / 2) & ~3;
@@ -352,28 +385,13 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
             const unsigned char* base = blob(ent);
             return base ? base + size_t(r_begin + row - ent * I) * ROWB : nullptr;
         };
-        // The row at `src` into the next stage of the warp's ring, by one elected lane with operands that are the same in the warp (lanes that
-        // ask side by side are taken one by one; this took the DeepSeek shape from 19.3 to 17.8 us a layer). A bad slot's row is whatever
-        // was there: the status word says so.
-        auto ask = [&](const unsigned char* src) {
-            if (elect_one()) {
-                if (src) {
-                    mbar_arrive_expect_tx(bar0 + 8u * st_in, ROWB);
-                    bulk_g2s(ring0 + uint32_t(st_in) * ROWB, src, ROWB, bar0 + 8u * st_in, policy_evict_first());
-                } else {
-                    mbar_arrive(bar0 + 8u * st_in);
-                }
-            }
-            __syncwarp();
-            st_in = st_in + 1 == depth ? 0 : st_in + 1;
-        };
         int n_in = n_first;                 // rows that the warp has asked for
         if constexpr (Q4) {
             tiles.fill(0, min(depth, (span + kQ4Rows - 1) / kQ4Rows), wi, lane, ROWB, row_at);
         } else {       // (the lanes look the rows up side by side)
-            const unsigned char* base = lane < n_first ? blob(first_ent) : nullptr;
+            const unsigned char* base = lane >= n_early && lane < n_first ? blob(first_ent) : nullptr;
             const unsigned long long at = base ? reinterpret_cast<unsigned long long>(base + size_t(first_j) * ROWB) : 0ull;
-            for (int i = 0; i < n_first; ++i) ask(reinterpret_cast<const unsigned char*>(__shfl_sync(0xffffffffu, at, i)));
+            for (int i = n_early; i < n_first; ++i) ask(reinterpret_cast<const unsigned char*>(__shfl_sync(0xffffffffu, at, i)));
         }
         // Routing weights: the router tail's softmax over all experts, by every warp for itself. The four butterflies are the sums
         // of that tail's four warps, added in their order.
@@ -434,23 +452,20 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
                     dead = 1;
                     break;
                 }
-                gemv_row<WT, NSEG>(ring0 + uint32_t(st_out) * ROWB + lane * 16, xr, __shfl_sync(0xffffffffu, wk, (r_begin + wi + done * nw) / I), ya);
+                int ent, j;
+                share.row(wi + done * nw, ent, j);
+                gemv_row<WT, NSEG>(ring0 + uint32_t(st_out) * ROWB + lane * 16, xr, __shfl_sync(0xffffffffu, wk, ent), ya);
                 __syncwarp();
                 st_out = st_out + 1 == depth ? 0 : st_out + 1;
                 if (st_out == 0) ph ^= 1;
                 if (n_in < my_n) {
-                    const int r = r_begin + wi + n_in * nw, e = r / I;
-                    const unsigned char* base = blob(e);
-                    ask(base ? base + size_t(r - e * I) * ROWB : nullptr);
+                    share.row(wi + n_in * nw, ent, j);
+                    const unsigned char* base = blob(ent);
+                    ask(base ? base + size_t(j) * ROWB : nullptr);
                     ++n_in;
                 }
             }
-            if (dead)           // leave no copy in flight
-                for (; done < n_in; ++done) {
-                    if (!mbar_wait_bounded(bar0 + 8u * st_out, ph, kWaitLimitNs)) break;
-                    st_out = st_out + 1 == depth ? 0 : st_out + 1;
-                    if (st_out == 0) ph ^= 1;
-                }
+            if (dead) drain(n_in - done);
             if (wi < nw && !dead) gemv_stage_y<NSEG>(ring, lane, ya);
             if (__syncthreads_or(dead)) return;
 
@@ -464,6 +479,10 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
                     send(s * 32 * VEC + ln * VEC + 4 * h, y);
                 }
                 fence_proxy_async();            // the ring held partial sums: ordered before the next layer's copies
+                if (a.n_shared > 0 && l + 1 < a.L) {
+                    __syncthreads();
+                    ask_early(l + 1);
+                }
             }
         }
         if (l + 1 < a.L) preload(l + 1);

@@ -1024,7 +1024,7 @@ int run_ffn(spm_ctx* c, int layer, const float* x_norm, const int32_t* ids, cons
             a.wait_limit_ns = c->wait_limit_ns;
             a.early = 1;               // slot numbers are launch arguments: the first weight copies need not wait for the preceding kernel
             a.blob_bytes = c->blob;
-            a.I = m.inter; a.K = K; a.n_slots = c->S; a.n_shared = m.n_shared;
+            a.I = m.inter; a.K = K; a.n_slots = c->S; a.n_shared = m.n_shared; a.n_tail = first ? m.n_shared : 0;
             for (int tk = 0; tk < nb; ++tk) {
                 int cnt = 0;
                 for (int k = 0; k < K; ++k) {
@@ -1307,7 +1307,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             a.wait_limit_ns = c->wait_limit_ns;
             a.dev_code = codes;
             a.blob_bytes = c->blob;
-            a.I = m.inter; a.K = K; a.n_slots = c->S; a.n_shared = m.n_shared;
+            a.I = m.inter; a.K = K; a.n_slots = c->S; a.n_shared = m.n_shared; a.n_tail = m.n_shared;
             for (int tk = 0; tk < nb; ++tk) a.count[tk] = (unsigned char)(K + m.n_shared);   // launch shape only
         };
         if (use_tc) {
@@ -2262,7 +2262,7 @@ int spm_time_ffn_kernel(spm_ctx* c, int first_layer, const float* x_norm, const 
         a.wait_limit_ns = c->wait_limit_ns;
         a.early = pdl ? 1 : 0;
         a.blob_bytes = c->blob;
-        a.I = m.inter; a.K = K; a.n_slots = c->S; a.n_shared = m.n_shared;
+        a.I = m.inter; a.K = K; a.n_slots = c->S; a.n_shared = m.n_shared; a.n_tail = m.n_shared;
         int cnt = 0;
         for (int k = 0; k < K; ++k) {
             a.code[cnt] = short(tb.slot_of(layer, ids[size_t(i) * K + k]));
