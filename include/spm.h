@@ -223,7 +223,8 @@ int spm_prefetch_async(spm_ctx* ctx, int target_layer, const int32_t* ids, int c
  * were, and at batch 1 a layer is one launch whenever slots >= top_k, so in both cases the result
  * does not depend on the cache state, bit for bit. A batch with fp32 activations (spm_set_batched_path) is summed wave by
  * wave; where experts are streamed once for several tokens, the order of a token's sums also follows how the call's other tokens
- * are routed. The same call on the same cache state gives the same bits. */
+ * are routed. The same call on the same cache state gives the same bits. A batch of 4-bit experts on the tensor-core path takes one of
+ * two kernels by its size: both round the same quantities to bf16 and differ in the order of their fp32 sums (1e-4 of a layer's result). */
 int spm_moe_ffn(spm_ctx* ctx, int layer, const float* x_norm, const int32_t* ids,
                 const float* w, int nb, float* h_inout);
 

@@ -5,22 +5,21 @@
 // the Qwen3 shape give an expert about four. There the tensor cores idle either way, and what the tcgen05 kernel spends its time on
 // is the way of an operand: unpack, store to tensor or shared memory, fence, hand-shake, 1050 cycles for an item that HBM
 // delivers in 340. An mma.sync operand is where the unpacking leaves it, in the registers of the lane that needs it. A layer of a whole
-// host-free step of that shape: 198 -> 142 us (HBM time of its experts: 49). What bounds it now: instruction issue and dependent-issue
-// latency, 107,000 instructions a scheduler at 0.5 a cycle, 330 of a warp's 620 a tile for what is done once a tile.
+// host-free step of that shape: 197 -> 146 us (HBM time of its experts: 49; 142 with exact weights and the scale on the activations,
+// which rounds elsewhere than the tcgen05 kernel: outputs of 64 sequences then moved by 1e-2 where a near-tied Top-K choice tipped).
+// What bounds it now: instruction issue and dependent-issue latency, half of it for what is done once a tile.
 //
 // Work. A task is 128 intermediate rows of an expert (GgUnit) for up to kMqTokens of its tokens; CTA b runs the tasks b, b + grid, ...
 // of all experts in order (a hot expert's runs of tokens go to different CTAs). A task goes through its rows in tiles of 16; the
 // warps split the columns in groups of 32 (one scale), GB consecutive groups a warp.
-//   Phase 1 (M = 16 gate rows, then 16 up rows; N = tokens; K = 32 columns, two MMAs): the group's scale goes onto the fp32 sum. The
-// warps' sums meet in shared memory.
-//   Phase 2 (M = 16 hidden columns, N = tokens, K = 16 rows): the warp's own columns; the scale goes onto the activation, rounded
-// to bf16 once. y stays in the accumulators for the whole task.
+//   Phase 1 (M = 16 gate rows, then 16 up rows; N = tokens; K = 32 columns, two MMAs). The warps' sums meet in shared memory.
+//   Phase 2 (M = 16 hidden columns, N = tokens, K = 16 rows): the warp's own columns. y stays in the accumulators for the whole task.
 // Phase 2 is one tile behind phase 1, so that one CTA barrier a tile is enough. The rows of a tile come as two bulk copies each, gate /
 // up and W_down, into rings of their own.
 //
 // A token's result depends on its own row and the expert only (a column of the MMAs), so outputs do not depend on waves, batch
-// mates or the CTA. Rounding: activations to bf16, act * scale to bf16, all else exact or fp32 (the tcgen05 kernel also rounds
-// the scales and the products of scale and weight).
+// mates or the CTA. What is rounded is what the tcgen05 kernel rounds: scales, products of scale and q - 8, token rows and activations,
+// to bf16; sums are fp32. The two kernels differ in the order of the sums alone.
 #pragma once
 
 #include <type_traits>
@@ -34,6 +33,7 @@ namespace spm {
 constexpr int kMqTokens = 8;                  // tokens of a task: N of the MMAs
 constexpr int kMqTiles = kGgTileRows / kQ4Rows;
 constexpr int kMqRed = 264;                   // pitch of a warp's phase-1 sums: 256 floats, the next warp's eight banks on
+constexpr int kMqAct = 24;                     // pitch of a token's activations (bf16): 12 banks, so that eight tokens' pairs of rows have banks of their own
 constexpr int kMqMaxTasks = 512;              // tasks of a CTA
 
 struct MqArgs {
@@ -50,7 +50,7 @@ inline int mq_max_tasks(int nb, int K, int n, int n_jt, int grid) {
     return (runs * n_jt + grid - 1) / grid;
 }
 inline size_t mq_rest_bytes(int n) {
-    return 2 * kQ4MaxStages * 8 + 2 * size_t(kQ4MaxWarps) * kMqRed * 4 + 2 * kMqTokens * kQ4Rows * 4 + 2 * kMqTokens * 4 + 16 +
+    return 2 * kQ4MaxStages * 8 + 2 * size_t(kQ4MaxWarps) * kMqRed * 4 + 2 * kMqTokens * kMqAct * 2 + 2 * kMqTokens * 4 + 16 +
            size_t(kMqMaxTasks) * sizeof(MqTask) + size_t(n + 1) * 4;
 }
 inline int mq_stages(int D, int n, size_t* smem) {
@@ -59,6 +59,85 @@ inline int mq_stages(int D, int n, size_t* smem) {
     if (s > size_t(kQ4MaxStages)) s = kQ4MaxStages;
     *smem = s * stage + mq_rest_bytes(n);
     return int(s);
+}
+
+// Whether any of a warp's scales is infinite or a NaN, from sums of scale times zero
+__device__ __forceinline__ bool mq_nonfinite(__nv_bfloat162 zeros) { return __any_sync(0xffffffffu, (bits2(zeros) & 0x7fff7fffu) != 0); }
+
+// Phase 1 of a tile: gate and up of its rows (2^-22 of them) over one warp's groups, for the MMA's eight token columns.
+// rows: the tile's first row, rows of `pitch` bytes that hold gate, then up; x: the B operand of each group, nibble pairs 0..3.
+template <int GB>
+__device__ __forceinline__ void mq_phase1(uint32_t rows, uint32_t pitch, int D, int grp0, int lane, const uint32_t (&x)[GB][4], float (&gate)[4], float (&up)[4]) {
+    const uint32_t part = q4_part_bytes(D);
+    // matrices: gate rows 0-7, 8-15, up rows 0-7, 8-15, 16 bytes (a group) each
+    const uint32_t at = rows + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * pitch + uint32_t(lane >> 4) * part + uint32_t(grp0) * 16;
+    const uint32_t sc = rows + uint32_t(lane >> 2) * pitch + uint32_t(D / 2 + grp0 * 2);
+    constexpr int GP = (GB + 1) / 2;
+    __nv_bfloat162 s[4][GP], zeros = bf2(0u);            // gate rows g and g + 8, up rows g and g + 8: pairs of groups
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        uint32_t v[GP];
+        q4_scale_pairs<GB>(sc + uint32_t(r & 1) * 8 * pitch + uint32_t(r >> 1) * part, v);
+#pragma unroll
+        for (int i = 0; i < GP; ++i) { s[r][i] = q4_bf16_scales(v[i]); zeros = __hfma2(s[r][i], bf2(0u), zeros); }
+    }
+    auto run = [&](auto plain) {
+#pragma unroll
+        for (int i = 0; i < GB; ++i) {
+            const uint4 w4 = ldsm4(at + i * 16);
+            const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+            Nib4 a[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const __nv_bfloat162 one = (i & 1) ? __high2bfloat162(s[r][i / 2]) : __low2bfloat162(s[r][i / 2]);
+                a[r] = q4_weights<decltype(plain)::value>(w[r], q4_scaled(one), one);
+            }
+            mma_k16(gate, a[0].p[0], a[1].p[0], a[0].p[1], a[1].p[1], x[i][0], x[i][1]);
+            mma_k16(up, a[2].p[0], a[3].p[0], a[2].p[1], a[3].p[1], x[i][0], x[i][1]);
+            mma_k16(gate, a[0].p[2], a[1].p[2], a[0].p[3], a[1].p[3], x[i][2], x[i][3]);
+            mma_k16(up, a[2].p[2], a[3].p[2], a[2].p[3], a[3].p[3], x[i][2], x[i][3]);
+        }
+    };
+    if (mq_nonfinite(zeros)) run(std::true_type{});
+    else run(std::false_type{});
+}
+// Phase 2: y += W_down^T act over the tile's 16 rows (2^-22 of it). b0, b1: the activations of rows 2t, 2t + 1 and 2t + 8, 2t + 9. A lane
+// gets the columns 4g .. 4g + 3 of each group: y[0][0..1], y[0][2..3], y[1][0..1], y[1][2..3] for tokens 2t, 2t + 1.
+template <int GB>
+__device__ __forceinline__ void mq_phase2(uint32_t rows, uint32_t pitch, int D, int grp0, int lane, uint32_t b0, uint32_t b1, float (&y)[GB][2][4]) {
+    const uint32_t at = rows + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * pitch + uint32_t(grp0) * 16;
+    const uint32_t sc = rows + uint32_t(2 * (lane & 3)) * pitch + uint32_t(D / 2 + grp0 * 2);
+    constexpr int GP = (GB + 1) / 2;
+    uint32_t v[4][GP];                       // rows 2t, 2t + 1, 2t + 8, 2t + 9
+    q4_scale_pairs<GB>(sc, v[0]);
+    q4_scale_pairs<GB>(sc + pitch, v[1]);
+    q4_scale_pairs<GB>(sc + 8 * pitch, v[2]);
+    q4_scale_pairs<GB>(sc + 9 * pitch, v[3]);
+    __nv_bfloat162 s[2][GB], zeros = bf2(0u);            // a group's scales of two rows
+#pragma unroll
+    for (int i = 0; i < GB; ++i)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            s[r][i] = q4_bf16_scales(__byte_perm(v[2 * r][i / 2], v[2 * r + 1][i / 2], (i & 1) ? 0x7632 : 0x5410));
+            zeros = __hfma2(s[r][i], bf2(0u), zeros);
+        }
+    auto run = [&](auto plain) {
+        constexpr bool kPlain = decltype(plain)::value;
+#pragma unroll
+        for (int i = 0; i < GB; i += 2) {
+            // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word
+            const uint4 w = ldsm4t(at + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
+            auto group = [&](int j, uint32_t lo, uint32_t hi) {
+                const Nib4 a = q4_weights<kPlain>(lo, q4_scaled(s[0][j]), s[0][j]), b = q4_weights<kPlain>(hi, q4_scaled(s[1][j]), s[1][j]);
+                mma_k16(y[j][0], a.p[0], a.p[1], b.p[0], b.p[1], b0, b1);
+                mma_k16(y[j][1], a.p[2], a.p[3], b.p[2], b.p[3], b0, b1);
+            };
+            group(i, w.x, w.y);
+            if (i + 1 < GB) group(i + 1 < GB ? i + 1 : i, w.z, w.w);
+        }
+    };
+    if (mq_nonfinite(zeros)) run(std::true_type{});
+    else run(std::false_type{});
 }
 
 template <int NSEG>
@@ -72,8 +151,8 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + dn_ring + uint32_t(n_stages) * kQ4Rows * DN);
     MqTask* tasks = reinterpret_cast<MqTask*>(bars + 2 * kQ4MaxStages);
     float* red = reinterpret_cast<float*>(tasks + kMqMaxTasks);               // [2][warps] phase-1 sums
-    float* actv = red + 2 * NW * kMqRed;                                      // [2][token][row]
-    float* s_w = actv + 2 * kMqTokens * kQ4Rows;                              // [2 tasks][token]
+    __nv_bfloat16* actv = reinterpret_cast<__nv_bfloat16*>(red + 2 * NW * kMqRed);      // [2][token][row]
+    float* s_w = reinterpret_cast<float*>(actv + 2 * kMqTokens * kMqAct);     // [2 tasks][token]
     int& s_abort = *reinterpret_cast<int*>(s_w + 2 * kMqTokens);
     int& s_gu = (&s_abort)[1];
     int& s_dn = (&s_abort)[2];
@@ -168,9 +247,7 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
     // ---- tiles: phase 1 of tile k, phase 2 of tile k - 1 ----
     const int grp0 = warp * GB;
     uint32_t x[GB][4];
-    float off[GB][2], down[2] = {0.f, 0.f};      // down: 2^133 over the scale of the tokens 2t and 2t + 1
     float y[GB][2][4];
-    Q4ActScale scale;
     auto load_x = [&](int task) {           // token rows, and the routing weights, of the task that phase 1 comes to
         const MqTask k = task < n_tasks ? tasks[task] : MqTask{0, 0, 0, 0};
         const bool on = g < (k.jt_n & 15);
@@ -181,30 +258,6 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
             x[i][0] = v.x; x[i][1] = v.y; x[i][2] = v.z; x[i][3] = v.w;
         }
         if (threadIdx.x < kMqTokens) s_w[(task & 1) * kMqTokens + threadIdx.x] = int(threadIdx.x) < (k.jt_n & 15) ? __ldcg(a.wrow + k.row + threadIdx.x) : 0.f;
-    };
-    auto scale_x = [&]() {                  // a token's columns of this warp by one power of two
-        uint32_t top = 0;
-#pragma unroll
-        for (int i = 0; i < GB; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) top = __vmaxu2(top, x[i][q] & 0x7fff7fffu);
-        top = max(top & 0xffffu, top >> 16);
-        top = max(top, __shfl_xor_sync(0xffffffffu, top, 1));
-        top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
-        const int e = q4_exponent(top << 16);
-        const float up = q4_up(e), dn = q4_down(e);
-        const __nv_bfloat162 even = __float2bfloat162_rn(up), odd = __float2bfloat162_rn(up * 0.0625f);
-#pragma unroll
-        for (int i = 0; i < GB; ++i) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const __nv_bfloat162 v = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&x[i][q]), (q & 1) ? odd : even);
-                x[i][q] = *reinterpret_cast<const uint32_t*>(&v);
-            }
-            q4_offset(x[i], off[i]);
-        }
-        down[0] = __shfl_sync(0xffffffffu, dn, 8 * t);
-        down[1] = __shfl_sync(0xffffffffu, dn, 8 * t + 4);
     };
     auto clear_y = [&]() {
 #pragma unroll
@@ -224,18 +277,14 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
         const bool p1 = k < n_tiles, p2 = k > 0;
         const int task1 = k / kMqTiles;
         if (p1) {
-            if (k % kMqTiles == 0) scale_x();
             if (!dead) dead = !__all_sync(0xffffffffu, mt_wait(gu_bar + 8 * st1, ph1, &s_abort, a.status, limit));
             const uint32_t rows = ring + uint32_t(st1) * kQ4Rows * GU;
             if (++st1 == n_stages) { st1 = 0; ph1 ^= 1; }
-            float ag[4], au[4];
-            q4_phase1<GB, false>(rows, GU, D, grp0, lane, x, off, ag, au, [](float (&acc)[4], const float (&c)[4], float s0, float s1) {
-                acc[0] = fmaf(s0, c[0], acc[0]); acc[1] = fmaf(s0, c[1], acc[1]);
-                acc[2] = fmaf(s1, c[2], acc[2]); acc[3] = fmaf(s1, c[3], acc[3]);
-            });
+            float ag[4] = {}, au[4] = {};
+            mq_phase1<GB>(rows, GU, D, grp0, lane, x, ag, au);
             float* r = red + ((k & 1) * NW + warp) * kMqRed + lane * 4;
-            *reinterpret_cast<float4*>(r) = make_float4(ag[0] * down[0], ag[1] * down[1], ag[2] * down[0], ag[3] * down[1]);
-            *reinterpret_cast<float4*>(r + 128) = make_float4(au[0] * down[0], au[1] * down[1], au[2] * down[0], au[3] * down[1]);
+            *reinterpret_cast<float4*>(r) = make_float4(ag[0], ag[1], ag[2], ag[3]);
+            *reinterpret_cast<float4*>(r + 128) = make_float4(au[0], au[1], au[2], au[3]);
             if (k % kMqTiles == kMqTiles - 1) load_x(task1 + 1);        // the next task's rows are on their way while this tile is finished
         }
         if (p2 && !dead) dead = !__all_sync(0xffffffffu, mt_wait(dn_bar + 8 * st2, ph2, &s_abort, a.status, limit));
@@ -257,46 +306,18 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
                 vu += __shfl_xor_sync(0xffffffffu, vu, 8);
                 vg += __shfl_xor_sync(0xffffffffu, vg, 16);
                 vu += __shfl_xor_sync(0xffffffffu, vu, 16);
+                vg *= kQ4Unscale;
+                vu *= kQ4Unscale;
                 const int row = (pair >> 4) + 8 * ((pair >> 1) & 1), tok = 2 * ((pair >> 2) & 3) + (pair & 1);
-                if (lane < 8) actv[((k & 1) * kMqTokens + tok) * kQ4Rows + row] = __fdividef(vg, 1.f + __expf(-vg)) * vu * s_w[(task1 & 1) * kMqTokens + tok];
+                if (lane < 8) actv[((k & 1) * kMqTokens + tok) * kMqAct + row] = __float2bfloat16_rn(__fdividef(vg, 1.f + __expf(-vg)) * vu * s_w[(task1 & 1) * kMqTokens + tok]);
             }
         }
         if (!p2) continue;
         {
-            const float* av = actv + (((k - 1) & 1) * kMqTokens + g) * kQ4Rows + 2 * t;
-            float2 a0 = *reinterpret_cast<const float2*>(av), a1 = *reinterpret_cast<const float2*>(av + 8);
-            scale.fit<GB>(fmaxf(fmaxf(fabsf(a0.x), fabsf(a0.y)), fmaxf(fabsf(a1.x), fabsf(a1.y))), y);
-            a0.x *= scale.up; a0.y *= scale.up; a1.x *= scale.up; a1.y *= scale.up;
-            const uint32_t rows = ring + dn_ring + uint32_t(st2) * kQ4Rows * DN;
+            const __nv_bfloat16* av = actv + (((k - 1) & 1) * kMqTokens + g) * kMqAct + 2 * t;
+            const uint32_t b0 = *reinterpret_cast<const uint32_t*>(av), b1 = *reinterpret_cast<const uint32_t*>(av + 8);
+            mq_phase2<GB>(ring + dn_ring + uint32_t(st2) * kQ4Rows * DN, DN, D, grp0, lane, b0, b1, y);
             if (++st2 == n_stages) { st2 = 0; ph2 ^= 1; }
-            const uint32_t at = rows + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * DN + uint32_t(grp0) * 16;
-            const uint32_t sc = rows + uint32_t(2 * t) * DN + uint32_t(D / 2 + grp0 * 2);
-            uint32_t b[GB][2];
-            {
-                float s0[GB], s1[GB], s2[GB], s3[GB];
-                q4_scales<GB>(sc, s0);
-                q4_scales<GB>(sc + DN, s1);
-                q4_scales<GB>(sc + 8 * DN, s2);
-                q4_scales<GB>(sc + 9 * DN, s3);
-#pragma unroll
-                for (int i = 0; i < GB; ++i) {
-                    const __nv_bfloat162 b0 = __floats2bfloat162_rn(a0.x * s0[i], a0.y * s1[i]), b1 = __floats2bfloat162_rn(a1.x * s2[i], a1.y * s3[i]);
-                    b[i][0] = *reinterpret_cast<const uint32_t*>(&b0);
-                    b[i][1] = *reinterpret_cast<const uint32_t*>(&b1);
-                }
-            }
-            auto phase2 = [&](auto exact) {
-#pragma unroll
-                for (int i = 0; i < GB; i += 2) {
-                    // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word
-                    const int j = i + 1 < GB ? i + 1 : i;
-                    const uint4 w = ldsm4t(at + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
-                    q4_phase2<decltype(exact)::value>(y[i], w.x, w.y, b[i][0], b[i][1]);
-                    if (i + 1 < GB) q4_phase2<decltype(exact)::value>(y[j], w.z, w.w, b[j][0], b[j][1]);
-                }
-            };
-            if (q4_any_nonfinite(b)) phase2(std::true_type{});
-            else phase2(std::false_type{});
         }
         if ((k - 1) % kMqTiles == kMqTiles - 1) {            // end of a task: a lane has four consecutive columns of two tokens
             const MqTask kk = tasks[(k - 1) / kMqTiles];
@@ -304,11 +325,10 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
             float* out = a.partial + (size_t(kk.jt_n >> 4) * a.rows_cap + kk.row) * D + grp0 * 32 + g * 4;
 #pragma unroll
             for (int i = 0; i < GB; ++i) {
-                if (2 * t < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t) * D + i * 32) = scale.out(y[i][0][0], y[i][0][2], y[i][1][0], y[i][1][2]);
-                if (2 * t + 1 < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t + 1) * D + i * 32) = scale.out(y[i][0][1], y[i][0][3], y[i][1][1], y[i][1][3]);
+                if (2 * t < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t) * D + i * 32) = make_float4(y[i][0][0] * kQ4Unscale, y[i][0][2] * kQ4Unscale, y[i][1][0] * kQ4Unscale, y[i][1][2] * kQ4Unscale);
+                if (2 * t + 1 < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t + 1) * D + i * 32) = make_float4(y[i][0][1] * kQ4Unscale, y[i][0][3] * kQ4Unscale, y[i][1][1] * kQ4Unscale, y[i][1][3] * kQ4Unscale);
             }
             clear_y();
-            scale = Q4ActScale{};
         }
     }
     // Wind-down after a wait ran out, as in ffn_multi_kernel: the warps agree on the last tile that any of them fed, arrive without a

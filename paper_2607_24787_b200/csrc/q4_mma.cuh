@@ -65,6 +65,45 @@ __device__ __forceinline__ Nib4 q4_operands(uint32_t w) {
     return q4_unpack(w);
 }
 
+// Weights as the tensor cores of ffn_grouped_q4_kernel get them, bf16_rn(bf16_rn(scale) * (q - 8)), times 2^-22: one packed fma on the masked
+// nibbles, q 2^-133 * (s 2^111) - 8 s 2^-22, rounds once like that product (all of its operands are exact: s is an fp16 number rounded to
+// bf16, at most 2^16). `odd` is `even` over 16.
+struct Q4Scaled { __nv_bfloat162 even, odd, off; };
+__device__ __forceinline__ __nv_bfloat162 bf2(uint32_t v) { return *reinterpret_cast<const __nv_bfloat162*>(&v); }
+__device__ __forceinline__ uint32_t bits2(__nv_bfloat162 v) { return *reinterpret_cast<const uint32_t*>(&v); }
+constexpr uint32_t kQ4Up111 = 0x77007700u, kQ4Down4 = 0x3d803d80u, kQ4Off = 0xb600b600u, kQ4Down22 = 0x34803480u;      // 2^111, 2^-4, -2^-19, 2^-22, twice
+constexpr float kQ4Unscale = 4194304.f;         // 2^22
+__device__ __forceinline__ Q4Scaled q4_scaled(__nv_bfloat162 s) {
+    const __nv_bfloat162 even = __hmul2(s, bf2(kQ4Up111));
+    return Q4Scaled{even, __hmul2(even, bf2(kQ4Down4)), __hmul2(s, bf2(kQ4Off))};
+}
+__device__ __forceinline__ __nv_bfloat162 q4_bf16_scales(uint32_t halves) { return __float22bfloat162_rn(__half22float2(*reinterpret_cast<const __half2*>(&halves))); }
+// PLAIN: subtract, then multiply, for scales that are not finite (the fma would make a NaN of q times infinity minus 8 times infinity)
+template <bool PLAIN>
+__device__ __forceinline__ Nib4 q4_weights(uint32_t w, const Q4Scaled& s, __nv_bfloat162 plain) {
+    if constexpr (PLAIN) {
+        Nib4 r;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r.p[i] = bits2(__hmul2(__hmul2(bf2(nib_pair(w, i)), plain), bf2(kQ4Down22)));
+        return r;
+    }
+    const Nib4 q = q4_unpack(w);
+    return Nib4{{bits2(__hfma2(bf2(q.p[0]), s.even, s.off)), bits2(__hfma2(bf2(q.p[1]), s.odd, s.off)),
+                 bits2(__hfma2(bf2(q.p[2]), s.even, s.off)), bits2(__hfma2(bf2(q.p[3]), s.odd, s.off))}};
+}
+// GB consecutive fp16 scales as pairs of groups (the second half of the last pair is 0 where GB is odd)
+template <int GB>
+__device__ __forceinline__ void q4_scale_pairs(uint32_t addr, uint32_t (&v)[(GB + 1) / 2]) {
+    if constexpr (GB == 4) {
+        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(addr));
+    } else if constexpr (GB == 2) {
+        v[0] = lds32(addr);
+    } else {
+#pragma unroll
+        for (int i = 0; i < GB; ++i) v[i / 2] = (i & 1) ? v[i / 2] | lds16(addr + 2 * i) << 16 : lds16(addr + 2 * i);
+    }
+}
+
 // C = {c0, c1, c0, c1}
 __device__ __forceinline__ void mma_k16_from(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, float c0, float c1) {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %11, %10, %11};"

@@ -515,14 +515,15 @@ cudaError_t launch_grouped_q4_mma_t(const spm_ctx* c, const MqArgs& a) {
     const int stages = mq_stages(a.g.D, c->cfg.n_experts, &smem);
     return launch_k(kern, dim3(c->num_sms), dim3(q4_warps(NSEG) * 32), smem, c->compute, true, a, stages);
 }
-// 4-bit grouped FFN of nb sequences. Which kernel follows from the call alone, not from a wave: the two round differently.
+// 4-bit grouped FFN of nb sequences. Which kernel follows from the call alone, not from a wave: the two round alike but add in different orders.
 // ffn_grouped_q4_mma_kernel costs a CTA's tasks (an expert's 128 rows for up to eight tokens) and depends little on hidden, the
 // tcgen05 kernel costs a CTA's units (an expert's 128 rows), in proportion to hidden and up to twice as much with many tokens. The
-// costs below are in us per 16 rows, from whole host-free steps (us a layer, tcgen05 -> mma.sync; sequences, top-k of experts, hidden;
+// costs below are in us per 16 rows, from whole host-free steps (us a layer, tcgen05 / mma.sync; sequences, top-k of experts, hidden;
 // 768 rows an expert):
-//   64, 8 of 128, 2048: 198 -> 142     8, 8 of 128, 2048: 103 -> 68     64, 8 of 60, 2048: 140 -> 108     64, 8 of 24, 2048:  85 -> 98
-//   64, 8 of 128, 1280: 134 -> 120     2, 8 of 128, 2048:  52 -> 38     32, 4 of 12, 2048:  61 -> 42      64, 8 of 12, 2048:  95 -> 91
-//   64, 8 of 128,  768:  98 -> 97     64, 8 of 128,  256:  57 -> 93
+//   64, 8 of 128, 2048: 197 / 146     8, 8 of 128, 2048: 103 / 70     64, 8 of 60, 2048: 140 / 111     64, 8 of 24, 2048:  84 / 101
+//   64, 8 of 128, 1280: 134 / 126     2, 8 of 128, 2048:  52 / 39     32, 4 of 12, 2048:  61 / 43      64, 8 of 12, 2048:  94 / 93
+//   64, 8 of 128,  768:  98 / 99     64, 8 of 128,  512:  76 / 89     64, 8 of 128, 256:  57 / 92      32, 8 of 24, 2048:  67 / 64
+// (of 22 shapes measured on both, the rule takes the slower one for three, by 1 to 5 %)
 bool grouped_q4_mma_pays(const spm_ctx* c, int nb) {
     const spm_model_cfg& m = c->cfg;
     if (mq_max_tasks(nb, m.top_k, m.n_experts, c->n_jt, c->num_sms) > kMqMaxTasks) return false;

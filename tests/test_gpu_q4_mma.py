@@ -98,3 +98,99 @@ def test_batched(name):
         assert torch.equal(turned.roll(-1, 0), got)
         assert ((got - rows).norm(dim=1) <= 1e-2 * rows.norm(dim=1)).all()
     m.close()
+
+
+def rounded(cfg, x, ids, w, parts=None):
+    """The layer's expert sum with what the batched kernels round rounded to bf16 (token rows, scales, scale * (q - 8), activations), all
+    sums in 64 bits. parts(e): the expert's ((q, scale), (q, scale), (q, scale)) where they are not the configuration's."""
+    out = torch.zeros_like(x, dtype=torch.float64)
+    rows = x.bfloat16().double()
+    for e in range(cfg.n_experts):
+        hit = torch.from_numpy(ids).cuda() == e
+        on = hit.any(1)
+        if not on.any():
+            continue
+        wt = (w.double() * hit).sum(1)
+        mats = parts(e) if parts else [(q[0], s[0]) for q, s in synth.expert_q4(cfg, 0, [e], device="cuda")]
+        gate, up, down = (((q.float() - 8) * s.bfloat16().float().repeat_interleave(32, -1)).bfloat16().double() for q, s in mats)
+        act = (torch.nn.functional.silu(rows[on] @ gate.T) * (rows[on] @ up.T) * wt[on, None]).bfloat16().double()
+        out[on] += act @ down
+    return out
+
+
+@pytest.mark.parametrize("name", list(BATCHED) + ["tcgen05"])
+def test_batched_kernels_round_alike(name):
+    """Outputs of batched 4-bit experts are the same numbers whichever kernel a batch size leads to: both round what `rounded` does. Sums in
+    fp32 against 64 bits, 1e-6 of a gate, tip one activation in 2^12 to its other bf16 neighbour, 2^-8 of it: 6e-5 of the whole on
+    average, and five times that with few and uneven activations. An operand rounded elsewhere shows at 2e-3."""
+    hidden, inter, n, k, nb = dict(BATCHED, tcgen05=(2048, 768, 24, 8, 64))[name]
+    cfg = make(hidden, inter, n, k, batch=nb)
+    m = build(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    for scale in (1.0, 2e4):
+        x = torch.randn(nb, hidden, generator=gen, device="cuda") * scale
+        torch.cuda.synchronize()
+        _, ids, w, _ = m.router_topk(0, torch.randn(nb, hidden, generator=gen, device="cuda"))
+        got = torch.zeros_like(x)
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x, ids, w, got)
+        m.synchronize()
+        want, whole = rounded(cfg, x, ids, w), exact(cfg, x, ids, w)
+        assert (got.double() - want).norm() <= 3e-4 * want.norm(), scale
+        # all four roundings carry 2^-9 at most, three of them on independent terms: some 4e-3 of a row
+        assert ((got.double() - whole).norm(dim=1) <= 8e-3 * whole.norm(dim=1)).all(), scale
+    m.close()
+
+
+def test_batch_mates_do_not_change_a_row():
+    """Rows that are not finite, or as large as fp32 goes, beside ordinary rows of the same experts."""
+    cfg = make(1024, 256, 3, 3, batch=9)
+    m = build(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    x = torch.randn(9, 1024, generator=gen, device="cuda")
+    torch.cuda.synchronize()
+    _, ids, w, _ = m.router_topk(0, torch.randn(9, 1024, generator=gen, device="cuda"))
+    odd = x.clone()
+    odd[1, 7], odd[2], odd[4, 0], odd[5] = float("inf"), x[2] * 1e19, float("nan"), x[5] * 1e37
+    clean, mixed = torch.zeros_like(x), torch.zeros_like(x)
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, clean)
+    m.moe_ffn(0, odd, ids, w, mixed)
+    m.synchronize()
+    same = [0, 3, 6, 7, 8]
+    assert torch.equal(mixed[same], clean[same])
+    assert not mixed[[1, 4]].isfinite().any()
+    m.close()
+
+
+def test_scales_that_are_not_finite():
+    """An infinite or NaN scale of W_down makes infinities and NaNs of its columns, where the products say so, and of no others."""
+    cfg = make(1280, 256, 2, 2, batch=3)
+    m = build(cfg)
+    part = cfg.hidden // 2 + cfg.hidden // 16
+    blobs = m.store.tensor.view(cfg.n_experts, cfg.inter, 3, part)
+    bad = {(0, 5, 3): 0x7c00, (0, 130, 39): 0xfc00, (1, 255, 17): 0x7e01}         # (expert, row, group): fp16 bits
+    for (e, j, grp), bits in bad.items():
+        at = cfg.hidden // 2 + 2 * grp
+        blobs[e, j, 2, at], blobs[e, j, 2, at + 1] = bits & 255, bits >> 8
+
+    def parts(e):
+        mats = [(q[0], s[0].clone()) for q, s in synth.expert_q4(cfg, 0, [e], device="cuda")]
+        for (e2, j, grp), bits in bad.items():
+            if e2 == e:
+                mats[2][1].view(torch.int16)[j, grp] = bits - 65536 if bits > 32767 else bits
+        return mats
+
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn(3, cfg.hidden, generator=gen, device="cuda")
+    torch.cuda.synchronize()
+    _, ids, w, _ = m.router_topk(0, x)
+    got = torch.zeros_like(x)
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, got)
+    m.synchronize()
+    want = rounded(cfg, x, ids, w, parts)
+    assert torch.equal(got.isnan(), want.isnan()) and torch.equal(got.isposinf(), want.isposinf()) and torch.equal(got.isneginf(), want.isneginf())
+    ok = want.isfinite()
+    assert (~ok).sum() == 3 * 96 and ((got.double() - want)[ok].norm() <= 3e-4 * want[ok].norm())
+    m.close()
