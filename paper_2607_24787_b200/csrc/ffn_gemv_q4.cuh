@@ -178,7 +178,7 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
 #pragma unroll
                 for (int w = 0; w < NW; ++w) sum += p[w * kQ4Red];
                 const float up = __shfl_xor_sync(0xffffffffu, sum, 1);
-                if (lane == 0) acts[r] = r < nr ? __fdividef(sum, 1.f + __expf(-sum)) * up * weight(k * kQ4Rows + r) : 0.f;
+                if (lane == 0) acts[r] = r < nr ? sum / (1.f + expf(-sum)) * up * weight(k * kQ4Rows + r) : 0.f;
             }
         };
         float a0, a1, a2, a3;            // activations of rows 2t, 2t + 1, 2t + 8, 2t + 9

@@ -523,7 +523,7 @@ cudaError_t launch_grouped_q4_mma_t(const spm_ctx* c, const MqArgs& a) {
 //   64, 8 of 128, 2048: 197 / 146     8, 8 of 128, 2048: 103 / 70     64, 8 of 60, 2048: 140 / 111     64, 8 of 24, 2048:  84 / 101
 //   64, 8 of 128, 1280: 134 / 126     2, 8 of 128, 2048:  52 / 39     32, 4 of 12, 2048:  61 / 43      64, 8 of 12, 2048:  94 / 93
 //   64, 8 of 128,  768:  98 / 99     64, 8 of 128,  512:  76 / 89     64, 8 of 128, 256:  57 / 92      32, 8 of 24, 2048:  67 / 64
-// (of 22 shapes measured on both, the rule takes the slower one for three, by 1 to 5 %)
+// (of 22 shapes measured on both, the rule takes the slower one for two, by 4 and 5 %)
 bool grouped_q4_mma_pays(const spm_ctx* c, int nb) {
     const spm_model_cfg& m = c->cfg;
     if (mq_max_tasks(nb, m.top_k, m.n_experts, c->n_jt, c->num_sms) > kMqMaxTasks) return false;

@@ -194,3 +194,27 @@ def test_scales_that_are_not_finite():
     ok = want.isfinite()
     assert (~ok).sum() == 3 * 96 and ((got.double() - want)[ok].norm() <= 3e-4 * want[ok].norm())
     m.close()
+
+
+def test_silu_of_negative_gates():
+    """One row, one column that is not zero: gate and up are exact, so what is left is exp (two units in the last place at most), a sum, a
+    quotient, three products and the split sum of the result, 2^-24 each: 6e-7 of an element. The fast exponential is off by more the
+    larger the gate."""
+    cfg = make(256, 1, 2, 1)
+    m = build(cfg)
+    (gq, gs), (uq, us), _ = synth.expert_q4(cfg, 0, [0], device="cuda")
+    gate = ((gq[0, 0].float() - 8) * gs[0, 0].float().repeat_interleave(32)).cpu()
+    up = ((uq[0, 0].float() - 8) * us[0, 0].float().repeat_interleave(32)).cpu()
+    col = int((gate + 1e3 * (up == 0)).argmin())
+    ids, w = np.zeros((1, 1), np.int32), torch.ones(1, 1, device="cuda")
+    m.prefetch_async(0, ids[0])
+    for target in np.linspace(1, 40, 40):
+        x = torch.zeros(1, 256, device="cuda")
+        x[0, col] = round(target / -float(gate[col]) * 4) / 4            # few bits: its products with the weights are exact
+        got = torch.zeros_like(x)
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x, ids, w, got)
+        m.synchronize()
+        want = exact(cfg, x, ids, w)
+        assert ((got.double() - want).abs() <= 6e-7 * want.abs()).all(), target
+    m.close()
