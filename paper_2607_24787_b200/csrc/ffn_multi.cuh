@@ -241,12 +241,18 @@ template <> struct MtWeight<Q4Tag> {         // (q - 8) through the MMA, a group
         const uint32_t row = rows + uint32_t(lane >> 2) * stride, PART = part_bytes(D);
         const uint32_t wg = lds32(row + grp * 16 + (lane & 3) * 4), wu = lds32(row + PART + grp * 16 + (lane & 3) * 4);
         const float sg = lds_half(row + D / 2 + grp * 2), su = lds_half(row + PART + D / 2 + grp * 2);
-        float c[2][4];
+        // (one chain, small parts of both halves first: a rounding less than two chains and a sum)
+        float c[4];
 #pragma unroll
-        for (int kb = 0; kb < 2; ++kb)
-            mma_chain_k16<NS>(c[kb], nib_pair(wg, 2 * kb), nib_pair(wu, 2 * kb), nib_pair(wg, 2 * kb + 1), nib_pair(wu, 2 * kb + 1), x[kb][0], x[kb][1]);
+        for (int p = NS - 1; p >= 0; --p)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = fmaf(i < 2 ? sg : su, c[0][i] + c[1][i], acc[i]);
+            for (int kb = 0; kb < 2; ++kb) {
+                const uint32_t a0 = nib_pair(wg, 2 * kb), a1 = nib_pair(wu, 2 * kb), a2 = nib_pair(wg, 2 * kb + 1), a3 = nib_pair(wu, 2 * kb + 1);
+                if (p == NS - 1 && kb == 0) mma_k16_first(c, a0, a1, a2, a3, x[kb][0][p], x[kb][1][p]);
+                else mma_k16(c, a0, a1, a2, a3, x[kb][0][p], x[kb][1][p]);
+            }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = fmaf(i < 2 ? sg : su, c[i], acc[i]);
     }
     template <int NS>
     static __device__ __forceinline__ void phase2(uint32_t rows, uint32_t stride, int D, int grp, int lane, float2 act, const uint32_t (&)[NS], float (&y)[2][4]) {
