@@ -10,14 +10,16 @@
 //   Phase 1 (M = 16 gate rows, then 16 up rows; K = the group): the group's scale goes onto the fp32 sum of its 32 products; the warps' sums
 // meet in shared memory, a warp takes a row's activation from them.
 //   Phase 2 (M = hidden columns, K = the tile's 16 rows): act * scale is the split operand; two groups, whose scales differ, use columns of
-// N of their own. y stays in the accumulators for all tiles of the CTA, each column in one warp: no sum over warps.
+// N of their own. y stays in registers for all tiles of the CTA, each column in one warp: no sum over warps.
 //
 // Why MMAs: with fp32 FMAs the kernel was bound by instruction issue, 27 warp instructions per eight weights and lane, eight of which
-// widened halves to floats and eight multiplied; an MMA operand needs five. A layer of the Qwen3 shape (a step as one kernel; with
-// separate launches before) 26.5 -> 18.6 us, of the DeepSeek shape 25.6 -> 16.1; its part of that, 14.6 -> 9. What bounds it now: the
-// chain of latencies of a tile, of which a CTA has three or four, and still instruction issue (some 400 a warp and tile).
-// Error against 64 bits, 18 shapes of hidden 256 to 2048: 0.93 of the FMAs' on normally distributed rows (2.4e-7 of the result at
-// worst, as before), 1.4 on log-normal ones (5e-7 at worst: the -8 is a sum of its own).
+// widened halves to floats and eight multiplied; an MMA operand needs nine. A layer of the Qwen3 shape (a step as one kernel; with
+// separate launches before) 26.5 -> 18.3 us, of the DeepSeek shape 25.6 -> 16.2; its part of that, 14.6 -> 9. What bounds it now: the
+// chain of latencies of a tile, of which a CTA has three or four, and still instruction issue.
+// The tensor cores cut a sum off where fp32 adds round it, always towards zero, so no chain of MMAs is longer than a group (phase 1) or a
+// tile (phase 2); longer sums are fp32 adds. (With y in the accumulators for all tiles a CTA of 384 tiles was off by 2.4e-6; 1 % faster.)
+// Error against 64 bits, 18 shapes of hidden 256 to 2048, rows that are normal, log-normal, of one sign, with outliers: 0.79 - 0.86 of the
+// FMAs' on average, 2.2e-7 of the result at worst (2.7e-7). Activations below 2^-110 lose bits: their third parts end at bf16's last one.
 #pragma once
 
 #include <type_traits>
@@ -96,58 +98,51 @@ struct Q4Ring {
     }
 };
 
-// B operand of phase 1: the lane's part (N column = part) of the activations of its eight columns in each of the warp's groups, scaled up
-// by the warp's power of two; returns its exponent. get(col, v): eight consecutive fp32 from column col on.
+// B operand of phase 1: the lane's part (N column = part) of the activations of its eight columns in each of the warp's groups.
+// get(col, v): eight consecutive fp32 from column col on.
 template <int GB, typename F>
-__device__ __forceinline__ int q4_operand(uint32_t (&x)[GB][4], float (&off)[GB][2], int warp, int lane, F get) {
+__device__ __forceinline__ void q4_operand(uint32_t (&x)[GB][4], int warp, int lane, F get) {
     const int g = lane >> 2, t = lane & 3;
     float v[GB][8];
-    uint32_t top = 0;
+    bool odd = false;
 #pragma unroll
     for (int i = 0; i < GB; ++i) {
         get((warp * GB + i) * 32 + t * 8, v[i]);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) top = max(top, __float_as_uint(v[i][q]) & 0x7fffffffu);
+        for (int q = 0; q < 8; ++q) odd |= !(fabsf(v[i][q]) < INFINITY);
     }
-    top = __reduce_max_sync(0xffffffffu, top);
-    const int e = q4_exponent(top);
-    const bool guarded = top >= 0x7f800000u;
-    const float even = g < 3 ? q4_up(e) : 0.f, odd = even * 0.0625f;
+    const bool guarded = __any_sync(0xffffffffu, odd);
     const Q4Part part(g);
 #pragma unroll
     for (int i = 0; i < GB; ++i) {
-        // (a NaN comes out as the one whose upper half is one too)
+        if (guarded)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float f = (q & 1) ? odd : even;
-            x[i][q] = guarded ? (g < 3 ? part.pair(v[i][q] * f, v[i][q + 4] * f, true) : 0u) : part.pair(v[i][q] * f, v[i][q + 4] * f);
-        }
-        q4_offset(x[i], off[i]);
+            for (int q = 0; q < 8; ++q) v[i][q] = v[i][q] != v[i][q] ? __uint_as_float(0x7fffffffu) : v[i][q];      // (a NaN whose upper half is one too)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[i][q] = g < 3 ? part.pair(v[i][q], v[i][q + 4], guarded) : 0u;
     }
-    return e;
 }
 
 // The CTA's rows 0 .. span - 1, tile by tile. fill(tile): ask for the warp's rows of a tile; the first `stages` tiles have been
 // asked for. weight(row): routing weight. Every thread of the CTA takes part. Returns false, in every
 // thread, when a wait ran out (the caller drains and leaves).
 template <int GB, int NW, typename Fill, typename Weight>
-__device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[GB][4], const float (&off)[GB][2], int x_exp, float (&y)[GB][2][4], Q4ActScale& scale,
-                                         int D, int span, int warp, int lane, unsigned long long limit, Fill fill, Weight weight) {
+__device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[GB][4], float (&y)[GB][2][4], int D, int span,
+                                         int warp, int lane, unsigned long long limit, Fill fill, Weight weight) {
     const int g = lane >> 2, t = lane & 3, grp0 = warp * GB;
     const int tiles = (span + kQ4Rows - 1) / kQ4Rows;
     const uint32_t P = ring.pitch, PART = q4_part_bytes(D);
-    const float x_down = q4_down(x_exp);
     for (int k = 0; k < tiles; ++k) {
         const int nr = span - k * kQ4Rows;
         const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(ring.bars + 8u * ring.st, ring.ph, limit));
         const uint32_t rows = ring.rows + uint32_t(ring.st * kQ4Rows) * P;
         if (++ring.st == ring.stages) { ring.st = 0; ring.ph ^= 1; }
         float* acts = ring.act + (k & 1) * kQ4Rows;
-        // `whole`: for the case below, exact operands, and a group's three parts added up before the scale goes onto them
+        // `whole`: for the case below, a group's three parts added up before the scale goes onto them
         auto phase1 = [&](auto whole) {
             constexpr bool kWhole = decltype(whole)::value;
             float ag[4], au[4];
-            q4_phase1<GB, kWhole>(rows, P, D, grp0, lane, x, off, ag, au, [](float (&acc)[4], const float (&c)[4], float s0, float s1) {
+            q4_phase1<GB>(rows, P, D, grp0, lane, x, ag, au, [](float (&acc)[4], const float (&c)[4], float s0, float s1) {
                 if constexpr (kWhole) {
                     float lo = c[0] + c[1], hi = c[2] + c[3];
                     lo += __shfl_xor_sync(0xffffffffu, lo, 1);
@@ -165,7 +160,7 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
                 for (int j = 0; j < 4; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], 1);
             if (t == 0) {
                 float* r = ring.red + warp * kQ4Red + g;
-                r[0] = v[0] * x_down; r[8] = v[1] * x_down; r[16] = v[2] * x_down; r[24] = v[3] * x_down;
+                r[0] = v[0] * kQ4ExactUnscale; r[8] = v[1] * kQ4ExactUnscale; r[16] = v[2] * kQ4ExactUnscale; r[24] = v[3] * kQ4ExactUnscale;
             }
         };
         auto activations = [&]() {       // warp w: rows w, w + NW; even lanes take a row's gate, odd ones its up
@@ -185,7 +180,6 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
         auto take = [&]() {
             const float2 lo = *reinterpret_cast<const float2*>(acts + 2 * t), hi = *reinterpret_cast<const float2*>(acts + 2 * t + 8);
             a0 = lo.x; a1 = lo.y; a2 = hi.x; a3 = hi.y;
-            return fmaxf(fmaxf(fabsf(a0), fabsf(a1)), fmaxf(fabsf(a2), fabsf(a3)));
         };
         phase1(std::false_type{});
         if (!__syncthreads_and(ok)) return false;
@@ -193,21 +187,18 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
         if (k > 0 && k - 1 + ring.stages < tiles) fill(k - 1 + ring.stages);
         activations();
         __syncthreads();
-        float largest = take();
+        take();
         if (__any_sync(0xffffffffu, !isfinite(a0 * 0.f + a1 * 0.f + a2 * 0.f + a3 * 0.f))) {       // (so in all warps or in none)
-            // An infinite scale times a part that is zero is a NaN where the scale times the sum is an infinity, and so are q and -8
-            // times an infinity where q - 8 times it is one.
+            // An infinite scale times a part that is zero is a NaN where the scale times the sum is an infinity.
             phase1(std::true_type{});
             __syncthreads();
             activations();
             __syncthreads();
-            largest = take();
+            take();
         }
-        scale.fit<GB>(largest, y);
         // N columns 0-2: the parts for one group, 4-6: for the next (where there is one)
         const bool second = g >= 4;
-        const float up = (g & 3) < 3 ? scale.up : 0.f;
-        a0 *= up; a1 *= up; a2 *= up; a3 *= up;
+        const bool idle = (g & 3) == 3;
         const uint32_t at = rows + 2 * PART + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * P + uint32_t(grp0) * 16;
         const uint32_t sc = rows + 2 * PART + uint32_t(2 * t) * P + uint32_t(D / 2 + grp0 * 2);
         float s0[GB], s1[GB], s2[GB], s3[GB];
@@ -231,24 +222,17 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
                 const float v0 = a0 * (second ? s0[j] : s0[i]), v1 = a1 * (second ? s1[j] : s1[i]), v2 = a2 * (second ? s2[j] : s2[i]), v3 = a3 * (second ? s3[j] : s3[i]);
                 b[i / 2][0] = part.pair(v0, v1, guarded);
                 b[i / 2][1] = part.pair(v2, v3, guarded);
-                if ((i + 1 >= GB && second) || (guarded && (g & 3) == 3)) b[i / 2][0] = b[i / 2][1] = 0u;
+                if (idle || (i + 1 >= GB && second)) b[i / 2][0] = b[i / 2][1] = 0u;
             }
         };
         operand(false);
-        auto phase2 = [&](auto exact) {
+        if (q4_any_nonfinite(b)) operand(true);
 #pragma unroll
-            for (int i = 0; i < GB; i += 2) {
-                // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word
-                const uint4 w = ldsm4t(at + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
-                q4_phase2<decltype(exact)::value>(y[i], w.x, w.y, b[i / 2][0], b[i / 2][1]);
-                if (i + 1 < GB) q4_phase2<decltype(exact)::value>(y[i + 1 < GB ? i + 1 : i], w.z, w.w, b[i / 2][0], b[i / 2][1]);
-            }
-        };
-        if (q4_any_nonfinite(b)) {
-            operand(true);
-            phase2(std::true_type{});
-        } else {
-            phase2(std::false_type{});
+        for (int i = 0; i < GB; i += 2) {
+            // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word
+            const uint4 w = ldsm4t(at + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
+            q4_phase2(y[i], w.x, w.y, b[i / 2][0], b[i / 2][1]);
+            if (i + 1 < GB) q4_phase2(y[i + 1 < GB ? i + 1 : i], w.z, w.w, b[i / 2][0], b[i / 2][1]);
         }
     }
     return true;
@@ -256,14 +240,14 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
 
 // After the last tile: put(column, four consecutive y) for the columns of the warp's groups
 template <int GB, typename F>
-__device__ __forceinline__ void q4_result(const float (&y)[GB][2][4], const Q4ActScale& scale, int warp, int lane, F put) {
+__device__ __forceinline__ void q4_result(const float (&y)[GB][2][4], int warp, int lane, F put) {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
     for (int i = 0; i < GB; ++i) {
         float4 o = make_float4(y[i][0][0] + y[i][0][1], y[i][0][2] + y[i][0][3], y[i][1][0] + y[i][1][1], y[i][1][2] + y[i][1][3]);
         o.x += __shfl_xor_sync(0xffffffffu, o.x, 1); o.y += __shfl_xor_sync(0xffffffffu, o.y, 1);
         o.z += __shfl_xor_sync(0xffffffffu, o.z, 1); o.w += __shfl_xor_sync(0xffffffffu, o.w, 1);
-        if (t == (i & 1) * 2) put((warp * GB + i) * 32 + g * 4, scale.out(o.x, o.y, o.z, o.w));
+        if (t == (i & 1) * 2) put((warp * GB + i) * 32 + g * 4, make_float4(o.x * kQ4ExactUnscale, o.y * kQ4ExactUnscale, o.z * kQ4ExactUnscale, o.w * kQ4ExactUnscale));
     }
 }
 
@@ -321,10 +305,9 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages)
     if (early) depend();
 
     uint32_t x[GB][4];
-    float off[GB][2];
     const float* xt = a.x + size_t(tok) * D;
     const bool vec = (reinterpret_cast<uintptr_t>(xt) & 15) == 0;       // the caller's rows may start at any float
-    const int x_exp = q4_operand<GB>(x, off, warp, lane, [&](int col, float (&v)[8]) {
+    q4_operand<GB>(x, warp, lane, [&](int col, float (&v)[8]) {
         if (vec) {
             const float4 lo = *reinterpret_cast<const float4*>(xt + col), hi = *reinterpret_cast<const float4*>(xt + col + 4);
             v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w; v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
@@ -334,8 +317,7 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages)
         }
     });
     float y[GB][2][4] = {};
-    Q4ActScale scale;
-    const bool ok = q4_tiles<GB, NW>(ring, x, off, x_exp, y, scale, D, span, warp, lane, limit,
+    const bool ok = q4_tiles<GB, NW>(ring, x, y, D, span, warp, lane, limit,
         [&](int tile) { ring.fill(tile, 1, warp, lane, ROWB, row_at); ++filled; },
         [&](int row) {
             const int kk = a.kidx_of(tok, (r_begin + row) / I);
@@ -348,7 +330,7 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages)
             if (!mbar_wait_bounded(ring.bars + 8u * (k % n_stages), (k / n_stages) & 1, kWaitLimitNs)) break;
     }
     float* out = a.partial + (size_t(tok) * G + c) * D;
-    q4_result<GB>(y, scale, warp, lane, [&](int col, float4 v) { *reinterpret_cast<float4*>(out + col) = v; });
+    q4_result<GB>(y, warp, lane, [&](int col, float4 v) { *reinterpret_cast<float4*>(out + col) = v; });
     if (a.clock) {
         __syncthreads();
         if (threadIdx.x == 0) atomicMax(a.clock + 1, global_timer_ns());

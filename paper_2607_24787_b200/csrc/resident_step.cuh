@@ -327,10 +327,8 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
         // the GEMV's copy of the row: like one 16-byte weight vector per lane and segment, or as an MMA operand
         float xr[Q4 ? 1 : NSEG][VEC];
         uint32_t xq[GB][4];
-        float xoff[GB][2];
-        int x_exp = 0;
         if constexpr (Q4) {
-            x_exp = q4_operand<GB>(xq, xoff, wi, lane, [&](int col, float (&f)[8]) {
+            q4_operand<GB>(xq, wi, lane, [&](int col, float (&f)[8]) {
                 const float4 lo = *reinterpret_cast<const float4*>(xs + col), hi = *reinterpret_cast<const float4*>(xs + col + 4);
                 f[0] = lo.x; f[1] = lo.y; f[2] = lo.z; f[3] = lo.w; f[4] = hi.x; f[5] = hi.y; f[6] = hi.z; f[7] = hi.w;
             });
@@ -425,8 +423,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
         };
         if constexpr (Q4) {
             float y[GB][2][4] = {};
-            Q4ActScale scale;
-            if (!q4_tiles<GB, kStepWarps>(tiles, xq, xoff, x_exp, y, scale, D, span, wi, lane, limit, [&](int tile) { tiles.fill(tile, 1, wi, lane, ROWB, row_at); },
+            if (!q4_tiles<GB, kStepWarps>(tiles, xq, y, D, span, wi, lane, limit, [&](int tile) { tiles.fill(tile, 1, wi, lane, ROWB, row_at); },
                                           [&](int row) { return s_w[(r_begin + row) / I]; })) {
                 if (tid == 0) StepSpin::raise(a);
                 // leave no copy in flight: the tile that was waited for and those asked for since
@@ -438,7 +435,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
                 } while (st != tiles.st_in);
                 return;
             }
-            q4_result<GB>(y, scale, wi, lane, send);
+            q4_result<GB>(y, wi, lane, send);
         } else {
             uint64_t ya[NSEG][VEC / 2];
 #pragma unroll
