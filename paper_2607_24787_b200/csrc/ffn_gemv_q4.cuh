@@ -70,13 +70,18 @@ struct Q4Ring {
         }
     }
     // The warp's rows (warp, warp + NW) of `count` tiles from `tile` on; row_at(row) is null for rows that are not there. The lanes look the rows up side
-    // by side, one elected lane asks for them (lanes that ask side by side are taken one by one).
+    // by side, one elected lane asks for them (lanes that ask side by side are taken one by one). `waited`: row_at waits for arrivals, which
+    // the lane that waited has seen, but the one that asks reads the bytes: the barrier and the fence hand them on.
     template <typename F>
-    __device__ __forceinline__ void fill(int tile, int count, int warp, int lane, uint32_t bytes, F row_at) {
+    __device__ __forceinline__ void fill(int tile, int count, int warp, int lane, uint32_t bytes, bool waited, F row_at) {
         constexpr int kPer = q4_rows_per_warp(NW);
         const int mine = warp + lane % kPer * NW;
         const bool in = lane < count * kPer && mine < kQ4Rows;
         const unsigned long long at = in ? reinterpret_cast<unsigned long long>(row_at((tile + lane / kPer) * kQ4Rows + mine)) : 0ull;
+        if (waited) {
+            __syncwarp();
+            asm volatile("fence.proxy.async;" ::: "memory");
+        }
         for (int k = 0; k < count; ++k) {
 #pragma unroll
             for (int r = 0; r < kPer; ++r) {
@@ -301,7 +306,7 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages)
         return src_base ? src_base + size_t(r_begin + row - ent * I) * ROWB : nullptr;
     };
     int filled = min(n_stages, (span + kQ4Rows - 1) / kQ4Rows);
-    ring.fill(0, filled, warp, lane, ROWB, row_at);
+    ring.fill(0, filled, warp, lane, ROWB, a.ready != nullptr, row_at);
     if (early) depend();
 
     uint32_t x[GB][4];
@@ -318,7 +323,7 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages)
     });
     float y[GB][2][4] = {};
     const bool ok = q4_tiles<GB, NW>(ring, x, y, D, span, warp, lane, limit,
-        [&](int tile) { ring.fill(tile, 1, warp, lane, ROWB, row_at); ++filled; },
+        [&](int tile) { ring.fill(tile, 1, warp, lane, ROWB, a.ready != nullptr, row_at); ++filled; },
         [&](int row) {
             const int kk = a.kidx_of(tok, (r_begin + row) / I);
             return kk == 255 ? 1.f : a.w[size_t(tok) * a.K + kk];

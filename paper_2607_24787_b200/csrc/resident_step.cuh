@@ -385,7 +385,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
         };
         int n_in = n_first;                 // rows that the warp has asked for
         if constexpr (Q4) {
-            tiles.fill(0, min(depth, (span + kQ4Rows - 1) / kQ4Rows), wi, lane, ROWB, row_at);
+            tiles.fill(0, min(depth, (span + kQ4Rows - 1) / kQ4Rows), wi, lane, ROWB, false, row_at);
         } else {       // (the lanes look the rows up side by side)
             const unsigned char* base = lane >= n_early && lane < n_first ? blob(first_ent) : nullptr;
             const unsigned long long at = base ? reinterpret_cast<unsigned long long>(base + size_t(first_j) * ROWB) : 0ull;
@@ -423,7 +423,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
         };
         if constexpr (Q4) {
             float y[GB][2][4] = {};
-            if (!q4_tiles<GB, kStepWarps>(tiles, xq, y, D, span, wi, lane, limit, [&](int tile) { tiles.fill(tile, 1, wi, lane, ROWB, row_at); },
+            if (!q4_tiles<GB, kStepWarps>(tiles, xq, y, D, span, wi, lane, limit, [&](int tile) { tiles.fill(tile, 1, wi, lane, ROWB, false, row_at); },
                                           [&](int row) { return s_w[(r_begin + row) / I]; })) {
                 if (tid == 0) StepSpin::raise(a);
                 // leave no copy in flight: the tile that was waited for and those asked for since

@@ -257,3 +257,22 @@ def test_one_token_long_shares():
     want = exact(cfg, x, ids, w)
     assert (got.double() - want).norm() <= 5e-7 * want.norm()
     m.close()
+
+
+@pytest.mark.parametrize("shape", [(512, 200, 12, 3, 0), (1280, 896, 16, 6, 2), (2048, 333, 16, 4, 0)])
+def test_one_token_device_side_wait_gives_the_same_bits(shape):
+    """The kernel waits for arrivals in one lane and asks for the bytes in another; a small cache, so that every layer waits."""
+    cfg = make(*shape, layers=4).replace(slots=shape[3] + 1)
+    h = torch.randn(6, 1, cfg.hidden, generator=torch.Generator(device="cuda").manual_seed(8), device="cuda")
+    m = build(cfg)
+    runs = []
+    for on in (0, 1):
+        m.cache_reset()
+        m.set_device_wait(on)
+        torch.cuda.synchronize()
+        out = [m.decode_step(row) for row in h]
+        m.synchronize()
+        runs.append((torch.stack(out), m.events()))
+    assert torch.equal(runs[0][0], runs[1][0]) and runs[0][1] == runs[1][1]
+    assert m.stats()["misses"] > 0
+    m.close()
