@@ -272,8 +272,10 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages)
     const unsigned long long limit = a.limit();
     Q4Ring<NW> ring(smem, D, n_stages, threadIdx.x);
     __syncthreads();
-    // Everything above is independent of the preceding kernel; with `early` so are the first weight copies (see ffn_gemv_kernel).
-    const bool early = a.early && !a.dev_code;
+    int filled = min(n_stages, (span + kQ4Rows - 1) / kQ4Rows);
+    // Everything above is independent of the preceding kernel; with `early` so are the first weight copies (see ffn_gemv_kernel), but for those
+    // of shared experts, which are the caller's and may have been written just before. They are the last entries.
+    const bool early = a.early && !a.dev_code && (span == 0 || a.code_of(tok, (r_begin + min(span, filled * kQ4Rows) - 1) / I) >= 0);
     auto depend = [&]() {
         grid_dep_wait();
         // window start: kernel entry, or the end of the dependency wait when launched ahead of its predecessor's end
@@ -305,7 +307,6 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages)
         if (ent != src_ent) { src_ent = ent; src_base = resolve(ent); }
         return src_base ? src_base + size_t(r_begin + row - ent * I) * ROWB : nullptr;
     };
-    int filled = min(n_stages, (span + kQ4Rows - 1) / kQ4Rows);
     ring.fill(0, filled, warp, lane, ROWB, a.ready != nullptr, row_at);
     if (early) depend();
 
