@@ -180,7 +180,9 @@ const char* spm_last_error(const spm_ctx* ctx);   /* ctx may be NULL: last error
 /* Native router of `layer` (Section 3.1, first equation): RMSNorm, gate GEMV, softmax, Top-K,
  * renormalise.   h dev [nb][D] -> x_norm dev [nb][D], w dev [nb][K] (rank order),
  * logits dev [nb][n] (may be NULL), ids HOST [nb][K] (rank order: ties to the lower id).
- * Returns after the ids have reached the host (bounded wait, SPM_ERR_TIMEOUT). */
+ * Returns after the ids have reached the host (bounded wait, SPM_ERR_TIMEOUT). Weights written by work that was enqueued on the compute
+ * stream before are seen, here and in spm_adapter_predict. (Shared experts of fp32 and bf16 models in spm_moe_ffn, and all weights in steps
+ * without a host turn, may be read ahead of a preceding kernel that lets its successors start early: synchronise after changing them.) */
 int spm_router_topk(spm_ctx* ctx, int layer, const float* h, int nb,
                     float* x_norm, int32_t* ids, float* w, float* logits);
 

@@ -54,6 +54,7 @@ struct RouterArgs {
     const short* slot_map;   // optional [n] slot of each expert of this layer (device memory) ...
     short* codes_out;        // ... and where to leave the slots of the routed experts, [nb][K]
     unsigned long long* clock;   // optional {first leader past its dependency wait, last leader done} in ns
+    int late_weights;        // 1: the weights, too, are read behind the preceding kernel (stand-alone calls: it may have written them)
     int* status;             // optional status word: kStatusNonFinite is set when a router logit is NaN or Inf
     const float* partial;    // optional [nb][G][D] partial rows of the preceding expert kernel: the hidden row is
     int G;                   //   then h + sum of them (summed here instead of by a combine kernel) ...
@@ -255,6 +256,7 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
     // memory: arrive now, wait just before the first remote store
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
+    if (a.late_weights) grid_dep_wait();
     // ---- weights first: none of them depends on the kernel before this one, so in a launch that
     // overlaps its predecessor they are already in registers (or on their way into L2) when the
     // hidden row becomes readable. Router rows then adapter-A rows, one warp per row, ROWS rows in flight.

@@ -572,6 +572,7 @@ struct RouterRoute {
     const float* partial;      // partial rows of the preceding layer's expert kernel to fold into the hidden row, or null
     int G;
     RankArgs* defer;           // several tokens: the caller's next kernel ranks the adapter's priorities and is told here with what
+    bool late_weights = false; // stand-alone calls: the launch overlaps its predecessor, but weights that this may have written are read behind it
 };
 
 int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int nb, float* x_norm,
@@ -606,6 +607,7 @@ int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int 
     a.h_out = const_cast<float*>(h);
     a.publish_seq = publish_seq;
     a.defer_rank = route && route->defer;
+    a.late_weights = route && route->late_weights;
     if (int rc = take_clock(c, kClkRouter, &a.clock)) return rc;
     // Sequence numbers whose low 16 bits are zero are skipped, and the words this launch will
     // publish are zeroed first, so a word left by an older launch can never carry the current tag.
@@ -1778,7 +1780,7 @@ int spm_router_topk(spm_ctx* c, int layer, const float* h, int nb, float* x_norm
     // The kernel leaves the weights where they are wanted (a copy behind it cost its launch, and the expert kernel its early start); anything
     // but this device's memory is copied to.
     const bool direct = device_memory(w);
-    const RouterRoute route{c->mb_dev, nullptr, nullptr, true, nullptr, 0, nullptr};
+    const RouterRoute route{c->mb_dev, nullptr, nullptr, true, nullptr, 0, nullptr, true};
     if (int rc = launch_router(c, layer, h, nullptr, nb, x_norm, logits, true, false, &route, true, direct ? w : nullptr)) return rc;
     if (!direct) CU(c, cudaMemcpyAsync(w, c->ws_w, size_t(nb) * c->cfg.top_k * 4, cudaMemcpyDeviceToDevice, c->compute));
     if (int rc = wait_mailbox(c)) return rc;
@@ -1791,7 +1793,7 @@ int spm_adapter_predict(spm_ctx* c, int layer, const float* x_norm, int nb, floa
     if (int rc = flush_trace(c)) return rc;
     if (layer > c->cfg.n_layers - 2) return fail(c, SPM_ERR_INVALID_ARG, "layer %d has no adapter (L-1 adapters)", layer);
     if (!x_norm || !scores || !order) return fail(c, SPM_ERR_INVALID_ARG, "null argument");
-    const RouterRoute route{c->mb_dev, nullptr, nullptr, true, nullptr, 0, nullptr};
+    const RouterRoute route{c->mb_dev, nullptr, nullptr, true, nullptr, 0, nullptr, true};
     if (int rc = launch_router(c, layer, nullptr, x_norm, nb, nullptr, nullptr, false, true, &route)) return rc;
     if (int rc = wait_mailbox(c)) return rc;
     memcpy(scores, c->mb_host->scores, size_t(c->cfg.n_experts) * 4);

@@ -48,6 +48,25 @@ def same_as_after_a_pause(call, row, a, write):
             assert torch.equal(p.view(torch.int32), q.view(torch.int32)) if torch.is_tensor(p) else np.array_equal(p, q)
 
 
+def test_router_and_adapter_read_weights_written_just_before():
+    a, write = writer(256)
+    m, (gamma, router_w, adapter_a, _, _) = on_stream_of(a, synth.get_config("tiny", n_layers=2, hidden=256))
+    h = torch.randn(1, 256, device="cuda")
+    torch.cuda.synchronize()
+    x = m.router_topk(0, h)[0]
+
+    def route():
+        x2, ids, w, logits = m.router_topk(0, h, want_logits=True)
+        return [x2, w, logits, ids]
+
+    same_as_after_a_pause(route, gamma[0:1], a, write)
+    gamma.fill_(1)
+    same_as_after_a_pause(route, router_w[0, 3:4], a, write)
+    same_as_after_a_pause(lambda: [x.new_tensor(t) if t.dtype == np.float32 else t for t in m.adapter_predict(0, x)], adapter_a[0, 2:3], a, write)
+    m.close()
+    a.close()
+
+
 def test_4bit_shared_experts_written_just_before():
     a, write = writer(256)
     cfg = synth.get_config("dsvl2_q4", n_layers=1, hidden=256, n_experts=4, inter=64, top_k=1, n_shared=2, slots=4, batch=1, budget=0, adapter_rank=2)
