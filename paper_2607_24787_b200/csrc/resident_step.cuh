@@ -366,7 +366,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
             rk += __shfl_xor_sync(0xffffffffu, rk, 1);
             if (u < 2 * n && (u & 1) == 0 && rk < a.K) {
                 isel[rk] = e;
-                s_code[rk] = smap[e];
+                s_code[rk] = smap[e] >= 0 ? smap[e] : 1 << 20;       // no slot: fails the range check below
                 if (c == 0) a.mailbox[l].ids[rk] = tagged(tag & 0xffffu, e);
             }
         }

@@ -140,3 +140,38 @@ def test_two_contexts_at_once():
             assert np.array_equal(a, b)
     for m in ms:
         m.close()
+
+
+@pytest.mark.parametrize("name", ["fp32_widest", "bf16_nine_warps", "q4_widest", "q4_shared"])
+def test_expert_without_a_slot_is_reported(name):
+    """A slot map that names no slot for a routed expert (written over here, where the step reads it) is a bad slot, not a shared expert."""
+    cfg = config(name)
+    m = build(cfg, store_layers=1)
+    preload(cfg, m)
+    h = torch.as_tensor(rows(cfg, 1)[0], dtype=torch.float32).cuda()
+    torch.cuda.synchronize()
+    want = m.decode_step(h).clone()
+    m.synchronize()
+    used = m.router_topk(0, h)[1][0]
+    m.synchronize()
+    table = np.full((cfg.n_layers, cfg.n_experts), -1, np.int16)
+    for l in range(cfg.n_layers):
+        in_slot = m.slot_table(l)
+        for slot, e in enumerate(in_slot):
+            if e >= 0:
+                table[l, e] = slot
+    at = m.arena.cpu().numpy().tobytes().rindex(table.tobytes())
+    entry = m.arena[at + 2 * int(used[-1]):at + 2 * int(used[-1]) + 2]
+    saved = entry.clone()
+    entry.fill_(255)                    # -1
+    torch.cuda.synchronize()
+    m.decode_step(h)
+    with pytest.raises(SpmError) as e:
+        m.synchronize()
+    assert e.value.code == -5
+    entry.copy_(saved)
+    torch.cuda.synchronize()
+    got = m.decode_step(h)
+    m.synchronize()
+    assert torch.equal(got, want)
+    m.close()
