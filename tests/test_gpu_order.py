@@ -76,7 +76,7 @@ def test_4bit_shared_experts_written_just_before():
     m.prefetch_async(0, ids[0])
     m.synchronize()
 
-    outs = iter(torch.zeros(10, 1, 256, device="cuda"))
+    outs = iter(torch.zeros(15, 1, 256, device="cuda"))
 
     def ffn():
         out = next(outs)

@@ -150,7 +150,7 @@ def test_expert_without_a_slot_is_reported(name):
     preload(cfg, m)
     h = torch.as_tensor(rows(cfg, 1)[0], dtype=torch.float32).cuda()
     torch.cuda.synchronize()
-    want = m.decode_step(h).clone()
+    want = m.decode_step(h)
     m.synchronize()
     used = m.router_topk(0, h)[1][0]
     m.synchronize()
