@@ -291,7 +291,8 @@ int spm_set_device_wait(spm_ctx* ctx, int on);
  * at the latest when a call reads or changes that state. Outputs, events and statistics are the
  * same as with the option off; per-layer event timings are not taken in such steps (the in-kernel
  * window still is). A step of one sequence in the default geometry is one cooperative kernel over all SMs (not with timing or an
- * attention stand-in set, nor for fp32 models of one or two layers). On the batched tensor-core path the wave plan (token rows sorted by expert,
+ * attention stand-in set, nor for fp32 models of one or two layers, nor where the compute stream may not use all SMs). It begins when every SM
+ * is free of other streams' kernels and holds them all to its end; off, or with spm_set_ffn_ctas, the kernels share the device. On the batched tensor-core path the wave plan (token rows sorted by expert,
  * work units, combine map) is then built by a kernel instead of the host.
  * spm_cache_reset() ends the state; it is re-entered once the pools are full again. */
 int spm_set_host_free(spm_ctx* ctx, int on);

@@ -154,7 +154,7 @@ struct spm_ctx {
     unsigned long long* step_hx = nullptr;
     uint32_t step_tag = 1;                    // tag of the next launch's first layer
     bool step_clean = false;                  // no other kernel has written the partial rows since the last such step
-    bool coop = false;                        // the device takes cooperative launches
+    bool coop = false;                        // all of its CTAs can be running at once
     std::vector<std::vector<int32_t>> prev_rank;   // Naive Prefetch: experts the preceding step used, per layer
     std::vector<std::vector<int32_t>> pending_protect;
     std::vector<uint8_t> has_plan;
@@ -1369,35 +1369,40 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
     return SPM_OK;
 }
 
+struct ResidentKernel { void (*kern)(StepArgs); int threads; cudaError_t (*allow_smem)(); };
 template <typename WT, int NSEG, bool Q4>
-cudaError_t launch_resident_t(const StepArgs& a, int G, size_t smem, cudaStream_t st) {
-    constexpr auto kern = resident_step_kernel<WT, NSEG, Q4>;
-    if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
+ResidentKernel resident_kernel_t() { return {resident_step_kernel<WT, NSEG, Q4>, step_warps(NSEG, Q4) * 32, allow_full_smem<resident_step_kernel<WT, NSEG, Q4>>}; }
+template <typename WT, bool Q4>
+ResidentKernel resident_kernel_seg(int nseg) {
+    switch (nseg) {
+        case 1: return resident_kernel_t<WT, 1, Q4>();
+        case 2: return resident_kernel_t<WT, 2, Q4>();
+        case 3: return resident_kernel_t<WT, 3, Q4>();
+        case 4: return resident_kernel_t<WT, 4, Q4>();
+        case 5: return resident_kernel_t<WT, 5, Q4>();
+        case 6: return resident_kernel_t<WT, 6, Q4>();
+        case 7: return resident_kernel_t<WT, 7, Q4>();
+        default: return resident_kernel_t<WT, 8, Q4>();
+    }
+}
+ResidentKernel resident_kernel(const spm_ctx* c) {
+    return c->cfg.dtype == SPM_DTYPE_FP32 ? resident_kernel_seg<float, false>(c->nseg)
+         : c->cfg.dtype == SPM_DTYPE_BF16 ? resident_kernel_seg<bf16_t, false>(c->nseg) : resident_kernel_seg<bf16_t, true>(c->nseg);
+}
+cudaError_t launch_resident(const spm_ctx* c, const StepArgs& a, int G, size_t smem) {
+    const ResidentKernel k = resident_kernel(c);
+    if (cudaError_t e = k.allow_smem(); e != cudaSuccess) return e;
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(G);
-    lc.blockDim = dim3(step_warps(NSEG, Q4) * 32);
+    lc.blockDim = dim3(k.threads);
     lc.dynamicSmemBytes = smem;
-    lc.stream = st;
+    lc.stream = c->compute;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;      // the CTAs wait for one another
     at[0].val.cooperative = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, kern, a);
-}
-template <typename WT, bool Q4>
-cudaError_t launch_resident_seg(int nseg, const StepArgs& a, int G, size_t smem, cudaStream_t st) {
-    switch (nseg) {
-        case 1: return launch_resident_t<WT, 1, Q4>(a, G, smem, st);
-        case 2: return launch_resident_t<WT, 2, Q4>(a, G, smem, st);
-        case 3: return launch_resident_t<WT, 3, Q4>(a, G, smem, st);
-        case 4: return launch_resident_t<WT, 4, Q4>(a, G, smem, st);
-        case 5: return launch_resident_t<WT, 5, Q4>(a, G, smem, st);
-        case 6: return launch_resident_t<WT, 6, Q4>(a, G, smem, st);
-        case 7: return launch_resident_t<WT, 7, Q4>(a, G, smem, st);
-        case 8: return launch_resident_t<WT, 8, Q4>(a, G, smem, st);
-    }
-    return cudaErrorInvalidValue;
+    return cudaLaunchKernelEx(&lc, k.kern, a);
 }
 
 // Shared memory of resident_step_kernel: the GEMV's ring first, as deep as the routing arrays leave room for. False where they
@@ -1421,6 +1426,34 @@ bool resident_shape(const spm_ctx* c, int G, StepArgs* a, size_t* smem) {
             a->xs_in_ring = in_ring;
             if (*smem <= kFfnSmemLimit - 1024) return true;
         }
+    return false;
+}
+
+// SMs that kernels of a stream may use: those of its green context, if it belongs to one
+int sms_of_stream(cudaStream_t st, int all) {
+    CUgreenCtx green = nullptr;
+    CUdevResource res{};
+    void *get_ctx = nullptr, *get_res = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuStreamGetGreenCtx", &get_ctx, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess ||
+        cudaGetDriverEntryPoint("cuGreenCtxGetDevResource", &get_res, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        return all;
+    }
+    if (reinterpret_cast<decltype(&cuStreamGetGreenCtx)>(get_ctx)(reinterpret_cast<CUstream>(st), &green) != CUDA_SUCCESS || !green) return all;
+    if (reinterpret_cast<decltype(&cuGreenCtxGetDevResource)>(get_res)(green, &res, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return all;
+    return std::min(all, int(res.sm.smCount));
+}
+// Whether every CTA of the one-kernel step can be running at once on the compute stream
+bool resident_step_fits(const spm_ctx* c) {
+    int dev = 0, coop = 0, per_sm = 0;
+    StepArgs a{};
+    size_t smem = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return false;
+    if (sms_of_stream(c->compute, c->num_sms) < c->num_sms || !resident_shape(c, c->num_sms, &a, &smem)) return false;
+    const ResidentKernel k = resident_kernel(c);
+    if (k.allow_smem() == cudaSuccess && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.kern, k.threads, smem) == cudaSuccess) return per_sm >= 1;
+    cudaGetLastError();
     return false;
 }
 
@@ -1474,10 +1507,11 @@ int enqueue_resident_step(spm_ctx* c, const float* h_in, float* h_out, int slot,
     if (c->step_tag > 0xffffffffu - 2u * m.n_layers) c->step_tag = 1;        // (the words hold tags of the last two layers)
     a.tag0 = c->step_tag;
     c->step_tag += m.n_layers;
-    const cudaError_t launched = m.dtype == SPM_DTYPE_FP32 ? launch_resident_seg<float, false>(c->nseg, a, G, smem, c->compute)
-                               : m.dtype == SPM_DTYPE_BF16 ? launch_resident_seg<bf16_t, false>(c->nseg, a, G, smem, c->compute)
-                                                           : launch_resident_seg<bf16_t, true>(c->nseg, a, G, smem, c->compute);
-    CU(c, launched);
+    if (launch_resident(c, a, G, smem) != cudaSuccess) {         // not here, then: the separate launches take over (and report what is not of this launch)
+        cudaGetLastError();
+        c->coop = false;
+        return SPM_OK;
+    }
     c->kernel_launches++;
     c->ffn_launches += m.n_layers;
     *done = true;
@@ -1631,8 +1665,6 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     cudaGetDevice(&dev);
     cudaDeviceProp prop{};
     if (cudaGetDeviceProperties(&prop, dev) == cudaSuccess) c->num_sms = prop.multiProcessorCount;
-    int coop = 0;
-    c->coop = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop;
     if (prop.major != 10) { c->err = "this library is built for sm_100a (B200) only"; return bail(SPM_ERR_CONFIG); }
 
     unsigned char* base = static_cast<unsigned char*>(b->arena);
@@ -1732,6 +1764,7 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
         if (!cu(cudaEventCreate(&c->ring_start[i]), "cudaEventCreate") || !cu(cudaEventCreate(&c->ring_end[i]), "cudaEventCreate")) return bail(SPM_ERR_CUDA);
     if (!cu(cudaStreamSynchronize(c->compute), "cudaStreamSynchronize")) return bail(SPM_ERR_CUDA);
 
+    c->coop = c->S >= cfg->n_experts && resident_step_fits(c);
     c->clock_kind.assign(kClockSlots, kClkFfn);
     if (arm_clock(c) != SPM_OK) return bail(SPM_ERR_CUDA);
     c->budget = budget < 0 ? 1 : budget;

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 import synth
+from paper_2607_24787_b200 import binding as B
 from paper_2607_24787_b200.binding import SpmError
 from test_gpu_host_free import build, preload, rows, run
 
@@ -175,3 +176,41 @@ def test_expert_without_a_slot_is_reported(name):
     m.synchronize()
     assert torch.equal(got, want)
     m.close()
+
+
+def test_compute_stream_that_may_not_use_all_sms():
+    """Where the CTAs of the one-kernel step cannot all be running at once, the step is separate launches with the same bits."""
+    cu = pytest.importorskip("cuda.bindings.driver")
+
+    def ok(result):
+        if result[0] != cu.CUresult.CUDA_SUCCESS:
+            pytest.skip(f"no green contexts here: {result[0]}")
+        return result[1] if len(result) > 1 else None
+
+    cfg = config("bf16_nine_warps")
+    H = torch.as_tensor(rows(cfg, 3), dtype=torch.float32).cuda()
+    m = build(cfg, store_layers=1)
+    preload(cfg, m)
+    torch.cuda.synchronize()
+    want = [m.decode_step(h) for h in H]
+    m.synchronize()
+    assert m.stats()["kernel_launches"] == 3
+    dev = ok(cu.cuDeviceGet(torch.cuda.current_device()))
+    sms = ok(cu.cuDeviceGetDevResource(dev, cu.CUdevResourceType.CU_DEV_RESOURCE_TYPE_SM))
+    part = ok(cu.cuDevSmResourceSplitByCount(1, sms, 0, 72))
+    green = ok(cu.cuGreenCtxCreate(ok(cu.cuDevResourceGenerateDesc(part, 1)), dev, cu.CUgreenCtxCreate_flags.CU_GREEN_CTX_DEFAULT_STREAM))
+    stream = ok(cu.cuGreenCtxStreamCreate(green, cu.CUstream_flags.CU_STREAM_NON_BLOCKING, 0))
+    ptr = [t.data_ptr() if t is not None else None for t in m._keep[:5]]
+    B.spm_destroy(m.ctx)
+    m.ctx = B.spm_init(m.cfg, m.slots, 0, B.Buffers(*ptr, m.store.ptr, (m.arena.data_ptr() + 255) // 256 * 256, m.arena.numel() - 256,
+                                                    int(stream), m.copy.cuda_stream, 1))
+    preload(cfg, m)
+    got = [m.decode_step(h) for h in H]
+    m.synchronize()
+    st = m.stats()
+    assert st["host_free_steps"] == 3 and st["kernel_launches"] == 3 * (2 * cfg.n_layers + 1)
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    m.close()
+    ok(cu.cuStreamDestroy(stream))
+    ok(cu.cuGreenCtxDestroy(green))
