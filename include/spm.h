@@ -316,7 +316,8 @@ int spm_set_event_log_limit(spm_ctx* ctx, size_t max_events);
 int spm_set_deadline_ms(spm_ctx* ctx, int ms);
 /* Limit of every wait inside the expert kernels (for a weight copy to land in shared memory, for an
  * arrival counter with spm_set_device_wait, for a pipeline barrier of the grouped kernels), in
- * microseconds; 0 restores the default of 2 s. A wait that runs out sets a status bit, the kernel
+ * microseconds; 0 restores the default of 2 s (30 s for the start of a one-kernel step, which other streams' kernels may hold up). The
+ * CTAs of a one-kernel step wait for one another under the same limit. A wait that runs out sets a status bit, the kernel
  * winds down (no copy left in flight, tensor memory released) and returns; the next
  * spm_synchronize / spm_get_stats reports SPM_ERR_TIMEOUT once and the context stays usable
  * (spm_cache_reset brings slot table and arrival counters back to a known state). */

@@ -36,9 +36,10 @@ namespace spm {
 // Warps of a CTA: as many as the GEMV may take (those it does not use only route). Rows of 9216 bytes and more leave it eight at most,
 // whose threads then have 255 registers.
 constexpr int step_warps(int nseg, bool q4) { return q4 ? q4_warps(nseg) : nseg >= 6 ? 8 : kFfnMaxWarps; }
+constexpr int kStatusStepTimeout = 16;            // status bit (1 to 8: expert and routing kernels)
 constexpr int kStepCols = 16;                     // columns of the hidden row that an owner adds up
 constexpr int kStepMaxCtas = kReduceGroupsR * kReduceChunkR;
-constexpr unsigned long long kStepStartNs = 30000000000ull;     // limit of the first exchange: kernels of other streams may hold SMs until then
+constexpr unsigned long long kStepStartNs = 30000000000ull;     // default limit of the first exchange: kernels of other streams may hold SMs until then
 
 struct StepArgs {
     const float* h_in;              // [D]
@@ -90,7 +91,7 @@ struct StepSpin {
     int polls = 0;
     __device__ StepSpin(const StepArgs& args, unsigned long long limit_ns) : a(args), limit(limit_ns) {}
     __device__ __forceinline__ bool give_up() {
-        if ((++polls & 63) != 0) return false;
+        if ((++polls & 15) != 0) return false;          // (a poll takes half a microsecond; the exchanges some three)
         unsigned flag;
         asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(flag) : "l"(a.abort_word) : "memory");
         if (flag == a.tag0) return true;
@@ -101,7 +102,7 @@ struct StepSpin {
         return true;
     }
     static __device__ __forceinline__ void raise(const StepArgs& a) {
-        atomicOr(a.status, kStatusCopyTimeout);
+        atomicOr(a.status, kStatusStepTimeout);
         asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(a.abort_word), "r"(a.tag0) : "memory");
     }
 };
@@ -342,7 +343,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
                 }
         }
         for (int i = tid; i < rows; i += kStepThreads) {
-            StepSpin spin(a, l == 0 ? max(limit, kStepStartNs) : limit);
+            StepSpin spin(a, l == 0 && !a.wait_limit_ns ? kStepStartNs : limit);
             unsigned long long w;
             while (uint32_t((w = ll_load(a.zx + i * a.z_stride)) >> 32) != tag)
                 if (spin.give_up()) { dead = 1; break; }

@@ -1597,6 +1597,7 @@ int check_status(spm_ctx* c) {
     if (st & kStatusCopyTimeout) return fail(c, SPM_ERR_TIMEOUT, "expert FFN kernel gave up waiting for a weight copy");
     if (st & kStatusBadSlot) return fail(c, SPM_ERR_NOT_RESIDENT, "expert FFN kernel received a slot number outside the pool");
     if (st & kStatusGroupedTimeout) return fail(c, SPM_ERR_TIMEOUT, "grouped expert FFN kernel gave up waiting on a pipeline barrier");
+    if (st & kStatusStepTimeout) return fail(c, SPM_ERR_TIMEOUT, "a step's kernel gave up waiting for a weight copy or for another of its CTAs");
     if (st & kStatusNonFinite) return fail(c, SPM_ERR_NUMERIC, "a routing kernel met a non-finite logit (NaN or Inf in the hidden rows or the weights)");
     return SPM_OK;
 }

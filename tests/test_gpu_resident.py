@@ -214,3 +214,47 @@ def test_compute_stream_that_may_not_use_all_sms():
     m.close()
     ok(cu.cuStreamDestroy(stream))
     ok(cu.cuGreenCtxDestroy(green))
+
+
+# many experts of a few rows: with the routing weights in host memory a layer's logits take tens of microseconds to arrive
+SLOW = {
+    "fp32": dict(base="tiny", hidden=1024, n_experts=900, inter=8, top_k=4, adapter_rank=16),
+    "bf16_shared": dict(base="dsvl2", hidden=1280, n_experts=900, inter=40, top_k=4, n_shared=2, adapter_rank=16),
+    "bf16_widest": dict(base="qwen3", hidden=2048, n_experts=700, inter=16, top_k=8, adapter_rank=16),
+    "q4": dict(base="qwen3_q4", hidden=2048, n_experts=700, inter=64, top_k=8, adapter_rank=16),
+}
+
+
+@pytest.mark.parametrize("name", list(SLOW))
+def test_exchange_that_runs_out(name):
+    """A limit of a microsecond, and logits that take longer: the CTAs give up, with rows of shared experts on their way in one case, the host reads
+    the time-out once, and the next step has the bits of any other."""
+    kw = dict(SLOW[name])
+    cfg = synth.get_config(kw.pop("base"), n_layers=3, slots=kw["n_experts"], budget=2, batch=1, **kw)
+    m = build(cfg, store_layers=1)
+    preload(cfg, m)
+    h = torch.as_tensor(rows(cfg, 1)[0], dtype=torch.float32).cuda()
+    torch.cuda.synchronize()
+    want = m.decode_step(h)
+    m.synchronize()
+    slow = m._keep[1].cpu().pin_memory()
+    ptr = [t.data_ptr() if t is not None else None for t in m._keep[:5]]
+    B.spm_destroy(m.ctx)
+    m.ctx = B.spm_init(m.cfg, m.slots, 0, B.Buffers(ptr[0], slow.data_ptr(), *ptr[2:], m.store.ptr, (m.arena.data_ptr() + 255) // 256 * 256,
+                                                    m.arena.numel() - 256, m.compute.cuda_stream, m.copy.cuda_stream, 1))
+    preload(cfg, m)
+    for _ in range(2):
+        got = m.decode_step(h)
+        m.synchronize()
+        assert torch.equal(got, want)
+        m.set_device_wait_limit_us(1)
+        m.decode_step(h)
+        with pytest.raises(SpmError) as e:
+            m.synchronize()
+        assert e.value.code == -4 and "another of its CTAs" in str(e.value)
+        m.synchronize()                         # reported once
+        m.set_device_wait_limit_us(0)
+    got = m.decode_step(h)
+    m.synchronize()
+    assert torch.equal(got, want) and m.stats()["kernel_launches"] == 5
+    m.close()
