@@ -160,8 +160,13 @@ def _ptr(x):
         return x
     if isinstance(x, np.ndarray):
         assert x.flags["C_CONTIGUOUS"]
-        # (x.ctypes builds an object: 1.0 us against 0.3, seven times a layer in the stand-alone calls)
-        return C.addressof(_NO_BYTES.from_buffer(x)) if x.flags.writeable else x.ctypes.data
+        if x.flags.writeable:
+            # (x.ctypes builds an object: 1.0 us against 0.3, seven times a layer in the stand-alone calls)
+            try:
+                return C.addressof(_NO_BYTES.from_buffer(x))
+            except (TypeError, ValueError):      # no buffer of this type (dates, extension types), or no bytes
+                pass
+        return x.ctypes.data
     assert x.is_contiguous()
     return x.data_ptr()
 

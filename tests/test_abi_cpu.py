@@ -271,3 +271,10 @@ def test_checkpoint_words_match_the_oracle_state_and_resume_identically():
     assert np.array_equal(resumed.export_state(), keep)
     for x in (sim, resumed):
         x.close()
+
+
+@pytest.mark.parametrize("array", [np.zeros(3, "datetime64[s]"), np.zeros((2, 0), np.int32), np.zeros(4, np.float16), np.zeros((), np.int64)])
+def test_addresses_of_arrays_of_any_type(array):
+    for writeable in (True, False):
+        array.flags.writeable = writeable
+        assert B._ptr(array) == array.ctypes.data
