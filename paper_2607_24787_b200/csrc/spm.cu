@@ -153,7 +153,8 @@ struct spm_ctx {
     // one sequence: the whole host-free step as one cooperative kernel
     unsigned long long* step_hx = nullptr;
     uint32_t step_tag = 1;                    // tag of the next launch's first layer
-    bool step_clean = false;                  // no other kernel has written the partial rows since the last such step
+    bool step_clean = false;                  // nothing else has written the partial rows or the exchange since the last such step
+    bool clock_dirty = false;                 // such a step has written clock slots since they were armed
     bool coop = false;                        // all of its CTAs can be running at once
     std::vector<std::vector<int32_t>> prev_rank;   // Naive Prefetch: experts the preceding step used, per layer
     std::vector<std::vector<int32_t>> pending_protect;
@@ -218,8 +219,11 @@ size_t blob_bytes_of(const spm_model_cfg* m) {
 }
 
 constexpr int kMaxCtasBatch1 = 296;
-constexpr int kClockSlots = 8192;     // in-kernel {start, end} pairs between two harvests
-constexpr size_t kStepExchangeBytes = 65536;     // resident_step_kernel: hidden row, logits and adapter rows as 8-byte words, abort word
+constexpr int kClockSlots = 12288;    // in-kernel {start, end} pairs between two harvests
+// resident_step_kernel's exchange (hidden row, logits and adapter rows as 8-byte words, abort word) lies in the last of them: slots are
+// handed out with timing on, that kernel runs with timing off
+constexpr size_t kStepExchangeBytes = 65536;
+constexpr int kClockSlotsBeforeStep = kClockSlots - int(kStepExchangeBytes / 16);
 constexpr int kDescRing = 8;          // wave descriptors in flight for the batched tensor-core path
 constexpr int kTraceRing = 8;         // host-free steps whose bookkeeping may be outstanding
 static_assert(sizeof(GgTask) == sizeof(GgTaskHost), "host plan and device task share one layout");
@@ -290,7 +294,6 @@ struct Carve {
 
 struct Layout {
     size_t pools, slot_gen, x, logits, pihat, w, scores, partial, h, ids, order, clock, slot_map, codes, counters, status, total;
-    size_t step;                                                                   // exchange buffers of resident_step_kernel
     size_t mt_map;                                                                 // several-sequences kernel only
     size_t tc_xs, tc_wrow, tc_desc, tc_n_units, tc_act, tc_ready;       // batched tensor-core path only
     size_t desc_bytes, off_rows, off_rowmap, off_chunks, chunk_cap, off_wait;
@@ -335,7 +338,6 @@ Layout layout_of(const spm_model_cfg* m, int S, bool with_multi = true) {
     l.ids = c.take(nb * SPM_MAX_TOPK * 4);
     l.order = c.take(n * 4);
     l.clock = c.take(size_t(kClockSlots) * 16);
-    l.step = c.take(kStepExchangeBytes);
     l.slot_map = c.take(size_t(m->n_layers) * n * sizeof(short));
     l.codes = c.take(size_t(m->n_layers) * nb * SPM_MAX_TOPK * sizeof(short));
     if (l.tc) {
@@ -808,6 +810,12 @@ int harvest_clock(spm_ctx* c) {
 int take_clock(spm_ctx* c, ClockKind kind, unsigned long long** out) {
     *out = nullptr;
     if (!c->timing) return SPM_OK;
+    if (c->clock_dirty) {
+        std::vector<unsigned long long> h(kStepExchangeBytes / 8);
+        for (size_t i = 0; i < h.size(); i += 2) { h[i] = ~0ull; h[i + 1] = 0; }
+        CU(c, cudaMemcpyAsync(c->step_hx, h.data(), kStepExchangeBytes, cudaMemcpyHostToDevice, c->compute));      // (pageable: staged before it returns)
+        c->clock_dirty = c->step_clean = false;
+    }
     if (c->clock_used == kClockSlots) if (int rc = harvest_clock(c)) return rc;
     c->clock_kind[c->clock_used] = kind;
     *out = c->ws_clock + 2 * size_t(c->clock_used++);
@@ -819,6 +827,7 @@ int arm_clock(spm_ctx* c) {   // whole ring to {max, 0}
     for (int i = 0; i < kClockSlots; ++i) { h[2 * i] = ~0ull; h[2 * i + 1] = 0; }
     CU(c, cudaMemcpy(c->ws_clock, h.data(), h.size() * 8, cudaMemcpyHostToDevice));
     c->clock_used = 0;
+    c->clock_dirty = c->step_clean = false;
     return SPM_OK;
 }
 
@@ -1498,6 +1507,8 @@ int enqueue_resident_step(spm_ctx* c, const float* h_in, float* h_out, int slot,
     a.I = m.inter; a.K = m.top_k; a.n = m.n_experts; a.r = m.adapter_rank; a.L = m.n_layers; a.n_slots = c->S; a.n_shared = m.n_shared;
     a.renorm = m.renormalize; a.predict = predict;
     a.eps = m.rms_eps;
+    if (c->clock_used > kClockSlotsBeforeStep) if (int rc = harvest_clock(c)) return rc;
+    c->clock_dirty = true;
     if (!c->step_clean) {           // words of other kernels (or of the memory's last owner) could carry a tag
         CU(c, cudaMemsetAsync(a.part, 0, size_t(G) * m.hidden * 8, c->compute));
         CU(c, cudaMemsetAsync(a.hx, 0, kStepExchangeBytes, c->compute));
@@ -1685,7 +1696,7 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
     c->ws_ids = reinterpret_cast<int32_t*>(base + lay.ids);
     c->ws_order = reinterpret_cast<int32_t*>(base + lay.order);
     c->ws_clock = reinterpret_cast<unsigned long long*>(base + lay.clock);
-    c->step_hx = reinterpret_cast<unsigned long long*>(base + lay.step);
+    c->step_hx = c->ws_clock + 2 * size_t(kClockSlotsBeforeStep);
     c->ws_slot_map = reinterpret_cast<short*>(base + lay.slot_map);
     c->ws_codes = reinterpret_cast<short*>(base + lay.codes);
     c->ws_counters = reinterpret_cast<unsigned*>(base + lay.counters);

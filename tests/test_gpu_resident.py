@@ -258,3 +258,30 @@ def test_exchange_that_runs_out(name):
     m.synchronize()
     assert torch.equal(got, want) and m.stats()["kernel_launches"] == 5
     m.close()
+
+
+def test_clock_slots_and_exchange_share_memory():
+    """More timed launches than there are clock slots ahead of the exchange, then one-kernel steps, and both again: no window is lost to the
+    other's words and no word to a window."""
+    cfg = config("fp32_smallest")
+    m = build(cfg, store_layers=1)
+    preload(cfg, m)
+    h = torch.as_tensor(rows(cfg, 1)[0], dtype=torch.float32).cuda()
+    torch.cuda.synchronize()
+    want = m.decode_step(h)
+    m.synchronize()
+    steps = 8192 // (2 * cfg.n_layers + 1) + 100
+    m.reset_stats()
+    for done in (1, 2):
+        m.set_timing(1)
+        for _ in range(steps):
+            m.decode_step(h)
+        m.set_timing(0)
+        got = m.decode_step(h)
+        m.synchronize()
+        assert torch.equal(got, want)
+        st = m.stats()
+        assert st["kernel_launches"] == done * (steps * (2 * cfg.n_layers + 1) + 1)
+        for key in ("ffn_window_us", "router_window_us"):
+            assert 0.5 < st[key] / (done * steps * cfg.n_layers) < 100, key
+    m.close()
