@@ -327,6 +327,10 @@ int spm_set_device_wait_limit_us(spm_ctx* ctx, int us);
  * so), so the kernel that waits for that batch gives up after the limit. Nothing on the GPU
  * faults or hangs. Cleared by spm_cache_reset. */
 int spm_test_withhold_arrivals(spm_ctx* ctx, int count);
+/* For tests of the two kernels that a batch of 4-bit experts may take on the tensor-core path: choice 0 leaves it to the rule on the call's
+ * size, 1 / 2 take the tcgen05 / mma.sync kernel (2: where its shape allows), a negative one changes nothing. launches (may be NULL)
+ * receives how often each has been launched since spm_init. */
+int spm_test_grouped_q4(spm_ctx* ctx, int choice, uint64_t launches[2]);
 
 /* Profile the overlap window (Section 3.3): window_us = median device time of the expert FFN of
  * one layer at max_batch tokens with every needed expert resident (kernel(s) + combine, the same

@@ -98,6 +98,7 @@ _SIG = {
     "spm_set_device_wait_limit_us": [_P, C.c_int],
     "spm_set_event_log_limit": [_P, C.c_size_t],
     "spm_test_withhold_arrivals": [_P, C.c_int],
+    "spm_test_grouped_q4": [_P, C.c_int, _P],
     "spm_cache_reset": [_P],
     "spm_reset_stats": [_P],
     "spm_get_stats": [_P, C.POINTER(Stats)],
@@ -356,6 +357,12 @@ def spm_set_device_wait_limit_us(ctx, us):
 
 def spm_test_withhold_arrivals(ctx, count):
     _check(load().spm_test_withhold_arrivals(ctx, count), ctx)
+
+
+def spm_test_grouped_q4(ctx, choice):
+    n = np.zeros(2, np.uint64)
+    _check(load().spm_test_grouped_q4(ctx, choice, _ptr(n)), ctx)
+    return n.tolist()
 
 
 def spm_cache_reset(ctx):

@@ -94,6 +94,8 @@ struct spm_ctx {
     std::vector<uint8_t> tc_desc_ev_valid;
     size_t tc_desc_pos = 0;
     uint64_t tc_launches = 0;
+    uint64_t q4_launches[2] = {0, 0};         // of ffn_grouped_q4_kernel, of ffn_grouped_q4_mma_kernel
+    int q4_choice = 0;                        // test hook: 0 the rule, 1 / 2 always the former / the latter
     // mailbox
     Mailbox* mb_host = nullptr;
     Mailbox* mb_dev = nullptr;
@@ -528,19 +530,21 @@ cudaError_t launch_grouped_q4_mma_t(const spm_ctx* c, const MqArgs& a) {
 // (of 22 shapes measured on both, the rule takes the slower one for two, by 4 and 5 %)
 bool grouped_q4_mma_pays(const spm_ctx* c, int nb) {
     const spm_model_cfg& m = c->cfg;
-    if (mq_max_tasks(nb, m.top_k, m.n_experts, c->n_jt, c->num_sms) > kMqMaxTasks) return false;
+    if (m.hidden < 512 || mq_max_tasks(nb, m.top_k, m.n_experts, c->n_jt, c->num_sms) > kMqMaxTasks) return false;      // (rows of 256: never worth it)
+    if (c->q4_choice) return c->q4_choice == 2;
     const double n = m.n_experts, used = n * (1.0 - std::pow(1.0 - m.top_k / n, nb)), tokens = double(nb) * m.top_k / used, seg = m.hidden / 256;
     auto rounds = [&](double work) { return std::ceil(work * c->n_jt / c->num_sms); };
     const double mma = rounds(used * std::max(1.0, (tokens + 3) / 8)) * (1.35 + 0.14 * seg);
     const double tc = rounds(used) * (0.2 + 0.49 * seg) * (1 + 0.5 * std::max(0.0, (std::min(tokens, 48.0) - 8) / 16));
     return mma < tc;
 }
-cudaError_t launch_grouped_q4(const spm_ctx* c, int nb, int grid, const GgArgs& a) {
+cudaError_t launch_grouped_q4(spm_ctx* c, int nb, int grid, const GgArgs& a) {
     const spm_model_cfg& m = c->cfg;
-    if (grouped_q4_mma_pays(c, nb)) {
+    const bool mma = grouped_q4_mma_pays(c, nb);
+    ++c->q4_launches[mma];
+    if (mma) {
         MqArgs q{c->pools, c->tc_xs, c->blob, a};
         switch (m.hidden / 256) {
-            case 1: return launch_grouped_q4_mma_t<1>(c, q);
             case 2: return launch_grouped_q4_mma_t<2>(c, q);
             case 3: return launch_grouped_q4_mma_t<3>(c, q);
             case 4: return launch_grouped_q4_mma_t<4>(c, q);
@@ -1555,7 +1559,7 @@ int enqueue_host_free_step(spm_ctx* c, const float* h_in, int nb, float* h_out) 
         if (!g && c->hf_warm && c->hf_graphs.size() < 64) {
             // (the first host-free step ran launch by launch, so every kernel attribute is already set)
             spm_ctx::HostFreeGraph ng{key, 0, 0, 0, nullptr};
-            const uint64_t k0 = c->kernel_launches, f0 = c->ffn_launches, t0 = c->tc_launches;
+            const uint64_t k0 = c->kernel_launches, f0 = c->ffn_launches, t0 = c->tc_launches, q0[2] = {c->q4_launches[0], c->q4_launches[1]};
             cudaGraph_t graph = nullptr;
             int rc = SPM_ERR_CUDA;
             cudaError_t ce = cudaStreamBeginCapture(c->compute, cudaStreamCaptureModeRelaxed);   // (fails on the legacy default stream)
@@ -1565,6 +1569,7 @@ int enqueue_host_free_step(spm_ctx* c, const float* h_in, int nb, float* h_out) 
             }
             ng.kernels = c->kernel_launches - k0; ng.ffns = c->ffn_launches - f0; ng.tcs = c->tc_launches - t0;
             c->kernel_launches = k0; c->ffn_launches = f0; c->tc_launches = t0;
+            c->q4_launches[0] = q0[0]; c->q4_launches[1] = q0[1];
             if (rc == SPM_OK && ce == cudaSuccess && graph && cudaGraphInstantiate(&ng.exec, graph, 0) == cudaSuccess) {
                 c->hf_graphs.push_back(ng);
                 g = &c->hf_graphs.back();
@@ -1577,6 +1582,7 @@ int enqueue_host_free_step(spm_ctx* c, const float* h_in, int nb, float* h_out) 
         if (g) {
             CU(c, cudaGraphLaunch(g->exec, c->compute));
             c->kernel_launches += g->kernels; c->ffn_launches += g->ffns; c->tc_launches += g->tcs;
+            if (m.dtype == SPM_DTYPE_Q4) c->q4_launches[g->tcs && grouped_q4_mma_pays(c, nb)] += g->tcs;
             done = true;
         }
     }
@@ -2047,6 +2053,17 @@ int spm_set_device_wait_limit_us(spm_ctx* c, int us) {
 int spm_test_withhold_arrivals(spm_ctx* c, int count) {
     if (!c || count < 0) return SPM_ERR_INVALID_ARG;
     c->withhold_arrivals = count;
+    return SPM_OK;
+}
+
+int spm_test_grouped_q4(spm_ctx* c, int choice, uint64_t launches[2]) {
+    if (!c || choice > 2) return SPM_ERR_INVALID_ARG;
+    if (choice >= 0 && choice != c->q4_choice) {
+        c->q4_choice = choice;
+        for (auto& g : c->hf_graphs) if (g.exec) cudaGraphExecDestroy(g.exec);       // (captured with the other choice)
+        c->hf_graphs.clear();
+    }
+    if (launches) std::copy(c->q4_launches, c->q4_launches + 2, launches);
     return SPM_OK;
 }
 

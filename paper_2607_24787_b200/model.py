@@ -163,6 +163,7 @@ class OffloadedMoE:
     def set_event_log_limit(self, n): B.spm_set_event_log_limit(self.ctx, n)
     def set_device_wait_limit_us(self, us): B.spm_set_device_wait_limit_us(self.ctx, us)
     def test_withhold_arrivals(self, count): B.spm_test_withhold_arrivals(self.ctx, count)
+    def test_grouped_q4(self, choice=-1): return B.spm_test_grouped_q4(self.ctx, choice)
     def cache_reset(self): B.spm_cache_reset(self.ctx)
     def check_invariants(self, with_device=True): B.spm_check_invariants(self.ctx, with_device)
     def cache_export(self): return B.spm_cache_export(self.ctx)

@@ -1,10 +1,13 @@
 """4-bit experts through mma.sync operands: the one-token kernel at the edges of its tiles against 64-bit sums, the batched kernel at
 the edges of its runs of tokens against the one-token kernel."""
+import time
+
 import numpy as np
 import pytest
 import torch
 
 import synth
+from paper_2607_24787_b200.binding import SpmError
 from test_gpu_edges import build
 
 pytestmark = pytest.mark.gpu
@@ -275,4 +278,120 @@ def test_one_token_device_side_wait_gives_the_same_bits(shape):
         runs.append((torch.stack(out), m.events()))
     assert torch.equal(runs[0][0], runs[1][0]) and runs[0][1] == runs[1][1]
     assert m.stats()["misses"] > 0
+    m.close()
+
+
+def moe(m, x, ids, w):
+    got = torch.zeros_like(x)
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, got)
+    m.synchronize()
+    return got
+
+
+# every split of the columns over warps that the mma.sync kernel has (hidden 512 to 2048), tokens an expert from one to 64 on both kernels
+BOTH = {f"hidden_{h}": (h, 256, 6, 2, 24) for h in range(512, 2049, 256)}
+BOTH |= {"wide_rows_many_tokens": (2048, 768, 24, 8, 64), "few_experts": (2048, 1024, 12, 8, 64), "deep": (1024, 1152, 12, 3, 17), "one_token_an_expert": (768, 384, 128, 3, 7)}
+
+
+@pytest.mark.parametrize("name", list(BOTH))
+def test_both_batched_kernels(name):
+    """The same call through each of the two kernels, and both against the roundings restated in 64 bits (see test_batched_kernels_round_alike)."""
+    hidden, inter, n, k, nb = BOTH[name]
+    cfg = make(hidden, inter, n, k, batch=nb)
+    m = build(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    x = torch.randn(nb, hidden, generator=gen, device="cuda")
+    torch.cuda.synchronize()
+    _, ids, w, _ = m.router_topk(0, torch.randn(nb, hidden, generator=gen, device="cuda"))
+    want = rounded(cfg, x, ids, w)
+    for choice in (1, 2):
+        m.test_grouped_q4(choice)
+        got = moe(m, x, ids, w)
+        assert m.test_grouped_q4() == [1, choice - 1]
+        assert (got.double() - want).norm() <= 3e-4 * want.norm(), choice
+    m.close()
+
+
+def test_every_number_of_tokens_an_expert_on_both_kernels():
+    """Experts with 64, 47, 33, 17, 16, 14 and 1 tokens in one launch, in narrow rows and in the widest."""
+    counts = [64, 47, 33, 17, 16, 14, 1, 0]
+    for hidden in (512, 2048):
+        cfg = make(hidden, 256, 8, 3, batch=64)
+        m = build(cfg)
+        gen = torch.Generator(device="cuda").manual_seed(10)
+        x = torch.randn(64, hidden, generator=gen, device="cuda")
+        w = torch.rand(64, 3, generator=gen, device="cuda") + 0.1
+        left, ids = list(counts), np.zeros((64, 3), np.int32)
+        for t in range(64):                # the experts with the most tokens left, no expert twice a token
+            for k, e in enumerate(sorted(range(8), key=lambda e: -left[e])[:3]):
+                ids[t, k] = e
+                left[e] -= 1
+        assert sorted(np.bincount(ids.reshape(-1), minlength=8).tolist()) == sorted(counts)
+        want = rounded(cfg, x, ids, w)
+        for choice in (1, 2):
+            m.test_grouped_q4(choice)
+            got = moe(m, x, ids, w)
+            assert ((got.double() - want).norm(dim=1) <= 2e-3 * want.norm(dim=1)).all(), (hidden, choice)
+        assert m.test_grouped_q4() == [1, 1]
+        m.close()
+
+
+@pytest.mark.parametrize("choice", [1, 2])
+def test_waves_and_host_free_steps_on_both_kernels(choice):
+    """A small cache (waves, copies, device-side waits) and a context that holds every expert give the same bits, launched and replayed."""
+    cfg = make(768, 384, 12, 4, batch=9, layers=3)
+    h = torch.randn(3, 9, cfg.hidden, generator=torch.Generator(device="cuda").manual_seed(11), device="cuda")
+    outs = []
+    for slots, wait in ((5, 0), (5, 1), (12, 0)):
+        m = build(cfg.replace(slots=slots))
+        m.test_grouped_q4(choice)
+        m.set_device_wait(wait)
+        torch.cuda.synchronize()
+        o = [m.decode_step(row) for row in h] + [m.decode_step(h[0]) for _ in range(20)]       # (captured per trace slot: the last ones are replays)
+        m.synchronize()
+        outs.append(torch.stack(o))
+        ran = m.test_grouped_q4()
+        assert ran[2 - choice] == 0 and ran[choice - 1] >= 23 * cfg.n_layers
+        m.close()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
+GIVE_UP = {          # (shape, slots, batch, batched kernel)
+    "one_token": ((1280, 896, 16, 6, 2), 8, 1, 0), "one_token_widest": ((2048, 333, 16, 4), 5, 1, 0),
+    "batched_mma": ((2048, 256, 12, 8), 8, 16, 2), "batched_tcgen05": ((2048, 256, 12, 8), 8, 16, 1),
+}
+
+
+@pytest.mark.parametrize("name", list(GIVE_UP))
+def test_wait_for_a_copy_runs_out(name):
+    """An arrival that is never published (withheld on the host; the bytes land): the kernel gives up after its limit with nothing in flight, the
+    host reads the time-out once, and after a cache reset the context gives the bits of before."""
+    shape, slots, nb, choice = GIVE_UP[name]
+    cfg = make(*shape, batch=nb, layers=2).replace(slots=slots)
+    h = torch.randn(2, nb, cfg.hidden, generator=torch.Generator(device="cuda").manual_seed(12), device="cuda")
+    m = build(cfg)
+    m.set_policy("on_demand")
+    m.test_grouped_q4(choice)
+    torch.cuda.synchronize()
+    want = [m.decode_step(row) for row in h]
+    m.synchronize()
+    assert m.test_grouped_q4()[2 - choice if choice else 0] == 0 and (nb == 1 or sum(m.test_grouped_q4()) > 0)
+    m.set_device_wait(1)
+    for withheld in (1, 2):
+        m.set_device_wait_limit_us(3000)
+        m.cache_reset()
+        m.test_withhold_arrivals(withheld)
+        t0 = time.perf_counter()
+        with pytest.raises(SpmError) as e:
+            m.decode_step(h[0])
+            m.synchronize()
+        assert e.value.code == -4 and time.perf_counter() - t0 < 1.9        # after the limit, not the 2 s default
+        m.synchronize()                                                     # reported once
+        m.set_device_wait_limit_us(0)
+        m.cache_reset()
+        got = [m.decode_step(row) for row in h]
+        m.synchronize()
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
     m.close()
