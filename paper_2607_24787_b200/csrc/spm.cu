@@ -1511,6 +1511,8 @@ int enqueue_resident_step(spm_ctx* c, const float* h_in, float* h_out, int slot,
     a.I = m.inter; a.K = m.top_k; a.n = m.n_experts; a.r = m.adapter_rank; a.L = m.n_layers; a.n_slots = c->S; a.n_shared = m.n_shared;
     a.renorm = m.renormalize; a.predict = predict;
     a.eps = m.rms_eps;
+    // (tags start over on a cleared exchange: words of adapter rows may be as old as the last step that predicted)
+    if (c->step_tag > 0xffffffffu - 2u * m.n_layers) c->step_clean = false;
     if (c->clock_used > kClockSlotsBeforeStep) if (int rc = harvest_clock(c)) return rc;
     c->clock_dirty = true;
     if (!c->step_clean) {           // words of other kernels (or of the memory's last owner) could carry a tag
@@ -1519,7 +1521,6 @@ int enqueue_resident_step(spm_ctx* c, const float* h_in, float* h_out, int slot,
         c->step_tag = 1;
         c->step_clean = true;
     }
-    if (c->step_tag > 0xffffffffu - 2u * m.n_layers) c->step_tag = 1;        // (the words hold tags of the last two layers)
     a.tag0 = c->step_tag;
     c->step_tag += m.n_layers;
     if (launch_resident(c, a, G, smem) != cudaSuccess) {         // not here, then: the separate launches take over (and report what is not of this launch)
