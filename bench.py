@@ -172,9 +172,13 @@ def config_block(cfg, args):
             "l2": "inputs larger than L2: every layer streams its own slot pool, 3.6 GB of weights per step"}
 
 
-def ffn_kernel_name(cfg):
+def ffn_kernel_name(cfg, m):
+    """The expert kernel of cfg's batches on context m (4-bit batches: the one that it has launched most, see spm_test_grouped_q4)."""
     if cfg.batch > 1 and cfg.n_shared == 0 and cfg.dtype in ("bf16", "q4"):
-        return "ffn_grouped_q4_mma_kernel" if cfg.dtype == "q4" else "ffn_grouped_kernel"
+        if cfg.dtype == "bf16":
+            return "ffn_grouped_kernel"
+        tcgen05, mma = m.test_grouped_q4()
+        return "ffn_grouped_q4_mma_kernel" if mma >= tcgen05 else "ffn_grouped_q4_kernel"
     if cfg.dtype == "q4":
         return "ffn_gemv_q4_kernel"
     return "ffn_gemv_kernel"
@@ -316,7 +320,7 @@ def run_ours(args):
     # duration of an HBM-streaming kernel on this machine; `isolated` (below, when the
     # resident leg runs) times the same entry point with no PCIe traffic.
     result["roofline"] = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                          "traffic": NCU_DRAM_BYTES_PER_LAUNCH.get(cfg.name), "kernel": ffn_kernel_name(cfg),
+                          "traffic": NCU_DRAM_BYTES_PER_LAUNCH.get(cfg.name), "kernel": ffn_kernel_name(cfg, m),
                           "peak_source": f"of {which}", "algorithmic_bytes_per_launch": algo_bytes,
                           "us_per_launch": ffn_us, "in_kernel_window_us": window_us,
                           "achieved_in_kernel_window": algo_bytes / (window_us * 1e-6) / 1e9 if window_us > 0 else None,
@@ -600,7 +604,7 @@ def grouped_alone(cfg, ctx, n_resident, peak, which, launches):
     us = st["ffn_us"] / max(st["ffn_launches"], 1)
     ach = mean_bytes / (us * 1e-6) / 1e9
     win = st["ffn_window_us"] / max(st["ffn_launches"], 1)      # in-kernel clock: first CTA past its dependency wait -> last CTA end
-    return {"bound": "hbm", "kernel": ffn_kernel_name(cfg), "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
+    return {"bound": "hbm", "kernel": ffn_kernel_name(cfg, ctx), "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
             "in_kernel_window_us": win, "frac_in_kernel_window": mean_bytes / (win * 1e-6) / 1e9 / peak if win > 0 else None,
             "traffic": NCU_DRAM_BYTES_PER_LAUNCH["batched_wave"] if (cfg.name == "batched" and n_resident == cfg.slots) else None,
             "peak_source": f"of {which}", "algorithmic_bytes_per_launch": mean_bytes, "us_per_launch": us,
@@ -781,7 +785,7 @@ def ffn_back_to_back(cfg, full, algo_bytes, peak, launches=480):
     e1.record(full.compute)
     full.synchronize()
     per_call = e0.elapsed_time(e1) * 1e3 / launches
-    out = {"launches": launches, "kernel": ffn_kernel_name(cfg),
+    out = {"launches": launches, "kernel": ffn_kernel_name(cfg, full),
            "algorithmic_bytes_per_launch": mean_bytes, "event_pair_each_us": per_kernel,
            "kernel_window_us": window if window > 0 else None, "call_us_incl_combine": per_call,
            "misses": st["misses"]}

@@ -1,5 +1,5 @@
-"""4-bit experts through mma.sync operands: the one-token kernel at the edges of its tiles against 64-bit sums, the batched kernel at
-the edges of its runs of tokens against the one-token kernel."""
+"""4-bit experts through mma.sync operands: the one-token kernel at the edges of its tiles against 64-bit sums, the batched kernels at the edges
+of their runs of tokens against the one-token kernel and against their roundings restated in 64 bits."""
 import time
 
 import numpy as np
@@ -39,7 +39,7 @@ def test_one_token(shape):
     cfg = make(*shape)
     m = build(cfg)
     gen = torch.Generator(device="cuda").manual_seed(1)
-    for scale in (1.0, 1e-6, 3e4, 1e9):         # the last two: activations that take phase 2's scale down
+    for scale in (1.0, 1e-6, 3e4, 1e9):         # the last two: activations beyond 2^15 and 2^60
         x = torch.randn(1, cfg.hidden, generator=gen, device="cuda") * scale
         x[0, 5] *= 100
         torch.cuda.synchronize()
