@@ -24,7 +24,7 @@
 // CTA (which owns no columns where there are fewer than 16 a CTA) while the others exchange the hidden row.
 //
 // Registers: nine warps leave a thread 168, sixteen 128. Three instances spill: hidden 1280 of bf16 (112 bytes stored, 144 loaded), hidden 1792 and
-// 2048 of 4 bits (88 / 128 and 116 / 160).
+// 2048 of 4 bits (96 / 140 and 116 / 160).
 //
 // The CTAs wait for one another, so the launch is cooperative (one CTA per SM, all resident or none). Every wait is
 // bounded: a CTA that gives up raises a flag that the others' waits look at, and all of them return with nothing in flight.
