@@ -55,7 +55,7 @@ __device__ __forceinline__ Nib4 q4_exact(uint32_t w) {
 
 // Weights as the tensor cores of ffn_grouped_q4_kernel get them, bf16_rn(bf16_rn(scale) * (q - 8)), times 2^-22: one packed fma on the masked
 // nibbles, q 2^-133 * (s 2^111) - 8 s 2^-22, rounds once like that product (all of its operands are exact: s is an fp16 number rounded to
-// bf16, at most 2^16). `odd` is `even` over 16.
+// bf16, at most 2^16). `odd` is `even` over 16. Sums stay at 2^-22 of the result, so results below 2^-100 or so lose bits.
 struct Q4Scaled { __nv_bfloat162 even, odd, off; };
 constexpr uint32_t kQ4Up111 = 0x77007700u, kQ4Down4 = 0x3d803d80u, kQ4Off = 0xb600b600u, kQ4Down22 = 0x34803480u;      // 2^111, 2^-4, -2^-19, 2^-22, twice
 constexpr float kQ4Unscale = 4194304.f;         // 2^22
