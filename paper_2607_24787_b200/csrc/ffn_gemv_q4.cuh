@@ -7,15 +7,15 @@
 //
 // All arithmetic on weights is mma.sync, with the fp32 operand as the sum of three bf16 numbers (split3) in three columns of N, so
 // that nothing is rounded to 16 bits. The warps split the columns in groups of 32 (one scale):
-//   Phase 1 (M = 16 gate rows, then 16 up rows; K = the group): the group's scale goes onto the fp32 sum of its 32 products; the warps' sums
+//   Phase 1 (M = eight gate rows and the same up rows; K = the group): the group's scale goes onto the fp32 sum of its 32 products; the warps' sums
 // meet in shared memory, a warp takes a row's activation from them.
 //   Phase 2 (M = hidden columns, K = the tile's 16 rows): act * scale is the split operand; two groups, whose scales differ, use columns of
 // N of their own. y stays in registers for all tiles of the CTA, each column in one warp: no sum over warps.
 //
 // Why MMAs: with fp32 FMAs the kernel was bound by instruction issue, 27 warp instructions per eight weights and lane, eight of which
 // widened halves to floats and eight multiplied; an MMA operand needs nine. A layer of the Qwen3 shape (a step as one kernel; with
-// separate launches before) 26.5 -> 18.3 us, of the DeepSeek shape 25.6 -> 16.2; its part of that, 14.6 -> 9. What bounds it now: the
-// chain of latencies of a tile, of which a CTA has three or four, and still instruction issue.
+// separate launches before) 26.5 -> 18.3 us, of the DeepSeek shape 25.6 -> 16.2; its part of that, 14.6 -> 9 (in rounds of tiles: see q4_tiles).
+// What bounds it now: latencies between dependent instructions (half of the issue slots are used), and still instruction issue.
 // The tensor cores cut a sum off where fp32 adds round it, always towards zero, so no chain of MMAs is longer than a group (phase 1) or a
 // tile (phase 2); longer sums are fp32 adds. (With y in the accumulators for all tiles a CTA of 384 tiles was off by 2.4e-6; 1 % faster.)
 // Error against 64 bits, 18 shapes of hidden 256 to 2048, rows that are normal, log-normal, of one sign, with outliers: 0.79 - 0.86 of the
@@ -48,8 +48,9 @@ struct Q4Part {
 };
 
 // Where the tiles of a CTA are: a ring of stages of kQ4Rows rows, one barrier a stage that completes when all rows of it have been asked for
-// and have landed, the phase-1 sums [warps][kQ4Red], gate and up of each row, and the activations [2][rows].
+// and have landed, the phase-1 sums [tile of a round][warps][kQ4Red], gate and up of each row, and the activations [tile of a round][rows].
 constexpr int kQ4Red = 33;             // (a lane reads one row's sum of one warp)
+constexpr int kQ4Super = 4;            // tiles of a round
 template <int NW>
 struct Q4Ring {
     uint32_t rows, bars, pitch;
@@ -63,7 +64,7 @@ struct Q4Ring {
         rows = smem_u32(smem);
         bars = smem_u32(b);
         red = reinterpret_cast<float*>(b + kQ4MaxStages);
-        act = red + (NW * kQ4Red + 3) / 4 * 4;
+        act = red + (kQ4Super * NW * kQ4Red + 3) / 4 * 4;
         if (thread == 0) {
             for (int s = 0; s < stages; ++s) mbar_init(bars + 8u * s, kQ4Rows);
             fence_barrier_init();
@@ -128,7 +129,11 @@ __device__ __forceinline__ void q4_operand(uint32_t (&x)[GB][4], int warp, int l
     }
 }
 
-// The CTA's rows 0 .. span - 1, tile by tile. fill(tile): ask for the warp's rows of a tile; the first `stages` tiles have been
+// The CTA's rows 0 .. span - 1, in rounds of up to four tiles: phase 1 of all of them, the warps' sums meet once, a warp a tile takes the
+// activations, phase 2 of all. What bounds a round is the latency between dependent instructions, which several tiles between two barriers
+// hide: whole steps of the 4-bit Qwen3 shape (three tiles a CTA), us a layer, 18.1 a tile at a time -> 17.3, DeepSeek shape (four, the last of one
+// row) 16.1 -> 13.8. (One barrier a tile, phase 2 a tile behind phase 1: 18.0 and 14.4.) Where the ring holds fewer tiles than the
+// CTA has, a round takes half of it, so that the other half is on its way. fill(tile): ask for the warp's rows of a tile; the first `stages` tiles have been
 // asked for. weight(row): routing weight. Every thread of the CTA takes part. Returns false, in every
 // thread, when a wait ran out (the caller drains and leaves).
 template <int GB, int NW, typename Fill, typename Weight>
@@ -137,108 +142,127 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
     const int g = lane >> 2, t = lane & 3, grp0 = warp * GB;
     const int tiles = (span + kQ4Rows - 1) / kQ4Rows;
     const uint32_t P = ring.pitch, PART = q4_part_bytes(D);
-    for (int k = 0; k < tiles; ++k) {
-        const int nr = span - k * kQ4Rows;
-        const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(ring.bars + 8u * ring.st, ring.ph, limit));
-        const uint32_t rows = ring.rows + uint32_t(ring.st * kQ4Rows) * P;
-        if (++ring.st == ring.stages) { ring.st = 0; ring.ph ^= 1; }
-        float* acts = ring.act + (k & 1) * kQ4Rows;
+    const int most = min(kQ4Super, tiles <= ring.stages ? tiles : (ring.stages + 1) / 2), rounds = (tiles + most - 1) / max(most, 1);
+    int before = 0;                  // tiles of the round before
+    for (int k = 0, left = rounds; left > 0; --left) {
+        const int nt = (tiles - k + left - 1) / left;
+        int st0 = ring.st;
+        auto rows_of = [&](int u) { return ring.rows + uint32_t((st0 + u < ring.stages ? st0 + u : st0 + u - ring.stages) * kQ4Rows) * P; };
         // `whole`: for the case below, a group's three parts added up before the scale goes onto them
-        auto phase1 = [&](auto whole) {
+        auto phase1 = [&](auto whole, auto blocks, int u) {
             constexpr bool kWhole = decltype(whole)::value;
-            float ag[4], au[4];
-            q4_phase1<GB>(rows, P, D, grp0, lane, x, ag, au, [](float (&acc)[4], const float (&c)[4], float s0, float s1) {
+            constexpr int H = decltype(blocks)::value;
+            float acc[H][4];
+            q4_phase1<GB, H>(rows_of(u), P, D, grp0, lane, x, acc, [](float (&a)[4], const float (&c)[4], float s0, float s1) {
                 if constexpr (kWhole) {
                     float lo = c[0] + c[1], hi = c[2] + c[3];
                     lo += __shfl_xor_sync(0xffffffffu, lo, 1);
                     hi += __shfl_xor_sync(0xffffffffu, hi, 1);
-                    acc[0] = fmaf(s0, lo, acc[0]); acc[2] = fmaf(s1, hi, acc[2]);
+                    a[0] = fmaf(s0, lo, a[0]); a[2] = fmaf(s1, hi, a[2]);
                 } else {
-                    acc[0] = fmaf(s0, c[0], acc[0]); acc[1] = fmaf(s0, c[1], acc[1]);
-                    acc[2] = fmaf(s1, c[2], acc[2]); acc[3] = fmaf(s1, c[3], acc[3]);
+                    a[0] = fmaf(s0, c[0], a[0]); a[1] = fmaf(s0, c[1], a[1]);
+                    a[2] = fmaf(s1, c[2], a[2]); a[3] = fmaf(s1, c[3], a[3]);
                 }
             });
             // columns 0 and 1 are in lane t = 0, column 2 in lane t = 1 (the others hold zeros)
-            float v[4] = {ag[0] + ag[1], ag[2] + ag[3], au[0] + au[1], au[2] + au[3]};
-            if constexpr (!kWhole)
+            float* r = ring.red + (u * NW + warp) * kQ4Red + g;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], 1);
-            if (t == 0) {
-                float* r = ring.red + warp * kQ4Red + g;
-                r[0] = v[0] * kQ4ExactUnscale; r[8] = v[1] * kQ4ExactUnscale; r[16] = v[2] * kQ4ExactUnscale; r[24] = v[3] * kQ4ExactUnscale;
+            for (int h = 0; h < H; ++h) {
+                float vg = acc[h][0] + acc[h][1], vu = acc[h][2] + acc[h][3];
+                if constexpr (!kWhole) { vg += __shfl_xor_sync(0xffffffffu, vg, 1); vu += __shfl_xor_sync(0xffffffffu, vu, 1); }
+                if (t == 0) { r[8 * h] = vg * kQ4ExactUnscale; r[16 + 8 * h] = vu * kQ4ExactUnscale; }
             }
         };
-        auto activations = [&]() {       // warp w: rows w, w + NW; even lanes take a row's gate, odd ones its up
-#pragma unroll
-            for (int r0 = 0; r0 < kQ4Rows; r0 += NW) {
-                const int r = r0 + warp;
-                if (kQ4Rows % NW != 0 && r >= kQ4Rows) continue;
-                const float* p = ring.red + (lane & 1) * 16 + r;
+        // warp u: tile u; even lanes take a row's gate, odd ones its up. True where an activation is not finite.
+        auto activations = [&]() -> bool {
+            bool odd = false;
+            if (warp < nt) {
+                const int r = lane >> 1, row = (k + warp) * kQ4Rows + r;
+                const float* p = ring.red + warp * NW * kQ4Red + (lane & 1) * 16 + r;
                 float sum = 0.f;         // (front to back: the loads overlap, so it takes no longer than shuffles between lanes)
 #pragma unroll
                 for (int w = 0; w < NW; ++w) sum += p[w * kQ4Red];
                 const float up = __shfl_xor_sync(0xffffffffu, sum, 1);
-                if (lane == 0) acts[r] = r < nr ? sum / (1.f + expf(-sum)) * up * weight(k * kQ4Rows + r) : 0.f;
+                if ((lane & 1) == 0) {
+                    const float act = row < span ? sum / (1.f + expf(-sum)) * up * weight(row) : 0.f;
+                    ring.act[warp * kQ4Rows + r] = act;
+                    odd = !isfinite(act);
+                }
             }
+            return odd;
         };
         float a0, a1, a2, a3;            // activations of rows 2t, 2t + 1, 2t + 8, 2t + 9
-        auto take = [&]() {
+        auto take = [&](int u) {
+            const float* acts = ring.act + u * kQ4Rows;
             const float2 lo = *reinterpret_cast<const float2*>(acts + 2 * t), hi = *reinterpret_cast<const float2*>(acts + 2 * t + 8);
             a0 = lo.x; a1 = lo.y; a2 = hi.x; a3 = hi.y;
         };
-        phase1(std::false_type{});
+        bool ok = true;
+        for (int u = 0; u < nt && ok; ++u) {
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(ring.bars + 8u * ring.st, ring.ph, limit));
+            if (++ring.st == ring.stages) { ring.st = 0; ring.ph ^= 1; }
+            if (span - (k + u) * kQ4Rows > 8) phase1(std::false_type{}, std::integral_constant<int, 2>{}, u);
+            else phase1(std::false_type{}, std::integral_constant<int, 1>{}, u);
+        }
         if (!__syncthreads_and(ok)) return false;
-        // every warp is done with the tile before this one
-        if (k > 0 && k - 1 + ring.stages < tiles) fill(k - 1 + ring.stages);
-        activations();
-        __syncthreads();
-        take();
-        if (__any_sync(0xffffffffu, !isfinite(a0 * 0.f + a1 * 0.f + a2 * 0.f + a3 * 0.f))) {       // (so in all warps or in none)
+        // every warp is done with the tiles of the round before this one
+        for (int u = k - before; u < k; ++u)
+            if (u + ring.stages < tiles) fill(u + ring.stages);
+        if (__syncthreads_or(activations())) {
             // An infinite scale times a part that is zero is a NaN where the scale times the sum is an infinity.
-            phase1(std::true_type{});
+            for (int u = 0; u < nt; ++u) {
+                take(u);
+                if (__any_sync(0xffffffffu, !isfinite(a0 * 0.f + a1 * 0.f + a2 * 0.f + a3 * 0.f))) phase1(std::true_type{}, std::integral_constant<int, 2>{}, u);       // (so in all warps or in none)
+            }
             __syncthreads();
             activations();
             __syncthreads();
-            take();
         }
-        // N columns 0-2: the parts for one group, 4-6: for the next (where there is one)
-        const bool second = g >= 4;
-        const bool idle = (g & 3) == 3;
-        const uint32_t at = rows + 2 * PART + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * P + uint32_t(grp0) * 16;
-        const uint32_t sc = rows + 2 * PART + uint32_t(2 * t) * P + uint32_t(D / 2 + grp0 * 2);
-        float s0[GB], s1[GB], s2[GB], s3[GB];
-        q4_scales<GB>(sc, s0);
-        q4_scales<GB>(sc + P, s1);
-        q4_scales<GB>(sc + 8 * P, s2);
-        q4_scales<GB>(sc + 9 * P, s3);
-        if (nr < kQ4Rows) {          // rows past the last one hold whatever was there: their activations are 0, so their scales must be finite
+        for (int u = 0; u < nt; ++u) {
+            const int nr = span - (k + u) * kQ4Rows;
+            const uint32_t rows = rows_of(u);
+            take(u);
+            // N columns 0-2: the parts for one group, 4-6: for the next (where there is one)
+            const bool second = g >= 4;
+            const bool idle = (g & 3) == 3;
+            const uint32_t at = rows + 2 * PART + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * P + uint32_t(grp0) * 16;
+            const uint32_t sc = rows + 2 * PART + uint32_t(2 * t) * P + uint32_t(D / 2 + grp0 * 2);
+            float s0[GB], s1[GB], s2[GB], s3[GB];
+            q4_scales<GB>(sc, s0);
+            q4_scales<GB>(sc + P, s1);
+            q4_scales<GB>(sc + 8 * P, s2);
+            q4_scales<GB>(sc + 9 * P, s3);
+            if (nr < kQ4Rows) {          // rows past the last one hold whatever was there: their activations are 0, so their scales must be finite
 #pragma unroll
-            for (int i = 0; i < GB; ++i) {
-                s0[i] = 2 * t < nr ? s0[i] : 0.f; s1[i] = 2 * t + 1 < nr ? s1[i] : 0.f;
-                s2[i] = 2 * t + 8 < nr ? s2[i] : 0.f; s3[i] = 2 * t + 9 < nr ? s3[i] : 0.f;
+                for (int i = 0; i < GB; ++i) {
+                    s0[i] = 2 * t < nr ? s0[i] : 0.f; s1[i] = 2 * t + 1 < nr ? s1[i] : 0.f;
+                    s2[i] = 2 * t + 8 < nr ? s2[i] : 0.f; s3[i] = 2 * t + 9 < nr ? s3[i] : 0.f;
+                }
             }
-        }
-        uint32_t b[(GB + 1) / 2][2];
-        const Q4Part part(g & 3);
-        auto operand = [&](bool guarded) {
+            uint32_t b[(GB + 1) / 2][2];
+            const Q4Part part(g & 3);
+            auto operand = [&](bool guarded) {
+#pragma unroll
+                for (int i = 0; i < GB; i += 2) {
+                    const int j = i + 1 < GB ? i + 1 : GB - 1;
+                    const float v0 = a0 * (second ? s0[j] : s0[i]), v1 = a1 * (second ? s1[j] : s1[i]), v2 = a2 * (second ? s2[j] : s2[i]), v3 = a3 * (second ? s3[j] : s3[i]);
+                    b[i / 2][0] = part.pair(v0, v1, guarded);
+                    b[i / 2][1] = part.pair(v2, v3, guarded);
+                    if (idle || (i + 1 >= GB && second)) b[i / 2][0] = b[i / 2][1] = 0u;
+                }
+            };
+            operand(false);
+            if (q4_any_nonfinite(b)) operand(true);
 #pragma unroll
             for (int i = 0; i < GB; i += 2) {
-                const int j = i + 1 < GB ? i + 1 : GB - 1;
-                const float v0 = a0 * (second ? s0[j] : s0[i]), v1 = a1 * (second ? s1[j] : s1[i]), v2 = a2 * (second ? s2[j] : s2[i]), v3 = a3 * (second ? s3[j] : s3[i]);
-                b[i / 2][0] = part.pair(v0, v1, guarded);
-                b[i / 2][1] = part.pair(v2, v3, guarded);
-                if (idle || (i + 1 >= GB && second)) b[i / 2][0] = b[i / 2][1] = 0u;
+                // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word
+                const uint4 w = ldsm4t(at + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
+                q4_phase2(y[i], w.x, w.y, b[i / 2][0], b[i / 2][1]);
+                if (i + 1 < GB) q4_phase2(y[i + 1 < GB ? i + 1 : i], w.z, w.w, b[i / 2][0], b[i / 2][1]);
             }
-        };
-        operand(false);
-        if (q4_any_nonfinite(b)) operand(true);
-#pragma unroll
-        for (int i = 0; i < GB; i += 2) {
-            // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word
-            const uint4 w = ldsm4t(at + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
-            q4_phase2(y[i], w.x, w.y, b[i / 2][0], b[i / 2][1]);
-            if (i + 1 < GB) q4_phase2(y[i + 1 < GB ? i + 1 : i], w.z, w.w, b[i / 2][0], b[i / 2][1]);
         }
+        k += nt;
+        before = nt;
     }
     return true;
 }
@@ -346,7 +370,7 @@ ffn_gemv_q4_kernel(const __grid_constant__ FfnArgs<MAXNB> a, const int n_stages)
 // Ring of a CTA with rows_per_cta rows: all its tiles where they fit beside `reserve` bytes. Returns the bytes of ring, barriers and sums.
 inline size_t ffn_gemv_q4_shape(int D, int rows_per_cta, size_t reserve, int* stages) {
     const size_t stage = size_t(kQ4Rows) * mt_pitch(3 * q4_part_bytes(D), false);
-    const size_t rest = kQ4MaxStages * 8 + size_t(kQ4MaxWarps) * kQ4Red * 4 + 16 + 2 * kQ4Rows * 4;
+    const size_t rest = kQ4MaxStages * 8 + size_t(kQ4Super) * kQ4MaxWarps * kQ4Red * 4 + 16 + size_t(kQ4Super) * kQ4Rows * 4;
     const size_t fit = (kFfnSmemLimit - 1024 - rest - reserve) / stage;
     const int want = rows_per_cta < kQ4Rows ? 1 : (rows_per_cta + kQ4Rows - 1) / kQ4Rows;
     *stages = int(fit < size_t(want) ? fit : size_t(want));

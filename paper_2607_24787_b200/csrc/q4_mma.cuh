@@ -111,36 +111,41 @@ __device__ __forceinline__ void q4_scales(uint32_t addr, float (&s)[GB]) {
     }
 }
 
-// Phase 1 of a tile: gate and up of its rows (2^-6 of them) over one warp's groups, for the MMA's eight N columns.
-// rows: the tile's first row, rows of `pitch` bytes that hold gate, then up; grp0: the warp's first group;
+// Phase 1: gate and up (2^-6 of them) of H blocks of eight rows over one warp's groups, for the MMA's eight N columns. A block's gate rows
+// are the upper half of M, its up rows the lower, so that the last rows of a share cost blocks of eight and not tiles of sixteen.
+// rows: the first row, rows of `pitch` bytes that hold gate, then up; grp0: the warp's first group;
 // x: the B operand of each group, four words: nibble pairs 0..3.
-// add(acc, c, s0, s1) puts a group's sums c onto acc: rows g (s0) and g + 8 (s1).
-template <int GB, typename Add>
+// add(acc, c, s0, s1) puts a group's sums c onto acc: gate row g (s0) and up row g (s1).
+template <int GB, int H, typename Add>
 __device__ __forceinline__ void q4_phase1(uint32_t rows, uint32_t pitch, int D, int grp0, int lane, const uint32_t (&x)[GB][4],
-                                          float (&gate)[4], float (&up)[4], Add add) {
+                                          float (&acc)[H][4], Add add) {
     const uint32_t part = q4_part_bytes(D);
-    // matrices: gate rows 0-7, 8-15, up rows 0-7, 8-15, 16 bytes (a group) each
-    const uint32_t at = rows + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * pitch + uint32_t(lane >> 4) * part + uint32_t(grp0) * 16;
+    // matrices: gate rows 0-7, up rows 0-7, 16 bytes (a group) each, then those of the next group
+    const uint32_t at = rows + uint32_t(lane & 7) * pitch + uint32_t((lane >> 3) & 1) * part + uint32_t(grp0) * 16;
     const uint32_t sc = rows + uint32_t(lane >> 2) * pitch + uint32_t(D / 2 + grp0 * 2);
-    float g0[GB], g1[GB], u0[GB], u1[GB];
-    q4_scales<GB>(sc, g0);
-    q4_scales<GB>(sc + 8 * pitch, g1);
-    q4_scales<GB>(sc + part, u0);
-    q4_scales<GB>(sc + 8 * pitch + part, u1);
+    float sg[H][GB], su[H][GB];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) gate[j] = up[j] = 0.f;
+    for (int h = 0; h < H; ++h) {
+        q4_scales<GB>(sc + uint32_t(h) * 8 * pitch, sg[h]);
+        q4_scales<GB>(sc + uint32_t(h) * 8 * pitch + part, su[h]);
 #pragma unroll
-    for (int i = 0; i < GB; ++i) {
-        const uint4 w = ldsm4(at + i * 16);
-        const Nib4 a = q4_exact(w.x), b = q4_exact(w.y), c = q4_exact(w.z), d = q4_exact(w.w);
-        float cg[4], cu[4];
-        mma_k16_first(cg, a.p[0], b.p[0], a.p[1], b.p[1], x[i][0], x[i][1]);
-        mma_k16_first(cu, c.p[0], d.p[0], c.p[1], d.p[1], x[i][0], x[i][1]);
-        mma_k16(cg, a.p[2], b.p[2], a.p[3], b.p[3], x[i][2], x[i][3]);
-        mma_k16(cu, c.p[2], d.p[2], c.p[3], d.p[3], x[i][2], x[i][3]);
-        add(gate, cg, g0[i], g1[i]);
-        add(up, cu, u0[i], u1[i]);
+        for (int j = 0; j < 4; ++j) acc[h][j] = 0.f;
     }
+#pragma unroll
+    for (int i = 0; i < GB; i += 2)
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const uint4 w = ldsm4(at + uint32_t(h) * 8 * pitch + uint32_t(i + (i + 1 < GB ? (lane >> 4) : 0)) * 16);
+            auto group = [&](int j, uint32_t wg, uint32_t wu) {
+                const Nib4 a = q4_exact(wg), b = q4_exact(wu);
+                float c[4];
+                mma_k16_first(c, a.p[0], b.p[0], a.p[1], b.p[1], x[j][0], x[j][1]);
+                mma_k16(c, a.p[2], b.p[2], a.p[3], b.p[3], x[j][2], x[j][3]);
+                add(acc[h], c, sg[h][j], su[h][j]);
+            };
+            group(i, w.x, w.y);
+            if (i + 1 < GB) group(i + 1 < GB ? i + 1 : i, w.z, w.w);
+        }
 }
 
 // Phase 2 for one group: y += W_down^T act over the tile's 16 rows (2^-6 of it). lo, hi: transposed matrices of the group's nibbles, rows 0-7

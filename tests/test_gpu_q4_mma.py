@@ -70,6 +70,35 @@ def test_infinite_operands_reach_the_result():
     m.close()
 
 
+# Rounds of tiles: 8, 9 and 17 rows a CTA (blocks of eight), 33 (a fourth tile of one row), 49 and 65 (five tiles), 70 and 144 rows with rings of
+# three and eight tiles. (hidden, inter, experts, top-k)
+ROUNDS = [(1024, 148, 9, 8), (512, 148, 10, 9), (1536, 148 * 17, 3, 1), (768, 148 * 3, 12, 11), (1280, 148 * 7, 8, 7), (1792, 148 * 13, 6, 5),
+          (2048, 1480, 8, 7), (256, 148 * 12, 13, 12)]
+
+
+@pytest.mark.parametrize("shape", ROUNDS)
+def test_rounds_of_tiles(shape):
+    """Against 64 bits, with the bound of test_one_token, and beyond fp32, where every tile's activations are infinite."""
+    hidden, inter, n, k = shape
+    cfg = make(hidden, inter, n, k)
+    m = build(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(1, hidden, generator=gen, device="cuda")
+    torch.cuda.synchronize()
+    _, ids, w, _ = m.router_topk(0, x)
+    got, huge = torch.zeros_like(x), torch.zeros_like(x)
+    big = x * 1e25                              # gate * up beyond fp32
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, got)
+    m.moe_ffn(0, big, ids, w, huge)
+    m.synchronize()
+    want = exact(cfg, x, ids, w)
+    assert (got.double() - want).norm() <= 1e-6 * want.norm()
+    far = exact(cfg, big, ids, w).abs() > 1e39
+    assert far.any() and not huge[far].isfinite().any()
+    m.close()
+
+
 # tokens of an expert: runs of eight (every expert in every token), one short and one over; few and many tasks a CTA; every split of the columns
 BATCHED = {
     "one_run": (2048, 128, 3, 3, 8), "run_and_one": (2048, 256, 3, 3, 9), "run_short": (1792, 384, 2, 2, 15), "eight_runs": (1536, 128, 2, 2, 64),
