@@ -22,6 +22,7 @@
 // FMAs' on average, 2.2e-7 of the result at worst (2.7e-7). Activations below 2^-110 lose bits: their third parts end at bf16's last one.
 #pragma once
 
+#include <climits>
 #include <type_traits>
 
 #include <cuda_bf16.h>
@@ -32,18 +33,20 @@
 
 namespace spm {
 
-// One of the three parts of split3 by a lane that wants only that: what is left of a number after the parts before it. An infinity
-// leaves NaNs (`guarded`: zeros).
+// One of the three parts of split3 by a lane that wants only that (p > 2: zero): what is left of a number after the parts before it. What is not
+// finite leaves NaNs; guarded: the number itself as the first part, zeros as the others.
 struct Q4Part {
     uint32_t m1, m2;               // masks of the parts that go first
-    __device__ __forceinline__ explicit Q4Part(int p) : m1(p >= 1 ? 0xffff0000u : 0u), m2(p >= 2 ? 0xffff0000u : 0u) {}
-    __device__ __forceinline__ float left(float v, bool guarded) const {
+    __device__ __forceinline__ explicit Q4Part(int p) : m1(p > 2 ? 0xffffffffu : p >= 1 ? 0xffff0000u : 0u), m2(p >= 2 ? 0xffff0000u : 0u) {}
+    template <bool GUARDED>
+    __device__ __forceinline__ float left(float v) const {
         float r = v - __uint_as_float(__float_as_uint(v) & m1);
-        if (guarded && m1 != 0 && !(fabsf(v) < INFINITY)) r = 0.f;
+        if (GUARDED && m1 != 0 && !(fabsf(v) < INFINITY)) r = 0.f;
         return r - __uint_as_float(__float_as_uint(r) & m2);
     }
-    __device__ __forceinline__ uint32_t pair(float a, float b, bool guarded = false) const {
-        return __byte_perm(__float_as_uint(left(a, guarded)), __float_as_uint(left(b, guarded)), 0x7632);
+    template <bool GUARDED = false>
+    __device__ __forceinline__ uint32_t pair(float a, float b) const {
+        return __byte_perm(__float_as_uint(left<GUARDED>(a)), __float_as_uint(left<GUARDED>(b)), 0x7632);
     }
 };
 
@@ -70,15 +73,15 @@ struct Q4Ring {
             fence_barrier_init();
         }
     }
-    // The warp's rows (warp, warp + NW) of `count` tiles from `tile` on; row_at(row) is null for rows that are not there. The lanes look the rows up side
-    // by side, one elected lane asks for them (lanes that ask side by side are taken one by one). `waited`: row_at waits for arrivals, which
+    // The warp's rows (warp, warp + NW) of `count` tiles from `tile` on; row_at(row), called by the whole warp, is null for rows that are not there. The
+    // lanes look the rows up side by side, one elected lane asks for them (lanes that ask side by side are taken one by one). `waited`: row_at waits for arrivals, which
     // the lane that waited has seen, but the one that asks reads the bytes: the barrier and the fence hand them on.
     template <typename F>
     __device__ __forceinline__ void fill(int tile, int count, int warp, int lane, uint32_t bytes, bool waited, F row_at) {
         constexpr int kPer = q4_rows_per_warp(NW);
         const int mine = warp + lane % kPer * NW;
         const bool in = lane < count * kPer && mine < kQ4Rows;
-        const unsigned long long at = in ? reinterpret_cast<unsigned long long>(row_at((tile + lane / kPer) * kQ4Rows + mine)) : 0ull;
+        const unsigned long long at = reinterpret_cast<unsigned long long>(row_at(in ? (tile + lane / kPer) * kQ4Rows + mine : INT_MAX));
         if (waited) {
             __syncwarp();
             asm volatile("fence.proxy.async;" ::: "memory");
@@ -109,24 +112,28 @@ struct Q4Ring {
 template <int GB, typename F>
 __device__ __forceinline__ void q4_operand(uint32_t (&x)[GB][4], int warp, int lane, F get) {
     const int g = lane >> 2, t = lane & 3;
-    float v[GB][8];
-    bool odd = false;
+    float v[GB][8], zeros[4] = {0.f, 0.f, 0.f, 0.f};         // (sums of products with zero: NaN where one is not finite)
 #pragma unroll
     for (int i = 0; i < GB; ++i) {
         get((warp * GB + i) * 32 + t * 8, v[i]);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) odd |= !(fabsf(v[i][q]) < INFINITY);
+        for (int q = 0; q < 8; ++q) zeros[q & 3] = fmaf(v[i][q], 0.f, zeros[q & 3]);
     }
-    const bool guarded = __any_sync(0xffffffffu, odd);
     const Q4Part part(g);
+    if (__any_sync(0xffffffffu, (zeros[0] + zeros[1]) + (zeros[2] + zeros[3]) != 0.f)) {
 #pragma unroll
-    for (int i = 0; i < GB; ++i) {
-        if (guarded)
+        for (int i = 0; i < GB; ++i) {
 #pragma unroll
             for (int q = 0; q < 8; ++q) v[i][q] = v[i][q] != v[i][q] ? __uint_as_float(0x7fffffffu) : v[i][q];      // (a NaN whose upper half is one too)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) x[i][q] = g < 3 ? part.pair(v[i][q], v[i][q + 4], guarded) : 0u;
+            for (int q = 0; q < 4; ++q) x[i][q] = part.pair<true>(v[i][q], v[i][q + 4]);
+        }
+        return;
     }
+#pragma unroll
+    for (int i = 0; i < GB; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[i][q] = part.pair(v[i][q], v[i][q + 4]);
 }
 
 // The CTA's rows 0 .. span - 1, in rounds of up to four tiles: phase 1 of all of them, the warps' sums meet once, a warp a tile takes the
@@ -224,7 +231,6 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
             take(u);
             // N columns 0-2: the parts for one group, 4-6: for the next (where there is one)
             const bool second = g >= 4;
-            const bool idle = (g & 3) == 3;
             const uint32_t at = rows + 2 * PART + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * P + uint32_t(grp0) * 16;
             const uint32_t sc = rows + 2 * PART + uint32_t(2 * t) * P + uint32_t(D / 2 + grp0 * 2);
             float s0[GB], s1[GB], s2[GB], s3[GB];
@@ -241,18 +247,18 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
             }
             uint32_t b[(GB + 1) / 2][2];
             const Q4Part part(g & 3);
-            auto operand = [&](bool guarded) {
+            auto operand = [&](auto guarded) {
 #pragma unroll
                 for (int i = 0; i < GB; i += 2) {
                     const int j = i + 1 < GB ? i + 1 : GB - 1;
                     const float v0 = a0 * (second ? s0[j] : s0[i]), v1 = a1 * (second ? s1[j] : s1[i]), v2 = a2 * (second ? s2[j] : s2[i]), v3 = a3 * (second ? s3[j] : s3[i]);
-                    b[i / 2][0] = part.pair(v0, v1, guarded);
-                    b[i / 2][1] = part.pair(v2, v3, guarded);
-                    if (idle || (i + 1 >= GB && second)) b[i / 2][0] = b[i / 2][1] = 0u;
+                    b[i / 2][0] = part.pair<decltype(guarded)::value>(v0, v1);
+                    b[i / 2][1] = part.pair<decltype(guarded)::value>(v2, v3);
+                    if (i + 1 >= GB && second) b[i / 2][0] = b[i / 2][1] = 0u;
                 }
             };
-            operand(false);
-            if (q4_any_nonfinite(b)) operand(true);
+            operand(std::false_type{});
+            if (q4_any_nonfinite(b)) operand(std::true_type{});
 #pragma unroll
             for (int i = 0; i < GB; i += 2) {
                 // matrices: rows 0-7 and 8-15 of group i, then of group i + 1; transposed: a lane has four columns of two rows a word

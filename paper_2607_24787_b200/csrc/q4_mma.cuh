@@ -163,10 +163,10 @@ __device__ __forceinline__ void q4_phase2(float (&y)[2][4], uint32_t lo, uint32_
 // Whether any of a warp's bf16 pairs holds an infinity or a NaN
 template <int N>
 __device__ __forceinline__ bool q4_any_nonfinite(const uint32_t (&b)[N][2]) {
-    uint32_t top = 0;
+    __nv_bfloat162 zeros = bf2(0u);            // sums of products with zero
 #pragma unroll
-    for (int i = 0; i < N; ++i) top = __vmaxu2(top, __vmaxu2(b[i][0] & 0x7fff7fffu, b[i][1] & 0x7fff7fffu));
-    return __any_sync(0xffffffffu, (top & 0xffffu) >= 0x7f80u || (top >> 16) >= 0x7f80u);
+    for (int i = 0; i < N; ++i) zeros = __hfma2(bf2(b[i][0]), bf2(0u), __hfma2(bf2(b[i][1]), bf2(0u), zeros));
+    return __any_sync(0xffffffffu, (bits2(zeros) & 0x7fff7fffu) != 0);
 }
 
 }  // namespace spm

@@ -15,16 +15,16 @@
 // One buffer per exchange is enough: a CTA overwrites a word one layer later, when it holds data that every reader of
 // the old word contributed to after reading it.
 //
-// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 16.2 (21): the FFN 11.5 - 13 and 8 - 10 with the slowest SM 2 us
-// behind the mean, and a chain of latencies of 6 (partial rows 1.4, hidden row 1, norm and dot products 1.5, logits 1.1, Top-K to the
-// first copies 1.3).
+// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 15.9 (21): the FFN 11.5 - 13 and 8 - 10 with the slowest SM 2 us
+// behind the mean, and a chain of latencies of 6 (partial rows 1.4, hidden row 1, norm and dot products 1.5, logits 1.1, Top-K 0.6, first
+// copies 0.5). With 4-bit experts 16.8 and 13.5, 6 and 4.5 of which are the tiles.
 //
 // The arithmetic, the orders of all sums and the split of the rows are those of router_adapter_kernel and ffn_gemv_kernel, so the
 // outputs have the same bits as host-driven steps. The adapter's ranking, which only the host reads, is done by the last
 // CTA (which owns no columns where there are fewer than 16 a CTA) while the others exchange the hidden row.
 //
-// Registers: nine warps leave a thread 168, sixteen 128. Three instances spill: hidden 1280 of bf16 (112 bytes stored, 144 loaded), hidden 1792 and
-// 2048 of 4 bits (96 / 140 and 116 / 160).
+// Registers: nine warps leave a thread 168, sixteen 128. Instances that spill: hidden 1280 of bf16 (132 bytes stored, 164 loaded), hidden 1792 and
+// 2048 of 4 bits (120 / 152 and 132 / 164); 20 bytes and less at 1280 and 1536 of 4 bits.
 //
 // The CTAs wait for one another, so the launch is cooperative (one CTA per SM, all resident or none). Every wait is
 // bounded: a CTA that gives up raises a flag that the others' waits look at, and all of them return with nothing in flight.
@@ -40,6 +40,7 @@ namespace spm {
 // whose threads then have 255 registers.
 constexpr int step_warps(int nseg, bool q4) { return q4 ? q4_warps(nseg) : nseg >= 6 ? 8 : kFfnMaxWarps; }
 constexpr int kStatusStepTimeout = 16;            // status bit (1 to 8: expert and routing kernels)
+constexpr int kStepKeys = 4;                      // logits of a lane that a warp's Top-K keeps in registers
 constexpr int kStepCols = 16;                     // columns of the hidden row that an owner adds up
 constexpr int kStepMaxCtas = kReduceGroupsR * kReduceChunkR;
 constexpr unsigned long long kStepStartNs = 30000000000ull;     // default limit of the first exchange: kernels of other streams may hold SMs until then
@@ -128,10 +129,10 @@ __device__ __forceinline__ int count_before(const int* k, int j0, int j1, int e)
 }
 
 // Shared memory behind the GEMV's ring and barriers, in floats: [normalised row][n logits][n probabilities, or sums of the owned columns]
-// [r adapter hidden][scratch 32][16 residuals][experts, weights and slots of the chosen, 3 x 16][slot map, shorts]
+// [r adapter hidden][scratch 32][16 residuals][experts and weights of the chosen, 2 x 16][slot map, shorts]
 __host__ __device__ constexpr size_t step_route_bytes(int D, int n, int r, bool xs_in_ring) {
     const size_t n4 = (size_t(n) + 3) & ~size_t(3), sums = size_t(kReduceGroupsR) * kStepCols;
-    return sizeof(float) * ((xs_in_ring ? 0 : size_t(D)) + n4 + (n4 > sums ? n4 : sums) + ((size_t(r) + 3) & ~size_t(3)) + 32 + kStepCols + 3 * SPM_MAX_TOPK) +
+    return sizeof(float) * ((xs_in_ring ? 0 : size_t(D)) + n4 + (n4 > sums ? n4 : sums) + ((size_t(r) + 3) & ~size_t(3)) + 32 + kStepCols + 2 * SPM_MAX_TOPK) +
            n4 * sizeof(short);
 }
 
@@ -161,8 +162,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
     float* hres = scratch + 32;             // residual of the owned columns
     int* isel = reinterpret_cast<int*>(hres + kStepCols);
     float* s_w = reinterpret_cast<float*>(isel + SPM_MAX_TOPK);
-    int* s_code = reinterpret_cast<int*>(s_w + SPM_MAX_TOPK);
-    short* smap = reinterpret_cast<short*>(s_code + SPM_MAX_TOPK);
+    short* smap = reinterpret_cast<short*>(s_w + SPM_MAX_TOPK);
 
     // even split of the (expert, j) rows over the CTAs, then over the warps, as in ffn_gemv_kernel
     const GemvShare share(I, a.K + a.n_shared, Q4 ? 0 : a.n_shared, c, G);
@@ -175,15 +175,18 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
     const int n_first = min(depth, my_n);
     const int n_early = Q4 || a.xs_in_ring ? 0 : min(n_first, share.n_shared_rows > wi ? (share.n_shared_rows - wi + nw - 1) / nw : 0);
     int first_ent, first_j;
-    share.row(wi + min(lane, max(n_first - 1, 0)) * nw, first_ent, first_j);
+    if constexpr (Q4) {              // (a tile's rows go round the warps)
+        constexpr int kPer = q4_rows_per_warp(kStepWarps);
+        share.row(min(lane / kPer * kQ4Rows + wi + lane % kPer * kStepWarps, max(span - 1, 0)), first_ent, first_j);
+    } else {
+        share.row(wi + min(lane, max(n_first - 1, 0)) * nw, first_ent, first_j);
+    }
     const unsigned long long limit = a.wait_limit_ns ? a.wait_limit_ns : kWaitLimitNs;
     Q4Ring<kStepWarps> tiles(smem, D, Q4 ? depth : 0, tid);         // (4-bit experts)
     if (!Q4 && wi < nw && lane == 0) {
         for (int d = 0; d < depth; ++d) mbar_init(bar0 + 8u * d, 1);
         fence_barrier_init();
     }
-    if (tid < a.n_shared) s_code[a.K + tid] = -1 - tid;
-
     const bool owner = c * kStepCols < D, ranks = c == G - 1;
     if (owner && tid < kStepCols) hres[tid] = a.h_in[c * kStepCols + tid];
 
@@ -362,47 +365,82 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
         if (a.xs_in_ring) fence_proxy_async();      // the row was written and read where copies are about to land
         if (__syncthreads_or(dead)) { drain(n_early); return; }
 
-        // ---- Top-K, two threads an expert; then the first weight copies go out, and the routing weights are computed behind them ----
-        const int half_n = (n / 2) & ~3;
-        for (int u0 = 0; u0 < 2 * n; u0 += kStepThreads) {
-            const int u = u0 + tid, e = u >> 1;
-            int rk = u < 2 * n ? count_before(reinterpret_cast<const int*>(zs), (u & 1) ? half_n : 0, (u & 1) ? n : half_n, e) : 0;
-            rk += __shfl_xor_sync(0xffffffffu, rk, 1);
-            if (u < 2 * n && (u & 1) == 0 && rk < a.K) {
-                isel[rk] = e;
-                s_code[rk] = smap[e] >= 0 ? smap[e] : 1 << 20;       // no slot: fails the range check below
-                if (c == 0) a.mailbox[l].ids[rk] = tagged(tag & 0xffffu, e);
+        // ---- Top-K; then the first weight copies go out, and the routing weights are computed behind them ----
+        int sel = 0, top_key = 0;           // lane k: the k-th expert; key of the first
+        // Up to 128 experts every warp ranks for itself: the lanes hold runs of consecutive keys, largest first, and a round takes the largest of all.
+        // (Two threads an expert counting what comes before it, and a barrier: 0.9 us of a layer with 128 experts, 0.5 with 64; this takes 0.6.)
+        if (n <= 32 * kStepKeys) {
+            const int per = (n + 31) / 32;
+            int key[kStepKeys], id[kStepKeys];
+#pragma unroll
+            for (int i = 0; i < kStepKeys; ++i) {
+                id[i] = lane * per + i;
+                key[i] = i < per && id[i] < n ? reinterpret_cast<const int*>(zs)[id[i]] : INT_MIN;
             }
+#pragma unroll
+            for (int i = 1; i < kStepKeys; ++i)         // largest first, equal ones in the order of their ids
+#pragma unroll
+                for (int j = i; j > 0; --j)
+                    if (key[j] > key[j - 1]) {
+                        const int tk = key[j], ti = id[j];
+                        key[j] = key[j - 1]; key[j - 1] = tk;
+                        id[j] = id[j - 1]; id[j - 1] = ti;
+                    }
+            for (int k = 0; k < a.K && (Q4 || wi < nw); ++k) {
+                const int most = __reduce_max_sync(0xffffffffu, key[0]);
+                const int from = __ffs(__ballot_sync(0xffffffffu, key[0] == most)) - 1;
+                const int e = __shfl_sync(0xffffffffu, id[0], from);
+                if (k == 0) top_key = most;
+                if (lane == k) sel = e;
+                if (lane == from) {
+#pragma unroll
+                    for (int i = 0; i + 1 < kStepKeys; ++i) { key[i] = key[i + 1]; id[i] = id[i + 1]; }
+                    key[kStepKeys - 1] = INT_MIN;
+                }
+            }
+        } else {                            // two threads an expert count what comes before it
+            const int half_n = (n / 2) & ~3;
+            for (int u0 = 0; u0 < 2 * n; u0 += kStepThreads) {
+                const int u = u0 + tid, e = u >> 1;
+                int rk = u < 2 * n ? count_before(reinterpret_cast<const int*>(zs), (u & 1) ? half_n : 0, (u & 1) ? n : half_n, e) : 0;
+                rk += __shfl_xor_sync(0xffffffffu, rk, 1);
+                if (u < 2 * n && (u & 1) == 0 && rk < a.K) isel[rk] = e;
+            }
+            __syncthreads();
+            if (lane < a.K) sel = isel[lane];
+            top_key = reinterpret_cast<const int*>(zs)[isel[0]];
         }
-        __syncthreads();
-        auto blob = [&](int ent) -> const unsigned char* {          // null after a bad slot number
-            const int code = s_code[ent];
+        // lane k: slot of entry k, routed or shared (negative)
+        const int code_of = lane >= a.K ? a.K - 1 - lane : smap[sel] >= 0 ? smap[sel] : 1 << 20;       // no slot: fails the range check below
+        if (c == 0 && wi == 0 && lane < a.K) a.mailbox[l].ids[lane] = tagged(tag & 0xffffu, sel);
+        auto blob = [&](int ent) -> const unsigned char* {          // by whole warps; null after a bad slot number
+            const int code = __shfl_sync(0xffffffffu, code_of, ent);
             if (code >= a.n_slots) { atomicOr(a.status, kStatusBadSlot); return nullptr; }
             return code < 0 ? a.shared + (size_t(l) * a.n_shared + size_t(-1 - code)) * a.blob_bytes
                             : a.pools + size_t(l) * a.pool_bytes + size_t(code) * a.blob_bytes;
         };
         auto row_at = [&](int row) -> const unsigned char* {        // (4-bit experts)
-            if (row >= span) return nullptr;
-            const int ent = (r_begin + row) / I;
+            const int ent = row < span ? (r_begin + row) / I : 0;
             const unsigned char* base = blob(ent);
-            return base ? base + size_t(r_begin + row - ent * I) * ROWB : nullptr;
+            return base && row < span ? base + size_t(r_begin + row - ent * I) * ROWB : nullptr;
         };
         int n_in = n_first;                 // rows that the warp has asked for
         if constexpr (Q4) {
-            tiles.fill(0, min(depth, (span + kQ4Rows - 1) / kQ4Rows), wi, lane, ROWB, false, row_at);
+            tiles.fill(0, min(depth, (span + kQ4Rows - 1) / kQ4Rows), wi, lane, ROWB, false, [&](int row) -> const unsigned char* {
+                const unsigned char* base = blob(first_ent);
+                return base && row < span ? base + size_t(first_j) * ROWB : nullptr;
+            });
         } else {       // (the lanes look the rows up side by side)
-            const unsigned char* base = lane >= n_early && lane < n_first ? blob(first_ent) : nullptr;
+            const unsigned char* base = blob(first_ent);
             const unsigned long long at = base ? reinterpret_cast<unsigned long long>(base + size_t(first_j) * ROWB) : 0ull;
             for (int i = n_early; i < n_first; ++i) ask(reinterpret_cast<const unsigned char*>(__shfl_sync(0xffffffffu, at, i)));
         }
         // Routing weights: the router tail's softmax over all experts, by every warp for itself. The four butterflies are the sums
         // of that tail's four warps, added in their order.
         float wk = 1.f;                     // lane k: weight of entry k
-        if (!Q4 || wi == 0) {
-            float top = -INFINITY, part[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int e = lane; e < n; e += 32) top = fmaxf(top, ps[e]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        if (Q4 ? wi == 0 : wi < nw) {
+            const float top = key_value(top_key);
+            float part[4] = {0.f, 0.f, 0.f, 0.f};
             for (int e0 = 0; e0 < n; e0 += 128)
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
@@ -412,7 +450,7 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) part[q] += __shfl_xor_sync(0xffffffffu, part[q], o);
             const float sum = ((part[0] + part[1]) + part[2]) + part[3];
-            const float p = lane < a.K ? expf(ps[isel[lane]] - top) / sum : 0.f;
+            const float p = lane < a.K ? expf(ps[sel] - top) / sum : 0.f;
             float tot = 0.f;
             for (int k = 0; k < a.K; ++k) tot += __shfl_sync(0xffffffffu, p, k);
             if (lane < a.K) wk = a.renorm ? p / tot : p;

@@ -105,6 +105,8 @@ __device__ __forceinline__ int order_key(float v) {
     return b ^ ((b >> 31) & 0x7fffffff);
 }
 
+__device__ __forceinline__ float key_value(int key) { return __int_as_float(key ^ ((key >> 31) & 0x7fffffff)); }      // (of -0: +0)
+
 // Position of element e in the ordering (key descending, index ascending) of k[0..n): the number
 // of elements that beat it. Element j beats e when k[j] > k[e], or k[j] == k[e] and j < e, i.e.
 // when k[j] > k[e] - (j < e): branch-free, four independent counters. Keys never equal INT_MIN

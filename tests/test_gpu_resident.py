@@ -62,6 +62,35 @@ def test_one_kernel_gives_the_bits_of_host_driven_steps(name, policy):
     assert ev_a == ev_b and st_a == st_b
 
 
+@pytest.mark.parametrize("base,n,k", [("tiny", 3, 3), ("tiny", 32, 2), ("bf16_nine_warps", 97, 6), ("q4_widest", 128, 8), ("tiny", 129, 4)])
+def test_equal_logits_go_to_the_lower_id(base, n, k):
+    """Experts with one and the same router row, on both sides of the number that a warp ranks by itself: the lowest ids of the largest logit,
+    in order, as in host-driven steps."""
+    if base == "tiny":
+        cfg = synth.get_config("tiny", n_layers=3, n_experts=n, top_k=k, slots=n, budget=2, batch=1)
+    else:
+        cfg = config(base, n_experts=n, top_k=k, inter=64)
+    H = rows(cfg, 3)
+    results = []
+    for host_free in (1, 0):
+        m = build(cfg, store_layers=1)
+        w = m._keep[1]
+        w[:, 1::2] = w[:, 1:2].clone()                # every second expert like expert 1, ...
+        w[2] = w[2, :1].clone()                       # ... and all of the last layer's alike
+        torch.cuda.synchronize()
+        m.set_host_free(host_free)
+        preload(cfg, m)
+        outs = run(m, H)
+        _, ids, _, logits = m.router_topk(2, torch.as_tensor(H[0], dtype=torch.float32).cuda(), want_logits=True)
+        assert list(ids[0]) == list(range(k))
+        results.append((outs, m.events()))
+        m.close()
+    (a, ev_a), (b, ev_b) = results
+    for s in range(3):
+        assert np.array_equal(a[s], b[s]), s
+    assert ev_a == ev_b
+
+
 def test_other_launches_in_between_and_rows_from_anywhere():
     """The exchange words share memory with other kernels' partial rows: steps before and after such kernels, in place, from rows
     at any float and from pinned host rows."""
