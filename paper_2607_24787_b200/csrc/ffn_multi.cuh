@@ -5,7 +5,8 @@
 // sizes that do not tile by 128, spm_set_batched_path(1)) and enough expert reads are shared (multi_pays). One GEMV
 // per sequence, the other kernel of that path, reads an expert once per token: 16 sequences of the DeepSeek shape
 // (1280 x 896, 6 of 64 and 2 shared experts) ask for 880 MB a layer where the distinct experts hold 350 MB.
-// Measured there, the kernel's window in a host-free step: 104 us a layer with it, 76 us here (350 MB at the card's copy rate: 54 us).
+// Measured there, the kernel's window in a host-free step: 104 us a layer with it, 72 us here (350 MB at the card's copy rate: 54 us; 76 with eight
+// warps instead of ten).
 //
 // Work. An entry is an expert with at most kMtTokens of its tokens. Its rows (row j = gate[j][:], up[j][:] and
 // column j of W_down, contiguous in the blob) are taken in blocks of kMtRows; the blocks of all entries, in
@@ -23,7 +24,7 @@
 // the lanes, this kernel needed 944 warp instructions per row of 1280 columns (its rows arrive every 1280 issue slots) and 108 us
 // for the layer above; with MMAs about 400.
 // mma.sync and not tcgen05: the accumulator has to come back to registers every 16 terms.
-//   Phase 1 (M = 8 gate rows over 8 up rows, N = tokens, K = hidden): the warps split the columns in groups
+//   Phase 1 (M = 8 gate rows over 8 up rows, N = tokens, K = hidden): the warps (eight to twenty) split the columns in groups
 // of 32; a lane ends up with gate and up of the same (row, token); the warps' sums meet in shared memory.
 //   Phase 2 (M = hidden, N = tokens, K = the block's 8 rows): the same groups of columns; y stays in registers
 // for the whole segment and is written once, to slot (segment, token) of `partial`.
@@ -52,8 +53,6 @@ namespace spm {
 
 constexpr int kMtTokens = 8;          // tokens of an entry: N of the MMAs
 constexpr int kMtRows = 8;            // rows of a block: gate and up rows together are M of the first MMA
-constexpr int kMtWarps = 8;
-constexpr int kMtThreads = kMtWarps * 32;
 constexpr int kMtMaxStages = 8;
 constexpr int kMtMaxPairs = SPM_MAX_BATCH * SPM_MAX_TOPK;
 
@@ -272,9 +271,11 @@ template <> struct MtWeight<Q4Tag> {         // (q - 8) through the MMA, a group
     }
 };
 
-template <typename WT, int GB>               // GB: groups of 32 columns per warp
-__global__ void __launch_bounds__(kMtThreads, 1)
+template <typename WT, int GB, int NW>       // GB: groups of 32 columns per warp; NW: warps
+__global__ void __launch_bounds__(NW * 32, 1)
 ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
+    static_assert(NW >= kMtRows && NW % 2 == 0, "a warp feeds, and sums up, a row of a block");
+    constexpr int kMtWarps = NW, kMtThreads = NW * 32;
     using W = MtWeight<WT>;
     extern __shared__ __align__(128) unsigned char smem[];
     const int D = a.D, I = a.I, n = a.n, n_pairs = a.nb * a.K, n_grp = D / 32;
@@ -326,7 +327,7 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
     const uint64_t pol = policy_evict_first();
     bool feeding = false;
     auto feed = [&](Feed& f, uint32_t ring_at, uint32_t bar, uint32_t pitch, uint32_t off, uint32_t bytes) {
-        if (!feeding || f.n >= steps) return;
+        if (!feeding || f.n >= steps || warp >= kMtRows) return;
         if (!f.src || f.row >= NB * kMtRows) {
             if (f.src) { ++f.u; f.row = warp; }
             int chunk;
@@ -359,7 +360,7 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
     auto feed_gu = [&]() { feed(fgu, ring, gu_bar, GU, 0, 2 * PART); };
     auto feed_dn = [&]() { feed(fdn, ring + dn_ring, dn_bar, DN, 2 * PART, PART); };
     const int g = lane >> 2, t = lane & 3;
-    // a warp's groups are warp, warp + 8, ...: the same number for every warp where hidden is a multiple of 256. Else (fp32) a
+    // a warp's groups are warp, warp + NW, ...: the same number for every warp but with fp32 weights, where a
     // warp without a last group computes group 0 there and drops it: straight-line code, so that the MMA chains interleave.
     const bool has_last = sizeof(WT) != 4 || warp + (GB - 1) * kMtWarps < n_grp;
     const int last_grp = has_last ? warp + (GB - 1) * kMtWarps : 0;
@@ -391,10 +392,10 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
                     for (int v = 0; v < 4; ++v) y[i][tile][v] = 0.f;
             }
         }
-        // Role in the meeting of the warps' phase-1 sums: warp i does row i. NS = 3: eight tokens, gate or up, four of the
-        // warps each. NS = 1: two tokens, gate or up, one warp's three parts each.
+        // Role in the meeting of the warps' phase-1 sums: warp i < 8 does row i. NS = 3: eight tokens, gate or up, half of the
+        // warps each. NS = 1: two tokens, gate or up, the three parts of every eighth warp each.
         const int m_row = warp, m_tok = lane & (NS == 3 ? 7 : 1), m_up = (lane >> (NS == 3 ? 3 : 1)) & 1;
-        const float* m_at = red + (NS == 3 ? (lane >> 4) * 4 * 128 + (m_row * 4 + (m_tok >> 1)) * 4 + (m_tok & 1) + 2 * m_up
+        const float* m_at = red + (NS == 3 ? (lane >> 4) * (kMtWarps / 2) * 128 + (m_row * 4 + (m_tok >> 1)) * 4 + (m_tok & 1) + 2 * m_up
                                            : (lane >> 2) * 128 + m_row * 16 + m_tok + 2 * m_up);
         const int wp = __shfl_sync(0xffffffffu, mine, min(m_tok, ntok - 1));
         const float wt = e >= n ? 1.f : a.w[wp];
@@ -438,10 +439,18 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
                 if constexpr (kP1) feed_gu();
                 if (i1 >= 2 && fdn.n < i1 - 1 + n_stages) feed_dn();
             }
-            if constexpr (kP1) {
+            if (kP1 && warp < kMtRows) {
                 float v = 0.f;
+                if constexpr (NS == 3) {
 #pragma unroll
-                for (int i = 0; i < (NS == 3 ? kMtWarps / 2 : 3); ++i) v += m_at[(i1 & 1) * (kMtWarps * 128) + i * (NS == 3 ? 128 : 4)];
+                    for (int i = 0; i < kMtWarps / 2; ++i) v += m_at[(i1 & 1) * (kMtWarps * 128) + i * 128];
+                } else {
+#pragma unroll
+                    for (int w = 0; w < kMtWarps; w += 8)
+#pragma unroll
+                        for (int i = 0; i < 3; ++i)
+                            if (kMtWarps % 8 == 0 || w + (lane >> 2) < kMtWarps) v += m_at[(i1 & 1) * (kMtWarps * 128) + w * 128 + i * 4];
+                }
                 if constexpr (NS == 1) {
                     v += __shfl_xor_sync(0xffffffffu, v, 4);
                     v += __shfl_xor_sync(0xffffffffu, v, 8);
@@ -577,7 +586,7 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
         if (lane == 0) { atomicMax(&s_entries, fgu.n); atomicMax(&s_routed, fdn.n); }
         __syncthreads();
         const int n_gu = s_entries, n_dn = s_routed;
-        if (elect_one()) {
+        if (warp < kMtRows && elect_one()) {
             for (int i = fgu.n; i < n_gu; ++i) mbar_arrive(gu_bar + 8 * (i % n_stages));
             for (int i = fdn.n; i < n_dn; ++i) mbar_arrive(dn_bar + 8 * (i % n_stages));
         }
@@ -709,8 +718,8 @@ inline size_t mt_partial_rows(int ctas, int nb, int K, int n, int n_shared) {
     return size_t(ctas + mt_max_entries(nb, K, n, n_shared)) * kMtTokens;
 }
 // Ring stages that fit beside the rest of the shared memory, and its total
-inline int mt_stages(size_t row_bytes, bool fp32, int n, int n_pairs, size_t* smem) {
-    const size_t rest = 2 * kMtMaxStages * 8 + 2 * (kMtWarps * 128 + kMtTokens * kMtRows) * 4 + size_t(n + 4) * 4 + size_t(n_pairs) * 2;
+inline int mt_stages(size_t row_bytes, bool fp32, int n, int n_pairs, int warps, size_t* smem) {
+    const size_t rest = 2 * kMtMaxStages * 8 + 2 * (size_t(warps) * 128 + kMtTokens * kMtRows) * 4 + size_t(n + 4) * 4 + size_t(n_pairs) * 2;
     const size_t stage = size_t(kMtRows) * (mt_pitch(uint32_t(row_bytes) / 3 * 2, fp32) + mt_pitch(uint32_t(row_bytes) / 3, fp32));
     size_t s = (kFfnSmemLimit - rest) / stage;
     if (s > size_t(kMtMaxStages)) s = kMtMaxStages;

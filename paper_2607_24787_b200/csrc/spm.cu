@@ -456,30 +456,43 @@ cudaError_t launch_gemv(const spm_ctx* c, const FfnArgs<MAXNB>& a, int G, int nb
     return launch_gemv_seg<float, MAXNB>(c->nseg, a, G, nb, warps, depth, smem, c->compute, pdl);
 }
 
-template <typename WT, int GB>
+template <typename WT, int GB, int NW>
 cudaError_t launch_multi_t(const spm_ctx* c, const MtArgs& a) {
-    constexpr auto kern = ffn_multi_kernel<WT, GB>;
+    constexpr auto kern = ffn_multi_kernel<WT, GB, NW>;
     if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
     size_t smem = 0;
-    const int stages = mt_stages(c->row_bytes, std::is_same<WT, float>::value, a.n, a.nb * a.K, &smem);
-    return launch_k(kern, dim3(mt_grid_for(c)), dim3(kMtThreads), smem, c->compute, true, a, stages);
+    const int stages = mt_stages(c->row_bytes, std::is_same<WT, float>::value, a.n, a.nb * a.K, NW, &smem);
+    return launch_k(kern, dim3(mt_grid_for(c)), dim3(NW * 32), smem, c->compute, true, a, stages);
 }
+// Groups of 32 columns over warps, evenly (but for fp32 rows of 128). A block is a chain of latencies, so more warps of fewer groups each pay until what every
+// warp does once a block outweighs it: 2048 columns, eight warps of eight -> sixteen of four, a layer of 16 sequences 107 -> 98 us; 1280, eight of
+// five -> ten of four 91 -> 87 (twenty of two: 96; 4-bit 111 -> 110, twenty of two 105); bf16 of 512, eight of two 34.2, sixteen of one 35.4 (4-bit 52.1, 51.4).
+// bf16 of 1536 keeps eight of six: the sums of sixteen would cost one of three ring stages.
 template <typename WT>
 cudaError_t launch_multi_g(const spm_ctx* c, const MtArgs& a) {
-    const int gb = (a.D / 32 + kMtWarps - 1) / kMtWarps;
-    switch (gb) {
-        case 1: return launch_multi_t<WT, 1>(c, a);
-        case 2: return launch_multi_t<WT, 2>(c, a);
-        case 3: return launch_multi_t<WT, 3>(c, a);
-        case 4: return launch_multi_t<WT, 4>(c, a);
-    }
-    if constexpr (sizeof(WT) != 4)      // (fp32: hidden <= 1024)
-        switch (gb) {
-            case 5: return launch_multi_t<WT, 5>(c, a);
-            case 6: return launch_multi_t<WT, 6>(c, a);
-            case 7: return launch_multi_t<WT, 7>(c, a);
-            case 8: return launch_multi_t<WT, 8>(c, a);
+    constexpr bool q4 = std::is_same<WT, Q4Tag>::value;
+    if constexpr (std::is_same<WT, float>::value) {
+        switch (a.D / 128) {
+            case 1: case 2: return launch_multi_t<WT, 1, 8>(c, a);
+            case 3: return launch_multi_t<WT, 1, 12>(c, a);
+            case 4: return launch_multi_t<WT, 1, 16>(c, a);
+            case 5: return launch_multi_t<WT, 2, 10>(c, a);
+            case 6: return launch_multi_t<WT, 2, 12>(c, a);
+            case 7: return launch_multi_t<WT, 2, 14>(c, a);
+            case 8: return launch_multi_t<WT, 2, 16>(c, a);
         }
+    } else {
+        switch (a.D / 256) {
+            case 1: return launch_multi_t<WT, 1, 8>(c, a);
+            case 2: return launch_multi_t<WT, q4 ? 1 : 2, q4 ? 16 : 8>(c, a);
+            case 3: return launch_multi_t<WT, 2, 12>(c, a);
+            case 4: return launch_multi_t<WT, 2, 16>(c, a);
+            case 5: return launch_multi_t<WT, q4 ? 2 : 4, q4 ? 20 : 10>(c, a);
+            case 6: return launch_multi_t<WT, q4 ? 3 : 6, q4 ? 16 : 8>(c, a);
+            case 7: return launch_multi_t<WT, 4, 14>(c, a);
+            case 8: return launch_multi_t<WT, 4, 16>(c, a);
+        }
+    }
     return cudaErrorInvalidValue;
 }
 

@@ -82,6 +82,32 @@ def test_several_sequences_equal_one_at_a_time(name):
     m.close()
 
 
+SPLITS = [("tiny", d) for d in (128, 256, 384, 512, 640, 768, 896, 1024)] + [(b, d) for b in ("qwen3", "qwen3_q4") for d in range(256, 2049, 256)]
+
+
+@pytest.mark.parametrize("base,hidden", SPLITS)
+def test_every_split_of_the_columns_over_warps(base, hidden):
+    """17 tokens of all four experts: two full runs and one token, against the batch-1 kernel's sums with the bound of the test above. One or two
+    rows in the last block."""
+    for inter in (1202, 1201) if hidden == 1280 else (1201 * 128 // hidden * 8 + 1,):
+        cfg = synth.get_config(base, n_layers=1, budget=1, hidden=hidden, n_experts=4, inter=inter, top_k=4, slots=4, batch=17)
+        assert takes_kernel(cfg, cfg.batch)
+        m = build(cfg)
+        gen = torch.Generator(device="cuda").manual_seed(hidden)
+        x = torch.randn(17, hidden, generator=gen, device="cuda")
+        torch.cuda.synchronize()
+        m.set_batched_path(1)
+        _, ids, w, _ = m.router_topk(0, x)
+        both = torch.zeros(2, 17, hidden, device="cuda")
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x, ids, w, both[0])
+        for t in range(17):
+            m.moe_ffn(0, x[t:t + 1], ids[t:t + 1], w[t:t + 1].contiguous(), both[1, t:t + 1])
+        m.synchronize()
+        assert (both[0] - both[1]).abs().max() <= 5e-6 * both[1].abs().max()
+        m.close()
+
+
 @pytest.mark.parametrize("offset", [1, 2, 3])
 def test_hidden_rows_may_start_at_any_float(offset):
     """spm_moe_ffn updates h_inout in place wherever it lies: an offset slice has the alignment of a float only. Same sums
