@@ -1348,7 +1348,7 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
                            (const int32_t*)c->ws_ids, (const short*)(c->ws_slot_map + size_t(l) * n), l * c->S, nb * K, K, n, c->n_jt, m.hidden,
                            units, rowmap, c->tc_n_units, c->tc_xs, c->tc_wrow, m.dtype == SPM_DTYPE_Q4 ? 1 : 0,
                            m.dtype == SPM_DTYPE_Q4 ? (int*)nullptr : c->tc_ready, m.dtype == SPM_DTYPE_Q4 ? 0 : c->max_units + 1, c->ws_status, rank));
-            // (no chunk list here: the plan is built on the device, a chunk is a whole unit)
+            // (no chunk list here: the plan is built on the device, the kernel cuts for itself)
             GgArgs ga{units, 0, c->tc_n_units, c->tc_wrow, c->tc_partial, c->rows_cap, m.hidden, m.inter, c->ws_status, c->wait_limit_ns,
                       nullptr, 0, c->tc_ready, c->tc_act, c->tc_ready + 1, clock_slot};
             if (m.dtype == SPM_DTYPE_Q4)

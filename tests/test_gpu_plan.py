@@ -34,3 +34,22 @@ def test_device_plan_and_ranking_equal_the_host_driven_step(name):
         m.close()
     (a, ev_a, st_a), (b, ev_b, st_b) = results
     assert np.array_equal(a, b) and ev_a == ev_b and st_a == st_b
+
+
+# (hidden, inter, experts, top-k, sequences): 2 to 16 d-tiles a unit, some that do not divide into parts evenly; fewer units than CTAs, about as many,
+# and up to three times as many with whole units in front
+@pytest.mark.parametrize("hidden,inter,n,k,nb", [(256, 384, 20, 2, 9), (768, 128, 40, 4, 30), (512, 256, 12, 3, 4), (1024, 1024, 24, 4, 16), (1280, 512, 48, 4, 40),
+                                                 (1792, 640, 64, 6, 48), (2048, 768, 16, 8, 5), (2048, 128, 149, 4, 64)])
+def test_units_cut_on_the_device_give_the_bits_of_the_host_plan(hidden, inter, n, k, nb):
+    cfg = synth.get_config("qwen3", n_layers=2, hidden=hidden, inter=inter, n_experts=n, top_k=k, slots=n, batch=nb, budget=1, adapter_rank=4)
+    H = rows(cfg, 2)
+    outs = []
+    for host_free in (1, 0):
+        m = build(cfg, store_layers=1)
+        m.set_host_free(host_free)
+        preload(cfg, m)
+        outs.append(run(m, H, sync_every=1))
+        assert m.stats()["host_free_steps"] == (2 if host_free else 0)
+        m.close()
+    for a, b in zip(*outs):
+        assert np.isfinite(a).all() and np.array_equal(a, b)
