@@ -14,8 +14,9 @@
 // warps split the columns in groups of 32 (one scale), GB consecutive groups a warp.
 //   Phase 1 (M = 16 gate rows, then 16 up rows; N = tokens; K = 32 columns, two MMAs). The warps' sums meet in shared memory.
 //   Phase 2 (M = 16 hidden columns, N = tokens, K = 16 rows): the warp's own columns. y stays in the accumulators for the whole task.
-// Phase 2 is one tile behind phase 1, so that one CTA barrier a tile is enough. The rows of a tile come as two bulk copies each, gate /
-// up and W_down, into rings of their own.
+// Phase 2 is one tile behind phase 1, so that one CTA barrier a tile is enough. A tile comes as three boxes of 16 rows by TMA, gate and up into one
+// ring, W_down into another. Where 16 rows of a part would start in the same banks (hidden a multiple of 512) a box is 16 bytes wider
+// than the part, which pads the rows. (Two bulk copies a row, asked for by all warps: 80 of some 640 instructions of a warp and tile. XXX)
 //
 // A token's result depends on its own row and the expert only (a column of the MMAs), so outputs do not depend on waves, batch
 // mates or the CTA. What is rounded is what the tcgen05 kernel rounds: scales, products of scale and q - 8, token rows and activations,
@@ -37,9 +38,7 @@ constexpr int kMqAct = 24;                     // pitch of a token's activations
 constexpr int kMqMaxTasks = 512;              // tasks of a CTA
 
 struct MqArgs {
-    const unsigned char* pools;     // all layers' slots
     const __nv_bfloat16* xs;        // sorted token rows, columns 8g .. 8g + 7 in the order 0 4 1 5 2 6 3 7
-    unsigned long long blob_bytes;
     GgArgs g;
 };
 struct MqTask { int slot, jt_n, row, unit; };         // global slot, 128-row tile * 16 + tokens, first token row, unit
@@ -54,7 +53,7 @@ inline size_t mq_rest_bytes(int n) {
            size_t(kMqMaxTasks) * sizeof(MqTask) + size_t(n + 1) * 4;
 }
 inline int mq_stages(int D, int n, size_t* smem) {
-    const size_t stage = size_t(kQ4Rows) * (mt_pitch(2 * q4_part_bytes(D), false) + mt_pitch(q4_part_bytes(D), false));
+    const size_t stage = 3 * size_t(kQ4Rows) * mt_pitch(q4_part_bytes(D), false);
     size_t s = (kFfnSmemLimit - mq_rest_bytes(n)) / stage;
     if (s > size_t(kQ4MaxStages)) s = kQ4MaxStages;
     *smem = s * stage + mq_rest_bytes(n);
@@ -65,10 +64,10 @@ inline int mq_stages(int D, int n, size_t* smem) {
 __device__ __forceinline__ bool mq_nonfinite(__nv_bfloat162 zeros) { return __any_sync(0xffffffffu, (bits2(zeros) & 0x7fff7fffu) != 0); }
 
 // Phase 1 of a tile: gate and up of its rows (2^-22 of them) over one warp's groups, for the MMA's eight token columns.
-// rows: the tile's first row, rows of `pitch` bytes that hold gate, then up; x: the B operand of each group, nibble pairs 0..3.
+// rows: the tile's first gate row, rows of `pitch` bytes, kQ4Rows of gate, then of up; x: the B operand of each group, nibble pairs 0..3.
 template <int GB>
 __device__ __forceinline__ void mq_phase1(uint32_t rows, uint32_t pitch, int D, int grp0, int lane, const uint32_t (&x)[GB][4], float (&gate)[4], float (&up)[4]) {
-    const uint32_t part = q4_part_bytes(D);
+    const uint32_t part = kQ4Rows * pitch;
     // matrices: gate rows 0-7, 8-15, up rows 0-7, 8-15, 16 bytes (a group) each
     const uint32_t at = rows + uint32_t((lane & 7) + ((lane >> 3) & 1) * 8) * pitch + uint32_t(lane >> 4) * part + uint32_t(grp0) * 16;
     const uint32_t sc = rows + uint32_t(lane >> 2) * pitch + uint32_t(D / 2 + grp0 * 2);
@@ -142,20 +141,18 @@ __device__ __forceinline__ void mq_phase2(uint32_t rows, uint32_t pitch, int D, 
 
 template <int NSEG>
 __global__ void __launch_bounds__(q4_warps(NSEG) * 32, 1)
-ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) {
+ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __grid_constant__ MqArgs m, const int n_stages) {
     constexpr int D = NSEG * 256, GB = q4_groups(NSEG), NW = q4_warps(NSEG);
-    constexpr uint32_t PART = q4_part_bytes(D), GU = mt_pitch(2 * PART, false), DN = mt_pitch(PART, false);      // row pitches
+    constexpr uint32_t PART = q4_part_bytes(D), PITCH = mt_pitch(PART, false), BOX = kQ4Rows * PITCH;      // a box: 16 rows of a part
     extern __shared__ __align__(128) unsigned char smem[];
     const GgArgs& a = m.g;
-    const uint32_t dn_ring = uint32_t(n_stages) * kQ4Rows * GU;               // the gate / up ring, then the W_down ring
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + dn_ring + uint32_t(n_stages) * kQ4Rows * DN);
+    const uint32_t dn_ring = uint32_t(n_stages) * 2 * BOX;                    // the gate / up ring, then the W_down ring
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + dn_ring + uint32_t(n_stages) * BOX);
     MqTask* tasks = reinterpret_cast<MqTask*>(bars + 2 * kQ4MaxStages);
     float* red = reinterpret_cast<float*>(tasks + kMqMaxTasks);               // [2][warps] phase-1 sums
     __nv_bfloat16* actv = reinterpret_cast<__nv_bfloat16*>(red + 2 * NW * kMqRed);      // [2][token][row]
     float* s_w = reinterpret_cast<float*>(actv + 2 * kMqTokens * kMqAct);     // [2 tasks][token]
     int& s_abort = *reinterpret_cast<int*>(s_w + 2 * kMqTokens);
-    int& s_gu = (&s_abort)[1];
-    int& s_dn = (&s_abort)[2];
     int* runs = &s_abort + 4;                                                 // [experts + 1] runs of tokens before each expert
     const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;      // (warp: uniform)
     const uint32_t ring = smem_u32(smem), gu_bar = smem_u32(bars), dn_bar = gu_bar + 8 * kQ4MaxStages;
@@ -163,7 +160,7 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
 
     grid_dep_launch();
     if (threadIdx.x == 0) {
-        for (int s = 0; s < n_stages; ++s) { mbar_init(gu_bar + 8 * s, kQ4Rows); mbar_init(dn_bar + 8 * s, kQ4Rows); }
+        for (int s = 0; s < n_stages; ++s) { mbar_init(gu_bar + 8 * s, 1); mbar_init(dn_bar + 8 * s, 1); }
         s_abort = 0;
         fence_barrier_init();
     }
@@ -204,44 +201,41 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
     }
     __syncthreads();
 
-    // ---- The warps fill the rings, warp i the rows i, i + NW of every tile. One elected lane asks, with operands that are the same in
-    // the warp: with a row a lane, which the compiler takes one by one, the two rings cost a warp 110 instructions a tile more. ----
-    struct Feed { int task, tile, n, st; const unsigned char* src; };       // next tile; tiles asked for; stage of the next; the tile's first row
+    // ---- The last warp fills the rings ----
+    struct Feed { int task, tile, n, st, row; };       // next tile; tiles asked for; stage of the next; the tile's row of the map
     const uint64_t pol = policy_evict_first();
-    bool feeding = true;
-    auto open = [&](Feed& f, uint32_t off, bool wait) {
-        if (f.task >= n_tasks) return;
+    bool feeding = warp == NW - 1;
+    auto open = [&](Feed& f, bool wait) {
+        if (!feeding || f.task >= n_tasks) return;
         const MqTask k = tasks[f.task];
-        f.src = m.pools + size_t(k.slot) * m.blob_bytes + size_t(k.jt_n >> 4) * kGgTileRows * (3 * PART) + off;
+        f.row = k.slot * a.I + (k.jt_n >> 4) * kGgTileRows;
         if (wait && a.unit_wait) {       // the expert's copy may still be on its way
             const GgWait uw = a.unit_wait[k.unit];
             const GgAbort ab{&s_abort, a.status, limit};
             if (uw.watch >= 0 && !__all_sync(0xffffffffu, gg_wait_arrival(a.ready + uw.watch, uw.want, ab))) feeding = false;
         }
     };
-    auto feed = [&](Feed& f, uint32_t ring_at, uint32_t bar, uint32_t pitch, uint32_t off, uint32_t bytes, bool wait) {
+    auto feed = [&](Feed& f, uint32_t ring_at, uint32_t bar, int part, int parts, bool wait) {
         if (!feeding || f.task >= n_tasks) return;
-        if (elect_one())
-#pragma unroll
-            for (int r = 0; r < kQ4Rows; r += NW)
-                if (kQ4Rows % NW == 0 || r + warp < kQ4Rows) {
-                    mbar_arrive_expect_tx(bar + 8 * f.st, bytes);
-                    bulk_g2s(ring_at + uint32_t(f.st * kQ4Rows + r + warp) * pitch, f.src + size_t(r + warp) * (3 * PART), bytes, bar + 8 * f.st, pol);
-                }
+        if (elect_one()) {
+            mbar_arrive_expect_tx(bar + 8 * f.st, uint32_t(parts) * BOX);
+            for (int i = 0; i < parts; ++i)
+                tma_load_2d_hint(ring_at + uint32_t(f.st * parts + i) * BOX, &rowmap, (part + i) * int(PART / 8), f.row, bar + 8 * f.st, pol);
+        }
         __syncwarp();
         ++f.n;
         f.st = f.st + 1 == n_stages ? 0 : f.st + 1;
-        f.src += size_t(kQ4Rows) * (3 * PART);
+        f.row += kQ4Rows;
         if (++f.tile < kMqTiles) return;
         f.tile = 0;
         ++f.task;
-        open(f, off, wait);
+        open(f, wait);
     };
-    Feed fgu{0, 0, 0, 0, nullptr}, fdn = fgu;
-    auto feed_gu = [&]() { feed(fgu, ring, gu_bar, GU, 0, 2 * PART, true); };
-    auto feed_dn = [&]() { feed(fdn, ring + dn_ring, dn_bar, DN, 2 * PART, PART, false); };     // (never ahead of the other)
-    open(fgu, 0, true);
-    open(fdn, 2 * PART, false);
+    Feed fgu{0, 0, 0, 0, 0}, fdn = fgu;
+    auto feed_gu = [&]() { feed(fgu, ring, gu_bar, 0, 2, true); };
+    auto feed_dn = [&]() { feed(fdn, ring + dn_ring, dn_bar, 2, 1, false); };     // (never ahead of the other)
+    open(fgu, true);
+    open(fdn, false);
     for (int i = 0; i < n_stages; ++i) { feed_gu(); feed_dn(); }
 
     // ---- tiles: phase 1 of tile k, phase 2 of tile k - 1 ----
@@ -278,10 +272,10 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
         const int task1 = k / kMqTiles;
         if (p1) {
             if (!dead) dead = !__all_sync(0xffffffffu, mt_wait(gu_bar + 8 * st1, ph1, &s_abort, a.status, limit));
-            const uint32_t rows = ring + uint32_t(st1) * kQ4Rows * GU;
+            const uint32_t rows = ring + uint32_t(st1) * 2 * BOX;
             if (++st1 == n_stages) { st1 = 0; ph1 ^= 1; }
             float ag[4] = {}, au[4] = {};
-            mq_phase1<GB>(rows, GU, D, grp0, lane, x, ag, au);
+            mq_phase1<GB>(rows, PITCH, D, grp0, lane, x, ag, au);
             float* r = red + ((k & 1) * NW + warp) * kMqRed + lane * 4;
             *reinterpret_cast<float4*>(r) = make_float4(ag[0], ag[1], ag[2], ag[3]);
             *reinterpret_cast<float4*>(r + 128) = make_float4(au[0], au[1], au[2], au[3]);
@@ -311,7 +305,7 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
         {
             const __nv_bfloat16* av = actv + (((k - 1) & 1) * kMqTokens + g) * kMqAct + 2 * t;
             const uint32_t b0 = *reinterpret_cast<const uint32_t*>(av), b1 = *reinterpret_cast<const uint32_t*>(av + 8);
-            mq_phase2<GB>(ring + dn_ring + uint32_t(st2) * kQ4Rows * DN, DN, D, grp0, lane, b0, b1, y);
+            mq_phase2<GB>(ring + dn_ring + uint32_t(st2) * BOX, PITCH, D, grp0, lane, b0, b1, y);
             if (++st2 == n_stages) { st2 = 0; ph2 ^= 1; }
         }
         if ((k - 1) % kMqTiles == kMqTiles - 1) {            // end of a task: a lane has four consecutive columns of two tokens
@@ -326,20 +320,9 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
             clear_y();
         }
     }
-    // Wind-down after a wait ran out, as in ffn_multi_kernel: the warps agree on the last tile that any of them fed, arrive without a
-    // copy for the tiles up to it, and wait for what is in flight.
+    // Wind-down after a wait ran out: the warp that asked waits for what is in flight.
     __syncthreads();
-    if (*reinterpret_cast<volatile int*>(&s_abort)) {
-        if (threadIdx.x == 0) { s_gu = 0; s_dn = 0; }
-        __syncthreads();
-        if (lane == 0) { atomicMax(&s_gu, fgu.n); atomicMax(&s_dn, fdn.n); }
-        __syncthreads();
-        const int n_gu = s_gu, n_dn = s_dn;
-        if (elect_one())
-            for (int r = warp; r < kQ4Rows; r += NW) {
-                for (int i = fgu.n; i < n_gu; ++i) mbar_arrive(gu_bar + 8 * (i % n_stages));
-                for (int i = fdn.n; i < n_dn; ++i) mbar_arrive(dn_bar + 8 * (i % n_stages));
-            }
+    if (warp == NW - 1 && *reinterpret_cast<volatile int*>(&s_abort)) {
         const unsigned long long t0 = global_timer_ns();
         auto drain = [&](uint32_t bar, int n_fed) {
             for (int i = max(0, n_fed - n_stages); i < n_fed; ++i) {
@@ -347,8 +330,8 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ MqArgs m, const int n_stages) 
                 mbar_wait_bounded(bar + 8 * (i % n_stages), (i / n_stages) & 1, spent < kWaitLimitNs ? kWaitLimitNs - spent : 0);
             }
         };
-        drain(gu_bar, n_gu);
-        drain(dn_bar, n_dn);
+        drain(gu_bar, fgu.n);
+        drain(dn_bar, fdn.n);
     }
     if (a.clock) {
         __syncthreads();

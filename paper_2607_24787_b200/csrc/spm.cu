@@ -78,7 +78,8 @@ struct spm_ctx {
     int rows_cap = 0, n_jt = 0, max_units = 0;
     CUtensorMap wmap{};
     GgTokenMaps xmaps{};
-    CUtensorMap qmapn{}, qmapsc{};            // 4-bit blobs: nibble box of 128 bytes, scale box of 16 bytes
+    CUtensorMap qmapn{}, qmapsc{};            // 4-bit blobs: nibble box of 128 bytes, scale box of 16 bytes ...
+    CUtensorMap qmaprow{};                    // ... and 16 rows of a part
     __nv_bfloat16* tc_xs = nullptr;
     float *tc_wrow = nullptr, *tc_partial = nullptr;
     unsigned char* tc_desc_dev = nullptr;     // kDescRing wave descriptors
@@ -530,7 +531,7 @@ cudaError_t launch_grouped_q4_mma_t(const spm_ctx* c, const MqArgs& a) {
     if (cudaError_t e = allow_full_smem<kern>(); e != cudaSuccess) return e;
     size_t smem = 0;
     const int stages = mq_stages(a.g.D, c->cfg.n_experts, &smem);
-    return launch_k(kern, dim3(c->num_sms), dim3(q4_warps(NSEG) * 32), smem, c->compute, true, a, stages);
+    return launch_k(kern, dim3(c->num_sms), dim3(q4_warps(NSEG) * 32), smem, c->compute, true, c->qmaprow, a, stages);
 }
 // 4-bit grouped FFN of nb sequences. Which kernel follows from the call alone, not from a wave: the two round alike but add in different orders.
 // ffn_grouped_q4_mma_kernel costs a CTA's tasks (an expert's 128 rows for up to eight tokens) and depends little on hidden, the
@@ -556,7 +557,7 @@ cudaError_t launch_grouped_q4(spm_ctx* c, int nb, int grid, const GgArgs& a) {
     const bool mma = grouped_q4_mma_pays(c, nb);
     ++c->q4_launches[mma];
     if (mma) {
-        MqArgs q{c->pools, c->tc_xs, c->blob, a};
+        MqArgs q{c->tc_xs, a};
         switch (m.hidden / 256) {
             case 2: return launch_grouped_q4_mma_t<2>(c, q);
             case 3: return launch_grouped_q4_mma_t<3>(c, q);
@@ -1778,7 +1779,8 @@ int spm_init(const spm_model_cfg* cfg, int slots_per_layer, int budget, const sp
         c->tc_desc_ev_valid.assign(kDescRing, 0);
         for (auto& ev : c->tc_desc_ev) if (!cu(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "cudaEventCreate")) return bail(SPM_ERR_CUDA);
         const bool maps_ok = cfg->dtype == SPM_DTYPE_Q4
-            ? make_q4_maps(&c->qmapn, &c->qmapsc, c->pools, cfg->hidden, cfg->inter, uint64_t(L) * c->S)
+            ? make_q4_maps(&c->qmapn, &c->qmapsc, c->pools, cfg->hidden, cfg->inter, uint64_t(L) * c->S) &&
+              make_q4_row_map(&c->qmaprow, c->pools, cfg->hidden, cfg->inter, uint64_t(L) * c->S, mt_pitch(q4_part_bytes(cfg->hidden), false), kQ4Rows)
             : make_weight_map(&c->wmap, c->pools, cfg->hidden, cfg->inter, uint64_t(L) * c->S);
         bool xmaps_ok = true;
         for (int b = 0; b < 3; ++b)

@@ -87,4 +87,19 @@ inline bool make_q4_maps(CUtensorMap* nib64, CUtensorMap* sc16, const void* base
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same blobs as rows [n_slots * I][3 * RB bytes]; a box is `box_rows` rows of one part, `box_bytes` wide (RB, or a little of what follows it with it,
+// which sets the pitch of the rows in shared memory), in elements of 8 bytes: a box has at most 256.
+inline bool make_q4_row_map(CUtensorMap* map, const void* base, int D, int I, uint64_t n_slots, uint32_t box_bytes, uint32_t box_rows) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const cuuint64_t row = 3 * (cuuint64_t(D) / 2 + cuuint64_t(D) / 16);
+    const cuuint64_t dims[2] = {row / 8, cuuint64_t(I) * n_slots};
+    const cuuint64_t strides[1] = {row};
+    const cuuint32_t box[2] = {box_bytes / 8, box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 2, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace spm
