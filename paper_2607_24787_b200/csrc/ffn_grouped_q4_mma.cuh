@@ -10,13 +10,18 @@
 // What bounds it now: instruction issue and dependent-issue latency, 106,000 instructions a scheduler at 0.57 a cycle.
 //
 // Work. A task is 128 intermediate rows of an expert (GgUnit) for up to kMqTokens of its tokens; CTA b runs the tasks b, b + grid, ...
-// of all experts in order (a hot expert's runs of tokens go to different CTAs). A task goes through its rows in tiles of 16; the
-// warps split the columns in groups of 32 (one scale), GB consecutive groups a warp.
+// of all experts in order (a hot expert's runs of tokens go to different CTAs), but for the last one to two tasks a CTA, which are split
+// evenly by tiles. A task that falls to two CTAs is begun by the first of them ahead of all else, which leaves its sums, unrounded, where the result goes, and
+// finished by the second after all else: a chain of sums is the same whoever adds, so outputs have the same bits. (760 tasks of 64 sequences of the
+// Qwen3 shape on 148 CTAs: six for some, where an even share is 5.1; 137.5 -> 133 us a layer; 16 sequences 87.6 -> 82, 8: 66.5 -> 60.3. 64 of 60
+// experts lose 1 %, two sequences, which give no CTA a second task, 0.6 us.)
+// A task goes through its rows in tiles of 16; the warps split the columns in groups of 32 (one scale), GB consecutive groups a warp.
 //   Phase 1 (M = 16 gate rows, then 16 up rows; N = tokens; K = 32 columns, two MMAs). The warps' sums meet in shared memory.
 //   Phase 2 (M = 16 hidden columns, N = tokens, K = 16 rows): the warp's own columns. y stays in the accumulators for the whole task.
 // Phase 2 is one tile behind phase 1, so that one CTA barrier a tile is enough. A tile comes as three boxes of 16 rows by TMA, gate and up into one
 // ring, W_down into another. Where 16 rows of a part would start in the same banks (hidden a multiple of 512) a box is 16 bytes wider
-// than the part, which pads the rows. (Two bulk copies a row, asked for by all warps: 80 of some 640 instructions of a warp and tile. XXX)
+// than the part, which pads the rows. (Two bulk copies a row, asked for by all warps: 80 of some 640 instructions of a warp and tile. 64
+// sequences of the Qwen3 shape 146 -> 137.5 us a layer.)
 //
 // A token's result depends on its own row and the expert only (a column of the MMAs), so outputs do not depend on waves, batch
 // mates or the CTA. What is rounded is what the tcgen05 kernel rounds: scales, products of scale and q - 8, token rows and activations,
@@ -35,13 +40,15 @@ constexpr int kMqTokens = 8;                  // tokens of a task: N of the MMAs
 constexpr int kMqTiles = kGgTileRows / kQ4Rows;
 constexpr int kMqRed = 264;                   // pitch of a warp's phase-1 sums: 256 floats, the next warp's eight banks on
 constexpr int kMqAct = 24;                     // pitch of a token's activations (bf16): 12 banks, so that eight tokens' pairs of rows have banks of their own
-constexpr int kMqMaxTasks = 512;              // tasks of a CTA
+constexpr int kMqMaxTasks = 512;              // tasks of a CTA (two more where some are split)
+constexpr int kMqTaskSlots = kMqMaxTasks + 4;
 
 struct MqArgs {
     const __nv_bfloat16* xs;        // sorted token rows, columns 8g .. 8g + 7 in the order 0 4 1 5 2 6 3 7
     GgArgs g;
 };
-struct MqTask { int slot, jt_n, row, unit; };         // global slot, 128-row tile * 16 + tokens, first token row, unit
+struct MqTask { int slot, jt_n, row, unit, span; };   // global slot, 128-row tile * 16 + tokens, first token row, unit, first tile | end << 8
+static_assert(kMqTaskSlots * sizeof(MqTask) % 16 == 0, "sums behind the tasks are stored four at a time");
 
 // Tasks of a CTA at worst: every expert's last run partly filled
 inline int mq_max_tasks(int nb, int K, int n, int n_jt, int grid) {
@@ -50,7 +57,7 @@ inline int mq_max_tasks(int nb, int K, int n, int n_jt, int grid) {
 }
 inline size_t mq_rest_bytes(int n) {
     return 2 * kQ4MaxStages * 8 + 2 * size_t(kQ4MaxWarps) * kMqRed * 4 + 2 * kMqTokens * kMqAct * 2 + 2 * kMqTokens * 4 + 16 +
-           size_t(kMqMaxTasks) * sizeof(MqTask) + size_t(n + 1) * 4;
+           size_t(kMqTaskSlots) * sizeof(MqTask) + size_t(n + 1) * 4;
 }
 inline int mq_stages(int D, int n, size_t* smem) {
     const size_t stage = 3 * size_t(kQ4Rows) * mt_pitch(q4_part_bytes(D), false);
@@ -149,7 +156,7 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
     const uint32_t dn_ring = uint32_t(n_stages) * 2 * BOX;                    // the gate / up ring, then the W_down ring
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + dn_ring + uint32_t(n_stages) * BOX);
     MqTask* tasks = reinterpret_cast<MqTask*>(bars + 2 * kQ4MaxStages);
-    float* red = reinterpret_cast<float*>(tasks + kMqMaxTasks);               // [2][warps] phase-1 sums
+    float* red = reinterpret_cast<float*>(tasks + kMqTaskSlots);                  // [2][warps] phase-1 sums
     __nv_bfloat16* actv = reinterpret_cast<__nv_bfloat16*>(red + 2 * NW * kMqRed);      // [2][token][row]
     float* s_w = reinterpret_cast<float*>(actv + 2 * kMqTokens * kMqAct);     // [2 tasks][token]
     int& s_abort = *reinterpret_cast<int*>(s_w + 2 * kMqTokens);
@@ -187,9 +194,25 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
     }
     __syncthreads();
     const int n_all = n_exp > 0 ? runs[n_exp] * n_jt : 0, G = int(gridDim.x);
-    const int n_tasks = min(kMqMaxTasks, int(blockIdx.x) < n_all ? (n_all - 1 - int(blockIdx.x)) / G + 1 : 0);
+    // Rounds of whole tasks, then the tiles s .. e of the tasks from `split` on: a head (the last of these tasks, begun here), which goes first, whole
+    // tasks, a tail (the first of them, begun by the CTA before), which goes last.
+    const int c = int(blockIdx.x), rounds = max(n_all / G - 1, 0), split = rounds * G;
+    int s = 0, e = c < n_all ? kMqTiles : 0, first = c;
+    if (n_all >= G) {
+        const int tiles = (n_all - split) * kMqTiles, q = tiles / G, rem = tiles - q * G;
+        s = q * c + min(c, rem);
+        e = s + q + (c < rem ? 1 : 0);
+        first = split + s / kMqTiles;
+        e -= s / kMqTiles * kMqTiles;
+        s %= kMqTiles;
+    }
+    const int head = e % kMqTiles ? 1 : 0, tail = s ? 1 : 0, whole = e / kMqTiles - tail;
+    const int n_tasks = min(kMqMaxTasks + 2, head + rounds + whole + tail), n_tiles = e - s + rounds * kMqTiles;
     for (int i = threadIdx.x; i < n_tasks; i += NW * 32) {
-        const int task = int(blockIdx.x) + i * G, run = task / n_jt, jt = task - run * n_jt;
+        const int j = i - head - rounds;             // >= 0: a whole task of the split ones, or the tail
+        const int task = i < head ? first + e / kMqTiles : j < 0 ? c + (i - head) * G : j < whole ? first + tail + j : first;
+        const int span = i < head ? (e % kMqTiles) << 8 : (j == whole ? s : 0) | kMqTiles << 8;
+        const int run = task / n_jt, jt = task - run * n_jt;
         int lo = 0, hi = n_exp;              // the expert whose runs hold this one
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -197,18 +220,20 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
         }
         const int4 v = __ldcg(reinterpret_cast<const int4*>(a.units + lo * n_jt + jt));      // GgUnit{slot, jt, row0, ntok}
         const int tok = (run - runs[lo]) * kMqTokens;
-        tasks[i] = MqTask{v.x, v.y * 16 + min(kMqTokens, v.w - tok), v.z + tok, lo * n_jt + jt};
+        tasks[i] = MqTask{v.x, v.y * 16 + min(kMqTokens, v.w - tok), v.z + tok, lo * n_jt + jt, span};
     }
     __syncthreads();
 
     // ---- The last warp fills the rings ----
-    struct Feed { int task, tile, n, st, row; };       // next tile; tiles asked for; stage of the next; the tile's row of the map
+    struct Feed { int task, tile, end, n, st, row; };  // next tile, its task's end; tiles asked for; stage of the next; the tile's row of the map
     const uint64_t pol = policy_evict_first();
     bool feeding = warp == NW - 1;
     auto open = [&](Feed& f, bool wait) {
         if (!feeding || f.task >= n_tasks) return;
         const MqTask k = tasks[f.task];
-        f.row = k.slot * a.I + (k.jt_n >> 4) * kGgTileRows;
+        f.tile = k.span & 255;
+        f.end = k.span >> 8;
+        f.row = k.slot * a.I + (k.jt_n >> 4) * kGgTileRows + f.tile * kQ4Rows;
         if (wait && a.unit_wait) {       // the expert's copy may still be on its way
             const GgWait uw = a.unit_wait[k.unit];
             const GgAbort ab{&s_abort, a.status, limit};
@@ -226,12 +251,11 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
         ++f.n;
         f.st = f.st + 1 == n_stages ? 0 : f.st + 1;
         f.row += kQ4Rows;
-        if (++f.tile < kMqTiles) return;
-        f.tile = 0;
+        if (++f.tile < f.end) return;
         ++f.task;
         open(f, wait);
     };
-    Feed fgu{0, 0, 0, 0, 0}, fdn = fgu;
+    Feed fgu{0, 0, 0, 0, 0, 0}, fdn = fgu;
     auto feed_gu = [&]() { feed(fgu, ring, gu_bar, 0, 2, true); };
     auto feed_dn = [&]() { feed(fdn, ring + dn_ring, dn_bar, 2, 1, false); };     // (never ahead of the other)
     open(fgu, true);
@@ -243,7 +267,7 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
     uint32_t x[GB][4];
     float y[GB][2][4];
     auto load_x = [&](int task) {           // token rows, and the routing weights, of the task that phase 1 comes to
-        const MqTask k = task < n_tasks ? tasks[task] : MqTask{0, 0, 0, 0};
+        const MqTask k = task < n_tasks ? tasks[task] : MqTask{0, 0, 0, 0, 0};
         const bool on = g < (k.jt_n & 15);
         const __nv_bfloat16* p = m.xs + size_t(k.row + g) * D + grp0 * 32 + t * 8;
 #pragma unroll
@@ -266,9 +290,21 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
     bool dead = false;
     int st1 = 0, st2 = 0;
     uint32_t ph1 = 0, ph2 = 0;
-    const int n_tiles = n_tasks * kMqTiles;
-    for (int k = 0; k <= n_tiles && n_tiles > 0; ++k) {
-        const bool p1 = k < n_tiles, p2 = k > 0;
+    // Tile k is tile k % 8 of the CTA's task k / 8: a head counts as the last tiles of its eight, so that all tasks end at multiples of eight but the tail,
+    // the last, which ends with the loop.
+    const int k0 = head ? kMqTiles - e % kMqTiles : 0, k1 = k0 + n_tiles;
+    auto finish = [&](int task, float unscale) {            // a lane has four consecutive columns of two tokens
+        const MqTask kk = tasks[task];
+        const int n_tok = kk.jt_n & 15;
+        float* out = a.partial + (size_t(kk.jt_n >> 4) * a.rows_cap + kk.row) * D + grp0 * 32 + g * 4;
+#pragma unroll
+        for (int i = 0; i < GB; ++i) {
+            if (2 * t < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t) * D + i * 32) = make_float4(y[i][0][0] * unscale, y[i][0][2] * unscale, y[i][1][0] * unscale, y[i][1][2] * unscale);
+            if (2 * t + 1 < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t + 1) * D + i * 32) = make_float4(y[i][0][1] * unscale, y[i][0][3] * unscale, y[i][1][1] * unscale, y[i][1][3] * unscale);
+        }
+    };
+    for (int k = k0; k <= k1 && n_tiles > 0; ++k) {
+        const bool p1 = k < k1, p2 = k > k0;
         const int task1 = k / kMqTiles;
         if (p1) {
             if (!dead) dead = !__all_sync(0xffffffffu, mt_wait(gu_bar + 8 * st1, ph1, &s_abort, a.status, limit));
@@ -286,7 +322,7 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
         // every warp is done with the gate / up rows of tile k and with the W_down rows of tile k - 2
         if (!dead) {
             if (p1) feed_gu();
-            if (k >= 2 && fdn.n < k - 1 + n_stages) feed_dn();
+            if (k >= k0 + 2 && fdn.n < k - k0 - 1 + n_stages) feed_dn();
         }
         // 128 (row, token) pairs, one a lane of four warps (with eight pairs in each of sixteen warps, the exponential and the division cost every
         // warp a tile's time: 64 sequences of the Qwen3 shape 155 us a layer against 146)
@@ -308,18 +344,34 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
             mq_phase2<GB>(ring + dn_ring + uint32_t(st2) * BOX, PITCH, D, grp0, lane, b0, b1, y);
             if (++st2 == n_stages) { st2 = 0; ph2 ^= 1; }
         }
-        if ((k - 1) % kMqTiles == kMqTiles - 1) {            // end of a task: a lane has four consecutive columns of two tokens
-            const MqTask kk = tasks[(k - 1) / kMqTiles];
-            const int n_tok = kk.jt_n & 15;
-            float* out = a.partial + (size_t(kk.jt_n >> 4) * a.rows_cap + kk.row) * D + grp0 * 32 + g * 4;
-#pragma unroll
-            for (int i = 0; i < GB; ++i) {
-                if (2 * t < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t) * D + i * 32) = make_float4(y[i][0][0] * kQ4Unscale, y[i][0][2] * kQ4Unscale, y[i][1][0] * kQ4Unscale, y[i][1][2] * kQ4Unscale);
-                if (2 * t + 1 < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t + 1) * D + i * 32) = make_float4(y[i][0][1] * kQ4Unscale, y[i][0][3] * kQ4Unscale, y[i][1][1] * kQ4Unscale, y[i][1][3] * kQ4Unscale);
+        if ((k - 1) % kMqTiles == kMqTiles - 1) {
+            const int task2 = (k - 1) / kMqTiles;
+            finish(task2, task2 < head ? 1.f : kQ4Unscale);
+            if (task2 < head) {              // the next CTA goes on from here
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(a.act_ready + blockIdx.x) : "memory");
             }
             clear_y();
+            if (tail && task2 == n_tasks - 2) {
+                const GgAbort ab{&s_abort, a.status, limit};
+                if (!dead) dead = !__all_sync(0xffffffffu, gg_wait_count(a.act_ready + blockIdx.x - 1, NW, ab));
+                const MqTask kk = tasks[task2 + 1];
+                const int n_tok = kk.jt_n & 15;
+                const float* in = a.partial + (size_t(kk.jt_n >> 4) * a.rows_cap + kk.row) * D + grp0 * 32 + g * 4;
+#pragma unroll
+                for (int i = 0; i < GB; ++i) {
+                    const float* p = in + size_t(2 * t) * D + i * 32;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {        // (one by one: loaded four at a time, they would want other registers than as sums of the MMAs)
+                        if (2 * t < n_tok) asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(y[i][q >> 1][(q & 1) * 2]) : "l"(p + q));
+                        if (2 * t + 1 < n_tok) asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(y[i][q >> 1][(q & 1) * 2 + 1]) : "l"(p + D + q));
+                    }
+                }
+            }
         }
     }
+    if (tail) finish(n_tasks - 1, kQ4Unscale);
     // Wind-down after a wait ran out: the warp that asked waits for what is in flight.
     __syncthreads();
     if (warp == NW - 1 && *reinterpret_cast<volatile int*>(&s_abort)) {

@@ -558,6 +558,7 @@ cudaError_t launch_grouped_q4(spm_ctx* c, int nb, int grid, const GgArgs& a) {
     ++c->q4_launches[mma];
     if (mma) {
         MqArgs q{c->tc_xs, a};
+        q.g.act_ready = reinterpret_cast<int*>(c->tc_act);       // (a counter a CTA, zeroed by the gather kernel; the space of the bf16 kernel's A^T)
         switch (m.hidden / 256) {
             case 2: return launch_grouped_q4_mma_t<2>(c, q);
             case 3: return launch_grouped_q4_mma_t<3>(c, q);
@@ -927,7 +928,7 @@ int launch_grouped_wave(spm_ctx* c, int layer, const float* x_norm, const int32_
     CU(c, launch_k(gg_gather_kernel, dim3(std::max(n_rows, 1)), dim3(128), 0, c->compute, true, x_norm, w,
                    reinterpret_cast<const GgRow*>(dd + c->tc_off_rows), n_rows, m.hidden, K,
                    c->tc_xs + size_t(off) * m.hidden, c->tc_wrow + off,
-                   q4 ? 1 : 0, q4 ? (int*)nullptr : c->tc_ready, q4 ? 0 : n_units + 1));
+                   q4 ? 1 : 0, q4 ? reinterpret_cast<int*>(c->tc_act) : c->tc_ready, q4 ? c->num_sms : n_units + 1));
     if (t && first) CU(c, cudaEventRecord(t->ffn_start[layer], c->compute));
     if (ring >= 0 && first) CU(c, cudaEventRecord(c->ring_start[ring], c->compute));
     GgArgs a{reinterpret_cast<const GgUnit*>(dd), n_units, nullptr, c->tc_wrow, c->tc_partial, c->rows_cap, m.hidden, m.inter, c->ws_status, c->wait_limit_ns,
@@ -1348,7 +1349,8 @@ int enqueue_host_free_layers(spm_ctx* c, int nb, float* h_out, int slot, bool pr
             CU(c, launch_k(gg_plan_gather_kernel, dim3(nb * K + (rank.pihat ? 1 : 0)), dim3(kGgPairThreads), 0, c->compute, true, (const float*)c->ws_x, (const float*)c->ws_w,
                            (const int32_t*)c->ws_ids, (const short*)(c->ws_slot_map + size_t(l) * n), l * c->S, nb * K, K, n, c->n_jt, m.hidden,
                            units, rowmap, c->tc_n_units, c->tc_xs, c->tc_wrow, m.dtype == SPM_DTYPE_Q4 ? 1 : 0,
-                           m.dtype == SPM_DTYPE_Q4 ? (int*)nullptr : c->tc_ready, m.dtype == SPM_DTYPE_Q4 ? 0 : c->max_units + 1, c->ws_status, rank));
+                           m.dtype == SPM_DTYPE_Q4 ? reinterpret_cast<int*>(c->tc_act) : c->tc_ready, m.dtype == SPM_DTYPE_Q4 ? c->num_sms : c->max_units + 1,
+                           c->ws_status, rank));
             // (no chunk list here: the plan is built on the device, the kernel cuts for itself)
             GgArgs ga{units, 0, c->tc_n_units, c->tc_wrow, c->tc_partial, c->rows_cap, m.hidden, m.inter, c->ws_status, c->wait_limit_ns,
                       nullptr, 0, c->tc_ready, c->tc_act, c->tc_ready + 1, clock_slot};

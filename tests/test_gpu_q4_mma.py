@@ -132,6 +132,36 @@ def test_batched(name):
     m.close()
 
 
+# (sequences, top-k), every pair an expert of its own: as many tasks as CTAs, one less, up to one a CTA more, two a CTA and either side of it, three
+# and a few; three tasks an expert in rows of other widths
+SPLIT = [(512, 128, 21, 7), (512, 128, 37, 4), (512, 128, 50, 3), (512, 128, 31, 5), (512, 128, 59, 5), (512, 128, 37, 8), (512, 128, 33, 9), (512, 128, 64, 7),
+         (1280, 384, 25, 2), (2048, 384, 64, 3)]
+
+
+@pytest.mark.parametrize("hidden,inter,nb,k", SPLIT)
+def test_tasks_split_between_two_ctas_keep_their_bits(hidden, inter, nb, k):
+    """Against the same rows in calls so small that no task is split."""
+    cfg = make(hidden, inter, nb * k, k, batch=nb)
+    m = build(cfg)
+    m.test_grouped_q4(2)
+    x = torch.randn(nb, hidden, generator=torch.Generator(device="cuda").manual_seed(4), device="cuda")
+    ids = np.random.default_rng(5).permutation(nb * k).astype(np.int32).reshape(nb, k)
+    w = torch.rand(nb, k, device="cuda")
+    got, want = torch.zeros_like(x), torch.zeros_like(x)
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, got)
+    few = max(2, 140 // (k * (inter // 128)))
+    for t in range(0, nb, few):
+        t = min(t, nb - 2)
+        want[t:t + few] = 0
+        torch.cuda.synchronize()
+        m.moe_ffn(0, x[t:t + few], ids[t:t + few], w[t:t + few].contiguous(), want[t:t + few])
+        m.synchronize()
+    assert m.test_grouped_q4(0)[0] == 0
+    assert got.abs().min(1).values.max() > 0 and torch.equal(got, want)
+    m.close()
+
+
 def rounded(cfg, x, ids, w, parts=None):
     """The layer's expert sum with what the batched kernels round rounded to bf16 (token rows, scales, scale * (q - 8), activations), all
     sums in 64 bits. parts(e): the expert's ((q, scale), (q, scale), (q, scale)) where they are not the configuration's."""
