@@ -40,7 +40,6 @@ namespace spm {
 // whose threads then have 255 registers.
 constexpr int step_warps(int nseg, bool q4) { return q4 ? q4_warps(nseg) : nseg >= 6 ? 8 : kFfnMaxWarps; }
 constexpr int kStatusStepTimeout = 16;            // status bit (1 to 8: expert and routing kernels)
-constexpr int kStepKeys = 4;                      // logits of a lane that a warp's Top-K keeps in registers
 constexpr int kStepCols = 16;                     // columns of the hidden row that an owner adds up
 constexpr int kStepMaxCtas = kReduceGroupsR * kReduceChunkR;
 constexpr unsigned long long kStepStartNs = 30000000000ull;     // default limit of the first exchange: kernels of other streams may hold SMs until then
@@ -367,37 +366,9 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
 
         // ---- Top-K; then the first weight copies go out, and the routing weights are computed behind them ----
         int sel = 0, top_key = 0;           // lane k: the k-th expert; key of the first
-        // Up to 128 experts every warp ranks for itself: the lanes hold runs of consecutive keys, largest first, and a round takes the largest of all.
-        // (Two threads an expert counting what comes before it, and a barrier: 0.9 us of a layer with 128 experts, 0.5 with 64; this takes 0.6.)
-        if (n <= 32 * kStepKeys) {
-            const int per = (n + 31) / 32;
-            int key[kStepKeys], id[kStepKeys];
-#pragma unroll
-            for (int i = 0; i < kStepKeys; ++i) {
-                id[i] = lane * per + i;
-                key[i] = i < per && id[i] < n ? reinterpret_cast<const int*>(zs)[id[i]] : INT_MIN;
-            }
-#pragma unroll
-            for (int i = 1; i < kStepKeys; ++i)         // largest first, equal ones in the order of their ids
-#pragma unroll
-                for (int j = i; j > 0; --j)
-                    if (key[j] > key[j - 1]) {
-                        const int tk = key[j], ti = id[j];
-                        key[j] = key[j - 1]; key[j - 1] = tk;
-                        id[j] = id[j - 1]; id[j - 1] = ti;
-                    }
-            for (int k = 0; k < a.K && (Q4 || wi < nw); ++k) {
-                const int most = __reduce_max_sync(0xffffffffu, key[0]);
-                const int from = __ffs(__ballot_sync(0xffffffffu, key[0] == most)) - 1;
-                const int e = __shfl_sync(0xffffffffu, id[0], from);
-                if (k == 0) top_key = most;
-                if (lane == k) sel = e;
-                if (lane == from) {
-#pragma unroll
-                    for (int i = 0; i + 1 < kStepKeys; ++i) { key[i] = key[i + 1]; id[i] = id[i + 1]; }
-                    key[kStepKeys - 1] = INT_MIN;
-                }
-            }
+        // Up to 128 experts every warp ranks for itself. (Two threads an expert counting what comes before it, and a barrier: 0.9 us of a layer with 128 experts, 0.5 with 64; this takes 0.6.)
+        if (n <= kTopKeys * 32) {
+            if (Q4 || wi < nw) sel = warp_top_k(n, a.K, lane, [&](int e) { return reinterpret_cast<const int*>(zs)[e]; }, top_key);
         } else {                            // two threads an expert count what comes before it
             const int half_n = (n / 2) & ~3;
             for (int u0 = 0; u0 < 2 * n; u0 += kStepThreads) {

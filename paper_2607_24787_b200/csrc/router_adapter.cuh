@@ -17,6 +17,8 @@
 // Every reduction has a fixed order, so results are bitwise reproducible.
 #pragma once
 
+#include <climits>
+
 #include "ptx.cuh"
 #include "../../include/spm.h"
 
@@ -129,7 +131,44 @@ __device__ __forceinline__ int rank_of_key(const int* k, int n, int e) {
     return c0 + c1 + c2 + c3;
 }
 
-constexpr int kRouterCluster = 8;   // CTAs per token, one thread-block cluster
+// The K largest of n <= 32 * kTopKeys keys, equal ones by their ids, by one warp: the lanes hold runs of consecutive keys, largest first, and a round takes
+// the largest of all. Returns the k-th in lane k and the key of the first.
+constexpr int kTopKeys = 4;
+template <typename F>
+__device__ __forceinline__ int warp_top_k(int n, int K, int lane, F key_of, int& first) {
+    const int per = (n + 31) / 32;
+    int key[kTopKeys], id[kTopKeys], sel = 0;
+#pragma unroll
+    for (int i = 0; i < kTopKeys; ++i) {
+        id[i] = lane * per + i;
+        key[i] = i < per && id[i] < n ? key_of(id[i]) : INT_MIN;
+    }
+#pragma unroll
+    for (int i = 1; i < kTopKeys; ++i)         // (stable)
+#pragma unroll
+        for (int j = i; j > 0; --j)
+            if (key[j] > key[j - 1]) {
+                const int tk = key[j], ti = id[j];
+                key[j] = key[j - 1]; key[j - 1] = tk;
+                id[j] = id[j - 1]; id[j - 1] = ti;
+            }
+    for (int k = 0; k < K; ++k) {
+        const int most = __reduce_max_sync(0xffffffffu, key[0]);
+        const int from = __ffs(__ballot_sync(0xffffffffu, key[0] == most)) - 1;
+        const int e = __shfl_sync(0xffffffffu, id[0], from);
+        if (k == 0) first = most;
+        if (lane == k) sel = e;
+        if (lane == from) {
+#pragma unroll
+            for (int i = 0; i + 1 < kTopKeys; ++i) { key[i] = key[i + 1]; id[i] = id[i + 1]; }
+            key[kTopKeys - 1] = INT_MIN;
+        }
+    }
+    return sel;
+}
+
+constexpr int kRouterCluster = 8;   // CTAs per token, one thread-block cluster ...
+constexpr int kRouterSmallCluster = 4;   // ... of a large batch
 constexpr int kStatusNonFinite = 8; // status bit (the expert kernels own bits 1, 2 and 4)
 constexpr int kReduceGroupsR = 8;   // runs of partial rows (= warps of a CTA); must equal the combine kernel's group count
 constexpr int kReduceChunkR = 20;   // partial rows a lane keeps in flight
@@ -208,7 +247,14 @@ struct RankArgs {
 __device__ __forceinline__ void rank_batch(const RankArgs& a, float* sm) {
     for (int e = threadIdx.x; e < a.n; e += blockDim.x) {
         float s = 0.f;
-        for (int t = 0; t < a.nb; ++t) s += __ldcg(a.pihat + size_t(t) * a.n + e);
+        constexpr int kAhead = 16;          // loads in flight
+        for (int t0 = 0; t0 < a.nb; t0 += kAhead) {
+            float v[kAhead];
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) v[i] = t0 + i < a.nb ? __ldcg(a.pihat + size_t(t0 + i) * a.n + e) : 0.f;
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) s += v[i];
+        }
         sm[e] = s;
     }
     __syncthreads();
@@ -226,7 +272,9 @@ __device__ __forceinline__ void rank_batch(const RankArgs& a, float* sm) {
 // on its first four warps and the adapter tail (up-projection, softmax, ranking) on the other four.
 // MINB = 1: all registers to one CTA per SM (the fold keeps 40 partial-row quads in flight);
 // MINB = 2: register budget halved so two CTAs share an SM, for batches with more CTAs than SMs.
-template <typename WT, int MINB>
+// CL: CTAs of a cluster. 32 clusters of eight run at once with two CTAs an SM; more tokens than that take clusters of four, whose CTAs have twice the rows
+// but need no second wave (64 sequences of the Qwen3 shape: 15.4 us from the first leader's start to the last one's end with eight, 9.5 with four).
+template <typename WT, int MINB, int CL>
 __global__ void __launch_bounds__(kRouterThreads, MINB)
 router_adapter_kernel(const __grid_constant__ RouterArgs a) {
     constexpr int VEC = 16 / int(sizeof(WT));
@@ -264,7 +312,7 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
     // hidden row becomes readable. Router rows then adapter-A rows, one warp per row, ROWS rows in flight.
     const int n_r = a.do_router ? n : 0;
     const int rows = n_r + (a.do_adapter ? a.r : 0);
-    constexpr int STRIDE = kRouterCluster * kRouterWarps;
+    constexpr int STRIDE = CL * kRouterWarps;
     const bool fused = MINB == 1 && a.partial != nullptr;   // this launch also sums the preceding expert kernel's partial rows
     uint4 v[ROWS][MAXIT];
     auto row_ptr = [&](int row) {
@@ -444,6 +492,13 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
     const int half = threadIdx.x >> 7, ht = threadIdx.x & 127;
     if (half == 0 && a.do_router) {
         if (ht < a.K) { isel[ht] = 0; psel[ht] = 0.f; }     // stays in range even if NaN logits leave a rank unfilled
+        auto put = [&](int k, int e, float w) {
+            a.ids[size_t(tok) * a.K + k] = e;
+            a.w[size_t(tok) * a.K + k] = w;
+            if (mb) mb->ids[tok * a.K + k] = tagged(tag, e);      // the host may start on these at once
+            // slot numbers for an expert kernel that follows without a host turn
+            if (a.codes_out) a.codes_out[tok * a.K + k] = smap[e];
+        };
         for (int e = ht; e < n; e += 128) {
             float z = zs[e];
             if (!isfinite(z)) {      // ids of this token are meaningless then; keep the ordering total so every rank is filled
@@ -457,19 +512,26 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
         }
         asm volatile("bar.sync 1, 128;" ::: "memory");
         half_softmax(ps, n, scratch, 1);          // ps = p, zs = order keys of z (ranking is taken on the logits)
-        for (int e = ht; e < n; e += 128) {
-            const int rk = rank_of_key(reinterpret_cast<const int*>(zs), n, e);
-            if (rk < a.K) { isel[rk] = e; psel[rk] = ps[e]; }
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (ht < a.K) {
-            float tot = 0.f;
-            for (int k = 0; k < a.K; ++k) tot += psel[k];
-            a.ids[size_t(tok) * a.K + ht] = isel[ht];
-            a.w[size_t(tok) * a.K + ht] = a.renorm ? psel[ht] / tot : psel[ht];
-            if (mb) mb->ids[tok * a.K + ht] = tagged(tag, isel[ht]);      // the host may start on these at once
-            // slot numbers for an expert kernel that follows without a host turn
-            if (a.codes_out) a.codes_out[tok * a.K + ht] = smap[isel[ht]];
+        if (n <= 32 * kTopKeys) {                 // one warp ranks (128 threads that count what comes before their expert take 1.1 - 1.5 us, and a barrier)
+            if (wi == 0) {
+                int first;
+                const int e = warp_top_k(n, a.K, lane, [&](int i) { return reinterpret_cast<const int*>(zs)[i]; }, first);
+                const float p = lane < a.K ? ps[e] : 0.f;
+                float tot = 0.f;
+                for (int k = 0; k < a.K; ++k) tot += __shfl_sync(0xffffffffu, p, k);
+                if (lane < a.K) put(lane, e, a.renorm ? p / tot : p);
+            }
+        } else {
+            for (int e = ht; e < n; e += 128) {
+                const int rk = rank_of_key(reinterpret_cast<const int*>(zs), n, e);
+                if (rk < a.K) { isel[rk] = e; psel[rk] = ps[e]; }
+            }
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (ht < a.K) {
+                float tot = 0.f;
+                for (int k = 0; k < a.K; ++k) tot += psel[k];
+                put(ht, isel[ht], a.renorm ? psel[ht] / tot : psel[ht]);
+            }
         }
     }
     if (half == 1 && a.do_adapter) {

@@ -661,16 +661,18 @@ int launch_router(spm_ctx* c, int layer, const float* h, const float* x_in, int 
         at[1].val.programmaticStreamSerializationAllowed = 1;
         lc.numAttrs = 2;
     }
-    // more CTAs than SMs: the variant compiled for two CTAs per SM halves the number of waves
-    const bool dense = kRouterCluster * nb > c->num_sms && !a.partial;
+    // more CTAs than SMs: the variants compiled for two CTAs per SM halve the number of waves
+    const bool dense = kRouterCluster * nb > c->num_sms && !a.partial, small = dense && nb > 32;
+    if (small) { lc.gridDim.x = kRouterSmallCluster; at[0].val.clusterDim.x = kRouterSmallCluster; }
     auto go = [&](auto kern) -> int {
         if (smem > 48 * 1024) CU(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
         CU(c, cudaLaunchKernelEx(&lc, kern, a));
         return SPM_OK;
     };
     int rc;
-    if (m.dtype != SPM_DTYPE_FP32) rc = dense ? go(router_adapter_kernel<bf16_t, 2>) : go(router_adapter_kernel<bf16_t, 1>);
-    else rc = dense ? go(router_adapter_kernel<float, 2>) : go(router_adapter_kernel<float, 1>);
+    constexpr int C8 = kRouterCluster, C4 = kRouterSmallCluster;
+    if (m.dtype != SPM_DTYPE_FP32) rc = small ? go(router_adapter_kernel<bf16_t, 2, C4>) : dense ? go(router_adapter_kernel<bf16_t, 2, C8>) : go(router_adapter_kernel<bf16_t, 1, C8>);
+    else rc = small ? go(router_adapter_kernel<float, 2, C4>) : dense ? go(router_adapter_kernel<float, 2, C8>) : go(router_adapter_kernel<float, 1, C8>);
     if (rc) return rc;
     CU(c, cudaGetLastError());
     c->kernel_launches++;

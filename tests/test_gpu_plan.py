@@ -1,6 +1,7 @@
 """Edges of the device-side plan of a batched host-free step and of the ranking made beside it."""
 import numpy as np
 import pytest
+import torch
 
 import synth
 from test_gpu_edges import build
@@ -53,3 +54,29 @@ def test_units_cut_on_the_device_give_the_bits_of_the_host_plan(hidden, inter, n
         m.close()
     for a, b in zip(*outs):
         assert np.isfinite(a).all() and np.array_equal(a, b)
+
+
+# sequences on either side of the lines between clusters of eight, one and two CTAs an SM, and clusters of four; experts on either side of what one warp ranks
+@pytest.mark.parametrize("nb", [18, 19, 32, 33, 47, 64])
+@pytest.mark.parametrize("hidden,n,k", [(256, 128, 16), (512, 131, 5), (2048, 37, 8)])
+def test_routing_of_a_batch_equals_one_sequence_at_a_time(nb, hidden, n, k):
+    cfg = synth.get_config("qwen3", n_layers=2, hidden=hidden, inter=128, n_experts=n, top_k=k, slots=n, batch=nb, budget=1, adapter_rank=5)
+    m = build(cfg)
+    h = torch.randn(nb, hidden, generator=torch.Generator(device="cuda").manual_seed(nb), device="cuda")
+    h[nb // 2] = h[0]
+    m._keep[1][0, 3] = m._keep[1][0, 9]         # two experts that always tie
+    torch.cuda.synchronize()
+    x, ids, w, logits = m.router_topk(0, h, want_logits=True)
+    scores, order = m.adapter_predict(0, x)
+    one = [m.router_topk(0, h[t:t + 1].contiguous(), want_logits=True) for t in range(nb)]
+    each = [m.adapter_predict(0, x[t:t + 1].contiguous())[0] for t in range(nb)]
+    m.synchronize()
+    for t, (xt, it, wt, lt) in enumerate(one):
+        assert torch.equal(x[t], xt[0]) and np.array_equal(ids[t], it[0]) and torch.equal(w[t], wt[0]) and torch.equal(logits[t], lt[0]), t
+        ranked = sorted(range(n), key=lambda e: (-float(lt[0, e]), e))
+        assert list(it[0]) == ranked[:k], t
+    want = np.zeros(n, np.float32)
+    for s in each:
+        want += s                               # (fp32, in token order)
+    assert np.array_equal(scores, want) and list(order) == sorted(range(n), key=lambda e: (-want[e], e))
+    m.close()
