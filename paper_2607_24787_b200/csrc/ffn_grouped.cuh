@@ -586,15 +586,31 @@ inline size_t ffn_grouped_smem() {
            2 * kGgQueue * sizeof(uint64_t) + kGgQueue * sizeof(GgTask);
 }
 
-// One token row as bf16, by all threads of the block.
-__device__ __forceinline__ void gg_copy_row(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int D, int perm8) {
-    if (perm8) {
-        // columns 8g .. 8g+7 are stored in the order 0 4 1 5 2 6 3 7: the order in which the 4-bit
-        // kernel unpacks a word of eight weights, so that its operand needs no re-ordering
-        for (int i = threadIdx.x * 8; i < D; i += blockDim.x * 8) {
-            const float4 v0 = *reinterpret_cast<const float4*>(src + i), v1 = *reinterpret_cast<const float4*>(src + i + 4);
-            const __nv_bfloat162 p0 = __floats2bfloat162_rn(v0.x, v1.x), p1 = __floats2bfloat162_rn(v0.y, v1.y);
-            const __nv_bfloat162 p2 = __floats2bfloat162_rn(v0.z, v1.z), p3 = __floats2bfloat162_rn(v0.w, v1.w);
+// One token row as bf16, by the kGgPairThreads threads of a block, in two halves: a thread's loads, which need not know where the row goes, and its stores.
+// (The loads ahead of the counting, and the residual's ahead of the sums in gg_combine_kernel: 2.7 us a layer at 5 and 4.6 at 64 sequences of the Qwen3 shape.)
+constexpr int kGgPairThreads = 128;
+struct GgRowCopy {
+    static constexpr int kChunks = 2;          // of eight columns a thread: hidden <= 2048
+    float4 v[kChunks][2];
+    __device__ __forceinline__ void load(const float* __restrict__ src, int D) {
+#pragma unroll
+        for (int c = 0; c < kChunks; ++c) {
+            const int i = (c * kGgPairThreads + int(threadIdx.x)) * 8;
+            if (i < D) { v[c][0] = *reinterpret_cast<const float4*>(src + i); v[c][1] = *reinterpret_cast<const float4*>(src + i + 4); }
+        }
+    }
+    // perm8: columns 8g .. 8g + 7 in the order 0 4 1 5 2 6 3 7: the order in which the 4-bit
+    // kernel unpacks a word of eight weights, so that its operand needs no re-ordering
+    __device__ __forceinline__ void store(__nv_bfloat16* __restrict__ dst, int D, int perm8) const {
+#pragma unroll
+        for (int c = 0; c < kChunks; ++c) {
+            const int i = (c * kGgPairThreads + int(threadIdx.x)) * 8;
+            if (i >= D) continue;
+            const float4 v0 = v[c][0], v1 = v[c][1];
+            const __nv_bfloat162 p0 = perm8 ? __floats2bfloat162_rn(v0.x, v1.x) : __floats2bfloat162_rn(v0.x, v0.y);
+            const __nv_bfloat162 p1 = perm8 ? __floats2bfloat162_rn(v0.y, v1.y) : __floats2bfloat162_rn(v0.z, v0.w);
+            const __nv_bfloat162 p2 = perm8 ? __floats2bfloat162_rn(v0.z, v1.z) : __floats2bfloat162_rn(v1.x, v1.y);
+            const __nv_bfloat162 p3 = perm8 ? __floats2bfloat162_rn(v0.w, v1.w) : __floats2bfloat162_rn(v1.z, v1.w);
             uint4 o;
             o.x = *reinterpret_cast<const uint32_t*>(&p0);
             o.y = *reinterpret_cast<const uint32_t*>(&p1);
@@ -602,17 +618,8 @@ __device__ __forceinline__ void gg_copy_row(const float* __restrict__ src, __nv_
             o.w = *reinterpret_cast<const uint32_t*>(&p3);
             *reinterpret_cast<uint4*>(dst + i) = o;
         }
-    } else {
-        for (int i = threadIdx.x * 4; i < D; i += blockDim.x * 4) {
-            const float4 v = *reinterpret_cast<const float4*>(src + i);
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-            uint2 o;
-            o.x = *reinterpret_cast<const uint32_t*>(&lo);
-            o.y = *reinterpret_cast<const uint32_t*>(&hi);
-            *reinterpret_cast<uint2*>(dst + i) = o;
-        }
     }
-}
+};
 
 // Sorted token rows of one wave: Xs[row][:] = bf16(x[token][:]), wrow[row] = w[token][k].
 struct GgRow { int32_t token, k; };
@@ -627,7 +634,9 @@ static __global__ void gg_gather_kernel(const float* __restrict__ x, const float
     const int r = blockIdx.x;
     if (r >= n_rows) return;
     const GgRow ri = rows[r];
-    gg_copy_row(x + size_t(ri.token) * D, xs + size_t(r) * D, D, perm8);
+    GgRowCopy row;
+    row.load(x + size_t(ri.token) * D, D);
+    row.store(xs + size_t(r) * D, D, perm8);
     if (threadIdx.x == 0) wrow[r] = w[size_t(ri.token) * K + ri.k];
 }
 
@@ -647,6 +656,7 @@ static __global__ void gg_combine_kernel(const float* __restrict__ partial, cons
     const int c = threadIdx.x % kCombineCols, k = threadIdx.x / kCombineCols;
     const int d = (blockIdx.x * kCombineCols + c) * 4;
     const int r = (k < K && d < D) ? rowmap[t * SPM_MAX_TOPK + k] : -1;
+    float4 tot = k == 0 && d < D ? *reinterpret_cast<const float4*>(h + size_t(t) * D + d) : make_float4(0.f, 0.f, 0.f, 0.f);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (r >= 0) {
         for (int j0 = 0; j0 < n_jt; j0 += kCombineMaxJt) {
@@ -663,7 +673,6 @@ static __global__ void gg_combine_kernel(const float* __restrict__ partial, cons
     if (k < K) part[k][c] = acc;
     __syncthreads();
     if (k == 0 && d < D) {
-        float4 tot = *reinterpret_cast<const float4*>(h + size_t(t) * D + d);
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int kk = 0; kk < K; ++kk) {
             if (rowmap[t * SPM_MAX_TOPK + kk] < 0) continue;
@@ -684,7 +693,6 @@ inline dim3 gg_combine_block(int K) { return dim3(kCombineCols * K); }
 // its expert and how many experts come before it, then copies its token row; the first pair of an expert writes the
 // expert's units. (With a plan kernel of one CTA ahead of the gather: 87.3 us a layer instead of 85.5 at 5 sequences of the Qwen3 shape,
 // 229 instead of 226 at 64.)
-constexpr int kGgPairThreads = 128;
 static_assert(SPM_MAX_BATCH * SPM_MAX_TOPK < (1 << 21), "three counts of pairs share a 64-bit word");
 
 static __global__ void __launch_bounds__(kGgPairThreads)
@@ -711,6 +719,8 @@ gg_plan_gather_kernel(const float* __restrict__ x, const float* __restrict__ w, 
     // the grouped kernel that follows counts arrivals per unit from zero
     if (i == 0) for (int v = tid; v < n_ready; v += kGgPairThreads) act_ready[v] = 0;
     const int e = __ldcg(ids + i), t = i / K, k = i - t * K;
+    GgRowCopy row;                       // (on its way while the pairs are counted)
+    row.load(x + size_t(t) * D, D);
     __syncthreads();
     unsigned long long c = 0;            // pairs of lower experts | earlier pairs of this expert << 21 | all pairs of this expert << 42
     for (int j = tid; j < n_pairs; j += kGgPairThreads) {
@@ -744,7 +754,7 @@ gg_plan_gather_kernel(const float* __restrict__ x, const float* __restrict__ w, 
             for (int jt = tid; jt < n_jt; jt += kGgPairThreads) units[rank * n_jt + jt] = GgUnit{slot_base + (slot < 0 ? 0 : slot), jt, start, cnt};
         }
     }
-    gg_copy_row(x + size_t(t) * D, xs + size_t(r) * D, D, perm8);
+    row.store(xs + size_t(r) * D, D, perm8);
 }
 
 }  // namespace spm
