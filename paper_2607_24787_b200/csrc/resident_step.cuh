@@ -15,7 +15,7 @@
 // One buffer per exchange is enough: a CTA overwrites a word one layer later, when it holds data that every reader of
 // the old word contributed to after reading it.
 //
-// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 15.9 (21): the FFN 11.5 - 13 and 8 - 10 with the slowest SM 2 us
+// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 15.5 (21): the FFN 11.5 - 13 and 8 - 10 with the slowest SM 2 us
 // behind the mean, and a chain of latencies of 6 (partial rows 1.4, hidden row 1, norm and dot products 1.5, logits 1.1, Top-K 0.6, first
 // copies 0.5). With 4-bit experts 16.8 and 13.5, 6 and 4.5 of which are the tiles.
 //
@@ -23,7 +23,7 @@
 // outputs have the same bits as host-driven steps. The adapter's ranking, which only the host reads, is done by the last
 // CTA (which owns no columns where there are fewer than 16 a CTA) while the others exchange the hidden row.
 //
-// Registers: nine warps leave a thread 168, sixteen 128. Instances that spill: hidden 1280 of bf16 (132 bytes stored, 164 loaded), hidden 1792 and
+// Registers: nine or ten warps leave a thread 168, sixteen 128. Instances that spill: hidden 1280 of bf16 (68 bytes stored and loaded), hidden 1792 and
 // 2048 of 4 bits (120 / 152 and 132 / 164); 20 bytes and less at 1280 and 1536 of 4 bits.
 //
 // The CTAs wait for one another, so the launch is cooperative (one CTA per SM, all resident or none). Every wait is
@@ -37,8 +37,9 @@
 namespace spm {
 
 // Warps of a CTA: as many as the GEMV may take (those it does not use only route). Rows of 9216 bytes and more leave it eight at most,
-// whose threads then have 255 registers.
-constexpr int step_warps(int nseg, bool q4) { return q4 ? q4_warps(nseg) : nseg >= 6 ? 8 : kFfnMaxWarps; }
+// whose threads then have 255 registers. Rows of five segments have one more than the GEMV takes: the 320 quads of a hidden row of 1280 bf16 then are
+// one a thread (DeepSeek shape 15.8 -> 15.45 us a layer; twelve warps 15.8. Ten or twelve warps at fewer segments: within 2 % either way.)
+constexpr int step_warps(int nseg, bool q4) { return q4 ? q4_warps(nseg) : nseg >= 6 ? 8 : nseg == 5 ? kFfnMaxWarps + 1 : kFfnMaxWarps; }
 constexpr int kStatusStepTimeout = 16;            // status bit (1 to 8: expert and routing kernels)
 constexpr int kStepCols = 16;                     // columns of the hidden row that an owner adds up
 constexpr int kStepMaxCtas = kReduceGroupsR * kReduceChunkR;
