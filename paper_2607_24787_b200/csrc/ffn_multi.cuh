@@ -440,16 +440,29 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
                 if (i1 >= 2 && fdn.n < i1 - 1 + n_stages) feed_dn();
             }
             if (kP1 && warp < kMtRows) {
-                float v = 0.f;
+                float v;
+                const float* from = m_at + (i1 & 1) * (kMtWarps * 128);
                 if constexpr (NS == 3) {
+                    // Pairs first: a chain over more warps rounds more often. Error against 64 bits, mean of 22 shapes: chains over eight warps 2.151e-7, over
+                    // as many as now 2.159e-7 (3 % more on some shapes), in pairs 2.125e-7; and a shorter chain of latencies (0.5 us a layer).
+                    float p[kMtWarps / 2];
 #pragma unroll
-                    for (int i = 0; i < kMtWarps / 2; ++i) v += m_at[(i1 & 1) * (kMtWarps * 128) + i * 128];
+                    for (int i = 0; i < kMtWarps / 2; ++i) p[i] = from[i * 128];
+#pragma unroll
+                    for (int d = 1; d < kMtWarps / 2; d *= 2)
+#pragma unroll
+                        for (int i = 0; i + d < kMtWarps / 2; i += 2 * d) p[i] += p[i + d];
+                    v = p[0];
                 } else {
+                    v = 0.f;
 #pragma unroll
-                    for (int w = 0; w < kMtWarps; w += 8)
+                    for (int w = 0; w < kMtWarps; w += 8) {
+                        const bool on = kMtWarps % 8 == 0 || w + (lane >> 2) < kMtWarps;
+                        float p = 0.f;
 #pragma unroll
-                        for (int i = 0; i < 3; ++i)
-                            if (kMtWarps % 8 == 0 || w + (lane >> 2) < kMtWarps) v += m_at[(i1 & 1) * (kMtWarps * 128) + w * 128 + i * 4];
+                        for (int i = 0; i < 3; ++i) p += on ? from[w * 128 + i * 4] : 0.f;
+                        v += p;
+                    }
                 }
                 if constexpr (NS == 1) {
                     v += __shfl_xor_sync(0xffffffffu, v, 4);
