@@ -6,8 +6,10 @@
 // is the way of an operand: unpack, store to tensor or shared memory, fence, hand-shake, 1050 cycles for an item that HBM
 // delivers in 340. An mma.sync operand is where the unpacking leaves it, in the registers of the lane that needs it. A layer of a whole
 // host-free step of that shape: 197 -> 146 us (HBM time of its experts: 49; 142 with exact weights and the scale on the activations,
-// which rounds elsewhere than the tcgen05 kernel: outputs of 64 sequences then moved by 1e-2 where a near-tied Top-K choice tipped).
-// What bounds it now: instruction issue and dependent-issue latency, 106,000 instructions a scheduler at 0.57 a cycle.
+// which rounds elsewhere than the tcgen05 kernel: outputs of 64 sequences then moved by 1e-2 where a near-tied Top-K choice tipped), 133 with
+// TMA boxes and split tasks (below), 125 with shorter routing, gather and combine kernels around it.
+// What bounds it now: instruction issue and dependent-issue latency, 99,000 instructions a scheduler at 0.56 a cycle; the packed bf16 multiply-adds of the
+// unpacking run at half rate (FMA pipe 45 %, ALU 42 % of active cycles).
 //
 // Work. A task is 128 intermediate rows of an expert (GgUnit) for up to kMqTokens of its tokens; CTA b runs the tasks b, b + grid, ...
 // of all experts in order (a hot expert's runs of tokens go to different CTAs), but for the last one to two tasks a CTA, which are split

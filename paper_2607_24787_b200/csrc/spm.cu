@@ -538,10 +538,11 @@ cudaError_t launch_grouped_q4_mma_t(const spm_ctx* c, const MqArgs& a) {
 // tcgen05 kernel costs a CTA's units (an expert's 128 rows), in proportion to hidden and up to twice as much with many tokens. The
 // costs below are in us per 16 rows, from whole host-free steps (us a layer, tcgen05 / mma.sync; sequences, top-k of experts, hidden;
 // 768 rows an expert):
-//   64, 8 of 128, 2048: 197 / 146     8, 8 of 128, 2048: 103 / 70     64, 8 of 60, 2048: 140 / 111     64, 8 of 24, 2048:  84 / 101
-//   64, 8 of 128, 1280: 134 / 126     2, 8 of 128, 2048:  52 / 39     32, 4 of 12, 2048:  61 / 43      64, 8 of 12, 2048:  94 / 93
-//   64, 8 of 128,  768:  98 / 99     64, 8 of 128,  512:  76 / 89     64, 8 of 128, 256:  57 / 92      32, 8 of 24, 2048:  67 / 64
-// (of 22 shapes measured on both, the rule takes the slower one for two, by 4 and 5 %)
+//   64, 8 of 128, 2048: 189 / 125     8, 8 of 128, 2048: 101 / 58     64, 8 of 60, 2048: 131 / 95      64, 8 of 24, 2048:  74 / 83
+//   64, 8 of 128, 1280: 128 / 104     2, 8 of 128, 2048:  50 / 36     32, 4 of 12, 2048:  59 / 40      64, 8 of 12, 2048:  85 / 81
+//   64, 8 of 128,  768:  92 / 83      64, 8 of 128,  512:  71 / 76     64, 8 of 128, 1024: 108 / 91     32, 8 of 24, 2048:  62 / 60
+// (of these the rule takes the slower one for two, 64 sequences of 768 columns and 32 of 24 experts, by 11 and 4 %: its line was drawn before the mma.sync
+// kernel split its last tasks, and the two kernels' outputs differ by the order of sums)
 bool grouped_q4_mma_pays(const spm_ctx* c, int nb) {
     const spm_model_cfg& m = c->cfg;
     if (m.hidden < 512 || mq_max_tasks(nb, m.top_k, m.n_experts, c->n_jt, c->num_sms) > kMqMaxTasks) return false;      // (rows of 256: never worth it)
