@@ -270,6 +270,8 @@ int mt_grid_for(const spm_ctx* c) { return std::min(c->num_sms, kMtMaxCtas); }
 //          512 x 384, 64 tokens 3 + 1 of 96: 104 -> 91 (89)       640 x 735, 31 tokens 7 + 1 of 128: 173 -> 191 (160)
 // Of 124 shapes that it chooses four are slower than with the GEMV, by 2 - 3 %; of those above 64 Mi that it leaves to the GEMV
 // two would gain 7 - 8 %.
+// (All with eight warps a CTA. With as many as launch_multi_g takes now the kernel's steps are 0 - 18 % shorter, so the line errs towards the GEMV; it stays where
+// it is, because the two add in different orders.)
 constexpr size_t kMi = size_t(1) << 20;
 bool multi_pays(const spm_model_cfg& m, int nb) {
     const size_t D = m.hidden, expert = size_t(3) * m.inter * D;
