@@ -30,6 +30,7 @@
 
 #include "ffn_gemv.cuh"
 #include "q4_mma.cuh"
+#include "q4_rounds.h"
 
 namespace spm {
 
@@ -53,7 +54,7 @@ struct Q4Part {
 // Where the tiles of a CTA are: a ring of stages of kQ4Rows rows, one barrier a stage that completes when all rows of it have been asked for
 // and have landed, the phase-1 sums [tile of a round][warps][kQ4Red], gate and up of each row, and the activations [tile of a round][rows].
 constexpr int kQ4Red = 33;             // (a lane reads one row's sum of one warp)
-constexpr int kQ4Super = 4;            // tiles of a round
+static_assert(kQ4MaxStages <= 2 * kQ4Super, "half of a ring is a round");
 template <int NW>
 struct Q4Ring {
     uint32_t rows, bars, pitch;
@@ -140,8 +141,8 @@ __device__ __forceinline__ void q4_operand(uint32_t (&x)[GB][4], int warp, int l
 // activations, phase 2 of all. What bounds a round is the latency between dependent instructions, which several tiles between two barriers
 // hide: whole steps of the 4-bit Qwen3 shape (three tiles a CTA), us a layer, 18.1 a tile at a time -> 17.3, DeepSeek shape (four, the last of one
 // row) 16.1 -> 13.8. (One barrier a tile, phase 2 a tile behind phase 1: 18.0 and 14.4.) Where the ring holds fewer tiles than the
-// CTA has, a round takes half of it, so that the other half is on its way. fill(tile): ask for the warp's rows of a tile; the first `stages` tiles have been
-// asked for. weight(row): routing weight. Every thread of the CTA takes part. Returns false, in every
+// CTA has, two neighbouring rounds fill it (q4_rounds.h), so that one is on its way. fill(tile): ask for the warp's rows of a tile; the first
+// `stages` tiles have been asked for. weight(row): routing weight. Every thread of the CTA takes part. Returns false, in every
 // thread, when a wait ran out (the caller drains and leaves).
 template <int GB, int NW, typename Fill, typename Weight>
 __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[GB][4], float (&y)[GB][2][4], int D, int span,
@@ -149,10 +150,10 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
     const int g = lane >> 2, t = lane & 3, grp0 = warp * GB;
     const int tiles = (span + kQ4Rows - 1) / kQ4Rows;
     const uint32_t P = ring.pitch, PART = q4_part_bytes(D);
-    const int most = min(kQ4Super, tiles <= ring.stages ? tiles : (ring.stages + 1) / 2), rounds = (tiles + most - 1) / max(most, 1);
+    Q4Rounds rounds(tiles, ring.stages);
     int before = 0;                  // tiles of the round before
-    for (int k = 0, left = rounds; left > 0; --left) {
-        const int nt = (tiles - k + left - 1) / left;
+    for (int k = 0; rounds.left > 0;) {
+        const int nt = rounds.next(tiles - k);
         int st0 = ring.st;
         auto rows_of = [&](int u) { return ring.rows + uint32_t((st0 + u < ring.stages ? st0 + u : st0 + u - ring.stages) * kQ4Rows) * P; };
         // `whole`: for the case below, a group's three parts added up before the scale goes onto them

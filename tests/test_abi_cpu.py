@@ -148,6 +148,75 @@ def test_a_captured_step_is_replayed_only_where_everything_it_was_built_from_is_
     assert subprocess.run([str(tmp_path / "key")]).returncode == 0
 
 
+def test_rounds_of_tiles_never_wait_for_a_tile_that_nobody_asked_for(tmp_path):
+    """Rings of two to eight stages, none to 400 tiles, as the one-token 4-bit kernels walk them: a round's tiles have been asked for when it waits for
+    them, and a stage is filled again only behind the round that read it."""
+    import shutil
+    import subprocess
+    if not shutil.which("g++"):
+        pytest.skip("no host compiler")
+    src = tmp_path / "rounds.cpp"
+    src.write_text('''#include <cstdio>
+#include "q4_rounds.h"
+int main() {
+  int bad = 0;
+  for (int stages = 2; stages <= 8; ++stages)
+    for (int tiles = 0; tiles <= 400; ++tiles) {
+      spm::Q4Rounds r(tiles, stages);
+      int asked = tiles < stages ? tiles : stages, k = 0, before = 0, rounds = 0;
+      bool ok = true;
+      for (; ok && r.left > 0; ++rounds) {
+        const int nt = r.next(tiles - k);
+        ok = nt >= 1 && nt <= spm::kQ4Super && k + nt <= asked;          // (waited for: k .. k + nt - 1)
+        for (int u = k - before; u < k; ++u)                             // the stages of the round before
+          if (u + stages < tiles) ok = ok && asked++ == u + stages;
+        k += nt;
+        before = nt;
+      }
+      ok = ok && k == tiles && asked == tiles && rounds <= 2 * ((tiles + stages - 1) / stages);
+      if (!ok && bad++ < 20) std::printf("ring of %d, %d tiles: tile %d of round %d, %d asked for\\n", stages, tiles, k, rounds, asked);
+    }
+  return bad != 0;
+}
+''')
+    subprocess.run(["g++", "-std=c++17", "-Wall", "-I", os.path.join(ROOT, "paper_2607_24787_b200", "csrc"), "-o", str(tmp_path / "rounds"), str(src)], check=True)
+    walk = subprocess.run([str(tmp_path / "rounds")], capture_output=True, text=True)
+    assert walk.returncode == 0, walk.stdout
+
+
+def test_gpu_tests_of_odd_rings_have_rings_of_that_size(tmp_path):
+    """The shapes with which the one-token 4-bit kernels are run on odd rings have the number of stages that the tests state (148 SMs), and more tiles."""
+    import subprocess
+    import test_gpu_q4_mma as Q
+    import test_gpu_resident as R
+    cases = []              # hidden, rows, stages, experts and adapter rank of a one-kernel step (else 0)
+    cases += [(d, inter, st, 0, 0) for d, inter, st in Q.ODD_RINGS]
+    cases += [(d, -(-(k + shared) * inter // (296 // nb)), st, 0, 0) for d, inter, n, k, shared, nb, st in Q.ODD_RINGS_BATCHED]
+    for name, kw in R.CASES.items():
+        if name.startswith("q4_ring_of"):
+            st = {"three": 3, "five": 5, "seven": 7}[name.split("_")[3]]
+            cases.append((kw["hidden"], -(-(kw["top_k"] + kw.get("n_shared", 0)) * kw["inter"] // 148), st, kw["n_experts"], kw["adapter_rank"]))
+    src = tmp_path / "ring.cu"
+    src.write_text('#include <cstdio>\n#include "resident_step.cuh"\nint main() {\n  const int cases[][5] = {'
+                   + ", ".join("{%d, %d, %d, %d, %d}" % c for c in cases)
+                   + """};
+  int bad = 0;
+  for (auto& c : cases) {
+    int stages = 0;
+    spm::ffn_gemv_q4_shape(c[0], c[1], c[3] ? spm::step_route_bytes(c[0], c[3], c[4], false) + 16 : 0, &stages);
+    const int tiles = (c[1] + spm::kQ4Rows - 1) / spm::kQ4Rows;
+    if (stages != c[2] || stages % 2 == 0 || tiles <= stages) { ++bad; std::printf("hidden %d, %d rows: %d stages, %d tiles\\n", c[0], c[1], stages, tiles); }
+  }
+  return bad != 0;
+}
+""")
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "--expt-relaxed-constexpr", "-I",
+                    os.path.join(ROOT, "paper_2607_24787_b200", "csrc"), "-o", str(tmp_path / "ring"), str(src)], check=True)
+    got = subprocess.run([str(tmp_path / "ring")], capture_output=True, text=True)
+    assert got.returncode == 0, got.stdout
+
+
 def test_noalloc_argument_checks_run_before_any_gpu_work():
     """The allocation-free entry point refuses bad shapes, indices and misaligned pointers on the
     host, before it touches the device: so this runs without a GPU (addresses below are never

@@ -9,6 +9,7 @@ import torch
 import synth
 from paper_2607_24787_b200.binding import SpmError
 from test_gpu_edges import build
+from test_gpu_multi import takes_kernel
 
 pytestmark = pytest.mark.gpu
 
@@ -70,8 +71,8 @@ def test_infinite_operands_reach_the_result():
     m.close()
 
 
-# Rounds of tiles: 8, 9 and 17 rows a CTA (blocks of eight), 33 (a fourth tile of one row), 49 and 65 (five tiles), 70 and 144 rows with rings of
-# three and eight tiles. (hidden, inter, experts, top-k)
+# Rounds of tiles: 8, 9 and 17 rows a CTA (blocks of eight), 33 and 49 (a last tile of one row), 65 and 70 (five tiles, rings of four), 144 (nine, a ring of
+# eight). (hidden, inter, experts, top-k)
 ROUNDS = [(1024, 148, 9, 8), (512, 148, 10, 9), (1536, 148 * 17, 3, 1), (768, 148 * 3, 12, 11), (1280, 148 * 7, 8, 7), (1792, 148 * 13, 6, 5),
           (2048, 1480, 8, 7), (256, 148 * 12, 13, 12)]
 
@@ -96,6 +97,51 @@ def test_rounds_of_tiles(shape):
     assert (got.double() - want).norm() <= 1e-6 * want.norm()
     far = exact(cfg, big, ids, w).abs() > 1e39
     assert far.any() and not huge[far].isfinite().any()
+    m.close()
+
+
+# Rings of an odd number of stages, and more tiles: (hidden, rows of an expert, stages), an expert a CTA; one tile more than stages, one row either side of a
+# tile, two and three times the ring, and several hundred tiles. (tests/test_abi_cpu.py holds the stages against the kernel's own rule.)
+ODD_RINGS = [(1536, 81, 5), (1536, 96, 5), (1536, 97, 5), (1536, 161, 5), (1536, 240, 5), (1536, 5000, 5),
+             (1024, 113, 7), (1024, 128, 7), (1024, 129, 7), (1024, 180, 7), (1024, 336, 7), (1024, 5000, 7)]
+
+
+@pytest.mark.parametrize("hidden,inter,stages", ODD_RINGS)
+def test_odd_rings(hidden, inter, stages):
+    """Against 64 bits, with the bound of test_one_token_long_shares."""
+    cfg = make(hidden, inter, 5, 4, 1)
+    m = build(cfg)
+    m.set_ffn_ctas(5)
+    x = torch.randn(1, hidden, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda")
+    torch.cuda.synchronize()
+    _, ids, w, _ = m.router_topk(0, x)
+    got = torch.zeros_like(x)
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, got)
+    m.synchronize()
+    want = exact(cfg, x, ids, w)
+    assert (got.double() - want).norm() <= 5e-7 * want.norm()
+    m.close()
+
+
+# (hidden, inter, experts, top-k, shared, sequences, stages): one GEMV a sequence, on 296 CTAs over the sequences
+ODD_RINGS_BATCHED = [(1536, 600, 40, 8, 0, 5, 5), (1536, 1000, 24, 8, 0, 3, 5), (1536, 768, 24, 6, 2, 4, 5), (1024, 550, 40, 8, 0, 8, 7), (1024, 768, 36, 6, 2, 6, 7)]
+
+
+@pytest.mark.parametrize("hidden,inter,n,k,shared,nb,stages", ODD_RINGS_BATCHED)
+def test_odd_rings_of_several_sequences(hidden, inter, n, k, shared, nb, stages):
+    cfg = make(hidden, inter, n, k, shared, nb)
+    assert not takes_kernel(cfg, nb) and (shared or inter % 128)           # (neither of the batched kernels)
+    m = build(cfg)
+    x = torch.randn(nb, hidden, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda")
+    torch.cuda.synchronize()
+    _, ids, w, _ = m.router_topk(0, x)
+    got = torch.zeros_like(x)
+    torch.cuda.synchronize()
+    m.moe_ffn(0, x, ids, w, got)
+    m.synchronize()
+    want = exact(cfg, x, ids, w)
+    assert ((got.double() - want).norm(dim=1) <= 5e-7 * want.norm(dim=1)).all()
     m.close()
 
 

@@ -27,6 +27,12 @@ CASES = {
     "q4_shared": dict(base="dsvl2_q4", hidden=1280, n_experts=16, inter=224, top_k=6, n_shared=2, adapter_rank=16),
     "q4_widest": dict(base="qwen3_q4", hidden=2048, n_experts=20, inter=450, top_k=8, adapter_rank=16),
     "q4_many_experts": dict(base="qwen3_q4", hidden=768, n_experts=300, inter=33, top_k=10, adapter_rank=2),
+    "q4_ring_of_three": dict(base="qwen3_q4", hidden=2048, n_experts=12, inter=896, top_k=8, adapter_rank=16),       # (three and four tiles)
+    "q4_ring_of_three_full": dict(base="qwen3_q4", hidden=2048, n_experts=128, inter=1024, top_k=8, adapter_rank=16),
+    "q4_ring_of_three_shared": dict(base="qwen3_q4", hidden=2048, n_experts=12, inter=768, top_k=8, n_shared=2, adapter_rank=16),
+    "q4_ring_of_three_long": dict(base="qwen3_q4", hidden=2048, n_experts=9, inter=1600, top_k=8, adapter_rank=16),
+    "q4_ring_of_five": dict(base="qwen3_q4", hidden=1536, n_experts=10, inter=1517, top_k=8, adapter_rank=16),
+    "q4_ring_of_seven": dict(base="qwen3_q4", hidden=1024, n_experts=9, inter=2202, top_k=8, adapter_rank=16),
     "bf16_raw_weights": dict(base="qwen3", hidden=1792, n_experts=9, inter=100, top_k=3, renormalize=0, adapter_rank=4),
 }
 
