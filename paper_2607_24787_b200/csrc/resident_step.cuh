@@ -450,6 +450,9 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
                 return;
             }
             q4_result<GB>(y, wi, lane, send);
+            // (a CTA without rows has met no barrier since the logits: its warps may still be ranking them and adding up their exponentials,
+            // where sums of the owned columns and the adapter's logits are about to go)
+            if (span == 0) __syncthreads();
         } else {
             uint64_t ya[NSEG][VEC / 2];
 #pragma unroll

@@ -27,6 +27,9 @@ CASES = {
     "q4_shared": dict(base="dsvl2_q4", hidden=1280, n_experts=16, inter=224, top_k=6, n_shared=2, adapter_rank=16),
     "q4_widest": dict(base="qwen3_q4", hidden=2048, n_experts=20, inter=450, top_k=8, adapter_rank=16),
     "q4_many_experts": dict(base="qwen3_q4", hidden=768, n_experts=300, inter=33, top_k=10, adapter_rank=2),
+    # owners of columns, and the CTA that ranks the adapter's logits, without a row
+    "q4_fewer_rows_than_ctas": dict(base="qwen3_q4", hidden=2048, n_experts=128, inter=9, top_k=3, adapter_rank=16),
+    "q4_one_row": dict(base="qwen3_q4", hidden=512, n_experts=100, inter=1, top_k=1, adapter_rank=40),
     "q4_ring_of_three": dict(base="qwen3_q4", hidden=2048, n_experts=12, inter=896, top_k=8, adapter_rank=16),       # (three and four tiles)
     "q4_ring_of_three_full": dict(base="qwen3_q4", hidden=2048, n_experts=128, inter=1024, top_k=8, adapter_rank=16),
     "q4_ring_of_three_shared": dict(base="qwen3_q4", hidden=2048, n_experts=12, inter=768, top_k=8, n_shared=2, adapter_rank=16),
