@@ -16,13 +16,17 @@ namespace spm {
 constexpr int kQ4Super = 4;            // tiles of a round at most
 
 struct Q4Rounds {
-    int both;                          // tiles of two neighbouring rounds at most
+    int both;                          // tiles of two neighbouring rounds at most (0: all tiles are in the ring)
     int left;                          // rounds to come
     // All tiles in the ring: nothing is filled again. Else as many rounds as halves of the ring, rounded up and down in turn, take.
     SPM_HD Q4Rounds(int tiles, int stages) {
-        both = tiles <= stages ? 2 * kQ4Super : stages;
-        const int pairs = tiles / both, rest = tiles - pairs * both;
-        left = 2 * pairs + (rest > (both + 1) / 2 ? 2 : rest > 0 ? 1 : 0);
+        both = tiles <= stages ? 0 : stages;
+        if (both == 0) {
+            left = tiles > kQ4Super ? 2 : tiles > 0 ? 1 : 0;
+        } else {
+            const int pairs = tiles / both, rest = tiles - pairs * both;
+            left = 2 * pairs + (rest > (both + 1) / 2 ? 2 : rest > 0 ? 1 : 0);
+        }
     }
     // Tiles of the next round, of `tiles` to come. In a ring that is filled again the last round takes half of it, rounded up, the one ahead of it half
     // rounded down, and so on, and the first what is left, which gives stages back early. Whole steps of one sequence, us a layer, a tile at a time :
@@ -30,7 +34,7 @@ struct Q4Rounds {
     // 1600 (six tiles) 25.6 : 27.4 : 26.2 : 25.5, 1536 x 1517 (five stages, six tiles) 22.2 : 23.0 : 22.3 : 21.4.
     SPM_HD int next(int tiles) {
         --left;
-        if (both == 2 * kQ4Super) return (tiles + left) / (left + 1);
+        if (both == 0) return (tiles + left) >> left;
         return tiles - (left / 2 * both + (left & 1) * ((both + 1) / 2));
     }
 };

@@ -24,7 +24,7 @@
 // CTA (which owns no columns where there are fewer than 16 a CTA) while the others exchange the hidden row.
 //
 // Registers: nine or ten warps leave a thread 168, sixteen 128. Instances that spill: hidden 1280 of bf16 (68 bytes stored and loaded), hidden 1792 and
-// 2048 of 4 bits (116 / 148 and 128 / 160); 4 bytes at 1536 of 4 bits.
+// 2048 of 4 bits (116 / 148 and 128 / 160); 12 bytes at 1280 of 4 bits.
 //
 // The CTAs wait for one another, so the launch is cooperative (one CTA per SM, all resident or none). Every wait is
 // bounded: a CTA that gives up raises a flag that the others' waits look at, and all of them return with nothing in flight.
