@@ -17,6 +17,9 @@
 // finished by the second after all else: a chain of sums is the same whoever adds, so outputs have the same bits. (760 tasks of 64 sequences of the
 // Qwen3 shape on 148 CTAs: six for some, where an even share is 5.1; 137.5 -> 133 us a layer; 16 sequences 87.6 -> 82, 8: 66.5 -> 60.3. 64 of 60
 // experts lose 1 %, two sequences, which give no CTA a second task, 0.6 us.)
+// Tasks are split, too, where the kernel waits for copies of experts. What a CTA begins first may then be of an expert that is on its way, and holds up the
+// rest; but so may any task of a list in order, and a wave's copies are one arrival. Offloaded steps of the Qwen3 shape with device-side waits, us a
+// layer, split : in order: 4 sequences, 120 slots 109 : 115, 16 sequences, 96 slots 997 : 1004, 64 sequences, 32 slots 4982 : 4999.
 // A task goes through its rows in tiles of 16; the warps split the columns in groups of 32 (one scale), GB consecutive groups a warp.
 //   Phase 1 (M = 16 gate rows, then 16 up rows; N = tokens; K = 32 columns, two MMAs). The warps' sums meet in shared memory.
 //   Phase 2 (M = 16 hidden columns, N = tokens, K = 16 rows): the warp's own columns. y stays in the accumulators for the whole task.
