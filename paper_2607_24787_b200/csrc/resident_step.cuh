@@ -24,7 +24,7 @@
 // CTA (which owns no columns where there are fewer than 16 a CTA) while the others exchange the hidden row.
 //
 // Registers: nine or ten warps leave a thread 168, sixteen 128. Instances that spill: hidden 1280 of bf16 (68 bytes stored and loaded), hidden 1792 and
-// 2048 of 4 bits (116 / 148 and 128 / 160); 12 bytes at 1280 of 4 bits.
+// 2048 of 4 bits (116 / 148 and 128 / 160); 16 bytes at 1280 of 4 bits.
 //
 // The CTAs wait for one another, so the launch is cooperative (one CTA per SM, all resident or none). Every wait is
 // bounded: a CTA that gives up raises a flag that the others' waits look at, and all of them return with nothing in flight.
@@ -367,9 +367,13 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
 
         // ---- Top-K; then the first weight copies go out, and the routing weights are computed behind them ----
         int sel = 0, top_key = 0;           // lane k: the k-th expert; key of the first
-        // Up to 128 experts every warp ranks for itself. (Two threads an expert counting what comes before it, and a barrier: 0.9 us of a layer with 128 experts, 0.5 with 64; this takes 0.6.)
-        if (n <= kTopKeys * 32) {
-            if (Q4 || wi < nw) sel = warp_top_k(n, a.K, lane, [&](int e) { return reinterpret_cast<const int*>(zs)[e]; }, top_key);
+        // Up to 64 experts, and up to 128 of 4 bits, every warp ranks for itself; else two threads an expert count what comes before it. Whole steps, us a
+        // layer, counting : every warp, four keys a lane : two keys: DeepSeek shape (6 of 64) 15.7 : 15.5 : 15.4, 1024 x 512 (4 of 64) 10.0 : 10.2 : 9.95,
+        // 512 x 768 (6 and a shared one of 64) 9.2 : 9.5 : 9.2, 256 x 512 (6 of 64) 6.8 : 7.25 : 7.0; Qwen3 shape (8 of 128) 20.95 : 21.05.
+        constexpr int kFew = 64;
+        auto key_of = [&](int e) { return reinterpret_cast<const int*>(zs)[e]; };
+        if (n <= kFew || (Q4 && n <= kTopKeys * 32)) {
+            if (Q4 || wi < nw) sel = !Q4 || n <= kFew ? warp_top_k<kFew / 32>(n, a.K, lane, key_of, top_key) : warp_top_k<kTopKeys>(n, a.K, lane, key_of, top_key);
         } else {                            // two threads an expert count what comes before it
             const int half_n = (n / 2) & ~3;
             for (int u0 = 0; u0 < 2 * n; u0 += kStepThreads) {

@@ -131,20 +131,20 @@ __device__ __forceinline__ int rank_of_key(const int* k, int n, int e) {
     return c0 + c1 + c2 + c3;
 }
 
-// The K largest of n <= 32 * kTopKeys keys, equal ones by their ids, by one warp: the lanes hold runs of consecutive keys, largest first, and a round takes
+// The K largest of n <= 32 * KEYS keys, equal ones by their ids, by one warp: the lanes hold runs of consecutive keys, largest first, and a round takes
 // the largest of all. Returns the k-th in lane k and the key of the first.
-constexpr int kTopKeys = 4;
-template <typename F>
+constexpr int kTopKeys = 4;                 // most keys of a lane
+template <int KEYS, typename F>
 __device__ __forceinline__ int warp_top_k(int n, int K, int lane, F key_of, int& first) {
     const int per = (n + 31) / 32;
-    int key[kTopKeys], id[kTopKeys], sel = 0;
+    int key[KEYS], id[KEYS], sel = 0;
 #pragma unroll
-    for (int i = 0; i < kTopKeys; ++i) {
+    for (int i = 0; i < KEYS; ++i) {
         id[i] = lane * per + i;
         key[i] = i < per && id[i] < n ? key_of(id[i]) : INT_MIN;
     }
 #pragma unroll
-    for (int i = 1; i < kTopKeys; ++i)         // (stable)
+    for (int i = 1; i < KEYS; ++i)         // (stable)
 #pragma unroll
         for (int j = i; j > 0; --j)
             if (key[j] > key[j - 1]) {
@@ -160,8 +160,8 @@ __device__ __forceinline__ int warp_top_k(int n, int K, int lane, F key_of, int&
         if (lane == k) sel = e;
         if (lane == from) {
 #pragma unroll
-            for (int i = 0; i + 1 < kTopKeys; ++i) { key[i] = key[i + 1]; id[i] = id[i + 1]; }
-            key[kTopKeys - 1] = INT_MIN;
+            for (int i = 0; i + 1 < KEYS; ++i) { key[i] = key[i + 1]; id[i] = id[i + 1]; }
+            key[KEYS - 1] = INT_MIN;
         }
     }
     return sel;
@@ -515,7 +515,7 @@ router_adapter_kernel(const __grid_constant__ RouterArgs a) {
         if (n <= 32 * kTopKeys) {                 // one warp ranks (128 threads that count what comes before their expert take 1.1 - 1.5 us, and a barrier)
             if (wi == 0) {
                 int first;
-                const int e = warp_top_k(n, a.K, lane, [&](int i) { return reinterpret_cast<const int*>(zs)[i]; }, first);
+                const int e = warp_top_k<kTopKeys>(n, a.K, lane, [&](int i) { return reinterpret_cast<const int*>(zs)[i]; }, first);
                 const float p = lane < a.K ? ps[e] : 0.f;
                 float tot = 0.f;
                 for (int k = 0; k < a.K; ++k) tot += __shfl_sync(0xffffffffu, p, k);
