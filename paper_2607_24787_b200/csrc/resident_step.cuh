@@ -38,7 +38,8 @@ namespace spm {
 
 // Warps of a CTA: as many as the GEMV may take (those it does not use only route). Rows of 9216 bytes and more leave it eight at most,
 // whose threads then have 255 registers. Rows of five segments have one more than the GEMV takes: the 320 quads of a hidden row of 1280 bf16 then are
-// one a thread (DeepSeek shape 15.8 -> 15.45 us a layer; twelve warps 15.8. Ten or twelve warps at fewer segments: within 2 % either way.)
+// one a thread (DeepSeek shape 15.8 -> 15.45 us a layer; twelve warps 15.8. Ten or twelve warps at fewer segments: within 2 % either way). fp32 rows of five
+// segments, 640 columns, have half as many quads and take as long with nine warps (8.93 : 8.91 us a layer, 512 rows, 4 of 64).
 constexpr int step_warps(int nseg, bool q4) { return q4 ? q4_warps(nseg) : nseg >= 6 ? 8 : nseg == 5 ? kFfnMaxWarps + 1 : kFfnMaxWarps; }
 constexpr int kStatusStepTimeout = 16;            // status bit (1 to 8: expert and routing kernels)
 constexpr int kStepCols = 16;                     // columns of the hidden row that an owner adds up
