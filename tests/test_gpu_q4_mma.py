@@ -442,13 +442,14 @@ def test_every_number_of_tokens_an_expert_on_both_kernels():
         m.close()
 
 
-@pytest.mark.parametrize("choice", [1, 2])
-def test_waves_and_host_free_steps_on_both_kernels(choice):
+# (choice, hidden, inter, experts, top-k, slots): the last with 148 tasks and more in a wave, some of which fall to two CTAs
+@pytest.mark.parametrize("choice,hidden,inter,n,k,few", [(1, 768, 384, 12, 4, 5), (2, 768, 384, 12, 4, 5), (2, 512, 1024, 40, 8, 30)])
+def test_waves_and_host_free_steps_on_both_kernels(choice, hidden, inter, n, k, few):
     """A small cache (waves, copies, device-side waits) and a context that holds every expert give the same bits, launched and replayed."""
-    cfg = make(768, 384, 12, 4, batch=9, layers=3)
+    cfg = make(hidden, inter, n, k, batch=9, layers=3)
     h = torch.randn(3, 9, cfg.hidden, generator=torch.Generator(device="cuda").manual_seed(11), device="cuda")
     outs = []
-    for slots, wait in ((5, 0), (5, 1), (12, 0)):
+    for slots, wait in ((few, 0), (few, 1), (n, 0)):
         m = build(cfg.replace(slots=slots))
         m.test_grouped_q4(choice)
         m.set_device_wait(wait)
@@ -465,6 +466,7 @@ def test_waves_and_host_free_steps_on_both_kernels(choice):
 GIVE_UP = {          # (shape, slots, batch, batched kernel)
     "one_token": ((1280, 896, 16, 6, 2), 8, 1, 0), "one_token_widest": ((2048, 333, 16, 4), 5, 1, 0),
     "batched_mma": ((2048, 256, 12, 8), 8, 16, 2), "batched_tcgen05": ((2048, 256, 12, 8), 8, 16, 1),
+    "batched_mma_split": ((512, 1024, 40, 8), 30, 16, 2),       # (240 tasks in a full wave: CTAs that go on from what another has begun)
 }
 
 
