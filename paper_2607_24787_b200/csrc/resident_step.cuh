@@ -368,13 +368,16 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
 
         // ---- Top-K; then the first weight copies go out, and the routing weights are computed behind them ----
         int sel = 0, top_key = 0;           // lane k: the k-th expert; key of the first
-        // Up to 64 experts, and up to 128 of 4 bits, every warp ranks for itself; else two threads an expert count what comes before it. Whole steps, us a
-        // layer, counting : every warp, four keys a lane : two keys: DeepSeek shape (6 of 64) 15.7 : 15.5 : 15.4, 1024 x 512 (4 of 64) 10.0 : 10.2 : 9.95,
-        // 512 x 768 (6 and a shared one of 64) 9.2 : 9.5 : 9.2, 256 x 512 (6 of 64) 6.8 : 7.25 : 7.0; Qwen3 shape (8 of 128) 20.95 : 21.05.
-        constexpr int kFew = 64;
+        // Every warp ranks for itself, or two threads an expert count what comes before it, and a barrier. The first pays for 4 bits, whose rows are then looked up
+        // ahead, for fp32 rows of 1024 (both up to 128 experts), and with ten warps (up to 64; of 128 either takes as long); elsewhere it is the longer way to
+        // the first copies. Whole steps, us a layer, counting : every warp with two keys a lane (with four): DeepSeek shape (6 of 64) 15.7 : 15.4 (15.5),
+        // 1280 x 512 (4 of 24) 11.2 : 11.0; 512 x 768 (6 and a shared one of 64) 9.2 : 9.2 (9.5), 768 x 512 (6 of 64) 9.2 : 9.3 (9.4), 256 x 512 (6 of 64)
+        // 6.8 : 7.0 (7.25); fp32 1024 x 200 (8 of 128) 9.9 : (9.5), 1024 x 128 (2 of 16) 6.7 : (6.6), 896 x 200 (8 of 128) 9.4 : (9.5), 768 x 128 (2 of 16) 6.6 : (6.8).
+        constexpr bool kWideFp32 = sizeof(WT) == 4 && NSEG == 8;
+        constexpr int kFew = 64, kRanked = Q4 || kWideFp32 ? kTopKeys * 32 : NSEG == 5 ? kFew : 0;
         auto key_of = [&](int e) { return reinterpret_cast<const int*>(zs)[e]; };
-        if (n <= kFew || (Q4 && n <= kTopKeys * 32)) {
-            if (Q4 || wi < nw) sel = !Q4 || n <= kFew ? warp_top_k<kFew / 32>(n, a.K, lane, key_of, top_key) : warp_top_k<kTopKeys>(n, a.K, lane, key_of, top_key);
+        if (kRanked > 0 && n <= kRanked) {
+            if (Q4 || wi < nw) sel = kRanked <= kFew || (Q4 && n <= kFew) ? warp_top_k<kFew / 32>(n, a.K, lane, key_of, top_key) : warp_top_k<kTopKeys>(n, a.K, lane, key_of, top_key);
         } else {                            // two threads an expert count what comes before it
             const int half_n = (n / 2) & ~3;
             for (int u0 = 0; u0 < 2 * n; u0 += kStepThreads) {

@@ -72,7 +72,8 @@ def test_one_kernel_gives_the_bits_of_host_driven_steps(name, policy):
 
 
 @pytest.mark.parametrize("base,n,k", [("tiny", 3, 3), ("tiny", 32, 2), ("bf16_nine_warps", 97, 6), ("q4_widest", 128, 8), ("tiny", 129, 4),
-                                      ("tiny", 33, 3), ("tiny", 64, 4), ("tiny", 65, 2), ("bf16_nine_warps", 64, 6), ("q4_widest", 63, 5), ("q4_widest", 65, 8)])
+                                      ("tiny", 33, 3), ("tiny", 64, 4), ("tiny", 65, 2), ("bf16_nine_warps", 64, 6), ("q4_widest", 63, 5), ("q4_widest", 65, 8),
+                                      ("fp32_widest", 128, 4), ("fp32_widest", 129, 4), ("bf16_nine_warps", 65, 2)])
 def test_equal_logits_go_to_the_lower_id(base, n, k):
     """Experts with one and the same router row, on both sides of the number that a warp ranks by itself: the lowest ids of the largest logit,
     in order, as in host-driven steps."""
