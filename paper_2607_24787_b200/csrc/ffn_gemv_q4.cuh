@@ -74,9 +74,10 @@ struct Q4Ring {
             fence_barrier_init();
         }
     }
-    // The warp's rows (warp, warp + NW) of `count` tiles from `tile` on; row_at(row), called by the whole warp, is null for rows that are not there. The
-    // lanes look the rows up side by side, one elected lane asks for them (lanes that ask side by side are taken one by one). `waited`: row_at waits for arrivals, which
-    // the lane that waited has seen, but the one that asks reads the bytes: the barrier and the fence hand them on.
+    // The warp's rows (warp, warp + NW) of `count` tiles from `tile` on; row_at(row), called by the whole warp, is null for rows that are
+    // not there. The lanes look the rows up side by side, one elected lane asks for them (lanes that ask side by side are taken one by
+    // one). `waited`: row_at waits for arrivals, which the lane that waited has seen, but the one that asks reads the bytes: the barrier
+    // and the fence hand them on.
     template <typename F>
     __device__ __forceinline__ void fill(int tile, int count, int warp, int lane, uint32_t bytes, bool waited, F row_at) {
         constexpr int kPer = q4_rows_per_warp(NW);
@@ -220,7 +221,8 @@ __device__ __forceinline__ bool q4_tiles(Q4Ring<NW>& ring, const uint32_t (&x)[G
             // An infinite scale times a part that is zero is a NaN where the scale times the sum is an infinity.
             for (int u = 0; u < nt; ++u) {
                 take(u);
-                if (__any_sync(0xffffffffu, !isfinite(a0 * 0.f + a1 * 0.f + a2 * 0.f + a3 * 0.f))) phase1(std::true_type{}, std::integral_constant<int, 2>{}, u);       // (so in all warps or in none)
+                if (__any_sync(0xffffffffu, !isfinite(a0 * 0.f + a1 * 0.f + a2 * 0.f + a3 * 0.f)))       // (so in all warps or in none)
+                    phase1(std::true_type{}, std::integral_constant<int, 2>{}, u);
             }
             __syncthreads();
             activations();

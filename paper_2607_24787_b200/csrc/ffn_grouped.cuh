@@ -25,12 +25,11 @@
 // counter, by whichever CTA is free: a chunk's output tiles are its own and are computed by the same
 // sequence of MMAs whoever runs it, so results do not depend on who took what. A^T travels from the
 // CTA that ran P1 to the CTA(s) that run P2 through a 16 KB slot of global memory (L2-resident)
-// guarded by a per-unit arrival counter: the P1 epilogue warps store their rows, fence, and bump the
-// counter; the P2 side's producer warp polls it (bounded), then pulls the slot into shared memory
-// with one bulk copy. Every CTA finishes its P1 tasks before it takes its first chunk, so no CTA
-// ever waits for a counter while its owner waits for it. The host cuts the chunks finer towards the
-// end of the list (gg_plan_chunks) so that all CTAs finish together; without a list gg_cut_task does so. The producer warp tells the other warps of its CTA what it took through a small queue
-// in shared memory.
+// guarded by a per-unit arrival counter: the P1 epilogue warps store their rows, fence, and bump the counter; the P2 side's producer warp
+// polls it (bounded), then pulls the slot into shared memory with one bulk copy. Every CTA finishes its P1 tasks before it takes its first
+// chunk, so no CTA ever waits for a counter while its owner waits for it. The host cuts the chunks finer towards the end of the list
+// (gg_plan_chunks) so that all CTAs finish together; without a list gg_cut_task does so. The producer warp tells the other warps of its CTA
+// what it took through a small queue in shared memory.
 // One warp issues TMA, one thread issues tcgen05.mma, four warps run the epilogues;
 // all of them talk through mbarriers, every wait is bounded and an abort flag lets the whole CTA
 // leave together (freeing its TMEM) if a wait ever gives up. No multicast anywhere.
@@ -81,10 +80,10 @@ struct GgWait {
 constexpr int kGgActReady = 4;           // arrivals (one per epilogue warp) that complete a unit's A^T
 constexpr int kGgQueue = 4;              // tasks the producer warp may be ahead of the other warps
 
-// P2 task `idx` of a plan that is made on the device, where no list is cut: the units in order, the last `cut` / q of them in more than q parts,
-// of kGgMinChunk d-tiles at least. unit < 0 past the last task. With whole units the CTAs that took one last left the others idle for up to a third of
-// a unit's time. cut = one unit a CTA; us a layer of the Qwen3 shape, whole units / grid / 2 : grid : 2 grid: 5 sequences 81.2 / 78.0 / 77.6 / 79.3,
-// 64 sequences 221 / 218 / 219 / 221, 64 of 24 experts 96.3 / 93.6 / 90.8 / 90.5.
+// P2 task `idx` of a plan that is made on the device, where no list is cut: the units in order, the last `cut` / q of them in more than q
+// parts, of kGgMinChunk d-tiles at least. unit < 0 past the last task. With whole units the CTAs that took one last left the others idle
+// for up to a third of a unit's time. cut = one unit a CTA; us a layer of the Qwen3 shape, whole units / grid / 2 : grid : 2 grid: 5
+// sequences 81.2 / 78.0 / 77.6 / 79.3, 64 sequences 221 / 218 / 219 / 221, 64 of 24 experts 96.3 / 93.6 / 90.8 / 90.5.
 __host__ __device__ inline GgTask gg_cut_task(int idx, int n_units, int n_dt, int cut) {
     const int most = n_dt / kGgMinChunk > 1 ? n_dt / kGgMinChunk : 1;
     int u = 0;
@@ -586,8 +585,10 @@ inline size_t ffn_grouped_smem() {
            2 * kGgQueue * sizeof(uint64_t) + kGgQueue * sizeof(GgTask);
 }
 
-// One token row as bf16, by the kGgPairThreads threads of a block, in two halves: a thread's loads, which need not know where the row goes, and its stores.
-// (The loads ahead of the counting, and the residual's ahead of the sums in gg_combine_kernel: 2.7 us a layer at 5 and 4.6 at 64 sequences of the Qwen3 shape.)
+// One token row as bf16, by the kGgPairThreads threads of a block, in two halves: a thread's loads, which need not know where the row goes,
+// and its stores.
+// (The loads ahead of the counting, and the residual's ahead of the sums in gg_combine_kernel: 2.7 us a layer at 5 and 4.6 at 64 sequences
+// of the Qwen3 shape.)
 constexpr int kGgPairThreads = 128;
 struct GgRowCopy {
     static constexpr int kChunks = 2;          // of eight columns a thread: hidden <= 2048

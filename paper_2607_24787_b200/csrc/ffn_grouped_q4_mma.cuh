@@ -8,18 +8,19 @@
 // host-free step of that shape: 197 -> 146 us (HBM time of its experts: 49; 142 with exact weights and the scale on the activations,
 // which rounds elsewhere than the tcgen05 kernel: outputs of 64 sequences then moved by 1e-2 where a near-tied Top-K choice tipped), 133 with
 // TMA boxes and split tasks (below), 125 with shorter routing, gather and combine kernels around it.
-// What bounds it now: instruction issue and dependent-issue latency, 99,000 instructions a scheduler at 0.56 a cycle; the packed bf16 multiply-adds of the
-// unpacking run at half rate (FMA pipe 45 %, ALU 42 % of active cycles).
+// What bounds it now: instruction issue and dependent-issue latency, 99,000 instructions a scheduler at 0.56 a cycle; the packed bf16
+// multiply-adds of the unpacking run at half rate (FMA pipe 45 %, ALU 42 % of active cycles).
 //
 // Work. A task is 128 intermediate rows of an expert (GgUnit) for up to kMqTokens of its tokens; CTA b runs the tasks b, b + grid, ...
 // of all experts in order (a hot expert's runs of tokens go to different CTAs), but for the last one to two tasks a CTA, which are split
-// evenly by tiles. A task that falls to two CTAs is begun by the first of them ahead of all else, which leaves its sums, unrounded, where the result goes, and
-// finished by the second after all else: a chain of sums is the same whoever adds, so outputs have the same bits. (760 tasks of 64 sequences of the
-// Qwen3 shape on 148 CTAs: six for some, where an even share is 5.1; 137.5 -> 133 us a layer; 16 sequences 87.6 -> 82, 8: 66.5 -> 60.3. 64 of 60
-// experts lose 1 %, two sequences, which give no CTA a second task, 0.6 us.)
-// Tasks are split, too, where the kernel waits for copies of experts. What a CTA begins first may then be of an expert that is on its way, and holds up the
-// rest; but so may any task of a list in order, and a wave's copies are one arrival. Offloaded steps of the Qwen3 shape with device-side waits, us a
-// layer, split : in order: 4 sequences, 120 slots 109 : 115, 16 sequences, 96 slots 997 : 1004, 64 sequences, 32 slots 4982 : 4999.
+// evenly by tiles. A task that falls to two CTAs is begun by the first of them ahead of all else, which leaves its sums, unrounded, where
+// the result goes, and finished by the second after all else: a chain of sums is the same whoever adds, so outputs have the same bits. (760
+// tasks of 64 sequences of the Qwen3 shape on 148 CTAs: six for some, where an even share is 5.1; 137.5 -> 133 us a layer; 16 sequences
+// 87.6 -> 82, 8: 66.5 -> 60.3. 64 of 60 experts lose 1 %, two sequences, which give no CTA a second task, 0.6 us.)
+// Tasks are split, too, where the kernel waits for copies of experts. What a CTA begins first may then be of an expert that is on its way,
+// and holds up the rest; but so may any task of a list in order, and a wave's copies are one arrival. Offloaded steps of the Qwen3 shape
+// with device-side waits, us a layer, split : in order: 4 sequences, 120 slots 109 : 115, 16 sequences, 96 slots 997 : 1004, 64 sequences,
+// 32 slots 4982 : 4999.
 // A task goes through its rows in tiles of 16; the warps split the columns in groups of 32 (one scale), GB consecutive groups a warp.
 //   Phase 1 (M = 16 gate rows, then 16 up rows; N = tokens; K = 32 columns, two MMAs). The warps' sums meet in shared memory.
 //   Phase 2 (M = 16 hidden columns, N = tokens, K = 16 rows): the warp's own columns. y stays in the accumulators for the whole task.
@@ -199,8 +200,8 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
     }
     __syncthreads();
     const int n_all = n_exp > 0 ? runs[n_exp] * n_jt : 0, G = int(gridDim.x);
-    // Rounds of whole tasks, then the tiles s .. e of the tasks from `split` on: a head (the last of these tasks, begun here), which goes first, whole
-    // tasks, a tail (the first of them, begun by the CTA before), which goes last.
+    // Rounds of whole tasks, then the tiles s .. e of the tasks from `split` on: a head (the last of these tasks, begun here), which goes
+    // first, whole tasks, a tail (the first of them, begun by the CTA before), which goes last.
     const int c = int(blockIdx.x), rounds = max(n_all / G - 1, 0), split = rounds * G;
     int s = 0, e = c < n_all ? kMqTiles : 0, first = c;
     if (n_all >= G) {
@@ -295,8 +296,8 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
     bool dead = false;
     int st1 = 0, st2 = 0;
     uint32_t ph1 = 0, ph2 = 0;
-    // Tile k is tile k % 8 of the CTA's task k / 8: a head counts as the last tiles of its eight, so that all tasks end at multiples of eight but the tail,
-    // the last, which ends with the loop.
+    // Tile k is tile k % 8 of the CTA's task k / 8: a head counts as the last tiles of its eight, so that all tasks end at multiples of
+    // eight but the tail, the last, which ends with the loop.
     const int k0 = head ? kMqTiles - e % kMqTiles : 0, k1 = k0 + n_tiles;
     auto finish = [&](int task, float unscale) {            // a lane has four consecutive columns of two tokens
         const MqTask kk = tasks[task];
@@ -304,8 +305,12 @@ ffn_grouped_q4_mma_kernel(const __grid_constant__ CUtensorMap rowmap, const __gr
         float* out = a.partial + (size_t(kk.jt_n >> 4) * a.rows_cap + kk.row) * D + grp0 * 32 + g * 4;
 #pragma unroll
         for (int i = 0; i < GB; ++i) {
-            if (2 * t < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t) * D + i * 32) = make_float4(y[i][0][0] * unscale, y[i][0][2] * unscale, y[i][1][0] * unscale, y[i][1][2] * unscale);
-            if (2 * t + 1 < n_tok) *reinterpret_cast<float4*>(out + size_t(2 * t + 1) * D + i * 32) = make_float4(y[i][0][1] * unscale, y[i][0][3] * unscale, y[i][1][1] * unscale, y[i][1][3] * unscale);
+            if (2 * t < n_tok)
+                *reinterpret_cast<float4*>(out + size_t(2 * t) * D + i * 32) =
+                    make_float4(y[i][0][0] * unscale, y[i][0][2] * unscale, y[i][1][0] * unscale, y[i][1][2] * unscale);
+            if (2 * t + 1 < n_tok)
+                *reinterpret_cast<float4*>(out + size_t(2 * t + 1) * D + i * 32) =
+                    make_float4(y[i][0][1] * unscale, y[i][0][3] * unscale, y[i][1][1] * unscale, y[i][1][3] * unscale);
         }
     };
     for (int k = k0; k <= k1 && n_tiles > 0; ++k) {

@@ -443,8 +443,9 @@ ffn_multi_kernel(const __grid_constant__ MtArgs a, const int n_stages) {
                 float v;
                 const float* from = m_at + (i1 & 1) * (kMtWarps * 128);
                 if constexpr (NS == 3) {
-                    // Pairs first: a chain over more warps rounds more often. Error against 64 bits, mean of 22 shapes: chains over eight warps 2.151e-7, over
-                    // as many as now 2.159e-7 (3 % more on some shapes), in pairs 2.125e-7; and a shorter chain of latencies (0.5 us a layer).
+                    // Pairs first: a chain over more warps rounds more often. Error against 64 bits, mean of 22 shapes: chains over eight
+                    // warps 2.151e-7, over as many as now 2.159e-7 (3 % more on some shapes), in pairs 2.125e-7; and a shorter chain of
+                    // latencies (0.5 us a layer).
                     float p[kMtWarps / 2];
 #pragma unroll
                     for (int i = 0; i < kMtWarps / 2; ++i) p[i] = from[i * 128];
@@ -677,8 +678,8 @@ static __global__ void mt_combine_kernel(const __grid_constant__ MtCombineArgs a
     if (a.clock && threadIdx.x == 0) atomicMin(a.clock, global_timer_ns());
     const int D = a.D, t = blockIdx.y, c = threadIdx.x & 31, k = threadIdx.x >> 5;
     const int d = (blockIdx.x * 32 + c) * 4;
-    // (the number of entries and the residual are on their way with the pair's place: where they are needed they would cost a latency each: 0.1 - 0.8 us a
-    // layer, fp32 1024 x 250 49 -> 47.6)
+    // (the number of entries and the residual are on their way with the pair's place: where they are needed they would cost a latency each:
+    // 0.1 - 0.8 us a layer, fp32 1024 x 250 49 -> 47.6)
     const int32_t code = a.map[4 + 2 * (t * SPM_MAX_TOPK + k)], entries = a.map[0];
     float* hp = a.h + size_t(t) * D + d;
     const bool mine = k == 0 && d < D, vec = (reinterpret_cast<uintptr_t>(hp) & 15) == 0;       // the caller's rows may start at any float (spm_moe_ffn)

@@ -23,8 +23,8 @@
 // outputs have the same bits as host-driven steps. The adapter's ranking, which only the host reads, is done by the last
 // CTA (which owns no columns where there are fewer than 16 a CTA) while the others exchange the hidden row.
 //
-// Registers: nine or ten warps leave a thread 168, sixteen 128. Instances that spill: hidden 1280 of bf16 (68 bytes stored and loaded), hidden 1792 and
-// 2048 of 4 bits (116 / 148 and 128 / 160); 16 bytes at 1280 of 4 bits.
+// Registers: nine or ten warps leave a thread 168, sixteen 128. Instances that spill: hidden 1280 of bf16 (68 bytes stored and loaded),
+// hidden 1792 and 2048 of 4 bits (116 / 148 and 128 / 160); 16 bytes at 1280 of 4 bits.
 //
 // The CTAs wait for one another, so the launch is cooperative (one CTA per SM, all resident or none). Every wait is
 // bounded: a CTA that gives up raises a flag that the others' waits look at, and all of them return with nothing in flight.
@@ -37,9 +37,10 @@
 namespace spm {
 
 // Warps of a CTA: as many as the GEMV may take (those it does not use only route). Rows of 9216 bytes and more leave it eight at most,
-// whose threads then have 255 registers. Rows of five segments have one more than the GEMV takes: the 320 quads of a hidden row of 1280 bf16 then are
-// one a thread (DeepSeek shape 15.8 -> 15.45 us a layer; twelve warps 15.8. Ten or twelve warps at fewer segments: within 2 % either way). fp32 rows of five
-// segments, 640 columns, have half as many quads and take as long with nine warps (8.93 : 8.91 us a layer, 512 rows, 4 of 64).
+// whose threads then have 255 registers. Rows of five segments have one more than the GEMV takes: the 320 quads of a hidden row of 1280
+// bf16 then are one a thread (DeepSeek shape 15.8 -> 15.45 us a layer; twelve warps 15.8. Ten or twelve warps at fewer segments: within 2 %
+// either way). fp32 rows of five segments, 640 columns, have half as many quads and take as long with nine warps (8.93 : 8.91 us a layer,
+// 512 rows, 4 of 64).
 constexpr int step_warps(int nseg, bool q4) { return q4 ? q4_warps(nseg) : nseg >= 6 ? 8 : nseg == 5 ? kFfnMaxWarps + 1 : kFfnMaxWarps; }
 constexpr int kStatusStepTimeout = 16;            // status bit (1 to 8: expert and routing kernels)
 constexpr int kStepCols = 16;                     // columns of the hidden row that an owner adds up
@@ -368,16 +369,19 @@ resident_step_kernel(const __grid_constant__ StepArgs a) {
 
         // ---- Top-K; then the first weight copies go out, and the routing weights are computed behind them ----
         int sel = 0, top_key = 0;           // lane k: the k-th expert; key of the first
-        // Every warp ranks for itself, or two threads an expert count what comes before it, and a barrier. The first pays for 4 bits, whose rows are then looked up
-        // ahead, for fp32 rows of 1024 (both up to 128 experts), and with ten warps (up to 64; of 128 either takes as long); elsewhere it is the longer way to
-        // the first copies. Whole steps, us a layer, counting : every warp with two keys a lane (with four): DeepSeek shape (6 of 64) 15.7 : 15.4 (15.5),
-        // 1280 x 512 (4 of 24) 11.2 : 11.0; 512 x 768 (6 and a shared one of 64) 9.2 : 9.2 (9.5), 768 x 512 (6 of 64) 9.2 : 9.3 (9.4), 256 x 512 (6 of 64)
-        // 6.8 : 7.0 (7.25); fp32 1024 x 200 (8 of 128) 9.9 : (9.5), 1024 x 128 (2 of 16) 6.7 : (6.6), 896 x 200 (8 of 128) 9.4 : (9.5), 768 x 128 (2 of 16) 6.6 : (6.8).
+        // Every warp ranks for itself, or two threads an expert count what comes before it, and a barrier. The first pays for 4 bits, whose
+        // rows are then looked up ahead, for fp32 rows of 1024 (both up to 128 experts), and with ten warps (up to 64; of 128 either takes
+        // as long); elsewhere it is the longer way to the first copies. Whole steps, us a layer, counting : every warp with two keys a lane
+        // (with four): DeepSeek shape (6 of 64) 15.7 : 15.4 (15.5), 1280 x 512 (4 of 24) 11.2 : 11.0; 512 x 768 (6 and a shared one of 64)
+        // 9.2 : 9.2 (9.5), 768 x 512 (6 of 64) 9.2 : 9.3 (9.4), 256 x 512 (6 of 64) 6.8 : 7.0 (7.25); fp32, four keys, 1024 x 200 (8 of
+        // 128) 9.9 : 9.5, 1024 x 128 (2 of 16) 6.7 : 6.6, 896 x 200 (8 of 128) 9.4 : 9.5, 768 x 128 (2 of 16) 6.6 : 6.8.
         constexpr bool kWideFp32 = sizeof(WT) == 4 && NSEG == 8;
         constexpr int kFew = 64, kRanked = Q4 || kWideFp32 ? kTopKeys * 32 : NSEG == 5 ? kFew : 0;
         auto key_of = [&](int e) { return reinterpret_cast<const int*>(zs)[e]; };
         if (kRanked > 0 && n <= kRanked) {
-            if (Q4 || wi < nw) sel = kRanked <= kFew || (Q4 && n <= kFew) ? warp_top_k<kFew / 32>(n, a.K, lane, key_of, top_key) : warp_top_k<kTopKeys>(n, a.K, lane, key_of, top_key);
+            if (Q4 || wi < nw)
+                sel = kRanked <= kFew || (Q4 && n <= kFew) ? warp_top_k<kFew / 32>(n, a.K, lane, key_of, top_key)
+                                                           : warp_top_k<kTopKeys>(n, a.K, lane, key_of, top_key);
         } else {                            // two threads an expert count what comes before it
             const int half_n = (n / 2) & ~3;
             for (int u0 = 0; u0 < 2 * n; u0 += kStepThreads) {

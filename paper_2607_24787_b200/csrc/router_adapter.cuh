@@ -131,8 +131,8 @@ __device__ __forceinline__ int rank_of_key(const int* k, int n, int e) {
     return c0 + c1 + c2 + c3;
 }
 
-// The K largest of n <= 32 * KEYS keys, equal ones by their ids, by one warp: the lanes hold runs of consecutive keys, largest first, and a round takes
-// the largest of all. Returns the k-th in lane k and the key of the first.
+// The K largest of n <= 32 * KEYS keys, equal ones by their ids, by one warp: the lanes hold runs of consecutive keys, largest first, and a
+// round takes the largest of all. Returns the k-th in lane k and the key of the first.
 constexpr int kTopKeys = 4;                 // most keys of a lane
 template <int KEYS, typename F>
 __device__ __forceinline__ int warp_top_k(int n, int K, int lane, F key_of, int& first) {
@@ -272,8 +272,9 @@ __device__ __forceinline__ void rank_batch(const RankArgs& a, float* sm) {
 // on its first four warps and the adapter tail (up-projection, softmax, ranking) on the other four.
 // MINB = 1: all registers to one CTA per SM (the fold keeps 40 partial-row quads in flight);
 // MINB = 2: register budget halved so two CTAs share an SM, for batches with more CTAs than SMs.
-// CL: CTAs of a cluster. 32 clusters of eight run at once with two CTAs an SM; more tokens than that take clusters of four, whose CTAs have twice the rows
-// but need no second wave (64 sequences of the Qwen3 shape: 15.4 us from the first leader's start to the last one's end with eight, 9.5 with four).
+// CL: CTAs of a cluster. 32 clusters of eight run at once with two CTAs an SM; more tokens than that take clusters of four, whose CTAs have
+// twice the rows but need no second wave (64 sequences of the Qwen3 shape: 15.4 us from the first leader's start to the last one's end with
+// eight, 9.5 with four).
 template <typename WT, int MINB, int CL>
 __global__ void __launch_bounds__(kRouterThreads, MINB)
 router_adapter_kernel(const __grid_constant__ RouterArgs a) {

@@ -270,8 +270,8 @@ int mt_grid_for(const spm_ctx* c) { return std::min(c->num_sms, kMtMaxCtas); }
 //          512 x 384, 64 tokens 3 + 1 of 96: 104 -> 91 (89)       640 x 735, 31 tokens 7 + 1 of 128: 173 -> 191 (160)
 // Of 124 shapes that it chooses four are slower than with the GEMV, by 2 - 3 %; of those above 64 Mi that it leaves to the GEMV
 // two would gain 7 - 8 %.
-// (All with eight warps a CTA. With as many as launch_multi_g takes now the kernel's steps are 0 - 18 % shorter, so the line errs towards the GEMV; it stays where
-// it is, because the two add in different orders.)
+// (All with eight warps a CTA. With as many as launch_multi_g takes now the kernel's steps are 0 - 18 % shorter, so the line errs towards
+// the GEMV. It has not been drawn again.)
 constexpr size_t kMi = size_t(1) << 20;
 bool multi_pays(const spm_model_cfg& m, int nb) {
     const size_t D = m.hidden, expert = size_t(3) * m.inter * D;
@@ -467,9 +467,10 @@ cudaError_t launch_multi_t(const spm_ctx* c, const MtArgs& a) {
     const int stages = mt_stages(c->row_bytes, std::is_same<WT, float>::value, a.n, a.nb * a.K, NW, &smem);
     return launch_k(kern, dim3(mt_grid_for(c)), dim3(NW * 32), smem, c->compute, true, a, stages);
 }
-// Groups of 32 columns over warps, evenly (but for fp32 rows of 128). A block is a chain of latencies, so more warps of fewer groups each pay until what every
-// warp does once a block outweighs it: 2048 columns, eight warps of eight -> sixteen of four, a layer of 16 sequences 107 -> 98 us; 1280, eight of
-// five -> ten of four 91 -> 87 (twenty of two: 96; 4-bit 111 -> 110, twenty of two 105); bf16 of 512, eight of two 34.2, sixteen of one 35.4 (4-bit 52.1, 51.4).
+// Groups of 32 columns over warps, evenly (but for fp32 rows of 128). A block is a chain of latencies, so more warps of fewer groups each
+// pay until what every warp does once a block outweighs it: 2048 columns, eight warps of eight -> sixteen of four, a layer of 16 sequences
+// 107 -> 98 us; 1280, eight of five -> ten of four 91 -> 87 (twenty of two: 96; 4-bit 111 -> 110, twenty of two 105); bf16 of 512, eight of
+// two 34.2, sixteen of one 35.4 (4-bit 52.1, 51.4).
 // bf16 of 1536 keeps eight of six: the sums of sixteen would cost one of three ring stages.
 template <typename WT>
 cudaError_t launch_multi_g(const spm_ctx* c, const MtArgs& a) {
@@ -543,8 +544,8 @@ cudaError_t launch_grouped_q4_mma_t(const spm_ctx* c, const MqArgs& a) {
 //   64, 8 of 128, 2048: 189 / 125     8, 8 of 128, 2048: 101 / 58     64, 8 of 60, 2048: 131 / 95      64, 8 of 24, 2048:  74 / 83
 //   64, 8 of 128, 1280: 128 / 104     2, 8 of 128, 2048:  50 / 36     32, 4 of 12, 2048:  59 / 40      64, 8 of 12, 2048:  85 / 81
 //   64, 8 of 128,  768:  92 / 83      64, 8 of 128,  512:  71 / 76     64, 8 of 128, 1024: 108 / 91     32, 8 of 24, 2048:  62 / 60
-// (of these the rule takes the slower one for two, 64 sequences of 768 columns and 32 of 24 experts, by 11 and 4 %: its line was drawn before the mma.sync
-// kernel split its last tasks, and the two kernels' outputs differ by the order of sums)
+// (of these the rule takes the slower one for two, 64 sequences of 768 columns and 32 of 24 experts, by 11 and 4 %: its line was drawn
+// before the mma.sync kernel split its last tasks and has not been drawn again)
 bool grouped_q4_mma_pays(const spm_ctx* c, int nb) {
     const spm_model_cfg& m = c->cfg;
     if (m.hidden < 512 || mq_max_tasks(nb, m.top_k, m.n_experts, c->n_jt, c->num_sms) > kMqMaxTasks) return false;      // (rows of 256: never worth it)

@@ -87,8 +87,8 @@ inline bool make_q4_maps(CUtensorMap* nib64, CUtensorMap* sc16, const void* base
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The same blobs as rows [n_slots * I][3 * RB bytes]; a box is `box_rows` rows of one part, `box_bytes` wide (RB, or a little of what follows it with it,
-// which sets the pitch of the rows in shared memory), in elements of 8 bytes: a box has at most 256.
+// The same blobs as rows [n_slots * I][3 * RB bytes]; a box is `box_rows` rows of one part, `box_bytes` wide (RB, or a little of what
+// follows it with it, which sets the pitch of the rows in shared memory), in elements of 8 bytes: a box has at most 256.
 inline bool make_q4_row_map(CUtensorMap* map, const void* base, int D, int I, uint64_t n_slots, uint32_t box_bytes, uint32_t box_rows) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
