@@ -15,9 +15,9 @@
 // One buffer per exchange is enough: a CTA overwrites a word one layer later, when it holds data that every reader of
 // the old word contributed to after reading it.
 //
-// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 15.5 (21): the FFN 11.5 - 13 and 8 - 10 with the slowest SM 2 us
+// A layer of the Qwen3 shape now takes 19.5 us, of the DeepSeek shape 15.3 (21): the FFN 11.5 - 13 and 8 - 10 with the slowest SM 2 us
 // behind the mean, and a chain of latencies of 6 (partial rows 1.4, hidden row 1, norm and dot products 1.5, logits 1.1, Top-K 0.6, first
-// copies 0.5). With 4-bit experts 16.8 and 13.5, 6 and 4.5 of which are the tiles.
+// copies 0.5). With 4-bit experts 16.3 and 13.1, 6 and 4.5 of which are the tiles.
 //
 // The arithmetic, the orders of all sums and the split of the rows are those of router_adapter_kernel and ffn_gemv_kernel, so the
 // outputs have the same bits as host-driven steps. The adapter's ranking, which only the host reads, is done by the last
